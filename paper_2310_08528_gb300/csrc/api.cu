@@ -153,13 +153,24 @@ struct Work {
   DevBuf grad_pair, gd, acts, wpartial;    // backward work memory
   DevBuf fd, dsh, dop;                     // colour and opacity heads: f_d [n][64] (work order),
                                            // deformed SH [n][48] and opacity logits [n]
+  DevBuf yparts, spos, srg, axis, band_pairs;  // frames composited straight from the depth order (direct.cu)
   int cap_color = 0;
   long long cap_pairs = 0;
   long long sort_parts_cap = 0;
   int cap_n = 0, cap_tiles = 0;
 };
 
+void release_work(Work& w) {
+  DevBuf* all[] = {&w.zero, &w.dmeans, &w.dquats, &w.dscales, &w.xy, &w.co, &w.rgb, &w.depth, &w.radius, &w.rect,
+                   &w.offsets, &w.emit_lb, &w.counters, &w.num_pairs, &w.hist, &w.dkeys, &w.dvals, &w.dkeys_alt,
+                   &w.dvals_alt, &w.keys, &w.values, &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges, &w.tile_count,
+                   &w.tile_order, &w.bitmap, &w.sxy, &w.sco, &w.srgb, &w.ts, &w.host_img, &w.grad_pair, &w.gd, &w.acts,
+                   &w.wpartial, &w.fd, &w.dsh, &w.dop, &w.yparts, &w.spos, &w.srg, &w.axis, &w.band_pairs};
+  for (DevBuf* b : all) release(*b);
+}
+
 constexpr int kSortMaxPasses = 8;
+constexpr int kMaxTileRows = 8192 / kTile;  // (valid_cam bounds the image)
 // Largest tile bitmap (one bit per (tile, Gaussian)) a frame bins through; larger
 // frames emit keys and radix-sort them.  At this size clearing and walking the
 // rows costs about as much memory traffic as the sort's passes over ~10 pairs per
@@ -243,6 +254,7 @@ struct fs4d_ctx {
   cudaEvent_t slot_rendered[2] = {}, slot_copied[2] = {};
   unsigned long long* h_pairs = nullptr;  // pinned, [h_pairs_cap]: each frame's pair count
   int h_pairs_cap = 0;
+  unsigned long long* h_band_pairs = nullptr;  // pinned, [kMaxTileRows]: pairs of a frame's bands
   uint32_t spin_limit = kSpinLimit;       // polls of a look-back wait (fs4d_set_wait_limit)
   // frames rendered in bands of tile rows (more pairs than one sort pass counts)
   int band_scene = -1, band_w = 0, band_h = 0, band_hint = 0;  // bands the last such frame used
@@ -250,7 +262,7 @@ struct fs4d_ctx {
   int last_bands = 1;
   long long last_launches = 0;  // kernels the last fs4d_render / fs4d_render_async call launched
   long long band_pairs = (1ll << 30) - 1;  // most pairs one band may hold (fs4d_set_band_pairs)
-  float stage_acc[6] = {};                // stage times summed over a banded frame's passes
+  float stage_acc[6] = {};                // stage times of a frame that went through two passes
   bool stage_acc_valid = false;
 };
 
@@ -613,7 +625,6 @@ struct Env {
   cudaStream_t s;
   uint32_t* status;
   bool timed;
-  int guard_w = 0, guard_h = 0;  // non-zero: the whole frame's size (a band's guard band is the frame's)
 };
 
 Env env_of(fs4d_ctx* c) { return Env{c, &c->w, c->stream, P<uint32_t>(c->status), true}; }
@@ -722,13 +733,13 @@ fs4d_status deform_part(fs4d_ctx* c, Work& w, const FramePart& q, fs4d_precision
   return FS4D_OK;
 }
 
-// Everything of a frame up to (and including) the key emission, over the union of
-// the parts' Gaussians.
-// cull: the tile lists may leave out Gaussians that no pixel of the tile blends
-// (same image; list positions, and so last-contributor indices, differ).
-fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_precision prec,
-                        const fs4d_camera& shape, const fs4d_camera* d_cam, const float* d_t, float t, long long cap,
-                        bool report, bool deform, bool offsets, bool cull = false) {
+// A frame up to its depth order, over the union of the parts' Gaussians: zeroed
+// state, deformation, projection and the sort of the depths.  *dsel: see launch_sort.
+// y_parts: the projection leaves each mean's row to be finished per band of tile
+// rows (ProjectArgs::y_parts).
+fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts, fs4d_precision prec,
+                              const fs4d_camera& shape, const fs4d_camera* d_cam, const float* d_t, float t,
+                              long long cap, bool deform, float2* y_parts, const uint32_t** dsel) {
   fs4d_ctx* c = e.c;
   Work& w = *e.w;
   const cudaStream_t stream = e.s;
@@ -767,10 +778,6 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
       pa.sh = P<float>(w.dsh) + 48 * q.off;
     }
     pa.cam = cam_params(shape);
-    if (e.guard_w > 0) {
-      pa.cam.guard_w = e.guard_w;
-      pa.cam.guard_h = e.guard_h;
-    }
     // world_to_cam applied to X + shift: the translation column absorbs W shift
     for (int r = 0; r < 3; ++r)
       pa.cam.m[4 * r + 3] += pa.cam.m[4 * r] * q.shift[0] + pa.cam.m[4 * r + 1] * q.shift[1] +
@@ -782,12 +789,12 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
     pa.depth_keys = P<unsigned long long>(w.dkeys) + q.off; pa.depth_vals = P<uint32_t>(w.dvals) + q.off;
     pa.index_base = (uint32_t)q.off;
     pa.depth_hist = z.hist;
+    if (y_parts) pa.y_parts = y_parts + q.off;
     FS4D_CUDA(c, launch_project(pa, stream));
   }
   mark(e, 2);
   // Gaussians in (float32 depth, index) order: the emission order
   bool dalt = false;
-  const uint32_t* dsel = nullptr;
   SortWork dsw;
   dsw.hist = z.hist; dsw.lookback = z.dlb; dsw.part_counters = z.counters + 8; dsw.max_parts = z.dparts;
   dsw.prezeroed = true;
@@ -795,8 +802,28 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
   dsw.grid_counter = z.counters + 56;  // (words 0..7 emission, 8..24 this sort, 32..48 the pair sort)
   FS4D_CUDA(c, launch_sort(P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), P<unsigned long long>(w.dkeys_alt),
                            P<uint32_t>(w.dvals_alt), nullptr, N, 0, 32, true, dsw, e.status, stream, &dalt,
-                           &dsel));
+                           dsel));
   mark(e, 3);
+  return FS4D_OK;
+}
+
+// Everything of a frame up to (and including) the key emission, over the union of
+// the parts' Gaussians.
+// cull: the tile lists may leave out Gaussians that no pixel of the tile blends
+// (same image; list positions, and so last-contributor indices, differ).
+fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_precision prec,
+                        const fs4d_camera& shape, const fs4d_camera* d_cam, const float* d_t, float t, long long cap,
+                        bool report, bool deform, bool offsets, bool cull = false) {
+  fs4d_ctx* c = e.c;
+  Work& w = *e.w;
+  const cudaStream_t stream = e.s;
+  const int tx = tiles_of(shape.width), ty = tiles_of(shape.height);
+  const int tile_bits = ceil_log2((long long)tx * ty);
+  const int N = (int)parts_total(parts, n_parts);
+  const uint32_t* dsel = nullptr;
+  const fs4d_status st0 = frame_depth_order(e, parts, n_parts, prec, shape, d_cam, d_t, t, cap, deform, nullptr, &dsel);
+  if (st0 != FS4D_OK) return st0;
+  const FrameZero& z = w.z;
   EmitArgs ea{};
   ea.n = N; ea.order = P<uint32_t>(w.dvals); ea.order_alt = P<uint32_t>(w.dvals_alt); ea.order_sel = dsel;
   ea.depth = P<float>(w.depth); ea.rect = P<int4>(w.rect); ea.tiles_x = tx;
@@ -912,86 +939,149 @@ fs4d_status read_pairs(fs4d_ctx* c, const uint32_t* d_num_pairs, long long* K) {
 }
 
 // One pair-sort pass counts at most 2^30 - 1 pairs (30-bit look-back values).  A
-// frame with more pairs renders in horizontal bands of tile rows: each band is a
-// frame of its own on the same deformed Gaussians, with the camera's principal
+// frame with more pairs renders in horizontal bands of tile rows: each band is an
+// image of its own of the same deformed Gaussians, with the camera's principal
 // point moved by the band's offset (a whole number of tiles, so every pixel keeps
-// its tile), composited into the band's rows of the image.
+// its tile).
 constexpr long long kMaxBandPairs = (1ll << 30) - 1;
 
-// Adds the stage times of the pass that just ended (timing on) to c->stage_acc.
-fs4d_status add_stage_times(fs4d_ctx* c, bool with_deform) {
-  if (!c->timing) return FS4D_OK;
+// Stage times of the frame last recorded (timing on).
+fs4d_status stage_times_of(fs4d_ctx* c, float* ms) {
   FS4D_CUDA(c, cudaEventSynchronize(c->ev[7]));
   const int from[6] = {0, 1, 2, 3, 5, 6}, to[6] = {1, 2, 3, 4, 6, 7};
-  for (int k = with_deform ? 0 : 1; k < 6; ++k) {
-    float ms = 0.f;
-    FS4D_CUDA(c, cudaEventElapsedTime(&ms, c->ev[from[k]], c->ev[to[k]]));
-    c->stage_acc[k] += ms;
-  }
+  for (int k = 0; k < 6; ++k) FS4D_CUDA(c, cudaEventElapsedTime(&ms[k], c->ev[from[k]], c->ev[to[k]]));
   return FS4D_OK;
 }
 
-// Bands of tile rows over the deformed Gaussians already in the work memory.
-// n_bands equal bands, or (reuse) the last banded frame's bands of tile rows, so that
-// frames of one scene and size are cut alike and render alike.
-fs4d_status render_bands(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t, int n_bands,
-                         float* d_image, float* d_t_final, int32_t* d_n_contrib, bool reuse = false) {
-  const int rows = tiles_of(cam->height), tx = tiles_of(cam->width);
-  n_bands = std::max(1, std::min(n_bands, rows));
-  std::vector<std::pair<int, int>> todo;  // tile-row ranges [r0, r1), taken from the back
-  if (reuse)
-    todo.assign(c->band_rows.rbegin(), c->band_rows.rend());
-  else
-    for (int b = n_bands - 1; b >= 0; --b) todo.push_back({rows * b / n_bands, rows * (b + 1) / n_bands});
-  std::vector<std::pair<int, int>> used;
-  long long total = 0;
-  int done = 0;
-  fs4d_status st;
-  const bool cull = !d_n_contrib;  // bands are never saved for the backward
-  Env be = env_of(c);
-  be.guard_w = cam->width;
-  be.guard_h = cam->height;
-  while (!todo.empty()) {
-    const std::pair<int, int> band = todo.back();
-    todo.pop_back();
-    const int r0 = band.first, r1 = band.second;
-    fs4d_camera bc = *cam;
-    bc.height = std::min(cam->height, kTile * r1) - kTile * r0;
-    bc.cy = cam->cy - (float)(kTile * r0);
-    if ((st = ensure_work(c, s->n, tx * (r1 - r0), c->w.cap_pairs)) != FS4D_OK) return st;
-    if ((st = frame_front(be, s, prec, bc, nullptr, nullptr, t, c->w.cap_pairs, false, false, false, cull)) != FS4D_OK)
-      return st;
-    long long K = 0;
-    if ((st = read_pairs(c, c->w.z.num_pairs, &K)) != FS4D_OK) return st;
-    if (K > c->band_pairs) {
-      if (r1 - r0 == 1) return fail(c, FS4D_ERR_CAPACITY, "one tile row of the frame holds more pairs than a band may");
-      const int mid = (r0 + r1) / 2;
-      todo.push_back({mid, r1});
-      todo.push_back({r0, mid});
-      continue;
-    }
-    if (K > c->w.cap_pairs) {
-      if ((st = ensure_work(c, s->n, tx * (r1 - r0), std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
-      if ((st = frame_front(be, s, prec, bc, nullptr, nullptr, t, c->w.cap_pairs, false, false, false, cull)) !=
-          FS4D_OK)
-        return st;
-    }
-    const size_t off = (size_t)kTile * r0 * cam->width;
-    if ((st = frame_back(c, bc, K, d_image + 3 * off, d_t_final ? d_t_final + off : nullptr,
-                         d_n_contrib ? d_n_contrib + off : nullptr)) != FS4D_OK)
-      return st;
-    if ((st = add_stage_times(c, false)) != FS4D_OK) return st;
-    total += K;
-    ++done;
-    used.push_back({r0, r1});
+// Bands [first, first + kMaxBands) of the list, as far as it goes.
+BandTab band_tab(const fs4d_camera* cam, const std::vector<std::pair<int, int>>& bands, size_t first) {
+  BandTab t{};
+  t.n = (int)std::min<size_t>(kMaxBands, bands.size() - first);
+  for (int b = 0; b < t.n; ++b) {
+    t.r0[b] = bands[first + b].first;
+    t.r0[b + 1] = bands[first + b].second;
+    t.cy[b] = cam->cy - (float)(kTile * t.r0[b]);
   }
+  return t;
+}
+
+// Device memory of the frames composited straight from the depth order.
+fs4d_status ensure_direct(fs4d_ctx* c, int n, int tiles_x, int tiles_y) {
+  Work& w = c->w;
+  const size_t m = (size_t)n, bits = 4 * (size_t)(tiles_x + tiles_y) * (size_t)bitmap_words(n);
+  if (w.yparts.bytes >= 8 * m && w.spos.bytes >= 16 * m && w.srg.bytes >= 8 * m && w.axis.bytes >= bits &&
+      w.band_pairs.bytes > 0)
+    return FS4D_OK;
+  FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
+  FS4D_CUDA(c, ensure(w.yparts, 8 * m));
+  FS4D_CUDA(c, ensure(w.spos, 16 * m));
+  FS4D_CUDA(c, ensure(w.srg, 8 * m));
+  FS4D_CUDA(c, ensure(w.axis, bits));
+  FS4D_CUDA(c, ensure(w.band_pairs, 8 * kMaxTileRows));
+  if (!c->h_band_pairs) FS4D_CUDA(c, cudaMallocHost(&c->h_band_pairs, 8 * kMaxTileRows));
+  return FS4D_OK;
+}
+
+// Pair counts of the bands [r0, r1) of tile rows, read back.
+fs4d_status count_bands(fs4d_ctx* c, DirectArgs a, const fs4d_camera* cam, const std::vector<std::pair<int, int>>& bands,
+                        std::vector<long long>& pairs) {
+  unsigned long long* d = P<unsigned long long>(c->w.band_pairs);
+  FS4D_CUDA(c, cudaMemsetAsync(d, 0, 8 * bands.size(), c->stream));
+  for (size_t i = 0; i < bands.size(); i += kMaxBands) {
+    a.bands = band_tab(cam, bands, i);
+    FS4D_CUDA(c, launch_band_pairs(a, d + i, c->stream));
+  }
+  FS4D_CUDA(c, cudaMemcpyAsync(c->h_band_pairs, d, 8 * bands.size(), cudaMemcpyDeviceToHost, c->stream));
+  FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
+  pairs.assign(c->h_band_pairs, c->h_band_pairs + bands.size());
+  return FS4D_OK;
+}
+
+// A frame composited straight from the depth order (direct.cu), in one image or,
+// when its pairs exceed c->band_pairs, in bands of tile rows.  deform: false if the
+// deformed Gaussians are in the work memory already.  Frames of one scene and size
+// are cut alike and so render alike: the bands of the last such frame are used again.
+fs4d_status render_direct(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t, bool deform,
+                          float* d_image, float* d_t_final, int32_t* d_n_contrib) {
+  Work& w = c->w;
+  const Env e = env_of(c);
+  const int rows = tiles_of(cam->height), tx = tiles_of(cam->width);
+  fs4d_status st = ensure_direct(c, s->n, tx, rows);
+  if (st != FS4D_OK) return st;
+  c->last_binning = FS4D_BINNING_SORT;
+  const uint32_t* dsel = nullptr;
+  const FramePart part{s, 0, {0.f, 0.f, 0.f}};
+  if ((st = frame_depth_order(e, &part, 1, prec, *cam, nullptr, nullptr, t, 0, deform, P<float2>(w.yparts), &dsel)) !=
+      FS4D_OK)
+    return st;
+  DirectArgs a{};
+  a.n = s->n; a.order = P<uint32_t>(w.dvals); a.order_alt = P<uint32_t>(w.dvals_alt); a.order_sel = dsel;
+  a.xy = P<float2>(w.xy); a.y_parts = P<float2>(w.yparts); a.rect = P<int4>(w.rect); a.radius = P<int>(w.radius);
+  a.conic_opacity = P<float4>(w.co); a.rgb = P<float>(w.rgb);
+  a.width = cam->width; a.height = cam->height; a.tiles_x = tx;
+  a.words = bitmap_words(s->n);
+  a.cols = P<uint32_t>(w.axis);
+  a.rows = a.cols + (size_t)tx * a.words;
+  a.s_pos = P<float4>(w.spos); a.s_co = P<float4>(w.sco); a.s_rg = P<float2>(w.srg);
+
+  std::vector<std::pair<int, int>> bands;  // tile rows [first, second), top to bottom
+  std::vector<long long> pairs;
+  if (c->band_hint > 1 && c->band_scene == s->id && c->band_w == cam->width && c->band_h == cam->height)
+    bands = c->band_rows;
+  else
+    bands.push_back({0, rows});
+  if ((st = count_bands(c, a, cam, bands, pairs)) != FS4D_OK) return st;
+  if (bands.size() == 1 && pairs[0] > c->band_pairs) {
+    const long long K = std::min<long long>(pairs[0], 0xffffffffll), per = std::max(c->band_pairs / 2, 1ll);
+    const int nb = std::max(1, std::min((int)std::min<long long>((K + per - 1) / per, 1 << 20), rows));
+    bands.clear();
+    for (int b = 0; b < nb; ++b) bands.push_back({rows * b / nb, rows * (b + 1) / nb});
+    if ((st = count_bands(c, a, cam, bands, pairs)) != FS4D_OK) return st;
+  }
+  // a band with more pairs than one may hold is halved
+  for (bool again = true; again;) {
+    again = false;
+    std::vector<std::pair<int, int>> cut;
+    for (size_t i = 0; i < bands.size(); ++i) {
+      const std::pair<int, int> q = bands[i];
+      if (pairs[i] <= c->band_pairs) {
+        cut.push_back(q);
+        continue;
+      }
+      if (q.second - q.first == 1)
+        return fail(c, FS4D_ERR_CAPACITY, "one tile row of the frame holds more pairs than a band may");
+      const int mid = (q.first + q.second) / 2;
+      cut.push_back({q.first, mid});
+      cut.push_back({mid, q.second});
+      again = true;
+    }
+    if (again) {
+      bands = cut;
+      if ((st = count_bands(c, a, cam, bands, pairs)) != FS4D_OK) return st;
+    }
+  }
+  mark(e, 4);
+  mark(e, 5);
+  for (size_t i = 0; i < bands.size(); i += kMaxBands) {
+    a.bands = band_tab(cam, bands, i);
+    FS4D_CUDA(c, launch_axis_bits(a, i == 0, c->stream));
+  }
+  mark(e, 6);
+  for (size_t i = 0; i < bands.size(); i += kMaxBands) {
+    a.bands = band_tab(cam, bands, i);
+    FS4D_CUDA(c, launch_composite_direct(a, d_image, d_t_final, d_n_contrib, c->stream));
+  }
+  mark(e, 7);
+  long long total = 0;
+  for (long long k : pairs) total += k;
   c->last_pairs = total;
-  c->last_bands = done;
-  // the next frame of this scene and size starts with as many bands, unless one would do
-  c->band_scene = s->id; c->band_w = cam->width; c->band_h = cam->height;
-  c->band_hint = total > c->band_pairs ? done : 0;
-  c->band_rows = used;
-  c->stage_acc_valid = c->timing;
+  c->last_bands = (int)bands.size();
+  if (bands.size() > 1) {
+    // the next frame of this scene and size starts with these bands, unless one would do
+    c->band_scene = s->id; c->band_w = cam->width; c->band_h = cam->height;
+    c->band_hint = total > c->band_pairs ? (int)bands.size() : 0;
+    c->band_rows = bands;
+  }
   return FS4D_OK;
 }
 
@@ -1002,21 +1092,12 @@ fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_c
   fs4d_status st = ensure_work(c, s->n, n_tiles, c->w.cap_pairs);
   if (st != FS4D_OK) return st;
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
-  std::fill(c->stage_acc, c->stage_acc + 6, 0.f);
   c->stage_acc_valid = false;
   c->last_bands = 1;
-  if (!offsets && c->band_hint > 1 && c->band_scene == s->id && c->band_w == cam->width && c->band_h == cam->height) {
-    // the last frame of this scene and size needed bands: deform, then bands straight away
-    mark(c, 0);
-    const FramePart part{s, 0, {0.f, 0.f, 0.f}};
-    if ((st = deform_part(c, c->w, part, prec, nullptr, t, c->stream, P<uint32_t>(c->status))) != FS4D_OK) return st;
-    mark(c, 1);
-    if (c->timing) {
-      FS4D_CUDA(c, cudaEventSynchronize(c->ev[1]));
-      FS4D_CUDA(c, cudaEventElapsedTime(&c->stage_acc[0], c->ev[0], c->ev[1]));
-    }
-    return render_bands(c, s, prec, cam, t, c->band_hint, d_image, d_t_final, d_n_contrib, true);
-  }
+  // too many tiles x Gaussians for the tile bitmap, or more pairs than a band may hold last time
+  const bool banded = c->band_hint > 1 && c->band_scene == s->id && c->band_w == cam->width && c->band_h == cam->height;
+  if (!offsets && (banded || (c->binning != FS4D_BINNING_SORT && !use_bitmap(c, c->w, s->n, n_tiles, false))))
+    return render_direct(c, s, prec, cam, t, true, d_image, d_t_final, d_n_contrib);
   // lists may drop Gaussians no pixel of their tile blends unless the frame reports
   // list positions (last contributors) or keeps the backward's pair slots
   const bool cull = !offsets && !d_n_contrib;
@@ -1026,11 +1107,18 @@ fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_c
   if ((st = read_pairs(c, c->w.z.num_pairs, &K)) != FS4D_OK) return st;
   if (K > c->band_pairs) {
     if (offsets) return fail(c, FS4D_ERR_CAPACITY, "a frame saved for the backward must fit one band of tile pairs");
-    if ((st = add_stage_times(c, true)) != FS4D_OK) return st;
-    // K saturates at 2^32 - 1; a band that still holds too many pairs is split again
-    const long long per = std::max(c->band_pairs / 2, 1ll);
-    return render_bands(c, s, prec, cam, t, (int)std::min<long long>((K + per - 1) / per, 1 << 20), d_image,
-                        d_t_final, d_n_contrib);
+    float deform_ms = 0.f;
+    if (c->timing) {
+      FS4D_CUDA(c, cudaEventSynchronize(c->ev[1]));
+      FS4D_CUDA(c, cudaEventElapsedTime(&deform_ms, c->ev[0], c->ev[1]));
+    }
+    st = render_direct(c, s, prec, cam, t, false, d_image, d_t_final, d_n_contrib);
+    if (st == FS4D_OK && c->timing) {  // the deformation is the pass above's
+      if ((st = stage_times_of(c, c->stage_acc)) != FS4D_OK) return st;
+      c->stage_acc[0] = deform_ms;
+      c->stage_acc_valid = true;
+    }
+    return st;
   }
   if (K > c->w.cap_pairs) {
     if ((st = ensure_work(c, s->n, n_tiles, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
@@ -1111,12 +1199,7 @@ fs4d_status fs4d_destroy(fs4d_ctx* c) {
     DeviceGuard g(c->device);
     cudaStreamSynchronize(c->stream);
     for (auto& kv : c->scenes) free_scene(kv.second);
-    Work& w = c->w;
-    DevBuf* all[] = {&w.dmeans, &w.dquats, &w.dscales, &w.xy, &w.co, &w.rgb, &w.depth, &w.radius, &w.rect,
-                     &w.offsets, &w.emit_lb, &w.counters, &w.num_pairs, &w.hist, &w.keys, &w.values,
-                     &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges, &w.tile_count, &w.tile_order, &w.zero, &w.bitmap, &w.sxy, &w.sco, &w.srgb, &w.ts, &w.host_img,
-                     &w.grad_pair, &w.gd, &w.acts, &w.wpartial};
-    for (DevBuf* b : all) release(*b);
+    release_work(c->w);
     release(c->status);
     if (c->h_pinned) cudaFreeHost(c->h_pinned);
     for (int i = 0; i < 8; ++i)
@@ -1132,6 +1215,7 @@ fs4d_status fs4d_destroy(fs4d_ctx* c) {
       if (c->slot_copied[i]) cudaEventDestroy(c->slot_copied[i]);
     }
     if (c->h_pairs) cudaFreeHost(c->h_pairs);
+    if (c->h_band_pairs) cudaFreeHost(c->h_band_pairs);
   }
   delete c;
   return FS4D_OK;
@@ -1602,14 +1686,11 @@ fs4d_status fs4d_stage_times(fs4d_ctx* c, float* h_ms) {
   if (!c || !h_ms) return FS4D_ERR_INVALID_ARG;
   if (!c->ev[0]) return fail(c, FS4D_ERR_INVALID_ARG, "stage_times: timing was never enabled");
   DeviceGuard g(c->device);
-  if (c->stage_acc_valid) {  // a frame rendered in bands: the sum over its passes
+  if (c->stage_acc_valid) {  // the last frame went through two passes
     for (int k = 0; k < 6; ++k) h_ms[k] = c->stage_acc[k];
     return FS4D_OK;
   }
-  FS4D_CUDA(c, cudaEventSynchronize(c->ev[7]));
-  const int from[6] = {0, 1, 2, 3, 5, 6}, to[6] = {1, 2, 3, 4, 6, 7};
-  for (int k = 0; k < 6; ++k) FS4D_CUDA(c, cudaEventElapsedTime(&h_ms[k], c->ev[from[k]], c->ev[to[k]]));
-  return FS4D_OK;
+  return stage_times_of(c, h_ms);
 }
 
 fs4d_status fs4d_backward_times(fs4d_ctx* c, float* h_ms) {
@@ -2511,12 +2592,8 @@ fs4d_status fs4d_server_destroy(fs4d_server* sv) {
   for (Slot* sl : sv->slots) {
     cudaStreamSynchronize(sl->stream);
     for (auto& kv : sl->graphs) cudaGraphExecDestroy(kv.second);
-    Work& w = sl->w;
-    DevBuf* all[] = {&w.dmeans, &w.dquats, &w.dscales, &w.xy, &w.co, &w.rgb, &w.depth, &w.radius, &w.rect,
-                     &w.offsets, &w.emit_lb, &w.counters, &w.num_pairs, &w.hist, &w.keys, &w.values,
-                     &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges, &w.tile_count, &w.tile_order, &w.zero, &w.bitmap, &w.sxy, &w.sco, &w.srgb, &sl->status, &sl->dcam, &sl->dt,
-                     &sl->image};
-    for (DevBuf* b : all) release(*b);
+    release_work(sl->w);
+    for (DevBuf* b : {&sl->status, &sl->dcam, &sl->dt, &sl->image}) release(*b);
     cudaFreeHost(sl->h_cam);
     cudaFreeHost(sl->h_t);
     cudaFreeHost(sl->h_out);

@@ -186,7 +186,128 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) composite_kernel(int wid
   write_pixel(inside, px, py, width, R, G, B, T, last, image, t_final, n_contrib, AUX);
 }
 
+// Tiles straight from the depth order (direct.cu): the tile's list is the set bits
+// of its column's and its row's bits, 32768 depth ranks per step (one 16-byte word of
+// each per thread).  The ranks of a step go into shared memory in order, at most
+// kQueue at a time, and are staged and blended as the listed tiles' are; the walk
+// ends when every pixel has saturated, so the far ranks of a covered tile are never
+// looked at.  Scanning costs two 16-byte loads per 128 ranks and tile against the
+// 5,000 instructions or so per warp that blending a batch of 256 takes.
+constexpr int kQueue = 4096;
+constexpr int kStepRanks = 128 * kThreads;
+static_assert(kStepRanks <= 65536, "queue entries are 16-bit offsets within a step");
+
+template <bool AUX>
+__global__ void __launch_bounds__(kThreads, 4) composite_direct_kernel(const __grid_constant__ DirectArgs a,
+                                                                       float* __restrict__ image,
+                                                                       float* __restrict__ t_final,
+                                                                       int* __restrict__ n_contrib) {
+  __shared__ float4 s_g0b[2][kBatch];   // x, y, a2, c2
+  __shared__ float4 s_g1b[2][kBatch];   // b2, opacity, red, green
+  __shared__ float s_blueb[2][kBatch];
+  __shared__ uint32_t s_maskb[2][kBatch];
+  __shared__ uint8_t s_list[kWarps][kBatch];
+  __shared__ uint16_t s_queue[kQueue];
+  __shared__ uint32_t s_warp[2][kWarps];
+  pdl_wait();
+  pdl_trigger();
+  const int tx = (int)blockIdx.x % a.tiles_x, row = a.bands.r0[0] + (int)blockIdx.x / a.tiles_x;
+  int band = 0;
+  while (band + 1 < a.bands.n && a.bands.r0[band + 1] <= row) ++band;
+  const float cy = a.bands.cy[band];
+  const int ty = row - a.bands.r0[band];  // rows and pixel rows count from the band's first
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int px = tx * kTile + (warp & 1) * 8 + (lane & 7), py = ty * kTile + (warp >> 1) * 4 + (lane >> 3);
+  const int gy = py + kTile * a.bands.r0[band];
+  const bool inside = px < a.width && gy < a.height;
+  const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
+  const uint4* col = reinterpret_cast<const uint4*>(a.cols + (size_t)tx * a.words);
+  const uint4* rowb = reinterpret_cast<const uint4*>(a.rows + (size_t)row * a.words);
+  const int nvec = a.words >> 2;
+
+  bool done = !inside;
+  float T = 1.f, R = 0.f, G = 0.f, B = 0.f;
+  int last = 0, listed = 0;  // listed: the tile's Gaussians in the steps before this one
+  int it = 0;
+  bool all_done = false;
+  for (int v0 = 0, step = 0; v0 < nvec && !all_done; v0 += kThreads, ++step) {
+    const int v = v0 + (int)threadIdx.x;
+    uint4 q = make_uint4(0u, 0u, 0u, 0u);
+    if (v < nvec) {
+      const uint4 c = col[v], r = rowb[v];
+      q = make_uint4(c.x & r.x, c.y & r.y, c.z & r.z, c.w & r.w);
+    }
+    const uint32_t cnt = __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += y;
+    }
+    uint32_t* sw = s_warp[step & 1];  // two buffers: one barrier before they are read, none after
+    if (lane == 31) sw[warp] = incl;
+    __syncthreads();
+    uint32_t first = incl - cnt, total = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t y = sw[w];
+      if (w < warp) first += y;
+      total += y;
+    }
+    for (uint32_t w0 = 0; w0 < total && !all_done; w0 += kQueue) {
+      // this thread's ranks whose list position falls into [w0, w0 + kQueue)
+      if (first < w0 + kQueue && first + cnt > w0) {
+        const uint32_t wd[4] = {q.x, q.y, q.z, q.w};
+        uint32_t pos = first;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t m = wd[j];
+          while (m) {
+            if (pos >= w0 && pos < w0 + kQueue)
+              s_queue[pos - w0] = (uint16_t)(128u * threadIdx.x + 32u * j + (uint32_t)(__ffs(m) - 1));
+            ++pos;
+            m &= m - 1u;
+          }
+        }
+      }
+      __syncthreads();
+      const int m = (int)min((uint32_t)kQueue, total - w0);
+      for (int b0 = 0; b0 < m; b0 += kBatch, ++it) {
+        const int b = it & 1, k = b0 + (int)threadIdx.x;
+        if (k < m) {
+          const uint32_t rank = 128u * (uint32_t)v0 + s_queue[k];
+          const float4 pos = a.s_pos[rank], co = a.s_co[rank];
+          const float2 rg = a.s_rg[rank], p = make_float2(pos.x, fmaf(pos.y, pos.z, cy));
+          s_g0b[b][threadIdx.x] = composite_coeffs(p, co);
+          s_g1b[b][threadIdx.x] = make_float4(composite_b2(co), co.w, rg.x, rg.y);
+          s_blueb[b][threadIdx.x] = pos.w;
+          s_maskb[b][threadIdx.x] = block_mask(p, co, composite_exp_threshold(co.w), tx, ty);
+        }
+        // (as in composite_kernel; the queue is refilled only after the last batch's barrier)
+        if (__syncthreads_count(done) == kThreads) {
+          all_done = true;
+          break;
+        }
+        if (__all_sync(0xffffffffu, done)) continue;  // warp-uniform
+        composite_batch<AUX>(min(kBatch, m - b0), listed + (int)w0 + b0, s_g0b[b], s_g1b[b], s_blueb[b], s_maskb[b],
+                             s_list[warp], warp, lane, fx, fy, done, T, R, G, B, last);
+      }
+    }
+    listed += (int)total;
+  }
+  write_pixel(inside, px, gy, a.width, R, G, B, T, last, image, t_final, n_contrib, AUX);
+}
+
 }  // namespace
+
+cudaError_t launch_composite_direct(const DirectArgs& a, float* image, float* t_final, int* n_contrib,
+                                    cudaStream_t s) {
+  const int rows = a.bands.r0[a.bands.n] - a.bands.r0[0];
+  if (a.tiles_x * rows <= 0) return cudaSuccess;
+  if (t_final || n_contrib)
+    return launch_pdl(composite_direct_kernel<true>, a.tiles_x * rows, kThreads, 0, s, a, image, t_final, n_contrib);
+  return launch_pdl(composite_direct_kernel<false>, a.tiles_x * rows, kThreads, 0, s, a, image, t_final, n_contrib);
+}
 
 cudaError_t launch_composite(int width, int height, const uint2* ranges, const uint32_t* values, const float2* xy,
                              const float4* conic_opacity, const float* rgb, float* image, float* t_final,

@@ -198,6 +198,9 @@ struct ProjectArgs {
   uint32_t* depth_vals;            // optional [n]: Gaussian index (index_base + g)
   uint32_t index_base;             // index of this call's first Gaussian in the frame's set
   uint32_t* depth_hist;            // optional [4][256] (zeroed): byte histograms of the depth keys
+  float2* y_parts;                 // optional [n]: (fy y, 1 / z) of the visible Gaussians, so that the mean's row
+                                   // is y_parts.x * y_parts.y + cy for any cy; a Gaussian is then culled by its
+                                   // columns only, and its rectangle's rows may be empty
 };
 
 // Tile-pair emission fused with the exclusive scan of per-Gaussian tile counts
@@ -283,6 +286,44 @@ cudaError_t launch_tile_scan(const uint32_t* tile_count, int n_tiles, uint32_t* 
 int bitmap_words(int n);        // words per tile row (a multiple of 4)
 cudaError_t launch_mark_tiles(const EmitArgs& a, cudaStream_t s);
 cudaError_t launch_extract_tiles(const EmitArgs& a, bool ids, cudaStream_t s);
+
+// ---- Frames composited straight from the depth order (direct.cu, composite.cu).
+// A tile rectangle is a column interval times a row interval, so the depth ranks of
+// tile (tx, ty) are the set bits of columns[tx] & rows[ty], one bit per depth rank.
+// Bands of tile rows [r0[b], r0[b + 1]) have a principal point of their own (cy[b],
+// relative to the band's first row), and so rows of their own.
+constexpr int kMaxBands = 64;
+struct BandTab {
+  int n;
+  int r0[kMaxBands + 1];
+  float cy[kMaxBands];
+};
+struct DirectArgs {
+  int n;
+  const uint32_t* order;        // depth order, as EmitArgs
+  const uint32_t* order_alt;
+  const uint32_t* order_sel;
+  const float2* xy;             // projection with y_parts
+  const float2* y_parts;
+  const int4* rect;
+  const int* radius;
+  const float4* conic_opacity;
+  const float* rgb;
+  int width, height, tiles_x;   // of the whole frame
+  int words;                    // 32-bit words per bit row: bitmap_words(n)
+  uint32_t* cols;               // [tiles_x][words]
+  uint32_t* rows;               // [tiles_y][words]
+  float4* s_pos;                // [n] by depth rank: u, fy y, 1 / z, blue
+  float4* s_co;                 // [n]
+  float2* s_rg;                 // [n]
+  BandTab bands;
+};
+// pairs[b] += tile pairs of band b (zeroed by the caller)
+cudaError_t launch_band_pairs(const DirectArgs& a, unsigned long long* pairs, cudaStream_t s);
+// the bit rows of the bands' tile rows; columns and rank-ordered copies with first
+cudaError_t launch_axis_bits(const DirectArgs& a, bool first, cudaStream_t s);
+cudaError_t launch_composite_direct(const DirectArgs& a, float* image, float* t_final, int* n_contrib,
+                                    cudaStream_t s);
 
 int sort_passes(int key_bits);
 long long sort_parts(long long n);

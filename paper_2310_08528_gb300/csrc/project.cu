@@ -186,13 +186,14 @@ __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   const float hd = 0.5f * (aa - dd);
   const float lmax = 0.5f * (ca + cc) + sqrtf(hd * hd + bb * bb);
   const int radius = (int)ceilf(3.f * sqrtf(lmax));
-  const float u = c.fx * px * iz + c.cx, v = c.fy * py * iz + c.cy;
+  const float u = c.fx * px * iz + c.cx, fpy = c.fy * py, v = fpy * iz + c.cy;
   const float fr = (float)radius;
   int x0 = (int)floorf((u - fr) * (1.f / kTile)), x1 = (int)floorf((u + fr) * (1.f / kTile)) + 1;
   int y0 = (int)floorf((v - fr) * (1.f / kTile)), y1 = (int)floorf((v + fr) * (1.f / kTile)) + 1;
   x0 = min(a.tiles_x, max(0, x0)); x1 = min(a.tiles_x, max(0, x1));
   y0 = min(a.tiles_y, max(0, y0)); y1 = min(a.tiles_y, max(0, y1));
-  if (x1 <= x0 || y1 <= y0) {
+  // (with y_parts the rows are decided later, per band of tile rows)
+  if (x1 <= x0 || (y1 <= y0 && !a.y_parts)) {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     return;
   }
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   a.rgb[3 * g + 1] = fmaxf(0.f, gg);
   a.rgb[3 * g + 2] = fmaxf(0.f, b);
   a.xy[g] = make_float2(u, v);
+  if (a.y_parts) a.y_parts[g] = make_float2(fpy, iz);
   a.conic_opacity[g] = make_float4(cc * idet, -cb * idet, ca * idet, opacity);
   a.radius[g] = radius;
   a.rect[g] = make_int4(x0, y0, x1, y1);

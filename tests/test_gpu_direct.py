@@ -1,0 +1,47 @@
+"""Frames composited straight from the depth order: columns and rows of tiles as
+bits per depth rank.  A frame whose pairs exceed a band goes that way; its first
+band has the whole frame's principal point, so its pixels are the listed tiles'
+bit for bit, with full lists (the last contributors are list positions)."""
+import numpy as np
+import pytest
+
+from paper_2310_08528_gb300 import scenegen as sg
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2310_08528_gb300 import fs4d  # noqa: E402
+
+
+# 32768 ranks are one step of a tile, 4096 of its list one queue, 1024 ranks one CTA of the bit rows
+@pytest.mark.parametrize("n,w,h,scale", [(33, 48, 40, -2.0), (1023, 130, 120, -2.5), (1025, 1100, 64, -3.0),
+                                         (6000, 64, 64, -1.0), (33000, 333, 211, -3.0)])
+def test_direct_frame_equals_listed_frame(n, w, h, scale):
+    s = sg.make_object(9, n=n, log_scale_mean=scale, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=w, height=h, seed=3)[2]
+    ctx = fs4d.Context(0)
+    try:
+        sid = ctx.load_scene(s)
+        want = ctx.render(sid, cam, 0.3, with_aux=True)
+        k = ctx.last_pairs()
+        assert ctx.last_bands() == 1
+        ctx.set_band_pairs(k - 1)
+        rows = (h + 15) // 16
+        for _ in range(2):  # cut into bands, then with the bands of the frame before
+            got = ctx.render(sid, cam, 0.3, with_aux=True)
+            bands = ctx.last_bands()
+            assert bands >= 2
+            first = 16 * (rows // 4)  # at most four bands at half the limit each: the first holds these rows
+            for a, b in zip(got, want):
+                assert torch.equal(a[:first], b[:first])
+                assert np.isfinite(a.float().cpu().numpy()).all()
+            # a row's principal point is rounded differently in the other bands
+            far = (got[0] - want[0]).abs().amax(-1) > 2e-2
+            assert int(far.sum()) <= 1e-3 * w * h
+        plain = ctx.render(sid, cam, 0.3)
+        assert torch.equal(plain, got[0])
+    finally:
+        ctx.close()
