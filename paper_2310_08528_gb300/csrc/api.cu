@@ -227,6 +227,9 @@ struct fs4d_frame {
   DevBuf xy, co, rgb, radius, rect, offsets;   // projection and emission offsets
   DevBuf values, ranges;                       // sorted Gaussian indices, per-tile ranges
   DevBuf t_final, n_contrib;                   // per pixel
+  cudaStream_t stream = nullptr;               // the stream of every launch that used the buffers,
+  bool one_stream = true;                      // unless there were several
+  int device = 0;
 };
 
 struct fs4d_server;
@@ -243,7 +246,11 @@ struct fs4d_ctx {
   DevBuf status;
   uint32_t* h_pinned = nullptr;  // [4] readback slots
   long long last_pairs = 0;
-  uint32_t* last_values = nullptr;  // sorted Gaussian indices of the last frame (work memory)
+  // Freed frames whose buffers the next saved frame takes over (at most kSpareFrames; all of
+  // their work is on `stream`, so the next frame's launches come after it).  A device
+  // allocation and its release cost a saved frame more than its kernels: 1.1 ms of the 2.65 ms
+  // of one 800x800 / 100k view and its backward went there.
+  std::vector<fs4d_frame*> spare;
   int binning = FS4D_BINNING_AUTO;
   int last_binning = FS4D_BINNING_SORT;
   bool timing = false;
@@ -254,6 +261,7 @@ struct fs4d_ctx {
   cudaEvent_t slot_rendered[2] = {}, slot_copied[2] = {};
   unsigned long long* h_pairs = nullptr;  // pinned, [h_pairs_cap]: each frame's pair count
   int h_pairs_cap = 0;
+  cudaEvent_t counted = nullptr;          // a frame's pair count is on the host
   unsigned long long* h_band_pairs = nullptr;  // pinned, [kMaxTileRows]: pairs of a frame's bands
   uint32_t spin_limit = kSpinLimit;       // polls of a look-back wait (fs4d_set_wait_limit)
   // frames rendered in bands of tile rows (more pairs than one sort pass counts)
@@ -928,7 +936,7 @@ fs4d_status frame_back(const Env& e, const fs4d_camera& shape, long long n_bound
 
 fs4d_status frame_back(fs4d_ctx* c, const fs4d_camera& shape, long long n_bound, float* d_image, float* d_t_final,
                        int* d_n_contrib) {
-  return frame_back(env_of(c), shape, n_bound, d_image, d_t_final, d_n_contrib, &c->last_values);
+  return frame_back(env_of(c), shape, n_bound, d_image, d_t_final, d_n_contrib, nullptr);
 }
 
 fs4d_status read_pairs(fs4d_ctx* c, const uint32_t* d_num_pairs, long long* K) {
@@ -1085,9 +1093,28 @@ fs4d_status render_direct(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d
   return FS4D_OK;
 }
 
-// offsets: the frame will be saved for a backward
+// The back half of a frame queued behind its front half before the pair count is
+// known on the host: the kernels take the count from the device, so only a frame whose
+// pairs overflow the capacity (or a band) has to be rendered again, and the host waits
+// for the count while the frame runs instead of between its halves.
+fs4d_status frame_queue(const Env& e, const fs4d_camera& cam, float* d_image, float* d_t_final, int* d_n_contrib,
+                        uint32_t** values_out, long long* K) {
+  fs4d_ctx* c = e.c;
+  const long long cap = e.w->cap_pairs;
+  FS4D_CUDA(c, cudaMemcpyAsync(c->h_pinned, e.w->z.num_pairs, 8, cudaMemcpyDeviceToHost, e.s));
+  if (!c->counted) FS4D_CUDA(c, cudaEventCreateWithFlags(&c->counted, cudaEventDisableTiming));
+  FS4D_CUDA(c, cudaEventRecord(c->counted, e.s));
+  if (cap > 0) {
+    const fs4d_status st = frame_back(e, cam, cap, d_image, d_t_final, d_n_contrib, values_out);
+    if (st != FS4D_OK) return st;
+  }
+  FS4D_CUDA(c, cudaEventSynchronize(c->counted));
+  *K = (long long)c->h_pinned[0];
+  return FS4D_OK;
+}
+
 fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t, float* d_image,
-                        float* d_t_final, int32_t* d_n_contrib, bool offsets = false) {
+                        float* d_t_final, int32_t* d_n_contrib) {
   const int n_tiles = tiles_of(cam->width) * tiles_of(cam->height);
   fs4d_status st = ensure_work(c, s->n, n_tiles, c->w.cap_pairs);
   if (st != FS4D_OK) return st;
@@ -1096,73 +1123,115 @@ fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_c
   c->last_bands = 1;
   // too many tiles x Gaussians for the tile bitmap, or more pairs than a band may hold last time
   const bool banded = c->band_hint > 1 && c->band_scene == s->id && c->band_w == cam->width && c->band_h == cam->height;
-  if (!offsets && (banded || (c->binning != FS4D_BINNING_SORT && !use_bitmap(c, c->w, s->n, n_tiles, false))))
+  if (banded || (c->binning != FS4D_BINNING_SORT && !use_bitmap(c, c->w, s->n, n_tiles, false)))
     return render_direct(c, s, prec, cam, t, true, d_image, d_t_final, d_n_contrib);
-  // lists may drop Gaussians no pixel of their tile blends unless the frame reports
-  // list positions (last contributors) or keeps the backward's pair slots
-  const bool cull = !offsets && !d_n_contrib;
-  st = frame_front(c, s, prec, *cam, nullptr, nullptr, t, c->w.cap_pairs, false, offsets, cull);
-  if (st != FS4D_OK) return st;
-  long long K = 0;
-  if ((st = read_pairs(c, c->w.z.num_pairs, &K)) != FS4D_OK) return st;
-  if (K > c->band_pairs) {
-    if (offsets) return fail(c, FS4D_ERR_CAPACITY, "a frame saved for the backward must fit one band of tile pairs");
-    float deform_ms = 0.f;
-    if (c->timing) {
-      FS4D_CUDA(c, cudaEventSynchronize(c->ev[1]));
-      FS4D_CUDA(c, cudaEventElapsedTime(&deform_ms, c->ev[0], c->ev[1]));
-    }
-    st = render_direct(c, s, prec, cam, t, false, d_image, d_t_final, d_n_contrib);
-    if (st == FS4D_OK && c->timing) {  // the deformation is the pass above's
-      if ((st = stage_times_of(c, c->stage_acc)) != FS4D_OK) return st;
-      c->stage_acc[0] = deform_ms;
-      c->stage_acc_valid = true;
-    }
-    return st;
-  }
-  if (K > c->w.cap_pairs) {
-    if ((st = ensure_work(c, s->n, n_tiles, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
-    st = frame_front(c, s, prec, *cam, nullptr, nullptr, t, c->w.cap_pairs, false, offsets, cull);
+  const bool cull = !d_n_contrib;  // lists may drop Gaussians unless the frame reports list positions
+  for (int pass = 0;; ++pass) {
+    st = frame_front(c, s, prec, *cam, nullptr, nullptr, t, c->w.cap_pairs, false, false, cull);
     if (st != FS4D_OK) return st;
+    long long K = 0;
+    if ((st = frame_queue(env_of(c), *cam, d_image, d_t_final, d_n_contrib, nullptr, &K)) != FS4D_OK) return st;
+    if (K > c->band_pairs) {
+      float deform_ms = 0.f;
+      if (c->timing) {
+        FS4D_CUDA(c, cudaEventSynchronize(c->ev[1]));
+        FS4D_CUDA(c, cudaEventElapsedTime(&deform_ms, c->ev[0], c->ev[1]));
+      }
+      st = render_direct(c, s, prec, cam, t, false, d_image, d_t_final, d_n_contrib);
+      if (st == FS4D_OK && c->timing) {  // the deformation is the pass above's
+        if ((st = stage_times_of(c, c->stage_acc)) != FS4D_OK) return st;
+        c->stage_acc[0] = deform_ms;
+        c->stage_acc_valid = true;
+      }
+      return st;
+    }
+    c->last_pairs = K;
+    if (K <= c->w.cap_pairs && c->w.cap_pairs > 0) return FS4D_OK;
+    if (pass > 0) return fail(c, FS4D_ERR_CAPACITY, "render: the frame's pairs changed between two passes");
+    if ((st = ensure_work(c, s->n, n_tiles, std::max(std::min(K + K / 4, c->band_pairs), 1ll))) != FS4D_OK) return st;
   }
-  c->last_pairs = K;
-  c->last_bands = 1;
-  return frame_back(c, *cam, K, d_image, d_t_final, d_n_contrib);
+}
+
+constexpr size_t kSpareFrames = 2;
+
+void release_frame(fs4d_frame& f) {
+  DevBuf* all[] = {&f.dmeans, &f.dquats, &f.dscales, &f.xy, &f.co, &f.rgb, &f.radius, &f.rect, &f.offsets,
+                   &f.values, &f.ranges, &f.t_final, &f.n_contrib};
+  for (DevBuf* b : all) release(*b);
+}
+
+void release_spare(fs4d_ctx* c) {  // (cudaFree waits for the work that uses the buffers)
+  for (fs4d_frame* f : c->spare) {
+    release_frame(*f);
+    delete f;
+  }
+  c->spare.clear();
+}
+
+// The buffers of a saved frame, grown where they are too small.
+fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, size_t npix, size_t pairs) {
+  const std::pair<DevBuf*, size_t> need[] = {
+      {&f->dmeans, 12 * n}, {&f->dquats, 16 * n}, {&f->dscales, 12 * n}, {&f->xy, 8 * n},       {&f->co, 16 * n},
+      {&f->rgb, 12 * n},    {&f->radius, 4 * n},  {&f->rect, 16 * n},    {&f->offsets, 4 * n},  {&f->values, 4 * pairs},
+      {&f->ranges, 8 * tiles}, {&f->t_final, 4 * npix}, {&f->n_contrib, 4 * npix}};
+  bool grow = false, first = true;
+  for (const auto& q : need) {
+    grow = grow || q.first->bytes < q.second;
+    first = first && !q.first->p;
+  }
+  if (!grow) return FS4D_OK;
+  if (!first) FS4D_CUDA(c, cudaStreamSynchronize(c->stream));  // the old buffers may still be read
+  for (const auto& q : need)
+    if (ensure(*q.first, q.second) != cudaSuccess) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
+  return FS4D_OK;
 }
 
 // Render with the state the backward needs, into f (its buffers are reused and
 // grown when needed, so a frame object can serve one training step after another).
+// The frame's kernels write that state where it stays: they run on a view of the
+// work memory in which the frame's buffers stand in for the context's.
 fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t,
                               float* d_image, fs4d_frame* f) {
   const size_t npix = (size_t)cam->width * cam->height;
-  if (ensure(f->t_final, 4 * npix) != cudaSuccess || ensure(f->n_contrib, 4 * npix) != cudaSuccess)
-    return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
-  fs4d_status st = render_sync(c, s, prec, cam, t, d_image, P<float>(f->t_final), P<int32_t>(f->n_contrib), true);
+  const int n_tiles = tiles_of(cam->width) * tiles_of(cam->height);
+  const bool odd = sort_passes(ceil_log2(n_tiles)) & 1;  // passes of the pair sort: where its result lands
+  fs4d_status st = ensure_work(c, s->n, n_tiles, std::max(c->w.cap_pairs, 4096ll));
   if (st != FS4D_OK) return st;
-  Work& w = c->w;
-  const size_t n = (size_t)s->n, K = (size_t)c->last_pairs;
-  const size_t tiles = (size_t)tiles_of(cam->width) * tiles_of(cam->height);
-  struct Item {
-    DevBuf* dst;
-    const void* src;
-    size_t bytes;
-  } items[] = {{&f->dmeans, w.dmeans.p, 12 * n}, {&f->dquats, w.dquats.p, 16 * n}, {&f->dscales, w.dscales.p, 12 * n},
-               {&f->xy, w.xy.p, 8 * n},          {&f->co, w.co.p, 16 * n},         {&f->rgb, w.rgb.p, 12 * n},
-               {&f->radius, w.radius.p, 4 * n},  {&f->rect, w.rect.p, 16 * n},     {&f->offsets, w.offsets.p, 4 * n},
-               {&f->values, c->last_values, 4 * std::max<size_t>(K, 1)},           {&f->ranges, w.ranges.p, 8 * tiles}};
-  for (Item& it : items) {
-    if (it.dst->bytes < it.bytes) {
-      FS4D_CUDA(c, cudaStreamSynchronize(c->stream));  // the old buffer may still be read
-      if (ensure(*it.dst, it.bytes) != cudaSuccess) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
+  if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
+  c->stage_acc_valid = false;
+  c->last_bands = 1;
+  c->last_binning = FS4D_BINNING_SORT;
+  if (f->stream != c->stream && f->dmeans.p) f->one_stream = false;
+  f->stream = c->stream;
+  f->device = c->device;
+  for (int pass = 0;; ++pass) {
+    if ((st = ensure_frame(c, f, (size_t)s->n, (size_t)n_tiles, npix, (size_t)c->w.cap_pairs)) != FS4D_OK) return st;
+    Work v = c->w;
+    v.dmeans = f->dmeans; v.dquats = f->dquats; v.dscales = f->dscales;
+    v.xy = f->xy; v.co = f->co; v.rgb = f->rgb; v.radius = f->radius; v.rect = f->rect;
+    v.offsets = f->offsets; v.ranges = f->ranges;
+    (odd ? v.values_alt : v.values) = f->values;
+    const Env e{c, &v, c->stream, P<uint32_t>(c->status), true};
+    if ((st = frame_front(e, s, prec, *cam, nullptr, nullptr, t, v.cap_pairs, false, true, true)) != FS4D_OK)
+      return st;
+    long long K = 0;
+    uint32_t* values = nullptr;
+    if ((st = frame_queue(e, *cam, d_image, P<float>(f->t_final), P<int32_t>(f->n_contrib), &values, &K)) != FS4D_OK)
+      return st;
+    if (K > c->band_pairs)
+      return fail(c, FS4D_ERR_CAPACITY, "a frame saved for the backward must fit one band of tile pairs");
+    f->pairs = c->last_pairs = K;
+    if (K <= c->w.cap_pairs) {
+      if (values != f->values.p) return fail(c, FS4D_ERR_CUDA, "render: the frame's list is not where it belongs");
+      break;
     }
-    if (cudaMemcpyAsync(it.dst->p, it.src, it.bytes, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
-      return fail(c, FS4D_ERR_CUDA, "render: saving the frame failed");
+    if (pass > 0) return fail(c, FS4D_ERR_CAPACITY, "render: the frame's pairs changed between two passes");
+    if ((st = ensure_work(c, s->n, n_tiles, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
   }
   f->scene = s->id;
   f->cam = *cam;
   f->t = t;
   f->n = s->n;
-  f->pairs = c->last_pairs;
   return FS4D_OK;
 }
 
@@ -1216,6 +1285,8 @@ fs4d_status fs4d_destroy(fs4d_ctx* c) {
     }
     if (c->h_pairs) cudaFreeHost(c->h_pairs);
     if (c->h_band_pairs) cudaFreeHost(c->h_band_pairs);
+    if (c->counted) cudaEventDestroy(c->counted);
+    release_spare(c);
   }
   delete c;
   return FS4D_OK;
@@ -1225,6 +1296,10 @@ const char* fs4d_last_error(const fs4d_ctx* c) { return c ? c->err.c_str() : "nu
 
 fs4d_status fs4d_set_stream(fs4d_ctx* c, void* cuda_stream) {
   if (!c) return FS4D_ERR_INVALID_ARG;
+  if (c->stream != reinterpret_cast<cudaStream_t>(cuda_stream) && !c->spare.empty()) {
+    DeviceGuard g(c->device);
+    release_spare(c);  // their work is on the old stream
+  }
   c->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   return FS4D_OK;
 }
@@ -1395,6 +1470,7 @@ fs4d_status fs4d_unload_scene(fs4d_ctx* c, fs4d_scene_id id) {
     return fail(c, FS4D_ERR_TIMEOUT, "unload_scene: serving requests on this scene did not finish");
   }
   cudaStreamSynchronize(c->stream);
+  release_spare(c);
   {
     std::lock_guard<std::mutex> lock(c->mu);
     c->scenes.erase(id);
@@ -1451,7 +1527,13 @@ fs4d_status render_impl(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision prec, cons
   DeviceGuard g(c->device);
   if (!saved) return render_sync(c, s, prec, cam, t, d_image, d_t_final, d_n_contrib);
   *saved = nullptr;
-  fs4d_frame* f = new (std::nothrow) fs4d_frame();
+  fs4d_frame* f = nullptr;
+  if (!c->spare.empty()) {
+    f = c->spare.back();
+    c->spare.pop_back();
+  } else {
+    f = new (std::nothrow) fs4d_frame();
+  }
   if (!f) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
   st = render_into_frame(c, s, prec, cam, t, d_image, f);
   if (st == FS4D_OK && d_t_final)
@@ -1716,6 +1798,7 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
     return fail(c, FS4D_ERR_UNIMPLEMENTED, "render_backward: no backward through the colour and opacity heads");
   if (s->n != f->n) return fail(c, FS4D_ERR_INVALID_ARG, "render_backward: the scene changed size since the frame");
   DeviceGuard g(c->device);
+  if (f->stream != c->stream) f->one_stream = false;
   Work& w = c->w;
   const long long n = s->n, K = f->pairs;
   const int hin = s->mg.hin;
@@ -1818,12 +1901,15 @@ fs4d_status fs4d_render_backward_stats(fs4d_ctx* c, fs4d_frame* f, const float* 
 
 fs4d_status fs4d_frame_free(fs4d_ctx* c, fs4d_frame* f) {
   if (!f) return FS4D_OK;
+  // kept for the context's next saved frame if all of its work is on the context's stream
+  if (c && f->one_stream && f->stream == c->stream && f->device == c->device && c->spare.size() < kSpareFrames) {
+    c->spare.push_back(f);
+    return FS4D_OK;
+  }
   {
-    DeviceGuard g(c ? c->device : 0);
+    DeviceGuard g(c ? c->device : f->device);
     if (c) cudaStreamSynchronize(c->stream);
-    DevBuf* all[] = {&f->dmeans, &f->dquats, &f->dscales, &f->xy, &f->co, &f->rgb, &f->radius,
-                     &f->rect, &f->offsets, &f->values, &f->ranges, &f->t_final, &f->n_contrib};
-    for (DevBuf* b : all) release(*b);
+    release_frame(*f);
   }
   delete f;
   return FS4D_OK;
@@ -2637,12 +2723,6 @@ struct fs4d_trainer {
 };
 
 namespace {
-void release_frame(fs4d_frame& f) {
-  DevBuf* all[] = {&f.dmeans, &f.dquats, &f.dscales, &f.xy, &f.co, &f.rgb, &f.radius, &f.rect, &f.offsets,
-                   &f.values, &f.ranges, &f.t_final, &f.n_contrib};
-  for (DevBuf* b : all) release(*b);
-}
-
 double lr_at(const float lr[2], long long k, long long total) {
   if (total <= 0 || !(lr[0] > 0.f) || !(lr[1] > 0.f)) return lr[0];
   const double f = std::min(1.0, (double)k / (double)total);
