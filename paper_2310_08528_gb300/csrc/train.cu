@@ -86,36 +86,46 @@ struct TvArgs {
 // Grid TV (reading of L_tv): per plane, mean squared neighbour difference along each
 // axis.  Each element's gradient needs only its 4 neighbours, so every element is
 // written by exactly one thread (g += ...), no atomics.  Per-block partial of the
-// loss (each pair counted by the element on its lower side).
+// loss (each pair counted by the element on its lower side).  A thread takes four
+// channels of a cell (h is a multiple of 16): one 16-byte access per neighbour and one
+// index calculation in 32 bits for four elements (4.7M elements: 44 us one at a time).
 __global__ void __launch_bounds__(kThreads) tv_kernel(const __grid_constant__ TvArgs a, const float* __restrict__ P,
                                                       float* __restrict__ g, float* __restrict__ partial) {
   __shared__ float tmp[kThreads / 32];
   float acc = 0.f;
-  for (long long i = blockIdx.x * (long long)kThreads + threadIdx.x; i < a.total;
+  const int hv = a.h / 4;
+  for (long long i = blockIdx.x * (long long)kThreads + threadIdx.x; i < a.total / 4;
        i += (long long)gridDim.x * kThreads) {
     int q = 0;
     long long rel = i;
-    while (q + 1 < a.n_planes && rel >= a.p[q].cells) rel -= a.p[q++].cells;
+    while (q + 1 < a.n_planes && rel >= a.p[q].cells / 4) rel -= a.p[q++].cells / 4;
     const TvPlane pl = a.p[q];
-    const long long e = pl.off + rel;
-    const long long cell = rel / a.h;
-    const int ai = (int)(cell % pl.ra), bi = (int)(cell / pl.ra);
+    const long long e = pl.off + 4 * rel;
+    const uint32_t cell = (uint32_t)rel / (uint32_t)hv;  // (launch_tv: fewer than 2^32 vectors a plane)
+    const int bi = (int)(cell / (uint32_t)pl.ra), ai = (int)cell - bi * pl.ra;
     const long long sa = a.h, sb = (long long)pl.ra * a.h;
-    const float v = P[e];
-    float gr = 0.f;
-    if (ai + 1 < pl.ra) {
-      const float d = P[e + sa] - v;
-      acc += d * d * (0.5f * pl.wa);
-      gr -= pl.wa * d;
-    }
-    if (ai > 0) gr += pl.wa * (v - P[e - sa]);
-    if (bi + 1 < pl.rb) {
-      const float d = P[e + sb] - v;
-      acc += d * d * (0.5f * pl.wb);
-      gr -= pl.wb * d;
-    }
-    if (bi > 0) gr += pl.wb * (v - P[e - sb]);
-    g[e] += gr;
+    auto at = [&](long long o) { return *reinterpret_cast<const float4*>(P + o); };
+    const float4 v = at(e);
+    float4 gr = make_float4(0.f, 0.f, 0.f, 0.f);
+    // the difference to the neighbour on the upper side counts for the loss, both for the gradient
+    auto upper = [&](const float4& n, float w) {
+      const float4 d = make_float4(n.x - v.x, n.y - v.y, n.z - v.z, n.w - v.w);
+      acc += d.x * d.x * (0.5f * w);
+      acc += d.y * d.y * (0.5f * w);
+      acc += d.z * d.z * (0.5f * w);
+      acc += d.w * d.w * (0.5f * w);
+      gr.x -= w * d.x; gr.y -= w * d.y; gr.z -= w * d.z; gr.w -= w * d.w;
+    };
+    auto lower = [&](const float4& n, float w) {
+      gr.x += w * (v.x - n.x); gr.y += w * (v.y - n.y); gr.z += w * (v.z - n.z); gr.w += w * (v.w - n.w);
+    };
+    if (ai + 1 < pl.ra) upper(at(e + sa), pl.wa);
+    if (ai > 0) lower(at(e - sa), pl.wa);
+    if (bi + 1 < pl.rb) upper(at(e + sb), pl.wb);
+    if (bi > 0) lower(at(e - sb), pl.wb);
+    float4* out = reinterpret_cast<float4*>(g + e);
+    const float4 o = *out;
+    *out = make_float4(o.x + gr.x, o.y + gr.y, o.z + gr.z, o.w + gr.w);
   }
   const float s = block_sum(acc, tmp);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
@@ -124,21 +134,56 @@ __global__ void __launch_bounds__(kThreads) tv_kernel(const __grid_constant__ Tv
 // Bias-corrected Adam over every segment; the gradient is cleared after use so the
 // next step accumulates afresh.  Element i of a segment takes lr_head where
 // (i mod period) < head (the degree-0 SH coefficients), else lr.
+// Four consecutive elements per thread (segments start 16-byte aligned and a vector
+// never crosses one), eight CTAs per SM so that enough of the four 16-byte loads are
+// in flight: bound by the 32 bytes per parameter.  22.6M parameters (the 300k room):
+// 290 us one element at a time with a 64-bit remainder for the SH rates.
+__device__ __forceinline__ void adam_one(const AdamArgs& a, float lr, float gv, float& p, float& m0, float& v0) {
+  const float m = a.beta1 * m0 + (1.f - a.beta1) * gv;
+  const float v = a.beta2 * v0 + (1.f - a.beta2) * gv * gv;
+  m0 = m;
+  v0 = v;
+  p -= lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
+}
 __global__ void __launch_bounds__(kThreads) adam_kernel(const __grid_constant__ AdamArgs a) {
   for (long long i = blockIdx.x * (long long)kThreads + threadIdx.x; i < a.total;
        i += (long long)gridDim.x * kThreads) {
     int q = 0;
-    long long j = i;
-    while (q + 1 < a.n_segs && j >= a.seg[q].n) j -= a.seg[q++].n;
+    long long j = i;  // vector within its segment
+    while (q + 1 < a.n_segs && j >= (a.seg[q].n + 3) / 4) j -= (a.seg[q++].n + 3) / 4;
     const AdamSeg& sgm = a.seg[q];
-    const float lr = (sgm.period > 0 && (int)(j % sgm.period) < sgm.head) ? sgm.lr_head : sgm.lr;
-    const float gv = sgm.g[j];
-    const float m = a.beta1 * sgm.m[j] + (1.f - a.beta1) * gv;
-    const float v = a.beta2 * sgm.v[j] + (1.f - a.beta2) * gv * gv;
-    sgm.m[j] = m;
-    sgm.v[j] = v;
-    sgm.p[j] -= lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
-    sgm.g[j] = 0.f;
+    j *= 4;
+    float lr[4] = {sgm.lr, sgm.lr, sgm.lr, sgm.lr};
+    if (sgm.period > 0) {
+      const int first = sgm.n < (1ll << 32) ? (int)((uint32_t)j % (uint32_t)sgm.period) : (int)(j % sgm.period);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {  // (period >= 3: at most two wraps)
+        int r = first + k;
+        r -= r >= sgm.period ? sgm.period : 0;
+        r -= r >= sgm.period ? sgm.period : 0;
+        if (r < sgm.head) lr[k] = sgm.lr_head;
+      }
+    }
+    if (j + 4 <= sgm.n) {
+      float4 p = *reinterpret_cast<float4*>(sgm.p + j), m = *reinterpret_cast<float4*>(sgm.m + j),
+             v = *reinterpret_cast<float4*>(sgm.v + j);
+      const float4 g = *reinterpret_cast<const float4*>(sgm.g + j);
+      adam_one(a, lr[0], g.x, p.x, m.x, v.x);
+      adam_one(a, lr[1], g.y, p.y, m.y, v.y);
+      adam_one(a, lr[2], g.z, p.z, m.z, v.z);
+      adam_one(a, lr[3], g.w, p.w, m.w, v.w);
+      *reinterpret_cast<float4*>(sgm.p + j) = p;
+      *reinterpret_cast<float4*>(sgm.m + j) = m;
+      *reinterpret_cast<float4*>(sgm.v + j) = v;
+      *reinterpret_cast<float4*>(sgm.g + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (j + k < sgm.n) {
+          adam_one(a, lr[k], sgm.g[j + k], sgm.p[j + k], sgm.m[j + k], sgm.v[j + k]);
+          sgm.g[j + k] = 0.f;
+        }
+    }
   }
 }
 
@@ -197,13 +242,14 @@ cudaError_t launch_tv(const PlaneGeom& pg, const float* planes, float weight, fl
       q.rb = axes[p][1] == 3 ? pg.res_time : pg.res[l];
       q.off = pg.off[l][p];
       q.cells = (long long)q.ra * q.rb * pg.feat_dim;
+      if (q.cells / 4 >= (1ll << 32) || pg.feat_dim % 4 != 0) return cudaErrorInvalidValue;
       const double na = (double)q.rb * (q.ra - 1) * pg.feat_dim, nb = (double)(q.rb - 1) * q.ra * pg.feat_dim;
       q.wa = (float)(2.0 * weight / na);
       q.wb = (float)(2.0 * weight / nb);
       total += q.cells;
     }
   a.total = total;
-  const int grid = grid_for(total);
+  const int grid = grid_for(total / 4);
   tv_kernel<<<grid, kThreads, 0, s>>>(a, planes, g_planes, partial);
   finish_sum_kernel<<<1, kThreads, 0, s>>>(partial, grid, 1.0, out);
   return cudaGetLastError();
@@ -211,7 +257,17 @@ cudaError_t launch_tv(const PlaneGeom& pg, const float* planes, float weight, fl
 
 cudaError_t launch_adam(const AdamArgs& a, cudaStream_t s) {
   if (a.total <= 0) return cudaSuccess;
-  adam_kernel<<<grid_for(a.total), kThreads, 0, s>>>(a);
+  AdamArgs b = a;
+  b.total = 0;  // in vectors of four
+  for (int q = 0; q < a.n_segs; ++q) {
+    const AdamSeg& sg = a.seg[q];
+    b.total += (sg.n + 3) / 4;
+    if (((reinterpret_cast<uintptr_t>(sg.p) | reinterpret_cast<uintptr_t>(sg.g) | reinterpret_cast<uintptr_t>(sg.m) |
+          reinterpret_cast<uintptr_t>(sg.v)) & 15u) != 0)
+      return cudaErrorMisalignedAddress;  // (the trainer allocates every group 16-byte aligned)
+  }
+  const long long most = 8LL * device_sm_count(), need = (b.total + kThreads - 1) / kThreads;
+  adam_kernel<<<(unsigned)std::min(need, most), kThreads, 0, s>>>(b);
   return cudaGetLastError();
 }
 
