@@ -1,4 +1,4 @@
-"""Frames composited straight from the depth order: columns and rows of tiles as
+"""Variants of a stage that are chosen by size give the same bits.  Frames composited straight from the depth order: columns and rows of tiles as
 bits per depth rank.  A frame whose pairs exceed a band goes that way; its first
 band has the whole frame's principal point, so its pixels are the listed tiles'
 bit for bit, with full lists (the last contributors are list positions)."""
@@ -43,5 +43,25 @@ def test_direct_frame_equals_listed_frame(n, w, h, scale):
             assert int(far.sum()) <= 1e-3 * w * h
         plain = ctx.render(sid, cam, 0.3)
         assert torch.equal(plain, got[0])
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 64 * 152, 64 * 152 + 1, 128 * 152 + 5])
+@pytest.mark.parametrize("levels", [1, 2, 3])
+def test_fp32_deform_tiles_agree(n, levels):
+    """Tiles of 32 and of 128 Gaussians give the same sums in the same order: a scene's first
+    Gaussians deform alike, bit for bit, alone and within a larger set."""
+    res = (8, 12, 16)[:levels]
+    s = sg.make_object(4, n=40000, res_spatial=res, res_time=5, mlp_std=0.2)
+    part = s.copy()
+    for k in ("means", "log_scales", "quats", "opacity_logits", "sh"):
+        setattr(part, k, np.ascontiguousarray(getattr(s, k)[:n]))
+    ctx = fs4d.Context(0)
+    try:
+        a = ctx.deform(ctx.load_scene(s), [0.37], fs4d.FP32)
+        b = ctx.deform(ctx.load_scene(part), [0.37], fs4d.FP32)
+        for x, y in zip(a, b):
+            assert torch.equal(x[:, :n], y)
     finally:
         ctx.close()
