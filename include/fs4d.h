@@ -68,11 +68,12 @@ typedef enum fs4d_precision {
  * (Sec. 3.1: the per-tile depth order of the tile-based rasteriser).  Both give the
  * same pair lists, bit for bit. */
 typedef enum fs4d_binning {
-  FS4D_BINNING_AUTO = 0,   /* the tile bitmap when it fits (at most 256 MB: tiles x Gaussians / 8
-                              bytes) and the frame keeps no state for a backward, else the sort */
+  FS4D_BINNING_AUTO = 0,   /* tile lists from column and row bits up to 2^31 tiles x Gaussians, else
+                              no lists at all (fs4d_render), or the sort where they are needed */
   FS4D_BINNING_SORT = 1,   /* emit one (tile | depth) key per pair and radix-sort on the tile bits */
-  FS4D_BINNING_BITMAP = 2  /* (only reported by fs4d_last_binning) one bit per (tile, depth rank),
-                              each tile's row read in rank order */
+  FS4D_BINNING_BITMAP = 2  /* (only reported by fs4d_last_binning) one bit per (tile column, depth rank)
+                              and (tile row, depth rank), ANDed and read in rank order; frames too large
+                              for it report FS4D_BINNING_SORT */
 } fs4d_binning;
 
 typedef struct fs4d_ctx fs4d_ctx;     /* one device + one stream; not thread-safe */
@@ -222,8 +223,8 @@ FS4D_API fs4d_status fs4d_deform(fs4d_ctx* ctx, fs4d_scene_id id, fs4d_precision
 /* Render one frame, I = S(M, G') with G' = G + F(G, t) (Sec. 4.1): deform at t
  * (Eq. 5, Eq. 6), project (Eq. 2, Eq. 3), bin, sort, composite (Eq. 1, Eq. 4).
  * A frame with more than 2^30 - 1 tile pairs (what one pair-sort pass counts) is
- * rendered in horizontal bands of whole tile rows, each binned, sorted and
- * composited on its own over the same deformed Gaussians (fs4d_last_pairs then
+ * rendered in horizontal bands of whole tile rows, each an image of its own
+ * over the same deformed Gaussians (fs4d_last_pairs then
  * gives the pairs of all bands); a frame saved for the backward must fit one
  * pass (FS4D_ERR_CAPACITY otherwise).  d_image:
  * device [height][width][3]; d_t_final [height][width] and d_n_contrib
@@ -280,9 +281,9 @@ FS4D_API fs4d_status fs4d_render_backward(fs4d_ctx* ctx, fs4d_frame* saved, cons
                                  const fs4d_grads* d_grads);
 FS4D_API fs4d_status fs4d_frame_free(fs4d_ctx* ctx, fs4d_frame* frame);
 /* Number of tile pairs K of a saved frame, and of the last render on the context:
- * the pairs of the Gaussians' tile rectangles (frames of the tile bitmap binning that
- * report no list positions list a Gaussian only in the tiles its ellipse
- * {alpha >= 1/255} reaches, which leaves the image unchanged and their lists shorter). */
+ * the pairs of the Gaussians' tile rectangles (frames with lists from column and row bits that
+ * report no list positions list a Gaussian only in the tiles that the bounding box of its
+ * ellipse {alpha >= 1/255} reaches, which leaves the image unchanged and their lists shorter). */
 FS4D_API fs4d_status fs4d_frame_pairs(const fs4d_frame* frame, int64_t* pairs);
 FS4D_API fs4d_status fs4d_last_pairs(const fs4d_ctx* ctx, int64_t* pairs);
 /* Number of kernels the last fs4d_render or fs4d_render_async call on the context

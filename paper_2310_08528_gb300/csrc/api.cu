@@ -1,6 +1,6 @@
 // C ABI of libfs4d.so: contexts, resident scenes, work memory and the per-frame
 // launch sequence: deform -> project -> depth sort of the N Gaussians -> tile
-// binning (tile bitmap: mark -> tile scan -> extract; or key emission -> tile
+// binning (column and row bits -> tile lists; or the bits alone; or key emission -> tile
 // scan -> stable pair sort on the tile bits) -> composite.  See include/fs4d.h
 // for the contract of every call.
 #include <nvtx3/nvToolsExt.h>
@@ -123,7 +123,8 @@ struct Scene {
 // ONE memset clears at the start of a frame.
 struct FrameZero {
   uint32_t* hist = nullptr;              // [8][256]: depth-key byte histograms, then the pair sort's
-  uint32_t* counters = nullptr;          // [64]: [0] emission ticket, [8, 25) depth sort, [32, 49) pair sort
+  uint32_t* counters = nullptr;          // [96]: [0] emission ticket, [8, 25) depth sort, [32, 49) pair sort,
+                                         // [56] grid barrier, [64, 96) tiles per length class
   uint32_t* num_pairs = nullptr;         // [4]
   uint32_t* tile_count = nullptr;        // [n_tiles]
   unsigned long long* emit_lb = nullptr; // [emit_parts(n) + 1]
@@ -138,48 +139,47 @@ struct Work {
   FrameZero z;                             // its layout for the frame in flight
   DevBuf dmeans, dquats, dscales;          // deformed Gaussians
   DevBuf xy, co, rgb, depth, radius, rect; // projected
-  DevBuf offsets, emit_lb, counters, num_pairs, hist;
+  DevBuf offsets, counters, hist;
   DevBuf dkeys, dvals, dkeys_alt, dvals_alt;  // per-Gaussian depth sort
   DevBuf keys, values, keys_alt, values_alt;
   DevBuf sort_lb;
-  DevBuf ranges, tile_count, tile_order;
-  DevBuf bitmap;                           // tile bitmap binning: [tiles][bitmap_words(n)], zero between frames
-  DevBuf sxy, sco, srgb;                   // with the bitmap: projected Gaussians in depth-rank order
-  bool bmp = false;                        // the frame in flight bins through the bitmap
+  DevBuf ranges, tile_order;
+  DevBuf axis;                             // column and row bits of the tiles: [tiles_x + tiles_y][bitmap_words(n)]
+  DevBuf sslot;                            // (a saved frame's, while it is rendered)
+  DevBuf sxy, sco, srgb, srect;      // with the lists: projected Gaussians in depth-rank order
+  bool bmp = false;                        // the frame in flight has tile lists from the column and row bits
   bool packed = false;                     // ... or sorts (tile | index) keys without values
-  bool bmp_dirty = false;                  // a frame set bits whose extraction was not launched
   DevBuf ts;
   DevBuf host_img;                         // device staging image of fs4d_render_host
   DevBuf grad_pair, gd, acts, wpartial;    // backward work memory
   DevBuf fd, dsh, dop;                     // colour and opacity heads: f_d [n][64] (work order),
                                            // deformed SH [n][48] and opacity logits [n]
-  DevBuf yparts, spos, srg, axis, band_pairs;  // frames composited straight from the depth order (direct.cu)
+  DevBuf yparts, spos, srg, band_pairs;  // frames composited straight from the depth order (direct.cu)
   int cap_color = 0;
   long long cap_pairs = 0;
   long long sort_parts_cap = 0;
   int cap_n = 0, cap_tiles = 0;
+  long long cap_rows = 0;                  // bit rows (tile columns + tile rows)
 };
 
 void release_work(Work& w) {
   DevBuf* all[] = {&w.zero, &w.dmeans, &w.dquats, &w.dscales, &w.xy, &w.co, &w.rgb, &w.depth, &w.radius, &w.rect,
-                   &w.offsets, &w.emit_lb, &w.counters, &w.num_pairs, &w.hist, &w.dkeys, &w.dvals, &w.dkeys_alt,
-                   &w.dvals_alt, &w.keys, &w.values, &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges, &w.tile_count,
-                   &w.tile_order, &w.bitmap, &w.sxy, &w.sco, &w.srgb, &w.ts, &w.host_img, &w.grad_pair, &w.gd, &w.acts,
-                   &w.wpartial, &w.fd, &w.dsh, &w.dop, &w.yparts, &w.spos, &w.srg, &w.axis, &w.band_pairs};
+                   &w.offsets, &w.counters, &w.hist, &w.dkeys, &w.dvals, &w.dkeys_alt,
+                   &w.dvals_alt, &w.keys, &w.values, &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges,
+                   &w.tile_order, &w.axis, &w.sxy, &w.sco, &w.srgb, &w.srect, &w.ts, &w.host_img, &w.grad_pair, &w.gd, &w.acts,
+                   &w.wpartial, &w.fd, &w.dsh, &w.dop, &w.yparts, &w.spos, &w.srg, &w.band_pairs};
   for (DevBuf* b : all) release(*b);
 }
 
 constexpr int kSortMaxPasses = 8;
 constexpr int kMaxTileRows = 8192 / kTile;  // (valid_cam bounds the image)
-// Largest tile bitmap (one bit per (tile, Gaussian)) a frame bins through; larger
-// frames emit keys and radix-sort them.  At this size clearing and walking the
-// rows costs about as much memory traffic as the sort's passes over ~10 pairs per
-// Gaussian, and the sort's latency chains are gone.
+// Frames of up to this many (tile, Gaussian) bits, 2^31, have tile lists from column and
+// row bits; larger ones are composited straight from those bits or, where lists are
+// needed, emit keys and radix-sort them.
 constexpr size_t kBitmapMaxBytes = size_t(256) << 20;
 
 size_t bitmap_bytes(int n, long long n_tiles) { return 4 * (size_t)n_tiles * (size_t)bitmap_words(std::max(n, 1)); }
 constexpr int kCounters = 32;  // [0] emit ticket, [8, 25) radix-sort tickets and selection words
-constexpr int kEmitCounters = 8;  // the words reset before an emission (the sort's words stay)
 
 // Byte layout of FrameZero for n Gaussians, n_tiles tiles, cap pairs and a pair
 // sort of pair_passes passes (256-byte aligned blocks); fills z when base != NULL.
@@ -192,7 +192,7 @@ size_t frame_zero_layout(int n, int n_tiles, long long cap, int pair_passes, uns
   };
   const long long dparts = sort_parts(std::max(n, 1)), pparts = sort_parts(std::max<long long>(cap, 1));
   const size_t o_hist = take(4 * 256 * (size_t)kSortMaxPasses);
-  const size_t o_cnt = take(4 * 64);
+  const size_t o_cnt = take(4 * 96);
   const size_t o_np = take(16);
   const size_t o_tc = take(4 * (size_t)n_tiles);
   const size_t o_elb = take(8 * (size_t)(emit_parts(std::max(n, 1)) + 1));
@@ -224,7 +224,9 @@ struct fs4d_frame {
   int n = 0;
   long long pairs = 0;
   DevBuf dmeans, dquats, dscales;              // deformed Gaussians
-  DevBuf xy, co, rgb, radius, rect, offsets;   // projection and emission offsets
+  DevBuf xy, co, rgb, radius, rect, offsets;   // projection and pair slots; lists of depth ranks: xy and rgb
+  DevBuf sco, slot;                            // by rank, with sco and (x0, y0, width, first slot) by rank
+  bool ranks = false;                          // the lists hold depth ranks
   DevBuf values, ranges;                       // sorted Gaussian indices, per-tile ranges
   DevBuf t_final, n_contrib;                   // per pixel
   cudaStream_t stream = nullptr;               // the stream of every launch that used the buffers,
@@ -536,12 +538,18 @@ fs4d_status ensure_color(fs4d_ctx* c, Work& w, cudaStream_t stream, int n) {
   return FS4D_OK;
 }
 
-fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int n_tiles, long long pairs) {
-  const bool bmp_ok = c->binning != FS4D_BINNING_SORT;
-  const size_t bmp_need =
-      std::max(bitmap_bytes(std::max(n, w.cap_n), std::max(n_tiles, w.cap_tiles)), w.bitmap.bytes);
-  const bool bmp_grow = bmp_ok && bmp_need <= kBitmapMaxBytes && bmp_need > w.bitmap.bytes;
-  bool grow = n > w.cap_n || n_tiles > w.cap_tiles || pairs > w.cap_pairs || bmp_grow;
+size_t axis_bytes(int n, long long rows) { return 4 * (size_t)rows * (size_t)bitmap_words(std::max(n, 1)); }
+
+fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx, int ty, long long pairs) {
+  const int n_tiles = tx * ty;
+  // bit rows for an image's tiles, or for lists of any number of tiles (bin_sort)
+  const bool image = tx <= kMaxTileRows && ty <= kMaxTileRows;
+  const bool bits = image || (c->binning != FS4D_BINNING_SORT && bitmap_bytes(n, (long long)tx * ty) <= kBitmapMaxBytes);
+  const long long rows = std::max(bits ? (long long)tx + ty : 0ll, w.cap_rows);
+  const size_t axis = axis_bytes(std::max(n, w.cap_n), rows);
+  const size_t order = 4 * (size_t)n_tiles * (image ? 32 : 1);  // 32 length classes
+  const bool grow = n > w.cap_n || n_tiles > w.cap_tiles || pairs > w.cap_pairs || axis > w.axis.bytes ||
+                    order > w.tile_order.bytes;
   if (!grow) return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(stream));
   if (n > w.cap_n) {
@@ -558,8 +566,8 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int n_
     FS4D_CUDA(c, ensure(w.sxy, 8 * m));
     FS4D_CUDA(c, ensure(w.sco, 16 * m));
     FS4D_CUDA(c, ensure(w.srgb, 12 * m));
+    FS4D_CUDA(c, ensure(w.srect, 16 * m));
     FS4D_CUDA(c, ensure(w.offsets, 4 * m));
-    FS4D_CUDA(c, ensure(w.emit_lb, 8 * (size_t)(emit_parts(n) + 1)));
     FS4D_CUDA(c, ensure(w.dkeys, 8 * m));
     FS4D_CUDA(c, ensure(w.dvals, 4 * m));
     FS4D_CUDA(c, ensure(w.dkeys_alt, 8 * m));
@@ -567,12 +575,9 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int n_
     w.cap_n = n;
   }
   FS4D_CUDA(c, ensure(w.counters, 4 * kCounters));
-  FS4D_CUDA(c, ensure(w.num_pairs, 4 * 4));
   FS4D_CUDA(c, ensure(w.hist, 4 * 256 * kSortMaxPasses));
   if (n_tiles > w.cap_tiles) {
     FS4D_CUDA(c, ensure(w.ranges, 8 * (size_t)n_tiles));
-    FS4D_CUDA(c, ensure(w.tile_count, 4 * (size_t)n_tiles));
-    FS4D_CUDA(c, ensure(w.tile_order, 4 * (size_t)n_tiles));
     w.cap_tiles = n_tiles;
   }
   if (pairs > w.cap_pairs) {
@@ -591,23 +596,20 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int n_
   const size_t zb = frame_zero_layout(w.cap_n, w.cap_tiles, w.cap_pairs,
                                       sort_passes(ceil_log2(std::max(w.cap_tiles, 1))), nullptr, nullptr);
   FS4D_CUDA(c, ensure(w.zero, zb));
-  if (bmp_grow) {  // zeroed once here; every frame that sets bits clears them again
-    FS4D_CUDA(c, ensure(w.bitmap, bmp_need));
-    FS4D_CUDA(c, cudaMemsetAsync(w.bitmap.p, 0, w.bitmap.bytes, stream));
-    w.bmp_dirty = false;
-    FS4D_CUDA(c, cudaStreamSynchronize(stream));
-  }
+  w.cap_rows = rows;
+  FS4D_CUDA(c, ensure(w.axis, axis));
+  FS4D_CUDA(c, ensure(w.tile_order, order));
   return FS4D_OK;
 }
 
-// Whether a frame of n Gaussians over n_tiles tiles bins through w's bitmap.
-bool use_bitmap(const fs4d_ctx* c, const Work& w, int n, int n_tiles, bool offsets) {
-  const size_t b = bitmap_bytes(n, n_tiles);
-  return c->binning != FS4D_BINNING_SORT && !offsets && n > 0 && b <= kBitmapMaxBytes && b <= w.bitmap.bytes;
+// Whether a frame of n Gaussians over tx x ty tiles has tile lists from column and row bits.
+bool use_lists(const fs4d_ctx* c, const Work& w, int n, int tx, int ty) {
+  return c->binning != FS4D_BINNING_SORT && n > 0 && bitmap_bytes(n, (long long)tx * ty) <= kBitmapMaxBytes &&
+         axis_bytes(n, (long long)tx + ty) <= w.axis.bytes;
 }
 
-fs4d_status ensure_work(fs4d_ctx* c, int n, int n_tiles, long long pairs) {
-  return ensure_work(c, c->w, c->stream, n, n_tiles, pairs);
+fs4d_status ensure_work(fs4d_ctx* c, int n, int tx, int ty, long long pairs) {
+  return ensure_work(c, c->w, c->stream, n, tx, ty, pairs);
 }
 
 SortWork sort_work(Work& w) {
@@ -621,6 +623,24 @@ SortWork sort_work(Work& w) {
 
 SortWork sort_work(fs4d_ctx* c) {
   SortWork sw = sort_work(c->w);
+  sw.spin_limit = c->spin_limit;
+  return sw;
+}
+
+// The depth sort's and the pair sort's share of a frame's zeroed state (counters: words
+// 0..7 emission, 8..24 depth sort, 32..48 pair sort, 56 grid barrier, 64..95 length classes).
+SortWork depth_sort_work(const fs4d_ctx* c, const FrameZero& z) {
+  SortWork sw;
+  sw.hist = z.hist; sw.lookback = z.dlb; sw.part_counters = z.counters + 8; sw.max_parts = z.dparts;
+  sw.prezeroed = true;
+  sw.spin_limit = c->spin_limit;
+  sw.grid_counter = z.counters + 56;
+  return sw;
+}
+SortWork pair_sort_work(const fs4d_ctx* c, const FrameZero& z) {
+  SortWork sw;
+  sw.hist = z.hist; sw.lookback = z.plb; sw.part_counters = z.counters + 32; sw.max_parts = z.pparts;
+  sw.prezeroed = true;
   sw.spin_limit = c->spin_limit;
   return sw;
 }
@@ -690,8 +710,6 @@ fs4d_status run_deform(fs4d_ctx* c, Scene* s, fs4d_precision prec, const DeformA
 }
 
 // Everything of a frame up to (and including) the key emission.
-// offsets: keep each Gaussian's emission offset (the backward's pair slots), which
-// only the key emission produces.
 // One scene's share of a frame's Gaussian set: its deformed Gaussians and
 // projections sit at [off, off + n) of the work arrays; shift translates the
 // scene in the world (composition, Sec. 5.4: G' = {G'_1, ..., G'_n}).
@@ -756,7 +774,8 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
   const int N = (int)parts_total(parts, n_parts);
   // every buffer the frame needs at zero, in one allocation (cleared below)
   FrameZero& z = w.z;
-  frame_zero_layout(N, tx * ty, cap, sort_passes(tile_bits), static_cast<unsigned char*>(w.zero.p), &z);
+  w.bmp = use_lists(c, w, N, tx, ty);
+  frame_zero_layout(N, tx * ty, cap, w.bmp ? 0 : sort_passes(tile_bits), static_cast<unsigned char*>(w.zero.p), &z);
   if (z.bytes > w.zero.bytes) return fail(c, FS4D_ERR_INVALID_ARG, "frame work memory was not reserved");
   mark(e, 0);
   for (int i = 0; i < n_parts; ++i)
@@ -803,13 +822,8 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
   mark(e, 2);
   // Gaussians in (float32 depth, index) order: the emission order
   bool dalt = false;
-  SortWork dsw;
-  dsw.hist = z.hist; dsw.lookback = z.dlb; dsw.part_counters = z.counters + 8; dsw.max_parts = z.dparts;
-  dsw.prezeroed = true;
-  dsw.spin_limit = c->spin_limit;
-  dsw.grid_counter = z.counters + 56;  // (words 0..7 emission, 8..24 this sort, 32..48 the pair sort)
   FS4D_CUDA(c, launch_sort(P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), P<unsigned long long>(w.dkeys_alt),
-                           P<uint32_t>(w.dvals_alt), nullptr, N, 0, 32, true, dsw, e.status, stream, &dalt,
+                           P<uint32_t>(w.dvals_alt), nullptr, N, 0, 32, true, depth_sort_work(c, z), e.status, stream, &dalt,
                            dsel));
   mark(e, 3);
   return FS4D_OK;
@@ -817,11 +831,12 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
 
 // Everything of a frame up to (and including) the key emission, over the union of
 // the parts' Gaussians.
+// saved: keep what the backward needs (each Gaussian's pair slots).
 // cull: the tile lists may leave out Gaussians that no pixel of the tile blends
 // (same image; list positions, and so last-contributor indices, differ).
 fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_precision prec,
                         const fs4d_camera& shape, const fs4d_camera* d_cam, const float* d_t, float t, long long cap,
-                        bool report, bool deform, bool offsets, bool cull = false) {
+                        bool report, bool deform, bool saved, bool cull = false) {
   fs4d_ctx* c = e.c;
   Work& w = *e.w;
   const cudaStream_t stream = e.s;
@@ -847,33 +862,37 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
   ea.status = e.status;
   ea.spin_limit = c->spin_limit;
   ea.report_overflow = report ? 1 : 0;
-  w.bmp = use_bitmap(c, w, N, tx * ty, offsets);
   // a frame kept for the backward needs each pair's (key, value) slots; any other
   // sorts one 8-byte (tile | Gaussian index) word per pair (16 instead of 24 bytes
   // per pair per pass)
-  w.packed = !w.bmp && !offsets;
+  w.packed = !w.bmp && !saved;
   ea.packed = w.packed ? 1 : 0;
 
   if (e.w == &c->w) c->last_binning = w.bmp ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
-  if (w.bmp) {
-    // bits per (tile, depth rank) and the projected Gaussians copied into rank order;
-    // ranges and launch order from the tile counts; each tile's row read in rank
-    // order is its list of depth ranks (no keys: the composite needs none)
-    ea.bitmap = P<uint32_t>(w.bitmap);
-    ea.words = bitmap_words(N);
-    ea.keys = nullptr;
-    ea.ranges = P<uint2>(w.ranges);
-    ea.tile_order = P<uint32_t>(w.tile_order);
-    ea.xy = P<float2>(w.xy); ea.conic_opacity = P<float4>(w.co); ea.rgb = P<float>(w.rgb);
-    ea.sorted_xy = P<float2>(w.sxy); ea.sorted_co = P<float4>(w.sco); ea.sorted_rgb = P<float>(w.srgb);
-    ea.cull = cull ? 1 : 0;  // bitmap frames only: the emission keeps the full rectangles
-    if (w.bmp_dirty) FS4D_CUDA(c, cudaMemsetAsync(w.bitmap.p, 0, w.bitmap.bytes, stream));
-    w.bmp_dirty = true;  // until the extraction (which clears every bit it reads) is launched
-    FS4D_CUDA(c, launch_mark_tiles(ea, stream));
-    FS4D_CUDA(c, launch_tile_scan(z.tile_count, tx * ty, z.num_pairs, P<uint2>(w.ranges), nullptr, 0,
-                                  P<uint32_t>(w.tile_order), stream, cap, report ? e.status : nullptr));
-    FS4D_CUDA(c, launch_extract_tiles(ea, false, stream));
-    w.bmp_dirty = false;
+  if (w.bmp) {  // lists of depth ranks into rank-ordered copies of the projected Gaussians
+    ListArgs la{};
+    la.n = N; la.order = ea.order; la.order_alt = ea.order_alt; la.order_sel = dsel;
+    la.rect = ea.rect; la.xy = P<float2>(w.xy); la.conic_opacity = P<float4>(w.co); la.rgb = P<float>(w.rgb);
+    la.tiles_x = tx; la.tiles_y = ty; la.n_tiles = tx * ty;
+    la.words = bitmap_words(N);
+    la.bits = P<uint32_t>(w.axis);
+    la.s_rect = P<int4>(w.srect); la.s_xy = P<float2>(w.sxy); la.s_co = P<float4>(w.sco);
+    la.s_rgb = P<float>(w.srgb);
+    la.cull = cull ? 1 : 0;
+    if (saved) {
+      la.offsets = ea.offsets;
+      la.s_slot = P<int4>(w.sslot);
+    }
+    la.num_pairs = z.num_pairs;
+    la.capacity = cap;
+    la.values = ea.values;
+    la.ranges = P<uint2>(w.ranges);
+    la.class_count = z.counters + 64;
+    la.class_tiles = P<uint32_t>(w.tile_order);
+    la.status = e.status;
+    la.report_overflow = report ? 1 : 0;
+    FS4D_CUDA(c, launch_tile_bits(la, stream));
+    FS4D_CUDA(c, launch_tile_lists(la, stream));
   } else {
     FS4D_CUDA(c, launch_scan_emit(ea, stream));
     // tile ranges and the pair sort's digit histograms straight from the tile counts
@@ -886,15 +905,15 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
 
 fs4d_status frame_front(const Env& e, Scene* s, fs4d_precision prec, const fs4d_camera& shape,
                         const fs4d_camera* d_cam, const float* d_t, float t, long long cap, bool report,
-                        bool deform = true, bool offsets = false, bool cull = false) {
+                        bool deform = true, bool saved = false, bool cull = false) {
   const FramePart part{s, 0, {0.f, 0.f, 0.f}};
-  return frame_front(e, &part, 1, prec, shape, d_cam, d_t, t, cap, report, deform, offsets, cull);
+  return frame_front(e, &part, 1, prec, shape, d_cam, d_t, t, cap, report, deform, saved, cull);
 }
 
 fs4d_status frame_front(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera& shape,
                         const fs4d_camera* d_cam, const float* d_t, float t, long long cap, bool report,
-                        bool offsets = false, bool cull = false) {
-  return frame_front(env_of(c), s, prec, shape, d_cam, d_t, t, cap, report, true, offsets, cull);
+                        bool saved = false, bool cull = false) {
+  return frame_front(env_of(c), s, prec, shape, d_cam, d_t, t, cap, report, true, saved, cull);
 }
 
 // Sort, ranges and composite with n_dev = the sortable pair count on device.
@@ -910,14 +929,10 @@ fs4d_status frame_back(const Env& e, const fs4d_camera& shape, long long n_bound
   mark(e, 5);
   if (!w.bmp) {
     // pairs arrive in depth order: a stable sort on the tile bits gives (tile, depth, index)
-    SortWork psw;
-    psw.hist = z.hist; psw.lookback = z.plb; psw.part_counters = z.counters + 32; psw.max_parts = z.pparts;
-    psw.prezeroed = true;
-    psw.spin_limit = c->spin_limit;
     if (sort_parts(n_bound) > z.pparts) return fail(c, FS4D_ERR_INVALID_ARG, "pair bound above the frame's capacity");
     FS4D_CUDA(c, launch_sort(P<unsigned long long>(w.keys), w.packed ? nullptr : P<uint32_t>(w.values),
                              P<unsigned long long>(w.keys_alt), w.packed ? nullptr : P<uint32_t>(w.values_alt), n_dev,
-                             n_bound, 32, tile_bits, true, psw, e.status, e.s, &alt));
+                             n_bound, 32, tile_bits, true, pair_sort_work(c, z), e.status, e.s, &alt));
   }
   // packed: the Gaussian index is the low word of each sorted 64-bit key
   uint32_t* values = w.packed ? reinterpret_cast<uint32_t*>(alt ? P<unsigned long long>(w.keys_alt)
@@ -925,11 +940,20 @@ fs4d_status frame_back(const Env& e, const fs4d_camera& shape, long long n_bound
                               : (alt ? P<uint32_t>(w.values_alt) : P<uint32_t>(w.values));
   if (values_out) *values_out = w.packed ? nullptr : values;
   mark(e, 6);
-  // with the bitmap the lists hold depth ranks into the rank-ordered copies
+  TileOrder order;
+  order.n_tiles = tx * ty;
+  if (w.bmp) {  // the lists hold depth ranks into the rank-ordered copies
+    order.class_count = z.counters + 64;
+    order.class_tiles = P<uint32_t>(w.tile_order);
+    order.listed = z.num_pairs + 1;
+    order.capacity = n_bound;
+  } else {
+    order.order = P<uint32_t>(w.tile_order);
+  }
   FS4D_CUDA(c, launch_composite(shape.width, shape.height, P<uint2>(w.ranges), values,
                                 w.bmp ? P<float2>(w.sxy) : P<float2>(w.xy), w.bmp ? P<float4>(w.sco) : P<float4>(w.co),
                                 w.bmp ? P<float>(w.srgb) : P<float>(w.rgb), d_image, d_t_final, d_n_contrib, e.s,
-                                P<uint32_t>(w.tile_order), w.packed ? 2 : 1));
+                                order, w.packed ? 2 : 1));
   mark(e, 7);
   return FS4D_OK;
 }
@@ -974,17 +998,15 @@ BandTab band_tab(const fs4d_camera* cam, const std::vector<std::pair<int, int>>&
 }
 
 // Device memory of the frames composited straight from the depth order.
-fs4d_status ensure_direct(fs4d_ctx* c, int n, int tiles_x, int tiles_y) {
+fs4d_status ensure_direct(fs4d_ctx* c, int n) {
   Work& w = c->w;
-  const size_t m = (size_t)n, bits = 4 * (size_t)(tiles_x + tiles_y) * (size_t)bitmap_words(n);
-  if (w.yparts.bytes >= 8 * m && w.spos.bytes >= 16 * m && w.srg.bytes >= 8 * m && w.axis.bytes >= bits &&
-      w.band_pairs.bytes > 0)
+  const size_t m = (size_t)n;
+  if (w.yparts.bytes >= 8 * m && w.spos.bytes >= 16 * m && w.srg.bytes >= 8 * m && w.band_pairs.bytes > 0)
     return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
   FS4D_CUDA(c, ensure(w.yparts, 8 * m));
   FS4D_CUDA(c, ensure(w.spos, 16 * m));
   FS4D_CUDA(c, ensure(w.srg, 8 * m));
-  FS4D_CUDA(c, ensure(w.axis, bits));
   FS4D_CUDA(c, ensure(w.band_pairs, 8 * kMaxTileRows));
   if (!c->h_band_pairs) FS4D_CUDA(c, cudaMallocHost(&c->h_band_pairs, 8 * kMaxTileRows));
   return FS4D_OK;
@@ -1014,7 +1036,7 @@ fs4d_status render_direct(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d
   Work& w = c->w;
   const Env e = env_of(c);
   const int rows = tiles_of(cam->height), tx = tiles_of(cam->width);
-  fs4d_status st = ensure_direct(c, s->n, tx, rows);
+  fs4d_status st = ensure_direct(c, s->n);
   if (st != FS4D_OK) return st;
   c->last_binning = FS4D_BINNING_SORT;
   const uint32_t* dsel = nullptr;
@@ -1115,15 +1137,15 @@ fs4d_status frame_queue(const Env& e, const fs4d_camera& cam, float* d_image, fl
 
 fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t, float* d_image,
                         float* d_t_final, int32_t* d_n_contrib) {
-  const int n_tiles = tiles_of(cam->width) * tiles_of(cam->height);
-  fs4d_status st = ensure_work(c, s->n, n_tiles, c->w.cap_pairs);
+  const int tx = tiles_of(cam->width), ty = tiles_of(cam->height);
+  fs4d_status st = ensure_work(c, s->n, tx, ty, c->w.cap_pairs);
   if (st != FS4D_OK) return st;
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
   c->stage_acc_valid = false;
   c->last_bands = 1;
   // too many tiles x Gaussians for the tile bitmap, or more pairs than a band may hold last time
   const bool banded = c->band_hint > 1 && c->band_scene == s->id && c->band_w == cam->width && c->band_h == cam->height;
-  if (banded || (c->binning != FS4D_BINNING_SORT && !use_bitmap(c, c->w, s->n, n_tiles, false)))
+  if (banded || (c->binning != FS4D_BINNING_SORT && !use_lists(c, c->w, s->n, tx, ty)))
     return render_direct(c, s, prec, cam, t, true, d_image, d_t_final, d_n_contrib);
   const bool cull = !d_n_contrib;  // lists may drop Gaussians unless the frame reports list positions
   for (int pass = 0;; ++pass) {
@@ -1148,7 +1170,7 @@ fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_c
     c->last_pairs = K;
     if (K <= c->w.cap_pairs && c->w.cap_pairs > 0) return FS4D_OK;
     if (pass > 0) return fail(c, FS4D_ERR_CAPACITY, "render: the frame's pairs changed between two passes");
-    if ((st = ensure_work(c, s->n, n_tiles, std::max(std::min(K + K / 4, c->band_pairs), 1ll))) != FS4D_OK) return st;
+    if ((st = ensure_work(c, s->n, tx, ty, std::max(std::min(K + K / 4, c->band_pairs), 1ll))) != FS4D_OK) return st;
   }
 }
 
@@ -1156,7 +1178,7 @@ constexpr size_t kSpareFrames = 2;
 
 void release_frame(fs4d_frame& f) {
   DevBuf* all[] = {&f.dmeans, &f.dquats, &f.dscales, &f.xy, &f.co, &f.rgb, &f.radius, &f.rect, &f.offsets,
-                   &f.values, &f.ranges, &f.t_final, &f.n_contrib};
+                   &f.sco, &f.slot, &f.values, &f.ranges, &f.t_final, &f.n_contrib};
   for (DevBuf* b : all) release(*b);
 }
 
@@ -1173,7 +1195,7 @@ fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, siz
   const std::pair<DevBuf*, size_t> need[] = {
       {&f->dmeans, 12 * n}, {&f->dquats, 16 * n}, {&f->dscales, 12 * n}, {&f->xy, 8 * n},       {&f->co, 16 * n},
       {&f->rgb, 12 * n},    {&f->radius, 4 * n},  {&f->rect, 16 * n},    {&f->offsets, 4 * n},  {&f->values, 4 * pairs},
-      {&f->ranges, 8 * tiles}, {&f->t_final, 4 * npix}, {&f->n_contrib, 4 * npix}};
+      {&f->sco, 16 * n},    {&f->slot, 16 * n},   {&f->ranges, 8 * tiles}, {&f->t_final, 4 * npix}, {&f->n_contrib, 4 * npix}};
   bool grow = false, first = true;
   for (const auto& q : need) {
     grow = grow || q.first->bytes < q.second;
@@ -1191,16 +1213,15 @@ fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, siz
 // The frame's kernels write that state where it stays: they run on a view of the
 // work memory in which the frame's buffers stand in for the context's.
 fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t,
-                              float* d_image, fs4d_frame* f) {
+                              float* d_image, fs4d_frame* f, bool cull) {
   const size_t npix = (size_t)cam->width * cam->height;
-  const int n_tiles = tiles_of(cam->width) * tiles_of(cam->height);
+  const int tx = tiles_of(cam->width), ty = tiles_of(cam->height), n_tiles = tx * ty;
   const bool odd = sort_passes(ceil_log2(n_tiles)) & 1;  // passes of the pair sort: where its result lands
-  fs4d_status st = ensure_work(c, s->n, n_tiles, std::max(c->w.cap_pairs, 4096ll));
+  fs4d_status st = ensure_work(c, s->n, tx, ty, std::max(c->w.cap_pairs, 4096ll));
   if (st != FS4D_OK) return st;
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
   c->stage_acc_valid = false;
   c->last_bands = 1;
-  c->last_binning = FS4D_BINNING_SORT;
   if (f->stream != c->stream && f->dmeans.p) f->one_stream = false;
   f->stream = c->stream;
   f->device = c->device;
@@ -1208,11 +1229,19 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
     if ((st = ensure_frame(c, f, (size_t)s->n, (size_t)n_tiles, npix, (size_t)c->w.cap_pairs)) != FS4D_OK) return st;
     Work v = c->w;
     v.dmeans = f->dmeans; v.dquats = f->dquats; v.dscales = f->dscales;
-    v.xy = f->xy; v.co = f->co; v.rgb = f->rgb; v.radius = f->radius; v.rect = f->rect;
+    v.co = f->co; v.radius = f->radius; v.rect = f->rect;
     v.offsets = f->offsets; v.ranges = f->ranges;
-    (odd ? v.values_alt : v.values) = f->values;
+    f->ranks = use_lists(c, c->w, s->n, tx, ty);
+    if (f->ranks) {
+      v.sxy = f->xy; v.srgb = f->rgb; v.sco = f->sco; v.sslot = f->slot;
+      v.values = f->values;
+    } else {
+      v.xy = f->xy; v.rgb = f->rgb;
+      (odd ? v.values_alt : v.values) = f->values;
+    }
+    c->last_binning = f->ranks ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
     const Env e{c, &v, c->stream, P<uint32_t>(c->status), true};
-    if ((st = frame_front(e, s, prec, *cam, nullptr, nullptr, t, v.cap_pairs, false, true, true)) != FS4D_OK)
+    if ((st = frame_front(e, s, prec, *cam, nullptr, nullptr, t, v.cap_pairs, false, true, true, cull)) != FS4D_OK)
       return st;
     long long K = 0;
     uint32_t* values = nullptr;
@@ -1226,7 +1255,7 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
       break;
     }
     if (pass > 0) return fail(c, FS4D_ERR_CAPACITY, "render: the frame's pairs changed between two passes");
-    if ((st = ensure_work(c, s->n, n_tiles, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
+    if ((st = ensure_work(c, s->n, tx, ty, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
   }
   f->scene = s->id;
   f->cam = *cam;
@@ -1535,7 +1564,7 @@ fs4d_status render_impl(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision prec, cons
     f = new (std::nothrow) fs4d_frame();
   }
   if (!f) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
-  st = render_into_frame(c, s, prec, cam, t, d_image, f);
+  st = render_into_frame(c, s, prec, cam, t, d_image, f, !d_n_contrib);
   if (st == FS4D_OK && d_t_final)
     st = cudaMemcpyAsync(d_t_final, f->t_final.p, 4 * (size_t)cam->width * cam->height, cudaMemcpyDeviceToDevice,
                          c->stream) == cudaSuccess ? FS4D_OK : fail(c, FS4D_ERR_CUDA, "render: copy of T failed");
@@ -1581,8 +1610,8 @@ fs4d_status fs4d_render_composed(fs4d_ctx* c, const fs4d_scene_id* ids, const fl
   }
   if (N >= (1ll << 31) - 1) return fail(c, FS4D_ERR_CAPACITY, "render_composed: more than 2^31 - 2 Gaussians");
   DeviceGuard g(c->device);
-  const int n_tiles = tiles_of(cam->width) * tiles_of(cam->height);
-  fs4d_status st = ensure_work(c, (int)N, n_tiles, c->w.cap_pairs);
+  const int tx = tiles_of(cam->width), ty = tiles_of(cam->height);
+  fs4d_status st = ensure_work(c, (int)N, tx, ty, c->w.cap_pairs);
   if (st != FS4D_OK) return st;
   for (const FramePart& q : parts)
     if (q.s->color_heads && (st = ensure_color(c, c->w, c->stream, (int)N)) != FS4D_OK) return st;
@@ -1594,7 +1623,7 @@ fs4d_status fs4d_render_composed(fs4d_ctx* c, const fs4d_scene_id* ids, const fl
   if ((st = read_pairs(c, c->w.z.num_pairs, &K)) != FS4D_OK) return st;
   if (K > c->band_pairs) return fail(c, FS4D_ERR_CAPACITY, "render_composed: the frame's pairs exceed one band");
   if (K > c->w.cap_pairs) {
-    if ((st = ensure_work(c, (int)N, n_tiles, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
+    if ((st = ensure_work(c, (int)N, tx, ty, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
     st = frame_front(env_of(c), parts.data(), n_scenes, prec, *cam, nullptr, nullptr, t, c->w.cap_pairs, false, true,
                      false, !d_n_contrib);
     if (st != FS4D_OK) return st;
@@ -1622,8 +1651,7 @@ fs4d_status fs4d_render_host(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision prec,
   // back with the image, so one host synchronisation per frame suffices; a frame
   // whose pairs overflowed the capacity (its image is incomplete) is rendered again
   // with the capacity grown.
-  const int n_tiles = tiles_of(cam->width) * tiles_of(cam->height);
-  if ((st = ensure_work(c, s->n, n_tiles, c->w.cap_pairs)) != FS4D_OK) return st;
+  if ((st = ensure_work(c, s->n, tiles_of(cam->width), tiles_of(cam->height), c->w.cap_pairs)) != FS4D_OK) return st;
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
   const long long cap = c->w.cap_pairs;
   if ((st = frame_front(c, s, prec, *cam, nullptr, nullptr, t, cap, false, false, true)) != FS4D_OK) return st;
@@ -1674,8 +1702,8 @@ fs4d_status fs4d_render_host_batch(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision
       }
     }
   }
-  const int n_tiles = tiles_of(cams[0].width) * tiles_of(cams[0].height);
-  if ((st = ensure_work(c, s->n, n_tiles, c->w.cap_pairs)) != FS4D_OK) return st;
+  if ((st = ensure_work(c, s->n, tiles_of(cams[0].width), tiles_of(cams[0].height), c->w.cap_pairs)) != FS4D_OK)
+    return st;
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
   const long long cap = c->w.cap_pairs;
   float* slot_img[2] = {P<float>(img), P<float>(img) + bytes / 4};
@@ -1715,7 +1743,7 @@ fs4d_status fs4d_reserve(fs4d_ctx* c, fs4d_scene_id id, int32_t width, int32_t h
   fs4d_status st = get_scene(c, id, &s);
   if (st != FS4D_OK) return st;
   DeviceGuard g(c->device);
-  st = ensure_work(c, s->n, tiles_of(width) * tiles_of(height), pair_capacity);
+  st = ensure_work(c, s->n, tiles_of(width), tiles_of(height), pair_capacity);
   if (st == FS4D_OK && s->color_heads) st = ensure_color(c, c->w, c->stream, s->n);
   if (st != FS4D_OK) return st;
   s->reserved_pairs = pair_capacity;
@@ -1828,7 +1856,8 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   CompositeBwdArgs cb{};
   cb.width = f->cam.width; cb.height = f->cam.height; cb.tiles_x = tx;
   cb.ranges = P<uint2>(f->ranges); cb.values = P<uint32_t>(f->values);
-  cb.xy = P<float2>(f->xy); cb.conic_opacity = P<float4>(f->co); cb.rgb = P<float>(f->rgb);
+  cb.xy = P<float2>(f->xy); cb.conic_opacity = P<float4>(f->ranks ? f->sco : f->co);
+  if (f->ranks) cb.slot = P<int4>(f->slot); cb.rgb = P<float>(f->rgb);
   cb.rect = P<int4>(f->rect); cb.offsets = P<uint32_t>(f->offsets);
   cb.t_final = P<float>(f->t_final); cb.n_contrib = P<int>(f->n_contrib);
   cb.dl_dimage = d_dl_dimage; cb.grad_pair = P<float>(w.grad_pair);
@@ -2034,66 +2063,71 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
     return fail(c, FS4D_ERR_INVALID_ARG, "bin_sort: bad argument");
   DeviceGuard g(c->device);
   const int n_tiles = tiles_x * tiles_y;
-  fs4d_status st = ensure_work(c, std::max(n, 1), n_tiles, capacity);
+  fs4d_status st = ensure_work(c, std::max(n, 1), tiles_x, tiles_y, capacity);
   if (st != FS4D_OK) return st;
   Work& w = c->w;
   const int tile_bits = ceil_log2(n_tiles);
-  // emission order: Gaussians sorted by (float32 depth, index)
-  FS4D_CUDA(c, launch_depth_keys(d_depth, n, P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), c->stream));
+  const bool bmp = use_lists(c, w, n, tiles_x, tiles_y);
+  c->last_binning = bmp ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
+  // everything that starts at zero, as a frame's (frame_depth_order)
+  FrameZero& z = w.z;
+  frame_zero_layout(n, n_tiles, capacity, bmp ? 0 : sort_passes(tile_bits), static_cast<unsigned char*>(w.zero.p), &z);
+  if (z.bytes > w.zero.bytes) return fail(c, FS4D_ERR_INVALID_ARG, "bin_sort: work memory was not reserved");
+  FS4D_CUDA(c, cudaMemsetAsync(w.zero.p, 0, z.bytes, c->stream));
+  // Gaussians sorted by (float32 depth, index)
+  FS4D_CUDA(c, launch_depth_keys(d_depth, n, P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), z.hist, c->stream));
   bool dalt = false;
   const uint32_t* dsel = nullptr;
   FS4D_CUDA(c, launch_sort(P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), P<unsigned long long>(w.dkeys_alt),
-                           P<uint32_t>(w.dvals_alt), nullptr, n, 0, 32, false, sort_work(c), P<uint32_t>(c->status),
-                           c->stream, &dalt, &dsel));
-  FS4D_CUDA(c, cudaMemsetAsync(w.counters.p, 0, 4 * kEmitCounters, c->stream));
-  FS4D_CUDA(c, cudaMemsetAsync(w.num_pairs.p, 0, 16, c->stream));
-  FS4D_CUDA(c, cudaMemsetAsync(w.tile_count.p, 0, 4 * (size_t)n_tiles, c->stream));
-  FS4D_CUDA(c, cudaMemsetAsync(w.emit_lb.p, 0, 8 * (size_t)emit_parts(std::max(n, 1)), c->stream));
-  EmitArgs ea{};
-  ea.n = n; ea.order = P<uint32_t>(w.dvals); ea.order_alt = P<uint32_t>(w.dvals_alt); ea.order_sel = dsel;
-  ea.depth = d_depth; ea.rect = reinterpret_cast<const int4*>(d_rect); ea.tiles_x = tiles_x;
-  ea.capacity = capacity;
-  ea.keys = reinterpret_cast<unsigned long long*>(d_keys); ea.values = d_values;
-  ea.offsets = P<uint32_t>(w.offsets);
-  ea.lookback = P<unsigned long long>(w.emit_lb);
-  ea.part_counter = P<uint32_t>(w.counters);
-  ea.num_pairs = P<uint32_t>(w.num_pairs);
-  ea.num_pairs_sort = P<uint32_t>(w.num_pairs) + 1;
-  ea.tile_count = P<uint32_t>(w.tile_count);
-  ea.n_tiles = n_tiles;
-  ea.status = P<uint32_t>(c->status);
-  ea.spin_limit = c->spin_limit;
-  ea.report_overflow = 0;
-  const bool bmp = use_bitmap(c, w, n, n_tiles, false);
-  c->last_binning = bmp ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
-  if (bmp) {
-    ea.bitmap = P<uint32_t>(w.bitmap);
-    ea.words = bitmap_words(n);
-    ea.ranges = reinterpret_cast<const uint2*>(d_ranges);
-    if (w.bmp_dirty) FS4D_CUDA(c, cudaMemsetAsync(w.bitmap.p, 0, w.bitmap.bytes, c->stream));
-    w.bmp_dirty = true;
-    FS4D_CUDA(c, launch_mark_tiles(ea, c->stream));
-    FS4D_CUDA(c, launch_tile_scan(P<uint32_t>(w.tile_count), n_tiles, P<uint32_t>(w.num_pairs),
-                                  reinterpret_cast<uint2*>(d_ranges), nullptr, 0, nullptr, c->stream, capacity));
-    FS4D_CUDA(c, launch_extract_tiles(ea, true, c->stream));  // also clears the bitmap when the pairs overflow
-    w.bmp_dirty = false;
+                           P<uint32_t>(w.dvals_alt), nullptr, n, 0, 32, true, depth_sort_work(c, z),
+                           P<uint32_t>(c->status), c->stream, &dalt, &dsel));
+  const int4* rect = reinterpret_cast<const int4*>(d_rect);
+  uint2* ranges = reinterpret_cast<uint2*>(d_ranges);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(d_keys);
+  if (bmp) {  // lists of depth ranks in the work memory, then copied in tile order
+    ListArgs la{};
+    la.n = n; la.order = P<uint32_t>(w.dvals); la.order_alt = P<uint32_t>(w.dvals_alt); la.order_sel = dsel;
+    la.rect = rect; la.depth = d_depth;
+    la.tiles_x = tiles_x; la.tiles_y = tiles_y; la.n_tiles = n_tiles;
+    la.words = bitmap_words(n);
+    la.bits = P<uint32_t>(w.axis); la.s_rect = P<int4>(w.srect);
+    la.num_pairs = z.num_pairs;
+    la.capacity = std::min<long long>(w.cap_pairs, capacity);
+    la.values = P<uint32_t>(w.values); la.ranges = P<uint2>(w.ranges);
+    la.tile_count = z.tile_count;
+    FS4D_CUDA(c, launch_tile_bits(la, c->stream));
+    FS4D_CUDA(c, launch_tile_lists(la, c->stream));
+    FS4D_CUDA(c, launch_tile_scan(z.tile_count, n_tiles, z.num_pairs, ranges, nullptr, 0, nullptr, c->stream, capacity));
+    FS4D_CUDA(c, launch_tile_keys(la, ranges, d_values, keys, c->stream));
   } else {
+    EmitArgs ea{};
+    ea.n = n; ea.order = P<uint32_t>(w.dvals); ea.order_alt = P<uint32_t>(w.dvals_alt); ea.order_sel = dsel;
+    ea.depth = d_depth; ea.rect = rect; ea.tiles_x = tiles_x;
+    ea.capacity = capacity;
+    ea.keys = keys; ea.values = d_values;
+    ea.offsets = P<uint32_t>(w.offsets);
+    ea.lookback = z.emit_lb;
+    ea.part_counter = z.counters;
+    ea.num_pairs = z.num_pairs;
+    ea.num_pairs_sort = z.num_pairs + 1;
+    ea.tile_count = z.tile_count;
+    ea.n_tiles = n_tiles;
+    ea.status = P<uint32_t>(c->status);
+    ea.spin_limit = c->spin_limit;
     FS4D_CUDA(c, launch_scan_emit(ea, c->stream));
-    FS4D_CUDA(c, launch_tile_scan(P<uint32_t>(w.tile_count), n_tiles, P<uint32_t>(w.num_pairs),
-                                  reinterpret_cast<uint2*>(d_ranges), P<uint32_t>(w.hist), sort_passes(tile_bits),
-                                  nullptr, c->stream));
+    FS4D_CUDA(c, launch_tile_scan(z.tile_count, n_tiles, z.num_pairs, ranges, z.hist, sort_passes(tile_bits), nullptr,
+                                  c->stream));
   }
   long long K = 0;
-  if ((st = read_pairs(c, P<uint32_t>(w.num_pairs), &K)) != FS4D_OK) return st;
+  if ((st = read_pairs(c, z.num_pairs, &K)) != FS4D_OK) return st;
   *h_num_pairs = K;
   if (K > capacity) {
     return fail(c, FS4D_ERR_CAPACITY, "bin_sort: " + std::to_string(K) + " pairs exceed the capacity");
   }
   if (bmp) return FS4D_OK;
   bool alt = false;
-  FS4D_CUDA(c, launch_sort(reinterpret_cast<unsigned long long*>(d_keys), d_values, P<unsigned long long>(w.keys_alt),
-                           P<uint32_t>(w.values_alt), nullptr, K, 32, tile_bits, true, sort_work(c),
-                           P<uint32_t>(c->status), c->stream, &alt));
+  FS4D_CUDA(c, launch_sort(keys, d_values, P<unsigned long long>(w.keys_alt), P<uint32_t>(w.values_alt), nullptr, K, 32,
+                           tile_bits, true, pair_sort_work(c, z), P<uint32_t>(c->status), c->stream, &alt));
   if (alt && K > 0) {
     FS4D_CUDA(c, cudaMemcpyAsync(d_keys, w.keys_alt.p, 8 * (size_t)K, cudaMemcpyDeviceToDevice, c->stream));
     FS4D_CUDA(c, cudaMemcpyAsync(d_values, w.values_alt.p, 4 * (size_t)K, cudaMemcpyDeviceToDevice, c->stream));
@@ -2107,7 +2141,7 @@ fs4d_status fs4d_sort_pairs(fs4d_ctx* c, int64_t n, int32_t key_bits, uint64_t* 
     return fail(c, FS4D_ERR_INVALID_ARG, "sort_pairs: bad argument");
   if (n == 0) return FS4D_OK;
   DeviceGuard g(c->device);
-  fs4d_status st = ensure_work(c, 1, 1, n);
+  fs4d_status st = ensure_work(c, 1, 1, 1, n);
   if (st != FS4D_OK) return st;
   Work& w = c->w;
   bool alt = false;
@@ -2301,11 +2335,11 @@ Slot* new_slot(fs4d_server* sv) {
 // Make the slot hold a frame of n Gaussians at w x h with `pairs` capacity.
 fs4d_status fit_slot(fs4d_server* sv, Slot* sl, int n, int w, int h, long long pairs) {
   fs4d_ctx* c = sv->c;
-  const void* before[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.bitmap.p};
-  fs4d_status st = ensure_work(c, sl->w, sl->stream, n, tiles_of(w) * tiles_of(h), pairs);
+  const void* before[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.axis.p};
+  fs4d_status st = ensure_work(c, sl->w, sl->stream, n, tiles_of(w), tiles_of(h), pairs);
   if (st != FS4D_OK) return st;
   if ((size_t)w * h * 12 > sl->image.bytes) FS4D_CUDA(c, ensure(sl->image, (size_t)w * h * 12));
-  const void* after[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.bitmap.p};
+  const void* after[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.axis.p};
   if (std::memcmp(before, after, sizeof(before)) != 0) {  // graphs captured on old buffers are stale
     cudaStreamSynchronize(sl->stream);
     for (auto& kv : sl->graphs) cudaGraphExecDestroy(kv.second);
@@ -2796,7 +2830,7 @@ fs4d_status fs4d_train_step(fs4d_trainer* tr, fs4d_precision prec, const fs4d_ca
   }
   float* losses = d_losses ? d_losses : P<float>(tr->losses);
   // 1. the frame, keeping the backward's state
-  if ((st = render_into_frame(c, s, prec, cam, t, P<float>(tr->image), &tr->frame)) != FS4D_OK) return st;
+  if ((st = render_into_frame(c, s, prec, cam, t, P<float>(tr->image), &tr->frame, true)) != FS4D_OK) return st;
   // 2. L1 loss and dL/dI (misaligned targets take the scalar path inside the kernel)
   FS4D_CUDA(c, launch_l1(P<float>(tr->image), d_target, (long long)pix3, P<float>(tr->dl), P<float>(tr->partial),
                          losses, c->stream));

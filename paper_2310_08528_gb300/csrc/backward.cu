@@ -123,8 +123,13 @@ __global__ void __launch_bounds__(kBatch) composite_bwd_kernel(CompositeBwdArgs 
       s_rgb[3 * threadIdx.x] = a.rgb[3 * g];
       s_rgb[3 * threadIdx.x + 1] = a.rgb[3 * g + 1];
       s_rgb[3 * threadIdx.x + 2] = a.rgb[3 * g + 2];
-      const int4 r = a.rect[g];
-      s_slot[threadIdx.x] = a.offsets[g] + (uint32_t)((ty - r.y) * (r.z - r.x) + (tx - r.x));
+      if (a.slot) {
+        const int4 r = a.slot[g];
+        s_slot[threadIdx.x] = (uint32_t)r.w + (uint32_t)((ty - r.y) * r.z + (tx - r.x));
+      } else {
+        const int4 r = a.rect[g];
+        s_slot[threadIdx.x] = a.offsets[g] + (uint32_t)((ty - r.y) * (r.z - r.x) + (tx - r.x));
+      }
       s_mask[threadIdx.x] = row_pair_mask(s_xy[threadIdx.x], cog, tx, ty);
     }
 #pragma unroll

@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) composite_kernel(int wid
                                                             const float4* __restrict__ conic_opacity,
                                                             const float* __restrict__ rgb, float* __restrict__ image,
                                                             float* __restrict__ t_final, int* __restrict__ n_contrib,
-                                                            const uint32_t* __restrict__ order, int vstride) {
+                                                            TileOrder to, int vstride) {
   // two staging buffers: batch i is staged while batch i - 1 may still be read
   __shared__ float4 s_g0b[2][kBatch];   // x, y, a2, c2
   __shared__ float4 s_g1b[2][kBatch];   // b2, opacity, red, green
@@ -156,15 +156,31 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) composite_kernel(int wid
   __shared__ uint8_t s_list[kWarps][kBatch];
   pdl_wait();
   pdl_trigger();
-  const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
-  const int tx = tile % tiles_x, ty = tile / tiles_x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int tile = (int)blockIdx.x;
+  bool empty = false;
+  if (to.order) {
+    tile = (int)to.order[blockIdx.x];
+  } else if (to.class_count) {  // each warp finds the CTA's place among the length classes
+    const uint32_t c = to.class_count[lane];
+    uint32_t incl = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += y;
+    }
+    const int cls = __ffs(__ballot_sync(0xffffffffu, incl > blockIdx.x)) - 1;
+    const uint32_t first = __shfl_sync(0xffffffffu, incl - c, cls);
+    tile = (int)to.class_tiles[(size_t)cls * to.n_tiles + (blockIdx.x - first)];
+    empty = (long long)*to.listed > to.capacity;
+  }
+  const int tx = tile % tiles_x, ty = tile / tiles_x;
   const int bx0 = tx * kTile + (warp & 1) * 8, by0 = ty * kTile + (warp >> 1) * 4;
   const int px = bx0 + (lane & 7), py = by0 + (lane >> 3);
   const bool inside = px < width && py < height;
   const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
   const uint2 range = ranges[tile];
-  const int n = (int)(range.y - range.x);
+  const int n = empty ? 0 : (int)(range.y - range.x);
 
   bool done = !inside;
   float T = 1.f, R = 0.f, G = 0.f, B = 0.f;
@@ -346,7 +362,7 @@ cudaError_t launch_composite_direct(const DirectArgs& a, float* image, float* t_
 
 cudaError_t launch_composite(int width, int height, const uint2* ranges, const uint32_t* values, const float2* xy,
                              const float4* conic_opacity, const float* rgb, float* image, float* t_final,
-                             int* n_contrib, cudaStream_t s, const uint32_t* order, int values_stride) {
+                             int* n_contrib, cudaStream_t s, const TileOrder& order, int values_stride) {
   const int tiles_x = (width + kTile - 1) / kTile, tiles_y = (height + kTile - 1) / kTile;
   if (tiles_x * tiles_y == 0) return cudaSuccess;
   if (t_final || n_contrib)

@@ -41,11 +41,11 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 extern thread_local unsigned long long g_kernel_launches;
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                              Args... args) {
+inline cudaError_t launch_pdl_2d(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                                 Args... args) {
   ++g_kernel_launches;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -57,6 +57,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned 
   cfg.attrs = attr;
   cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                              Args... args) {
+  return launch_pdl_2d(kernel, dim3(grid), block, smem, s, args...);
 }
 
 // Bounded spin limit for decoupled look-back waits (iterations of ~100 ns).  The
@@ -228,23 +234,6 @@ struct EmitArgs {
   uint32_t spin_limit;          // polls of the look-back wait before it gives up
   int packed;                   // 1: keys = (tile << 32) | Gaussian index, no values (the pairs
                                 // are sorted on the tile bits only and the index travels along)
-  // tile bitmap binning (launch_mark_tiles / launch_extract_tiles)
-  uint32_t* bitmap;             // [n_tiles][words], bit (i & 31) of word i >> 5 of row t: the
-                                // Gaussian of depth rank i touches tile t (all zero between frames)
-  int words;                    // words per row: bitmap_words(n)
-  const uint2* ranges;          // [n_tiles] tile [start, end) from the tile scan
-  const uint32_t* tile_order;   // NULL or a permutation of the tiles: extraction order
-  // with sorted_xy non-NULL, mark also copies the projected Gaussians into depth-rank order
-  const float2* xy;
-  const float4* conic_opacity;
-  const float* rgb;
-  float2* sorted_xy;            // [n]
-  float4* sorted_co;            // [n]
-  float* sorted_rgb;            // [n][3]
-  int cull;                     // 1 (mark): set a bit only for the tiles whose pixel centres the
-                                // Gaussian's ellipse {alpha >= 1/255} can reach.  The lists lose
-                                // Gaussians no pixel of the tile blends: the image is unchanged,
-                                // list positions are not the full rectangles'.
 };
 
 struct SortWork {
@@ -267,8 +256,10 @@ bool deform_bf16_supported(int feat_dim, int n_levels);
 cudaError_t launch_project(const ProjectArgs& a, cudaStream_t s);
 
 int emit_parts(int n);          // scan partitions of the emit kernel
-// keys[i] = float bits of depth[i] (upper word 0), vals[i] = i: input of the depth sort
-cudaError_t launch_depth_keys(const float* depth, int n, unsigned long long* keys, uint32_t* vals, cudaStream_t s);
+// keys[i] = float bits of depth[i] (upper word 0), vals[i] = i: input of the depth sort;
+// hist [4][256] (zeroed): byte histograms of the keys
+cudaError_t launch_depth_keys(const float* depth, int n, unsigned long long* keys, uint32_t* vals, uint32_t* hist,
+                              cudaStream_t s);
 cudaError_t launch_scan_emit(const EmitArgs& a, cudaStream_t s);
 // tile ranges (from the per-tile counts; all (0, 0) when num_pairs[1] == 0 < num_pairs[0]),
 // if hist != NULL the [passes][256] digit histograms of the pair sort on the tile bits, and
@@ -278,14 +269,47 @@ cudaError_t launch_scan_emit(const EmitArgs& a, cudaStream_t s);
 cudaError_t launch_tile_scan(const uint32_t* tile_count, int n_tiles, uint32_t* num_pairs, uint2* ranges,
                              uint32_t* hist, int passes, uint32_t* order, cudaStream_t s, long long capacity = -1,
                              uint32_t* status = nullptr);
-// Tile bitmap binning (the alternative to emission + pair sort when the bitmap is small):
-// mark sets the bit of every (tile, depth rank) pair and counts the pairs per tile
-// (tile_count, num_pairs[0]); after the tile scan, extract walks each tile's row in rank
-// order, writes the depth ranks at the tile's range -- or with ids the Gaussians (and
-// keys if non-NULL) -- and clears the row.
-int bitmap_words(int n);        // words per tile row (a multiple of 4)
-cudaError_t launch_mark_tiles(const EmitArgs& a, cudaStream_t s);
-cudaError_t launch_extract_tiles(const EmitArgs& a, bool ids, cudaStream_t s);
+// Tile lists from column and row bits (lists.cu), the alternative to emission + pair sort.
+struct ListArgs {
+  int n;
+  const uint32_t* order;        // depth order, as EmitArgs
+  const uint32_t* order_alt;
+  const uint32_t* order_sel;
+  const int4* rect;
+  const float2* xy;
+  const float4* conic_opacity;
+  const float* rgb;
+  const float* depth;
+  int tiles_x, tiles_y, n_tiles;
+  int words;                    // 32-bit words per bit row: bitmap_words(n)
+  uint32_t* bits;               // [tiles_x + tiles_y][words]
+  int4* s_rect;                 // [n] by depth rank
+  float2* s_xy;                 // [n] by depth rank, NULL: lists of Gaussians (bin_sort), else
+  float4* s_co;                 //   lists of depth ranks into these copies
+  float* s_rgb;                 // [n][3]
+  int cull;                     // 1: cut the rectangles to the tiles that the bounding box of the ellipse
+                                // {alpha >= 1/255} reaches.  The lists lose Gaussians no pixel of the tile
+                                // blends: the image is unchanged, list positions are not the full
+                                // rectangles'.
+  uint32_t* offsets;            // optional [n]: each Gaussian's first slot (one slot per tile of its rectangle)
+  int4* s_slot;                 // with offsets: [n] by depth rank: x0, y0, width of the rectangle, first slot
+  uint32_t* num_pairs;          // [0] += pairs of the rectangles, [1] += pairs listed (zeroed)
+  long long capacity;           // pairs `values` holds
+  uint32_t* values;
+  uint2* ranges;                // [n_tiles]
+  uint32_t* tile_count;         // optional [n_tiles]: pairs listed per tile
+  uint32_t* class_count;        // optional [32] (zeroed): tiles per length class, longest first
+  uint32_t* class_tiles;        // [32][n_tiles]
+  uint32_t* status;
+  int report_overflow;          // set kStatusCapacity in *status when num_pairs[1] > capacity
+};
+int bitmap_words(int n);        // words per bit row (a multiple of 4)
+cudaError_t launch_tile_bits(const ListArgs& a, cudaStream_t s);      // gather and bit rows
+// Lists of depth ranks and length classes (num_pairs[1] > capacity afterwards: not complete).
+cudaError_t launch_tile_lists(const ListArgs& a, cudaStream_t s);
+// ... copied as Gaussians and keys ((tile << 32) | depth bits) to the ranges `out`.
+cudaError_t launch_tile_keys(const ListArgs& a, const uint2* out, uint32_t* values, unsigned long long* keys,
+                             cudaStream_t s);
 
 // ---- Frames composited straight from the depth order (direct.cu, composite.cu).
 // A tile rectangle is a column interval times a row interval, so the depth ranks of
@@ -339,11 +363,21 @@ cudaError_t launch_sort(unsigned long long* keys, uint32_t* values, unsigned lon
                         uint32_t* values_alt, const uint32_t* n_dev, long long n_bound, int first_bit,
                         int key_bits, bool hist_ready, const SortWork& work, uint32_t* status, cudaStream_t s,
                         bool* result_in_alt, const uint32_t** result_sel = nullptr);
-// order (optional): CTA i composites tile order[i]; values_stride: 1 for a list of
-// uint32 indices, 2 for the low words of packed (tile | index) 64-bit keys
+// Launch order of the compositing: CTA i takes tile order[i], or the i-th tile of the
+// length classes (ListArgs; nothing is listed when *listed > capacity), or tile i.
+struct TileOrder {
+  const uint32_t* order = nullptr;
+  const uint32_t* class_count = nullptr;
+  const uint32_t* class_tiles = nullptr;
+  int n_tiles = 0;
+  const uint32_t* listed = nullptr;
+  long long capacity = 0;
+};
+// values_stride: 1 for a list of uint32 indices, 2 for the low words of packed
+// (tile | index) 64-bit keys
 cudaError_t launch_composite(int width, int height, const uint2* ranges, const uint32_t* values,
                              const float2* xy, const float4* conic_opacity, const float* rgb, float* image,
-                             float* t_final, int* n_contrib, cudaStream_t s, const uint32_t* order = nullptr,
+                             float* t_final, int* n_contrib, cudaStream_t s, const TileOrder& order = TileOrder(),
                              int values_stride = 1);
 }  // namespace fs4d
 
@@ -396,6 +430,7 @@ struct CompositeBwdArgs {
   const float* rgb;
   const int4* rect;
   const uint32_t* offsets;
+  const int4* slot;         // with lists of depth ranks: x0, y0, width, first slot by rank (rect, offsets unused)
   const float* t_final;
   const int* n_contrib;
   const float* dl_dimage;   // [H][W][3]

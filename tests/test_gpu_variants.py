@@ -65,3 +65,31 @@ def test_fp32_deform_tiles_agree(n, levels):
             assert torch.equal(x[:, :n], y)
     finally:
         ctx.close()
+
+
+# up to 131072 Gaussians a tile's words stay in registers
+@pytest.mark.parametrize("n,tx,ty,side", [(131072, 50, 41, 3), (131073, 7, 300, 2), (393217, 33, 9, 2),
+                                          (700, 40, 30, 30), (3000, 700, 1, 40)])
+def test_lists_equal_sorted_pairs(n, tx, ty, side):
+    """Tile lists from column and row bits are the radix-sorted pairs: keys, values, ranges, count."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    lo = torch.stack([torch.randint(0, t, (n,), generator=g, device="cuda") for t in (tx, ty)], 1)
+    size = torch.randint(0, side + 1, (n, 2), generator=g, device="cuda")  # (0: no tiles)
+    hi = torch.minimum(lo + size, torch.tensor([tx, ty], device="cuda"))
+    rect = torch.cat([lo, hi], 1).int().contiguous()
+    depth = (torch.rand(n, generator=g, device="cuda") * 4).round(decimals=3).contiguous()  # with ties
+    cap = int((hi - lo).prod(1).sum())
+    ctx = fs4d.Context(0)
+    try:
+        ctx.set_binning(fs4d.BINNING_SORT)
+        want = [v.clone() if torch.is_tensor(v) else v for v in ctx.bin_sort(depth, rect, tx, ty, cap)]
+        ctx.set_binning(fs4d.BINNING_AUTO)
+        got = ctx.bin_sort(depth, rect, tx, ty, cap)
+        assert ctx.last_binning() == fs4d.BINNING_BITMAP
+        assert got[3] == want[3] == cap
+        for a, b in zip(got[:3], want[:3]):
+            assert torch.equal(a, b)
+        with pytest.raises(fs4d.Fs4dError):
+            ctx.bin_sort(depth, rect, tx, ty, cap - 1)
+    finally:
+        ctx.close()
