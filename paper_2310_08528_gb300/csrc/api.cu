@@ -1830,12 +1830,12 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   Work& w = c->w;
   const long long n = s->n, K = f->pairs;
   const int hin = s->mg.hin;
-  const size_t act_floats = (size_t)n * (hin + 64 + 64 + 192 + 10 + 192 + 64 + 64);
+  const size_t act_floats = mlp_act_floats(n, hin);
   size_t wtot = 0;
   {
     size_t tot_floats;
     auto Ls = src_layers(hin, kWidth, &tot_floats);
-    wtot = (size_t)tot_floats;  // every layer's O*I + O entries
+    wtot = (size_t)tot_floats + kWidth;  // every block's O*I + O entries (d1 may be two blocks)
   }
   const size_t wp = (size_t)wgrad_chunks(n) * wtot;
   if (w.grad_pair.bytes < 4 * kPairStride * (size_t)std::max(K, 1ll) || w.gd.bytes < 40 * (size_t)n ||
@@ -1882,15 +1882,8 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   MlpBwdArgs mb{};
   mb.f = deform_args(s, nullptr, f->t, 1, nullptr, nullptr, nullptr);
   mb.gd = P<float>(w.gd);
-  float* A = P<float>(w.acts);
-  mb.act.fh = A; A += (size_t)n * hin;
-  mb.act.a1 = A; A += (size_t)n * 64;
-  mb.act.fd = A; A += (size_t)n * 64;
-  mb.act.hid = A; A += (size_t)n * 192;
-  mb.act.dout = A; A += (size_t)n * 10;
-  mb.act.dh = A; A += (size_t)n * 192;
-  mb.act.d2 = A; A += (size_t)n * 64;
-  mb.act.d1 = A;
+  mb.act = mlp_acts(P<float>(w.acts), n, hin);
+  mb.mlp = P<float>(s->mlp);
   mb.g_planes = gr->planes;
   mb.g_means = gr->means;
   FS4D_CUDA(c, launch_mlp_bwd(mb, c->stream));
@@ -1903,14 +1896,16 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
     WgradArgs wa{};
     wa.n = n;
     wa.partial = P<float>(w.wpartial);
-    auto add = [&](const float* D, const float* X, int O, int I, const SrcLayer& l) {
-      wa.l[wa.n_layers++] = WgradLayer{D, X, O, I, gr->mlp + l.w, gr->mlp + l.b, 0};
+    // weights [0, O) x [i0, i0 + I) of a layer
+    auto add = [&](const float* D, int ldd, const float* X, int ldx, int O, int i0, int I, const SrcLayer& l) {
+      wa.l[wa.n_layers++] = WgradLayer{D, X + i0, ldd, ldx, O, I, gr->mlp + l.w + i0, l.in, i0 ? nullptr : gr->mlp + l.b, 0};
     };
-    add(mb.act.d1, mb.act.fh, 64, hin, L[0]);
-    add(mb.act.d2, mb.act.a1, 64, 64, L[1]);
+    const MlpActs& q = mb.act;
+    for (int i0 = 0; i0 < hin; i0 += 64) add(q.d1, 64, q.fh, hin, 64, i0, std::min(64, hin - i0), L[0]);
+    add(q.d2, 64, q.a1, 64, 64, 0, 64, L[1]);
     for (int h = 0; h < 3; ++h) {
-      add(mb.act.dh + (size_t)64 * h * n, mb.act.fd, 64, 64, L[2 + 2 * h]);
-      add(mb.act.dout + (size_t)col0[h] * n, mb.act.hid + (size_t)64 * h * n, L[3 + 2 * h].out, 64, L[3 + 2 * h]);
+      add(q.dh + 64 * h, 192, q.fd, 64, 64, 0, 64, L[2 + 2 * h]);
+      add(q.dout + col0[h], 12, q.hid + 64 * h, 192, L[3 + 2 * h].out, 0, 64, L[3 + 2 * h]);
     }
     FS4D_CUDA(c, launch_wgrad(wa, c->stream));
   }

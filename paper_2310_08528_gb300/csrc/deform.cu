@@ -136,7 +136,31 @@ __device__ __forceinline__ void head_out(const float* __restrict__ W2, const flo
   }
 }
 
-template <int H, int L, int TG, int GROUPS>
+// The recompute for the backward: the thread's activations (after ReLU) as rows of out and
+// a bit for each that is positive.
+template <int TG>
+__device__ __forceinline__ void put_acts(const float (&acc)[TG / 32][8], int o8, float* __restrict__ out, int ld,
+                                         long long row0, long long n, uint32_t* mask_word) {
+  uint32_t mask = 0;
+#pragma unroll
+  for (int g = 0; g < TG / 32; ++g) {
+    float v[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      v[o] = fmaxf(acc[g][o], 0.f);
+      mask |= v[o] > 0.f ? 1u << (8 * g + o) : 0u;
+    }
+    if (row0 + g < n) {
+      float4* q = reinterpret_cast<float4*>(out + (row0 + g) * ld + o8);
+      q[0] = make_float4(v[0], v[1], v[2], v[3]);
+      q[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+  }
+  *mask_word = mask;
+}
+
+// ACT: the backward's recompute (DeformArgs::act_masks).
+template <int H, int L, int TG, int GROUPS, bool ACT>
 __global__ void __launch_bounds__(GROUPS * kThreads, 1) deform_fp32_kernel(const __grid_constant__ DeformArgs a) {
   constexpr int HL = H * L;
   constexpr int XR = HL > kWidth ? HL : kWidth;
@@ -248,6 +272,8 @@ __global__ void __launch_bounds__(GROUPS * kThreads, 1) deform_fp32_kernel(const
         const float v = e == 0 ? f[0] : (e == 1 ? f[1] : (e == 2 ? f[2] : f[3]));
         dst[e * kGS] = v;
       }
+      if (ACT && gi < total)
+        *reinterpret_cast<float4*>(a.act_fh + gi * HL + l * H + 4 * q) = make_float4(f[0], f[1], f[2], f[3]);
     }
     if (!loaded) {  // every thread takes part in this barrier once, here or after the loop
       asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -261,10 +287,22 @@ __global__ void __launch_bounds__(GROUPS * kThreads, 1) deform_fp32_kernel(const
     layer64<HL, TG>(sw + mg.w[0], sw + mg.b[0], X, g0, o8, acc);
     group_bar(grp);
     store_relu<TG>(X, g0, o8, acc);
+    uint32_t* masks = ACT ? a.act_masks + tile * 5 * kThreads + gt : nullptr;
+    if (ACT) put_acts<TG>(acc, o8, a.act_a1, kWidth, base + g0, total, masks);
     group_bar(grp);
     layer64<kWidth, TG>(sw + mg.w[1], sw + mg.b[1], X, g0, o8, acc);
     group_bar(grp);
     store_relu<TG>(X, g0, o8, acc);
+    if constexpr (ACT) {
+      put_acts<TG>(acc, o8, a.fd_out, kWidth, base + g0, total, masks + kThreads);
+      group_bar(grp);
+#pragma unroll
+      for (int h = 0; h < 3; ++h) {
+        layer64<kWidth, TG>(sw + mg.w[2 + 2 * h], sw + mg.b[2 + 2 * h], X, g0, o8, acc);
+        put_acts<TG>(acc, o8, a.act_hid + kWidth * h, 3 * kWidth, base + g0, total, masks + (2 + h) * kThreads);
+      }
+      continue;  // (the next tile writes X after a barrier)
+    }
     group_bar(grp);
     if (a.fd_out) {  // f_d for the colour and opacity heads, rows in work order
       for (int e = gt; e < TG * kWidth; e += kThreads) {
@@ -315,14 +353,14 @@ __global__ void __launch_bounds__(GROUPS * kThreads, 1) deform_fp32_kernel(const
   }
 }
 
-template <int H, int L, int TG, int GROUPS>
+template <int H, int L, int TG, int GROUPS, bool ACT>
 cudaError_t launch_tg(const DeformArgs& a, cudaStream_t s) {
   constexpr size_t smem = smem_bytes(H * L, TG, GROUPS);
   static_assert(smem <= 227 * 1024, "one CTA's shared memory");
   if (a.mg.total != mlp_floats(H * L)) return cudaErrorInvalidValue;
   static PerDeviceFlag attr;
   cudaError_t e = once_per_device(attr, [&] {
-    return cudaFuncSetAttribute(deform_fp32_kernel<H, L, TG, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(deform_fp32_kernel<H, L, TG, GROUPS, ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem);
   });
   if (e != cudaSuccess) return e;
@@ -330,7 +368,7 @@ cudaError_t launch_tg(const DeformArgs& a, cudaStream_t s) {
   const long long total = (long long)a.n * a.n_t;
   const long long need = (total + TG - 1) / TG;
   const int grid = (int)(need < sms ? need : sms);
-  return launch_pdl(deform_fp32_kernel<H, L, TG, GROUPS>, grid, GROUPS * kThreads, smem, s, a);
+  return launch_pdl(deform_fp32_kernel<H, L, TG, GROUPS, ACT>, grid, GROUPS * kThreads, smem, s, a);
 }
 
 template <int H, int L>
@@ -339,8 +377,9 @@ cudaError_t launch_t(const DeformArgs& a, cudaStream_t s) {
   constexpr int kGroups = smem_bytes(H * L, 128, 2) <= 227 * 1024 ? 2 : 1;
   const long long total = (long long)a.n * a.n_t;
   // tiles of 32 while all of them run at once
-  if (total <= 64ll * device_sm_count()) return launch_tg<H, L, 32, 2>(a, s);
-  return launch_tg<H, L, 128, kGroups>(a, s);
+  if (a.act_masks) return launch_tg<H, L, 128, kGroups, true>(a, s);
+  if (total <= 64ll * device_sm_count()) return launch_tg<H, L, 32, 2, false>(a, s);
+  return launch_tg<H, L, 128, kGroups, false>(a, s);
 }
 
 }  // namespace

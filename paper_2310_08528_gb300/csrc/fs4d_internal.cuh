@@ -149,6 +149,12 @@ struct DeformArgs {
   PlaneGeom pg;
   uint32_t* status;
   float* fd_out;                // FP32 kernel, optional [n][64]: f_d (after phi_d) in work order (n_t must be 1)
+  // FP32 kernel, the backward's recompute (act_masks non-NULL; needs fd_out, writes no
+  // deformed Gaussians): the other activations and the ReLU bits, see MlpActs
+  float* act_fh;
+  float* act_a1;
+  float* act_hid;
+  uint32_t* act_masks;
   uint4* zero;                  // optional: zero_n16 16-byte words the kernel sets to 0 (a frame's counters
   long long zero_n16;           // and look-back tables, cleared here instead of by a separate memset)
   uint4* fd_tiles;              // BF16 kernel, optional: f_d of each tile of 128 work-order rows as its BF16
@@ -460,21 +466,26 @@ struct ProjectBwdArgs {
   float* stat_visible;      // += 1 where visible (nullable)
 };
 
-// Per-Gaussian activations and deltas of the deformation MLP, feature-major
-// ([feature][n]) so that each thread's writes coalesce across the warp.
+// Activations and deltas of the deformation MLP, a row per Gaussian in work order, and a
+// bit per ReLU ([tile of 128][a1, f_d, three heads][256 threads of the tile's group]).
 struct MlpActs {
-  float* fh;    // [HL][n]  layer d1 input
-  float* a1;    // [64][n]  layer d2 input
-  float* fd;    // [64][n]  head hidden-layer input
-  float* hid;   // [192][n] head output-layer inputs (x, r, s)
-  float* dout;  // [10][n]  output deltas
-  float* dh;    // [192][n] head hidden pre-activation deltas
-  float* d2;    // [64][n]
-  float* d1;    // [64][n]
+  float* fh;       // [n][HL]  layer d1 input
+  float* a1;       // [n][64]  layer d2 input
+  float* fd;       // [n][64]  head hidden-layer input
+  float* hid;      // [n][192] head output-layer inputs (x, r, s)
+  float* dout;     // [n][12]  output deltas (10 used)
+  float* dh;       // [n][192] head hidden pre-activation deltas
+  float* d2;       // [n][64]
+  float* d1;       // [n][64]
+  float* dfh;      // [n][HL]  dL/df_h
+  uint32_t* masks;
 };
+size_t mlp_act_floats(long long n, int hin);
+MlpActs mlp_acts(float* base, long long n, int hin);
 
 struct MlpBwdArgs {
   DeformArgs f;             // canonical scene, t0, planes, transposed MLP
+  const float* mlp;         // the MLP in the source layout
   const float* gd;          // [n][10]
   MlpActs act;
   float* g_planes;          // += (nullable)
@@ -484,19 +495,21 @@ struct MlpBwdArgs {
 cudaError_t launch_composite_bwd(const CompositeBwdArgs& a, cudaStream_t s);
 cudaError_t launch_project_bwd(const ProjectBwdArgs& a, cudaStream_t s);
 cudaError_t launch_mlp_bwd(const MlpBwdArgs& a, cudaStream_t s);
-// dW[o][i] += sum_n D[o][n] X[i][n], db[o] += sum_n D[o][n] for up to 8 layers in one launch, through
-// per-chunk partial sums (deterministic two-stage reduction).  W and b in the source layout
-// (W[out][in] then b); D [O][n], X [I][n] feature-major.
+// dW[o][i] += sum_n D[n][o] X[n][i], db[o] += sum_n D[n][o] for up to 9 blocks of at most
+// 64 x 64 weights in one launch, through per-chunk partial sums (deterministic two-stage
+// reduction).
 struct WgradLayer {
-  const float* D;
-  const float* X;
-  int O, I;
-  float* gW;
-  float* gb;
+  const float* D;      // rows of ldd floats
+  const float* X;      // rows of ldx floats
+  int ldd, ldx;
+  int O, I;            // O 64 or at most 4; I a multiple of 4, at most 64
+  float* gW;           // rows of ldw floats
+  int ldw;
+  float* gb;           // optional
   long long part_off;  // set by launch_wgrad
 };
 struct WgradArgs {
-  WgradLayer l[8];
+  WgradLayer l[9];
   int n_layers;
   long long n;
   int chunks;          // set by launch_wgrad
