@@ -1830,7 +1830,7 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   Work& w = c->w;
   const long long n = s->n, K = f->pairs;
   const int hin = s->mg.hin;
-  const size_t act_floats = mlp_act_floats(n, hin);
+  const size_t act_floats = mlp_act_floats(n, s->pg);
   size_t wtot = 0;
   {
     size_t tot_floats;
@@ -1882,7 +1882,7 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   MlpBwdArgs mb{};
   mb.f = deform_args(s, nullptr, f->t, 1, nullptr, nullptr, nullptr);
   mb.gd = P<float>(w.gd);
-  mb.act = mlp_acts(P<float>(w.acts), n, hin);
+  mb.act = mlp_acts(P<float>(w.acts), n, s->pg);
   mb.mlp = P<float>(s->mlp);
   mb.g_planes = gr->planes;
   mb.g_means = gr->means;

@@ -479,9 +479,11 @@ struct MlpActs {
   float* d1;       // [n][64]
   float* dfh;      // [n][HL]  dL/df_h
   uint32_t* masks;
+  float* lines;    // time planes' gradients before the time weights: copies of [3 axes][line_cells][h]
+  int line_cells;  // spatial cells of all levels
 };
-size_t mlp_act_floats(long long n, int hin);
-MlpActs mlp_acts(float* base, long long n, int hin);
+size_t mlp_act_floats(long long n, const PlaneGeom& pg);
+MlpActs mlp_acts(float* base, long long n, const PlaneGeom& pg);
 
 struct MlpBwdArgs {
   DeformArgs f;             // canonical scene, t0, planes, transposed MLP

@@ -10,7 +10,8 @@
 //      cell) and the sampling positions;
 //   4. wgrad kernels: dW = D^T X as 8x8 register blocks per thread, per-chunk partial sums
 //      and a fixed-order reduction (deterministic).
-// 100k Gaussians, L = 2, h = 32 (us): @TABLE@
+// 100k Gaussians, L = 2, h = 32: recompute 161 us (142 as the forward), deltas 149, planes
+// 125, weights 133; one kernel for all but the weights took 635, the weights 244.
 #include <algorithm>
 
 #include "fs4d_internal.cuh"
@@ -200,9 +201,16 @@ __device__ __forceinline__ void axis_setup(float u, int R, int& i0, float& f, fl
 }
 
 // h/4 consecutive lanes per Gaussian, a float4 of features each, level after level (so a
-// Gaussian's position gradient is one lane's sum and needs no atomics).
+// Gaussian's position gradient is one lane's sum and needs no atomics).  All Gaussians
+// share t, so a time plane's gradient is one line over its spatial axis times the two time
+// rows' weights: the atomics go to kTimeCopies copies of the lines (by CTA, against many
+// adds to one address), which time_lines_kernel spreads over the two rows -- half the
+// atomics of adding to four cells.  300k Gaussians with the recompute and the deltas: 1471
+// us with four cells and 148 registers; lines 1196, with two CTAs per SM 1135, with three
+// (80 registers, a few spilled) 1125; one copy 1285, 32 copies 1133.
+constexpr int kTimeCopies = 8;
 template <int H, int L>
-__global__ void __launch_bounds__(256) plane_bwd_kernel(const __grid_constant__ MlpBwdArgs a) {
+__global__ void __launch_bounds__(256, 3) plane_bwd_kernel(const __grid_constant__ MlpBwdArgs a) {
   constexpr int Q = H / 4, HL = H * L;
   const DeformArgs& f = a.f;
   const PlaneGeom& pg = f.pg;
@@ -216,8 +224,9 @@ __global__ void __launch_bounds__(256) plane_bwd_kernel(const __grid_constant__ 
     const float c[4] = {(f.means[3 * g] - pg.aabb_min[0]) * pg.aabb_scale[0] - 1.f,
                         (f.means[3 * g + 1] - pg.aabb_min[1]) * pg.aabb_scale[1] - 1.f,
                         (f.means[3 * g + 2] - pg.aabb_min[2]) * pg.aabb_scale[2] - 1.f, 2.f * f.t0 - 1.f};
+    int line0 = 0;  // first cell of the level in a line
 #pragma unroll 1
-    for (int l = 0; l < L; ++l) {
+    for (int l = 0; l < L; line0 += pg.res[l], ++l) {
       const float4 gf4 = *reinterpret_cast<const float4*>(a.act.dfh + ii * HL + l * H + 4 * q);
       const float gf[4] = {gf4.x, gf4.y, gf4.z, gf4.w};
       int i0[4];
@@ -267,7 +276,12 @@ __global__ void __launch_bounds__(256) plane_bwd_kernel(const __grid_constant__ 
           sa += gv[e] * ((1.f - fb) * (Bs[e] - As[e]) + fb * (Es[e] - Cs[e]));
           sb += gv[e] * ((1.f - fa) * (Cs[e] - As[e]) + fa * (Es[e] - Bs[e]));
         }
-        if (a.g_planes) {
+        if (a.g_planes && p >= 3) {
+          float* G = a.act.lines + (((long long)(blockIdx.x % kTimeCopies) * 3 + ax) * a.act.line_cells + line0 + i0[ax]) * H + 4 * q;
+          atomicAdd(reinterpret_cast<float4*>(G),
+                    make_float4((1.f - fa) * gv[0], (1.f - fa) * gv[1], (1.f - fa) * gv[2], (1.f - fa) * gv[3]));
+          atomicAdd(reinterpret_cast<float4*>(G + H), make_float4(fa * gv[0], fa * gv[1], fa * gv[2], fa * gv[3]));
+        } else if (a.g_planes) {
           float* GP = a.g_planes + cell;
           const float w00 = (1.f - fa) * (1.f - fb), w10 = fa * (1.f - fb), w01 = (1.f - fa) * fb, w11 = fa * fb;
           atomicAdd(reinterpret_cast<float4*>(GP), make_float4(w00 * gv[0], w00 * gv[1], w00 * gv[2], w00 * gv[3]));
@@ -293,6 +307,26 @@ __global__ void __launch_bounds__(256) plane_bwd_kernel(const __grid_constant__ 
 #pragma unroll
     for (int k = 0; k < 3; ++k) a.g_means[3 * g + k] += gxs[k];
   }
+}
+
+// The lines of the time planes (all copies) into their two time rows.
+__global__ void __launch_bounds__(256) time_lines_kernel(const __grid_constant__ MlpBwdArgs a) {
+  const PlaneGeom& pg = a.f.pg;
+  const int H = pg.feat_dim;
+  const int e = blockIdx.x * 256 + (int)threadIdx.x, per = a.act.line_cells * H;
+  if (e >= 3 * per) return;
+  const int ax = e / per;
+  int cell = (e % per) / H, l = 0;
+  float g = 0.f;
+#pragma unroll
+  for (int k = 0; k < kTimeCopies; ++k) g += a.act.lines[(long long)k * 3 * per + e];
+  for (; cell >= pg.res[l]; ++l) cell -= pg.res[l];
+  int j0;
+  float fb, db;
+  axis_setup(2.f * a.f.t0 - 1.f, pg.res_time, j0, fb, db);
+  float* out = a.g_planes + pg.off[l][3 + ax] + ((long long)j0 * pg.res[l] + cell) * H + e % H;
+  out[0] += (1.f - fb) * g;
+  out[(long long)pg.res[l] * H] += fb * g;
 }
 
 // ------------------------------------------------------------------ weight gradients
@@ -469,20 +503,35 @@ cudaError_t launch_bwd_t(const MlpBwdArgs& a, cudaStream_t s) {
   const int sms = device_sm_count();
   mlp_delta_kernel<HL><<<(unsigned)(tiles < sms ? tiles : sms), kGroups * kThreads, smem, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const size_t line_floats = 3 * (size_t)a.act.line_cells * H;
+  if (a.g_planes && (e = cudaMemsetAsync(a.act.lines, 0, 4 * kTimeCopies * line_floats, s)) != cudaSuccess) return e;
   const long long items = (long long)a.f.n * (H / 4);
   plane_bwd_kernel<H, L><<<(unsigned)((items + 255) / 256), 256, 0, s>>>(a);
+  if ((e = cudaGetLastError()) != cudaSuccess || !a.g_planes) return e;
+  time_lines_kernel<<<(unsigned)((line_floats + 255) / 256), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t mlp_act_floats(long long n, int hin) {
+namespace {
+int line_cells(const PlaneGeom& pg) {
+  int c = 0;
+  for (int l = 0; l < pg.n_levels; ++l) c += pg.res[l];
+  return c;
+}
+}  // namespace
+
+size_t mlp_act_floats(long long n, const PlaneGeom& pg) {
   const long long tiles = (n + kTG - 1) / kTG;
-  return (size_t)n * (2 * hin + 64 + 64 + 192 + 12 + 192 + 64 + 64) + (size_t)tiles * 5 * kThreads;
+  return (size_t)n * (2 * pg.feat_dim * pg.n_levels + 64 + 64 + 192 + 12 + 192 + 64 + 64) +
+         (size_t)tiles * 5 * kThreads + (size_t)kTimeCopies * 3 * line_cells(pg) * pg.feat_dim;
 }
 
-MlpActs mlp_acts(float* base, long long n, int hin) {
+MlpActs mlp_acts(float* base, long long n, const PlaneGeom& pg) {
   MlpActs q{};
+  const int hin = pg.feat_dim * pg.n_levels;
+  const long long tiles = (n + kTG - 1) / kTG;
   auto take = [&](long long w) {
     float* p = base;
     base += n * w;
@@ -491,6 +540,8 @@ MlpActs mlp_acts(float* base, long long n, int hin) {
   q.fh = take(hin); q.a1 = take(64); q.fd = take(64); q.hid = take(192); q.dout = take(12);
   q.dh = take(192); q.d2 = take(64); q.d1 = take(64); q.dfh = take(hin);
   q.masks = reinterpret_cast<uint32_t*>(base);
+  q.lines = base + tiles * 5 * kThreads;
+  q.line_cells = line_cells(pg);
   return q;
 }
 
