@@ -145,7 +145,7 @@ struct Work {
   DevBuf sort_lb;
   DevBuf ranges, tile_order;
   DevBuf axis;                             // column and row bits of the tiles: [tiles_x + tiles_y][bitmap_words(n)]
-  DevBuf sslot;                            // (a saved frame's, while it is rendered)
+  DevBuf sslot, order_out;                 // (a saved frame's, while it is rendered)
   DevBuf sxy, sco, srgb, srect;      // with the lists: projected Gaussians in depth-rank order
   bool bmp = false;                        // the frame in flight has tile lists from the column and row bits
   bool packed = false;                     // ... or sorts (tile | index) keys without values
@@ -225,6 +225,7 @@ struct fs4d_frame {
   long long pairs = 0;
   DevBuf dmeans, dquats, dscales;              // deformed Gaussians
   DevBuf xy, co, rgb, radius, rect, offsets;   // projection and pair slots; lists of depth ranks: xy and rgb
+  DevBuf order;                                // launch order of the tiles, longest lists first
   DevBuf sco, slot;                            // by rank, with sco and (x0, y0, width, first slot) by rank
   bool ranks = false;                          // the lists hold depth ranks
   DevBuf values, ranges;                       // sorted Gaussian indices, per-tile ranges
@@ -942,6 +943,7 @@ fs4d_status frame_back(const Env& e, const fs4d_camera& shape, long long n_bound
   mark(e, 6);
   TileOrder order;
   order.n_tiles = tx * ty;
+  order.out = P<uint32_t>(w.order_out);
   if (w.bmp) {  // the lists hold depth ranks into the rank-ordered copies
     order.class_count = z.counters + 64;
     order.class_tiles = P<uint32_t>(w.tile_order);
@@ -1178,7 +1180,7 @@ constexpr size_t kSpareFrames = 2;
 
 void release_frame(fs4d_frame& f) {
   DevBuf* all[] = {&f.dmeans, &f.dquats, &f.dscales, &f.xy, &f.co, &f.rgb, &f.radius, &f.rect, &f.offsets,
-                   &f.sco, &f.slot, &f.values, &f.ranges, &f.t_final, &f.n_contrib};
+                   &f.order, &f.sco, &f.slot, &f.values, &f.ranges, &f.t_final, &f.n_contrib};
   for (DevBuf* b : all) release(*b);
 }
 
@@ -1195,7 +1197,7 @@ fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, siz
   const std::pair<DevBuf*, size_t> need[] = {
       {&f->dmeans, 12 * n}, {&f->dquats, 16 * n}, {&f->dscales, 12 * n}, {&f->xy, 8 * n},       {&f->co, 16 * n},
       {&f->rgb, 12 * n},    {&f->radius, 4 * n},  {&f->rect, 16 * n},    {&f->offsets, 4 * n},  {&f->values, 4 * pairs},
-      {&f->sco, 16 * n},    {&f->slot, 16 * n},   {&f->ranges, 8 * tiles}, {&f->t_final, 4 * npix}, {&f->n_contrib, 4 * npix}};
+      {&f->sco, 16 * n},    {&f->slot, 16 * n},   {&f->ranges, 8 * tiles}, {&f->order, 4 * tiles}, {&f->t_final, 4 * npix}, {&f->n_contrib, 4 * npix}};
   bool grow = false, first = true;
   for (const auto& q : need) {
     grow = grow || q.first->bytes < q.second;
@@ -1230,7 +1232,7 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
     Work v = c->w;
     v.dmeans = f->dmeans; v.dquats = f->dquats; v.dscales = f->dscales;
     v.co = f->co; v.radius = f->radius; v.rect = f->rect;
-    v.offsets = f->offsets; v.ranges = f->ranges;
+    v.offsets = f->offsets; v.ranges = f->ranges; v.order_out = f->order;
     f->ranks = use_lists(c, c->w, s->n, tx, ty);
     if (f->ranks) {
       v.sxy = f->xy; v.srgb = f->rgb; v.sco = f->sco; v.sslot = f->slot;
@@ -1857,7 +1859,8 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   cb.width = f->cam.width; cb.height = f->cam.height; cb.tiles_x = tx;
   cb.ranges = P<uint2>(f->ranges); cb.values = P<uint32_t>(f->values);
   cb.xy = P<float2>(f->xy); cb.conic_opacity = P<float4>(f->ranks ? f->sco : f->co);
-  if (f->ranks) cb.slot = P<int4>(f->slot); cb.rgb = P<float>(f->rgb);
+  if (f->ranks) cb.slot = P<int4>(f->slot);
+  cb.order = P<uint32_t>(f->order); cb.rgb = P<float>(f->rgb);
   cb.rect = P<int4>(f->rect); cb.offsets = P<uint32_t>(f->offsets);
   cb.t_final = P<float>(f->t_final); cb.n_contrib = P<int>(f->n_contrib);
   cb.dl_dimage = d_dl_dimage; cb.grad_pair = P<float>(w.grad_pair);

@@ -5,9 +5,8 @@
 //  composite_bwd_kernel  one CTA per tile, one pixel per thread, walking the
 //      tile's list back to front from each pixel's last blended term.  The
 //      contributions of the 256 pixels to each Gaussian are summed inside the
-//      CTA (warp shuffles, then shared-memory adds) and written ONCE per
-//      (tile, Gaussian) pair into that pair's emission slot, so no global
-//      atomics are needed: a Gaussian's slots are contiguous (offsets[g] ...
+//      CTA and written ONCE per (tile, Gaussian) pair into that pair's slot, so no
+//      global atomics are needed: a Gaussian's slots are contiguous (offsets[g] ...
 //      offsets[g] + rect area).
 //  project_bwd_kernel    one thread per Gaussian: sums its pair slots, then
 //      back-propagates through the conic inverse, Sigma' = A A^T + 0.3 I with
@@ -25,168 +24,188 @@ constexpr float kGuard = 1.3f;
 
 // ------------------------------------------------------------------ compositing
 
-// Bit w set iff some pixel centre of the 16x2 pixel rows (2w, 2w + 1) of tile
-// (tx, ty) -- warp w's pixels -- may reach alpha >= 1/255 (the rectangle minimum of
-// d^T K d against -2 thr with a 0.2% + 1e-3 margin, as the forward's block masks):
-// a warp skips, as a whole, the terms whose bit is clear, which no lane of it blends.
-__device__ __forceinline__ uint32_t row_pair_mask(float2 p, float4 co, int tx, int ty) {
-  const float thr = composite_exp_threshold(co.w);
-  if (!(thr < 0.f)) return 0u;
-  const float A = co.x, B = co.y, C = co.z;
-  if (!(A > 0.f && C > 0.f && A * C - B * B > 0.f)) return 0xffu;
-  const float s = -2.f * thr * 1.002f + 1e-3f;
-  const float kx = -B / C, ky = -B / A;
-  const float X0 = (float)(tx * kTile) + 0.5f - p.x, X1 = X0 + (float)(kTile - 1);
-  const float Y0 = (float)(ty * kTile) + 0.5f - p.y;
-  uint32_t mask = 0u;
-#pragma unroll
-  for (int w = 0; w < kBatch / 32; ++w) {
-    const float y0 = Y0 + 2.f * (float)w;
-    if (rect_min(A, B, C, kx, ky, X0, X1, y0, y0 + 1.f) <= s) mask |= 1u << w;
-  }
-  return mask;
-}
-
-// The warp's sums of nine per-lane values with 14 shuffles instead of 45: values
-// 0..7 are halved at each of the offsets 16, 8, 4 (a lane keeps one half and sends
-// the other to its partner) and the last one summed over offsets 2 and 1, so lane
-// 4k returns the sum of value k (k < 8); the sum of value 8 comes back in s8.
-__device__ __forceinline__ float warp_sum9(const float (&v)[kPairGrad], unsigned lane, float& s8) {
+// The warp's sums of the nine per-lane values of two terms with 21 shuffles (45 each one
+// by one): values 0..7 of both are halved at each of the offsets 16, 8, 4, 2 (a lane keeps
+// one half and sends the other to its partner) and the last one summed over offset 1, so
+// an even lane returns the sum of value (lane / 2) % 8 of term a (lanes 0..15) or b; the
+// sums of value 8 come back in s8 (a's in the lower half warp, b's in the upper).
+__device__ __forceinline__ float warp_sum18(const float (&a)[kPairGrad], const float (&b)[kPairGrad], unsigned lane,
+                                            float& s8) {
   static_assert(kPairGrad == 9, "eight halved values and one summed whole");
-  float h4[4], h2[2];
-  const bool u16 = (lane & 16u) != 0u, u8 = (lane & 8u) != 0u, u4 = (lane & 4u) != 0u;
+  float h8[8], h4[4], h2[2];
+  const bool u16 = (lane & 16u) != 0u, u8 = (lane & 8u) != 0u, u4 = (lane & 4u) != 0u, u2 = (lane & 2u) != 0u;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) h8[i] = (u16 ? b[i] : a[i]) + __shfl_xor_sync(0xffffffffu, u16 ? a[i] : b[i], 16);
 #pragma unroll
   for (int i = 0; i < 4; ++i)
-    h4[i] = (u16 ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, u16 ? v[i] : v[i + 4], 16);
+    h4[i] = (u8 ? h8[i + 4] : h8[i]) + __shfl_xor_sync(0xffffffffu, u8 ? h8[i] : h8[i + 4], 8);
 #pragma unroll
   for (int i = 0; i < 2; ++i)
-    h2[i] = (u8 ? h4[i + 2] : h4[i]) + __shfl_xor_sync(0xffffffffu, u8 ? h4[i] : h4[i + 2], 8);
-  float h1 = (u4 ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, u4 ? h2[0] : h2[1], 4);
-  h1 += __shfl_xor_sync(0xffffffffu, h1, 2);
+    h2[i] = (u4 ? h4[i + 2] : h4[i]) + __shfl_xor_sync(0xffffffffu, u4 ? h4[i] : h4[i + 2], 4);
+  float h1 = (u2 ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, u2 ? h2[0] : h2[1], 2);
   h1 += __shfl_xor_sync(0xffffffffu, h1, 1);
-  float w = v[8];
+  float w = (u16 ? b[8] : a[8]) + __shfl_xor_sync(0xffffffffu, u16 ? a[8] : b[8], 16);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  for (int o = 8; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
   s8 = w;
   return h1;
 }
 
-__global__ void __launch_bounds__(kBatch) composite_bwd_kernel(CompositeBwdArgs a) {
-  __shared__ float2 s_xy[kBatch];
-  __shared__ float4 s_co[kBatch];
-  __shared__ float s_rgb[3 * kBatch];
-  __shared__ uint32_t s_slot[kBatch];
-  __shared__ uint32_t s_mask[kBatch];
-  __shared__ float s_acc[kBatch][kPairGrad];
+// The state of a pixel on its way back to front.
+struct PixelBack {
+  float T, b0, b1, b2;     // transmittance before the current term, colour blended behind it
+  float dC0, dC1, dC2;     // dL/dC
+};
+
+// The gradients of one blended term (alpha > 0) at offset (dx, dy), zero otherwise.
+__device__ __forceinline__ void term_grads(PixelBack& p, float alpha, float G, const float4& co, const float4& col,
+                                           float dx, float dy, float (&gr)[kPairGrad]) {
+#pragma unroll
+  for (int k = 0; k < kPairGrad; ++k) gr[k] = 0.f;
+  if (!(alpha > 0.f)) return;
+  const float inv = 1.f / (1.f - alpha);
+  const float Ti = p.T * inv;
+  const float dalpha = p.dC0 * (col.x * Ti - p.b0 * inv) + p.dC1 * (col.y * Ti - p.b1 * inv) +
+                       p.dC2 * (col.z * Ti - p.b2 * inv);
+  const float w = alpha * Ti;
+  gr[6] = p.dC0 * w;
+  gr[7] = p.dC1 * w;
+  gr[8] = p.dC2 * w;
+  p.b0 += col.x * w;
+  p.b1 += col.y * w;
+  p.b2 += col.z * w;
+  p.T = Ti;
+  if (co.w * G <= kAlphaMax) {
+    const float dpow = dalpha * co.w * G;
+    gr[0] = -dpow * (co.x * dx + co.y * dy);
+    gr[1] = -dpow * (co.z * dy + co.y * dx);
+    gr[2] = -0.5f * dpow * dx * dx;
+    gr[3] = -dpow * dx * dy;
+    gr[4] = -0.5f * dpow * dy * dy;
+    gr[5] = dalpha * G;
+  }
+}
+
+// One CTA per tile in the forward's launch order (longest lists first), one pixel per
+// thread, the forward's 8x4 pixel blocks per warp.  Batches of kBack terms are staged with
+// the forward's block masks, and each warp compacts a batch to the terms its block may
+// blend and walks them back to front, two per step: both weights before the two updates,
+// one reduction for both.  A warp leaves its sums of a term in its own place in shared
+// memory (no atomics, nothing to clear: the output adds up the warps of the term's mask, in
+// order) and each (tile, Gaussian) slot is written once.  Bound by instruction issue, about
+// a hundred per term and warp: 240 -> 121 us at 800x800 / 100k, 992 -> 651 at 1352x1014 /
+// 300k against 16x2 blocks that test every term of a batch, reduce one term at a time and
+// add to shared memory with float atomics, in tile order.  At 80 registers and less (three,
+// four CTAs per SM): 123 and 660, 129 and 641.
+constexpr int kBack = 128;
+constexpr int kBackWarps = kBatch / 32;
+constexpr size_t kBackSmem = 4 * (size_t)kBackWarps * kBack * kPairGrad;
+
+__global__ void __launch_bounds__(kBatch, 2) composite_bwd_kernel(const __grid_constant__ CompositeBwdArgs a) {
+  extern __shared__ float s_part[];        // [kBackWarps][kBack][kPairGrad]
+  __shared__ float4 s_g0[kBack];           // x, y, a2, c2
+  __shared__ float4 s_co[kBack];           // conic, opacity
+  __shared__ float4 s_col[kBack];          // colour, b2
+  __shared__ uint32_t s_slot[kBack], s_mask[kBack];
+  __shared__ uint8_t s_list[kBackWarps][kBack];
   __shared__ int s_max_last;
-  const int tile = blockIdx.x;
+  const int tile = a.order ? (int)a.order[blockIdx.x] : (int)blockIdx.x;
   const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
-  const int px = tx * kTile + (threadIdx.x % kTile), py = ty * kTile + (threadIdx.x / kTile);
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const int px = tx * kTile + (int)(warp & 1) * 8 + (int)(lane & 7), py = ty * kTile + (int)(warp >> 1) * 4 + (int)(lane >> 3);
   const bool inside = px < a.width && py < a.height;
   const int pix = py * a.width + px;
   const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
   const uint2 range = a.ranges[tile];
   const int n = (int)(range.y - range.x);
   const int last = inside ? a.n_contrib[pix] : 0;
-  float T = inside ? a.t_final[pix] : 1.f;
-  float dC0 = 0.f, dC1 = 0.f, dC2 = 0.f;
+  PixelBack p{1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (inside) {
-    dC0 = a.dl_dimage[3 * pix];
-    dC1 = a.dl_dimage[3 * pix + 1];
-    dC2 = a.dl_dimage[3 * pix + 2];
+    p.T = a.t_final[pix];
+    p.dC0 = a.dl_dimage[3 * pix];
+    p.dC1 = a.dl_dimage[3 * pix + 1];
+    p.dC2 = a.dl_dimage[3 * pix + 2];
   }
-  float b0 = 0.f, b1 = 0.f, b2 = 0.f;  // colour blended behind the current term
   if (threadIdx.x == 0) s_max_last = 0;
   __syncthreads();
-  atomicMax(&s_max_last, last);
+  const int wlast = __reduce_max_sync(0xffffffffu, last);
+  if (lane == 0) atomicMax(&s_max_last, wlast);
   __syncthreads();
   const int max_last = min(s_max_last, n);
-  const unsigned lane = threadIdx.x & 31u;
+  const int term = (int)threadIdx.x % kBack, half = (int)threadIdx.x / kBack;
 
-  for (int bstart = ((max_last - 1) / kBatch) * kBatch; bstart >= 0 && max_last > 0; bstart -= kBatch) {
-    __syncthreads();
-    const int j = bstart + (int)threadIdx.x;
-    if (j < n) {
-      const uint32_t g = a.values[range.x + j];
-      s_xy[threadIdx.x] = a.xy[g];
-      const float4 cog = a.conic_opacity[g];
-      s_co[threadIdx.x] = cog;
-      s_rgb[3 * threadIdx.x] = a.rgb[3 * g];
-      s_rgb[3 * threadIdx.x + 1] = a.rgb[3 * g + 1];
-      s_rgb[3 * threadIdx.x + 2] = a.rgb[3 * g + 2];
-      if (a.slot) {
-        const int4 r = a.slot[g];
-        s_slot[threadIdx.x] = (uint32_t)r.w + (uint32_t)((ty - r.y) * r.z + (tx - r.x));
+  for (int bstart = ((max_last - 1) / kBack) * kBack; bstart >= 0 && max_last > 0; bstart -= kBack) {
+    __syncthreads();  // the previous batch's sums have been written out
+    const int jend = min(kBack, max_last - bstart);
+    if (term < jend) {
+      const uint32_t g = a.values[range.x + bstart + term];
+      const float4 co = a.conic_opacity[g];
+      if (half == 0) {
+        const float2 xy = a.xy[g];
+        s_g0[term] = composite_coeffs(xy, co);
+        s_co[term] = co;
+        s_mask[term] = block_mask(xy, co, composite_exp_threshold(co.w), tx, ty);
       } else {
-        const int4 r = a.rect[g];
-        s_slot[threadIdx.x] = a.offsets[g] + (uint32_t)((ty - r.y) * (r.z - r.x) + (tx - r.x));
-      }
-      s_mask[threadIdx.x] = row_pair_mask(s_xy[threadIdx.x], cog, tx, ty);
-    }
-#pragma unroll
-    for (int k = 0; k < kPairGrad; ++k) s_acc[threadIdx.x][k] = 0.f;
-    __syncthreads();
-    const int jend = min(kBatch, max_last - bstart);
-    const unsigned warp_bit = 1u << (threadIdx.x >> 5);
-    for (int jj = jend - 1; jj >= 0; --jj) {
-      if (!(s_mask[jj] & warp_bit)) continue;  // warp-uniform: no pixel of this warp blends term jj
-      float gr[kPairGrad];
-#pragma unroll
-      for (int k = 0; k < kPairGrad; ++k) gr[k] = 0.f;
-      bool contrib = false;
-      if (bstart + jj < last) {
-        const float2 p = s_xy[jj];
-        const float4 co = s_co[jj];
-        const float4 g0 = composite_coeffs(p, co);
-        const float dx = g0.x - fx, dy = g0.y - fy;
-        float G;
-        const float alpha = composite_alpha(g0, composite_b2(co), co.w, dx, dy, G);
-        if (alpha > 0.f) {
-          const float a_raw = co.w * G;
-          contrib = true;
-          const float inv = 1.f / (1.f - alpha);
-          const float Ti = T * inv;
-          const float c0 = s_rgb[3 * jj], c1 = s_rgb[3 * jj + 1], c2 = s_rgb[3 * jj + 2];
-          const float dalpha =
-              dC0 * (c0 * Ti - b0 * inv) + dC1 * (c1 * Ti - b1 * inv) + dC2 * (c2 * Ti - b2 * inv);
-          const float w = alpha * Ti;
-          gr[6] = dC0 * w;
-          gr[7] = dC1 * w;
-          gr[8] = dC2 * w;
-          b0 += c0 * w;
-          b1 += c1 * w;
-          b2 += c2 * w;
-          T = Ti;
-          if (a_raw <= kAlphaMax) {
-            const float dpow = dalpha * co.w * G;
-            gr[0] = -dpow * (co.x * dx + co.y * dy);
-            gr[1] = -dpow * (co.z * dy + co.y * dx);
-            gr[2] = -0.5f * dpow * dx * dx;
-            gr[3] = -dpow * dx * dy;
-            gr[4] = -0.5f * dpow * dy * dy;
-            gr[5] = dalpha * G;
-          }
+        s_col[term] = make_float4(a.rgb[3 * (size_t)g], a.rgb[3 * (size_t)g + 1], a.rgb[3 * (size_t)g + 2],
+                                  composite_b2(co));
+        if (a.slot) {
+          const int4 r = a.slot[g];
+          s_slot[term] = (uint32_t)r.w + (uint32_t)((ty - r.y) * r.z + (tx - r.x));
+        } else {
+          const int4 r = a.rect[g];
+          s_slot[term] = a.offsets[g] + (uint32_t)((ty - r.y) * (r.z - r.x) + (tx - r.x));
         }
       }
-      const unsigned mask = __ballot_sync(0xffffffffu, contrib);
-      if (mask == 0u) continue;
-      if (__popc(mask) > 4) {
-        float s8;
-        const float sk = warp_sum9(gr, lane, s8);
-        if ((lane & 3u) == 0u) atomicAdd(&s_acc[jj][lane >> 2], sk);
-        if (lane == 0u) atomicAdd(&s_acc[jj][8], s8);
-      } else if (contrib) {
-#pragma unroll
-        for (int k = 0; k < kPairGrad; ++k) atomicAdd(&s_acc[jj][k], gr[k]);
+    }
+    __syncthreads();
+    int cnt = 0;
+    for (int c0 = 0; c0 < jend; c0 += 32) {
+      const int j = c0 + (int)lane;
+      const bool hit = j < jend && ((s_mask[j] >> warp) & 1u);
+      const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+      if (hit) s_list[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = (uint8_t)j;
+      cnt += __popc(bal);
+    }
+    __syncwarp();
+    float* part = s_part + warp * kBack * kPairGrad;
+    for (int i = cnt - 1; i >= 0; i -= 2) {
+      const int ja = s_list[warp][i], jb = i > 0 ? s_list[warp][i - 1] : ja;
+      const float4 a0 = s_g0[ja], b0 = s_g0[jb], aco = s_co[ja], bco = s_co[jb], acol = s_col[ja], bcol = s_col[jb];
+      const float adx = a0.x - fx, ady = a0.y - fy, bdx = b0.x - fx, bdy = b0.y - fy;
+      float Ga, Gb;
+      float alpha_a = composite_alpha(a0, acol.w, aco.w, adx, ady, Ga);
+      float alpha_b = composite_alpha(b0, bcol.w, bco.w, bdx, bdy, Gb);
+      if (bstart + ja >= last) alpha_a = 0.f;
+      if (i == 0 || bstart + jb >= last) alpha_b = 0.f;
+      if (!__any_sync(0xffffffffu, alpha_a > 0.f || alpha_b > 0.f)) {
+        if (lane < kPairGrad) {
+          part[ja * kPairGrad + lane] = 0.f;
+          part[jb * kPairGrad + lane] = 0.f;
+        }
+        continue;
+      }
+      float ga[kPairGrad], gb[kPairGrad], s8;
+      term_grads(p, alpha_a, Ga, aco, acol, adx, ady, ga);
+      term_grads(p, alpha_b, Gb, bco, bcol, bdx, bdy, gb);
+      const float s = warp_sum18(ga, gb, lane, s8);
+      float* dst = part + (lane < 16 ? ja : jb) * kPairGrad;
+      if (lane < 16 || i > 0) {
+        if ((lane & 1u) == 0u) dst[(lane >> 1) & 7u] = s;
+        if ((lane & 15u) == 0u) dst[8] = s8;
       }
     }
     __syncthreads();
-    if ((int)threadIdx.x < jend && bstart + (int)threadIdx.x < n) {
-      float4* dst = reinterpret_cast<float4*>(a.grad_pair + (size_t)s_slot[threadIdx.x] * kPairStride);
-      const float* v = s_acc[threadIdx.x];
-      dst[0] = make_float4(v[0], v[1], v[2], v[3]);
-      dst[1] = make_float4(v[4], v[5], v[6], v[7]);
-      dst[2] = make_float4(v[8], 0.f, 0.f, 0.f);
+    if (term < jend) {  // half 0: values 0..3 of the term, half 1: values 4..8
+      float v[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      for (uint32_t m = s_mask[term]; m; m &= m - 1u) {
+        const float* src = s_part + ((__ffs((int)m) - 1) * kBack + term) * kPairGrad + 4 * half;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] += src[k];
+        if (half) v[4] += src[4];
+      }
+      float4* dst = reinterpret_cast<float4*>(a.grad_pair + (size_t)s_slot[term] * kPairStride);
+      dst[half] = make_float4(v[0], v[1], v[2], v[3]);
+      if (half) dst[2] = make_float4(v[4], 0.f, 0.f, 0.f);
     }
   }
 }
@@ -449,7 +468,12 @@ __global__ void __launch_bounds__(128) project_bwd_kernel(ProjectBwdArgs a) {
 cudaError_t launch_composite_bwd(const CompositeBwdArgs& a, cudaStream_t s) {
   const int tiles_y = (a.height + kTile - 1) / kTile;
   if (a.tiles_x * tiles_y == 0) return cudaSuccess;
-  composite_bwd_kernel<<<a.tiles_x * tiles_y, kBatch, 0, s>>>(a);
+  static PerDeviceFlag attr;
+  const cudaError_t e = once_per_device(attr, [] {
+    return cudaFuncSetAttribute(composite_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBackSmem);
+  });
+  if (e != cudaSuccess) return e;
+  composite_bwd_kernel<<<a.tiles_x * tiles_y, kBatch, kBackSmem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -22,35 +22,6 @@ constexpr int kWarps = kThreads / 32;
 constexpr float kTMin = 1e-4f;
 constexpr int kMinBlocks = 5;  // CTAs per SM the register budget must allow
 
-// Bit b set iff some pixel centre of warp block b (8x4 pixels at ((b%2)*8, (b/2)*4)
-// of tile (tx, ty)) may reach alpha >= 1/255: the minimum of q(d) = d^T K d over
-// the block's pixel-centre rectangle (d relative to the mean) is compared with
-// s = -2 * thr.  The minimum of a positive-definite quadratic over a rectangle is
-// 0 if the mean lies inside, else on one of the four edges (each minimised in
-// closed form, rect_min).  If
-// all four corner pixel centres of the tile lie in the ellipse q <= s, so does the
-// whole tile (the ellipse is convex) and every block is set at once.  A 0.2% +
-// 1e-3 margin keeps the test conservative against float32 rounding.
-__device__ __forceinline__ uint32_t block_mask(float2 p, float4 co, float thr, int tx, int ty) {
-  if (!(thr < 0.f)) return 0u;                         // alpha can never reach 1/255
-  const float A = co.x, B = co.y, C = co.z;
-  if (!(A > 0.f && C > 0.f && A * C - B * B > 0.f)) return 0xffu;  // no usable bound: test every pixel
-  const float s = -2.f * thr * 1.002f + 1e-3f;
-  const float X0 = (float)(tx * kTile) + 0.5f - p.x, X1 = X0 + (float)(kTile - 1);
-  const float Y0 = (float)(ty * kTile) + 0.5f - p.y, Y1 = Y0 + (float)(kTile - 1);
-  auto q = [&](float x, float y) { return A * x * x + 2.f * B * x * y + C * y * y; };
-  if (fmaxf(fmaxf(q(X0, Y0), q(X1, Y0)), fmaxf(q(X0, Y1), q(X1, Y1))) <= s) return 0xffu;
-  const float kx = -B / C, ky = -B / A;
-  uint32_t mask = 0u;
-#pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    const float x0 = X0 + (float)((b & 1) * 8), x1 = x0 + 7.f;
-    const float y0 = Y0 + (float)((b >> 1) * 4), y1 = y0 + 3.f;
-    if (rect_min(A, B, C, kx, ky, x0, x1, y0, y1) <= s) mask |= 1u << b;
-  }
-  return mask;
-}
-
 // One staged batch of m Gaussians (list positions base .. base + m - 1) for the
 // calling thread's pixel: the warp compacts the batch to the Gaussians whose mask
 // holds its block (ballot, order kept) and walks them two per step -- both weights
@@ -174,6 +145,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) composite_kernel(int wid
     tile = (int)to.class_tiles[(size_t)cls * to.n_tiles + (blockIdx.x - first)];
     empty = (long long)*to.listed > to.capacity;
   }
+  if (to.out && threadIdx.x == 0) to.out[blockIdx.x] = (uint32_t)tile;
   const int tx = tile % tiles_x, ty = tile / tiles_x;
   const int bx0 = tx * kTile + (warp & 1) * 8, by0 = ty * kTile + (warp >> 1) * 4;
   const int px = bx0 + (lane & 7), py = by0 + (lane >> 3);

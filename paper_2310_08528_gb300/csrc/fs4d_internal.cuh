@@ -378,6 +378,7 @@ struct TileOrder {
   int n_tiles = 0;
   const uint32_t* listed = nullptr;
   long long capacity = 0;
+  uint32_t* out = nullptr;      // optional [n_tiles]: the tile that CTA i took
 };
 // values_stride: 1 for a list of uint32 indices, 2 for the low words of packed
 // (tile | index) 64-bit keys
@@ -439,6 +440,7 @@ struct CompositeBwdArgs {
   const int4* slot;         // with lists of depth ranks: x0, y0, width, first slot by rank (rect, offsets unused)
   const float* t_final;
   const int* n_contrib;
+  const uint32_t* order;    // [n_tiles] launch order of the tiles
   const float* dl_dimage;   // [H][W][3]
   float* grad_pair;         // [K][kPairStride] (9 used), indexed by emission slot; zeroed by the caller
 };
@@ -611,5 +613,34 @@ __device__ __forceinline__ float rect_min(float A, float B, float C, float kx, f
 // the rounding of either exponent form) is used for conservative culling.
 __device__ __forceinline__ float composite_exp_threshold(float opacity) {
   return logf((1.f / 255.f) / opacity) - 1e-3f;
+}
+
+// Bit b set iff some pixel centre of warp block b (8x4 pixels at ((b%2)*8, (b/2)*4)
+// of tile (tx, ty)) may reach alpha >= 1/255: the minimum of q(d) = d^T K d over
+// the block's pixel-centre rectangle (d relative to the mean) is compared with
+// s = -2 * thr.  The minimum of a positive-definite quadratic over a rectangle is
+// 0 if the mean lies inside, else on one of the four edges (each minimised in
+// closed form, rect_min).  If
+// all four corner pixel centres of the tile lie in the ellipse q <= s, so does the
+// whole tile (the ellipse is convex) and every block is set at once.  A 0.2% +
+// 1e-3 margin keeps the test conservative against float32 rounding.
+__device__ __forceinline__ uint32_t block_mask(float2 p, float4 co, float thr, int tx, int ty) {
+  if (!(thr < 0.f)) return 0u;                         // alpha can never reach 1/255
+  const float A = co.x, B = co.y, C = co.z;
+  if (!(A > 0.f && C > 0.f && A * C - B * B > 0.f)) return 0xffu;  // no usable bound: test every pixel
+  const float s = -2.f * thr * 1.002f + 1e-3f;
+  const float X0 = (float)(tx * kTile) + 0.5f - p.x, X1 = X0 + (float)(kTile - 1);
+  const float Y0 = (float)(ty * kTile) + 0.5f - p.y, Y1 = Y0 + (float)(kTile - 1);
+  auto q = [&](float x, float y) { return A * x * x + 2.f * B * x * y + C * y * y; };
+  if (fmaxf(fmaxf(q(X0, Y0), q(X1, Y0)), fmaxf(q(X0, Y1), q(X1, Y1))) <= s) return 0xffu;
+  const float kx = -B / C, ky = -B / A;
+  uint32_t mask = 0u;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const float x0 = X0 + (float)((b & 1) * 8), x1 = x0 + 7.f;
+    const float y0 = Y0 + (float)((b >> 1) * 4), y1 = y0 + 3.f;
+    if (rect_min(A, B, C, kx, ky, x0, x1, y0, y1) <= s) mask |= 1u << b;
+  }
+  return mask;
 }
 }  // namespace fs4d
