@@ -222,7 +222,7 @@ struct fs4d_frame {
   fs4d_camera cam{};
   float t = 0.f;
   int n = 0;
-  long long pairs = 0;
+  long long pairs = 0, slots = 0;              // tile pairs; slots of the backward's per-pair sums
   DevBuf dmeans, dquats, dscales;              // deformed Gaussians
   DevBuf xy, co, rgb, radius, rect, offsets;   // projection and pair slots; lists of depth ranks: xy and rgb
   DevBuf order;                                // launch order of the tiles, longest lists first
@@ -873,7 +873,7 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
   if (w.bmp) {  // lists of depth ranks into rank-ordered copies of the projected Gaussians
     ListArgs la{};
     la.n = N; la.order = ea.order; la.order_alt = ea.order_alt; la.order_sel = dsel;
-    la.rect = ea.rect; la.xy = P<float2>(w.xy); la.conic_opacity = P<float4>(w.co); la.rgb = P<float>(w.rgb);
+    la.rect = P<int4>(w.rect); la.xy = P<float2>(w.xy); la.conic_opacity = P<float4>(w.co); la.rgb = P<float>(w.rgb);
     la.tiles_x = tx; la.tiles_y = ty; la.n_tiles = tx * ty;
     la.words = bitmap_words(N);
     la.bits = P<uint32_t>(w.axis);
@@ -1125,7 +1125,7 @@ fs4d_status frame_queue(const Env& e, const fs4d_camera& cam, float* d_image, fl
                         uint32_t** values_out, long long* K) {
   fs4d_ctx* c = e.c;
   const long long cap = e.w->cap_pairs;
-  FS4D_CUDA(c, cudaMemcpyAsync(c->h_pinned, e.w->z.num_pairs, 8, cudaMemcpyDeviceToHost, e.s));
+  FS4D_CUDA(c, cudaMemcpyAsync(c->h_pinned, e.w->z.num_pairs, 16, cudaMemcpyDeviceToHost, e.s));
   if (!c->counted) FS4D_CUDA(c, cudaEventCreateWithFlags(&c->counted, cudaEventDisableTiming));
   FS4D_CUDA(c, cudaEventRecord(c->counted, e.s));
   if (cap > 0) {
@@ -1252,6 +1252,7 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
     if (K > c->band_pairs)
       return fail(c, FS4D_ERR_CAPACITY, "a frame saved for the backward must fit one band of tile pairs");
     f->pairs = c->last_pairs = K;
+    f->slots = f->ranks ? (long long)c->h_pinned[2] : K;
     if (K <= c->w.cap_pairs) {
       if (values != f->values.p) return fail(c, FS4D_ERR_CUDA, "render: the frame's list is not where it belongs");
       break;
@@ -1830,7 +1831,7 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   DeviceGuard g(c->device);
   if (f->stream != c->stream) f->one_stream = false;
   Work& w = c->w;
-  const long long n = s->n, K = f->pairs;
+  const long long n = s->n, K = f->slots;
   const int hin = s->mg.hin;
   const size_t act_floats = mlp_act_floats(n, s->pg);
   size_t wtot = 0;
@@ -2085,7 +2086,8 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
   if (bmp) {  // lists of depth ranks in the work memory, then copied in tile order
     ListArgs la{};
     la.n = n; la.order = P<uint32_t>(w.dvals); la.order_alt = P<uint32_t>(w.dvals_alt); la.order_sel = dsel;
-    la.rect = rect; la.depth = d_depth;
+    la.rect = const_cast<int4*>(rect);  // (written only with offsets)
+    la.depth = d_depth;
     la.tiles_x = tiles_x; la.tiles_y = tiles_y; la.n_tiles = n_tiles;
     la.words = bitmap_words(n);
     la.bits = P<uint32_t>(w.axis); la.s_rect = P<int4>(w.srect);

@@ -281,7 +281,7 @@ struct ListArgs {
   const uint32_t* order;        // depth order, as EmitArgs
   const uint32_t* order_alt;
   const uint32_t* order_sel;
-  const int4* rect;
+  int4* rect;                   // with offsets set to the cut rectangles, whose tiles the slots are
   const float2* xy;
   const float4* conic_opacity;
   const float* rgb;
@@ -297,9 +297,9 @@ struct ListArgs {
                                 // {alpha >= 1/255} reaches.  The lists lose Gaussians no pixel of the tile
                                 // blends: the image is unchanged, list positions are not the full
                                 // rectangles'.
-  uint32_t* offsets;            // optional [n]: each Gaussian's first slot (one slot per tile of its rectangle)
+  uint32_t* offsets;            // optional [n]: each Gaussian's first slot (one slot per tile of the cut rectangle)
   int4* s_slot;                 // with offsets: [n] by depth rank: x0, y0, width of the rectangle, first slot
-  uint32_t* num_pairs;          // [0] += pairs of the rectangles, [1] += pairs listed (zeroed)
+  uint32_t* num_pairs;          // [0] += pairs of the rectangles, [1] += pairs listed, [2] += slots (zeroed)
   long long capacity;           // pairs `values` holds
   uint32_t* values;
   uint2* ranges;                // [n_tiles]

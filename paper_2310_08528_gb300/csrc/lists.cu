@@ -49,18 +49,18 @@ __device__ __forceinline__ int4 cut_rect(int4 r, float2 p, float4 co) {
 
 // Bound by the gathers' latency: everything is requested at once after the index.
 __global__ void __launch_bounds__(kThreads) gather_kernel(const __grid_constant__ ListArgs a) {
-  __shared__ uint32_t s_warp[kWarps], s_slot;
+  __shared__ uint32_t s_warp[kWarps], s_sum[kWarps], s_slot;
   pdl_wait();
   pdl_trigger();
   const uint32_t* order = (a.order_sel && *a.order_sel) ? a.order_alt : a.order;
   const int pos = blockIdx.x * kThreads + (int)threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t g = 0, cnt = 0;
-  int4 r = make_int4(0, 0, 0, 0);
+  int4 cut = make_int4(0, 0, 0, 0);
   if (pos < a.n) {
     g = order[pos];
-    r = a.rect[g];
+    const int4 r = a.rect[g];
     cnt = (uint32_t)max(0, r.z - r.x) * (uint32_t)max(0, r.w - r.y);
-    int4 cut = r;
+    cut = cnt ? r : cut;
     if (a.s_xy) {
       const float2 p = a.xy[g];
       const float4 co = a.conic_opacity[g];
@@ -74,29 +74,42 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const __grid_constant_
     }
     a.s_rect[pos] = cut;
   }
-  uint32_t incl = cnt;
+  // the pairs of the rectangles; a saved frame's slots, one per tile of the cut rectangle
+  // (each Gaussian's consecutive, anywhere: an atomic per CTA)
+  const uint32_t sum = __reduce_add_sync(0xffffffffu, cnt);
+  const uint32_t slots = a.offsets ? (uint32_t)(cut.z - cut.x) * (uint32_t)(cut.w - cut.y) : 0u;
+  uint32_t incl = slots;
+  if (a.offsets) {
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += y;
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += y;
+    }
   }
-  if (lane == 31) s_warp[warp] = incl;
+  if (lane == 31) {
+    s_sum[warp] = sum;
+    s_warp[warp] = incl;
+  }
   __syncthreads();
-  uint32_t before = 0, total = 0;
+  uint32_t before = 0, total = 0, pairs = 0;
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) {
     const uint32_t y = s_warp[w];
     if (w < warp) before += y;
     total += y;
+    pairs += s_sum[w];
   }
-  // (the CTA's first slot: any disjoint place will do, each Gaussian's slots are consecutive)
-  if (threadIdx.x == 0) s_slot = total ? atomicAdd(&a.num_pairs[0], total) : 0u;
+  if (threadIdx.x == 0) {
+    if (pairs) atomicAdd(&a.num_pairs[0], pairs);
+    s_slot = total ? atomicAdd(&a.num_pairs[2], total) : 0u;
+  }
   if (!a.offsets) return;
   __syncthreads();
   if (pos < a.n) {
-    const uint32_t first = s_slot + before + incl - cnt;
+    const uint32_t first = s_slot + before + incl - slots;
     a.offsets[g] = first;
-    a.s_slot[pos] = make_int4(r.x, r.y, r.z - r.x, (int)first);
+    a.rect[g] = cut;
+    a.s_slot[pos] = make_int4(cut.x, cut.y, cut.z - cut.x, (int)first);
   }
 }
 
