@@ -589,25 +589,6 @@ __device__ __forceinline__ float composite_alpha(const float4& g0, float b2, flo
   return alpha < 1.f / 255.f ? 0.f : alpha;
 }
 
-// Minimum over t in [t0, t1] of A u^2 + 2 B u t + C t^2 for fixed u (C > 0), whose
-// unconstrained minimiser is t = k u with k = -B / C.
-__device__ __forceinline__ float edge_min(float A, float B, float C, float k, float u, float t0, float t1) {
-  const float t = fminf(t1, fmaxf(t0, k * u));
-  return A * u * u + 2.f * B * u * t + C * t * t;
-}
-
-// Minimum of the positive-definite quadratic q(x, y) = A x^2 + 2 B x y + C y^2 over
-// the rectangle [x0, x1] x [y0, y1] (coordinates relative to the mean): 0 if the
-// mean lies inside, else the least of the four edges' minima (each in closed form;
-// a rounded minimiser only raises q by a second-order amount).  kx = -B / C,
-// ky = -B / A.
-__device__ __forceinline__ float rect_min(float A, float B, float C, float kx, float ky, float x0, float x1,
-                                          float y0, float y1) {
-  if (x0 <= 0.f && x1 >= 0.f && y0 <= 0.f && y1 >= 0.f) return 0.f;
-  return fminf(fminf(edge_min(A, B, C, kx, x0, y0, y1), edge_min(A, B, C, kx, x1, y0, y1)),
-               fminf(edge_min(C, B, A, ky, y0, x0, x1), edge_min(C, B, A, ky, y1, x0, x1)));
-}
-
 // Natural-log exponent bound: a term reaches alpha >= 1/255 only where
 // -d^T K d / 2 >= ln(1/(255 o)); the bound minus 1e-3 (0.1% in alpha, far above
 // the rounding of either exponent form) is used for conservative culling.
@@ -615,31 +596,59 @@ __device__ __forceinline__ float composite_exp_threshold(float opacity) {
   return logf((1.f / 255.f) / opacity) - 1e-3f;
 }
 
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// A C - B^2 of a conic to about an ulp (the rounding of each product is recovered by an
+// FMA): for a thin ellipse the difference is far smaller than its terms.
+__device__ __forceinline__ float conic_det(const float4& co) {
+  const float p = co.y * co.y;
+  return fmaf(co.x, co.z, -p) - fmaf(co.y, co.y, -p);
+}
+// Whether the bounds on the ellipse's extent hold: positive definite, and not so thin and
+// oblique (A C over a thousand times the determinant) that the rounding of a pixel's own
+// exponent comes near the margins.
+__device__ __forceinline__ bool conic_bounded(const float4& co, float det) {
+  return co.x > 0.f && co.z > 0.f && det > 0.f && co.x * co.z <= 1000.f * det;
+}
+
 // Bit b set iff some pixel centre of warp block b (8x4 pixels at ((b%2)*8, (b/2)*4)
-// of tile (tx, ty)) may reach alpha >= 1/255: the minimum of q(d) = d^T K d over
-// the block's pixel-centre rectangle (d relative to the mean) is compared with
-// s = -2 * thr.  The minimum of a positive-definite quadratic over a rectangle is
-// 0 if the mean lies inside, else on one of the four edges (each minimised in
-// closed form, rect_min).  If
-// all four corner pixel centres of the tile lie in the ellipse q <= s, so does the
-// whole tile (the ellipse is convex) and every block is set at once.  A 0.2% +
-// 1e-3 margin keeps the test conservative against float32 rounding.
+// of tile (tx, ty)) may reach alpha >= 1/255, that is iff the ellipse q(d) = d^T K d <= s
+// = -2 thr (d relative to the mean, a 0.2% + 1e-3 margin) meets the block's pixel-centre
+// rectangle.  Per band of four pixel rows [ya, yb], the ellipse covers an interval of
+// columns: x(y) = -B/A y +- sqrt(s/A - det/A^2 y^2) at the band's ends (clipped to the
+// ellipse), or its extreme column where the extreme point lies in the band.  Intervals are
+// widened by 1e-5 of the ellipse and 0.01 pixels for the rounding; a comparison with a NaN
+// keeps the block.  About 150 instructions, against 400 for the least value of the
+// quadratic over each of the eight rectangles: a third of the compositing of a 100k object.
 __device__ __forceinline__ uint32_t block_mask(float2 p, float4 co, float thr, int tx, int ty) {
   if (!(thr < 0.f)) return 0u;                         // alpha can never reach 1/255
-  const float A = co.x, B = co.y, C = co.z;
-  if (!(A > 0.f && C > 0.f && A * C - B * B > 0.f)) return 0xffu;  // no usable bound: test every pixel
+  const float A = co.x, B = co.y, C = co.z, det = conic_det(co);
+  if (!conic_bounded(co, det)) return 0xffu;  // no usable bound: test every pixel
   const float s = -2.f * thr * 1.002f + 1e-3f;
-  const float X0 = (float)(tx * kTile) + 0.5f - p.x, X1 = X0 + (float)(kTile - 1);
-  const float Y0 = (float)(ty * kTile) + 0.5f - p.y, Y1 = Y0 + (float)(kTile - 1);
-  auto q = [&](float x, float y) { return A * x * x + 2.f * B * x * y + C * y * y; };
-  if (fmaxf(fmaxf(q(X0, Y0), q(X1, Y0)), fmaxf(q(X0, Y1), q(X1, Y1))) <= s) return 0xffu;
-  const float kx = -B / C, ky = -B / A;
+  const float X0 = (float)(tx * kTile) + 0.5f - p.x, Y0 = (float)(ty * kTile) + 0.5f - p.y;
+  const float iA = 1.f / A, sd = s / det, k = B * iA, wA = s * iA, wd = det * iA * iA;
+  const float hx = sqrt_approx(sd * C), hy = sqrt_approx(sd * A) * 1.00001f + 0.01f;
+  const float yr = -B / C * hx;  // the row of the greatest column
+  const float slack = 1e-5f * hx + 0.01f;
   uint32_t mask = 0u;
 #pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    const float x0 = X0 + (float)((b & 1) * 8), x1 = x0 + 7.f;
-    const float y0 = Y0 + (float)((b >> 1) * 4), y1 = y0 + 3.f;
-    if (rect_min(A, B, C, kx, ky, x0, x1, y0, y1) <= s) mask |= 1u << b;
+  for (int r = 0; r < 4; ++r) {
+    const float ya = Y0 + (float)(4 * r), yb = ya + 3.f;
+    const float a = fmaxf(ya, -hy), b = fminf(yb, hy);
+    const float va = sqrt_approx(fmaxf(0.f, wA - wd * a * a)), vb = sqrt_approx(fmaxf(0.f, wA - wd * b * b));
+    float hi = fmaxf(va - k * a, vb - k * b), lo = fminf(-va - k * a, -vb - k * b);
+    if (yr >= a && yr <= b) hi = hx;
+    if (-yr >= a && -yr <= b) lo = -hx;
+    hi += slack;
+    lo -= slack;
+    if (!(a > b)) {
+      if (!(hi < X0) && !(lo > X0 + 7.f)) mask |= 1u << (2 * r);
+      if (!(hi < X0 + 8.f) && !(lo > X0 + 15.f)) mask |= 2u << (2 * r);
+    }
   }
   return mask;
 }

@@ -30,13 +30,13 @@ constexpr int kRowsPerCta = 256;    // bit rows per CTA of the bits kernel
 // The rectangle of a projected Gaussian cut to the tiles that have a pixel centre within
 // the bounding box of its ellipse {alpha >= 1/255}: d^T K d <= S, a 0.4% + 2e-3 margin
 // over the compositing's own bound, reaches sqrt(S C / det) in x and sqrt(S A / det) in y
-// (1e-3 of it and 0.01 pixels for the rounding).  Without a usable bound (not positive
-// definite) the rectangle stays.
+// (1e-3 of it and 0.01 pixels for the rounding).  Without a usable bound the rectangle
+// stays.
 __device__ __forceinline__ int4 cut_rect(int4 r, float2 p, float4 co) {
   const float thr = composite_exp_threshold(co.w);
   if (!(thr < 0.f)) return make_int4(0, 0, 0, 0);  // alpha never reaches 1/255
-  const float det = co.x * co.z - co.y * co.y;
-  if (!(co.x > 0.f && co.z > 0.f && det > 0.f)) return r;
+  const float det = conic_det(co);
+  if (!conic_bounded(co, det)) return r;
   const float S = (-2.f * thr * 1.004f + 2e-3f) / det;
   const float hx = sqrtf(S * co.z) * 1.001f + 0.01f, hy = sqrtf(S * co.x) * 1.001f + 0.01f;
   if (!(hx < 1e6f && hy < 1e6f)) return r;

@@ -93,3 +93,41 @@ def test_lists_equal_sorted_pairs(n, tx, ty, side):
             ctx.bin_sort(depth, rect, tx, ty, cap - 1)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("thin", [1.0, 30.0, 1000.0])
+def test_block_masks_miss_no_pixel(thin):
+    """One Gaussian per tile, round to a thousand times longer than wide, its mean within a few
+    of its sizes of the tile: every pixel whose alpha passes the threshold in 64 bits is
+    blended.  (alpha = 1.01 / 255 is a 1% margin on an exponent whose rounding is below 1e-7 of
+    the conic's terms, under 1e-2 here.)"""
+    tiles = 48
+    n = tiles * tiles
+    rng = np.random.default_rng(int(thin))
+    long, wide = np.exp(rng.uniform(0, 3, n)) * thin ** 0.5 + 0.55, rng.uniform(0.55, 3, n)
+    th, k, ph = rng.uniform(0, np.pi, n), rng.uniform(0, 3.3, n), rng.uniform(0, 2 * np.pi, n)
+    c, s = np.cos(th), np.sin(th)
+    u, v = k * long * np.cos(ph), k * wide * np.sin(ph)
+    t = np.arange(n)
+    xy = np.stack([t % tiles * 16 + 8 + u * c - v * s, t // tiles * 16 + 8 + u * s + v * c], 1).astype(np.float32)
+    a, b, d = [x.astype(np.float32) for x in ((c / long) ** 2 + (s / wide) ** 2, c * s * (long ** -2.0 - wide ** -2.0),
+                                             (s / long) ** 2 + (c / wide) ** 2)]
+    op = rng.uniform(0.02, 0.98, n).astype(np.float32)
+    co = np.stack([a, b, d, op], 1)
+    dev = lambda z: torch.from_numpy(np.ascontiguousarray(z)).cuda()  # noqa: E731
+    ranges = np.stack([t, t + 1], 1).astype(np.int32)
+    ctx = fs4d.Context(0)
+    try:
+        img, _, _ = ctx.composite(16 * tiles, 16 * tiles, dev(ranges), dev(t.astype(np.int32)), dev(xy), dev(co),
+                                  dev(np.ones((n, 3), np.float32)))
+        got = img[..., 0].cpu().numpy().reshape(tiles, 16, tiles, 16).transpose(0, 2, 1, 3).reshape(n, 16, 16)
+    finally:
+        ctx.close()
+    px = np.arange(16) + 0.5
+    dx = (xy[:, 0].astype(np.float64) - t % tiles * 16)[:, None, None] - px[None, None, :]
+    dy = (xy[:, 1].astype(np.float64) - t // tiles * 16)[:, None, None] - px[None, :, None]
+    A, B, C, O = [co[:, i].astype(np.float64)[:, None, None] for i in range(4)]
+    alpha = np.minimum(0.99, O * np.exp(-0.5 * (A * dx * dx + 2 * B * dx * dy + C * dy * dy)))
+    need = alpha > 1.01 / 255
+    assert need.sum() > n
+    assert (np.abs(got - alpha)[need] <= 2e-2 * alpha[need]).all()
