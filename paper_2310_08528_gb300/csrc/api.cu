@@ -127,6 +127,7 @@ struct FrameZero {
                                          // [56] grid barrier, [64, 96) tiles per length class
   uint32_t* num_pairs = nullptr;         // [4]
   uint32_t* tile_count = nullptr;        // [n_tiles]
+  uint32_t* bucket_hist = nullptr;       // [kBuckets] Gaussians per depth bucket
   unsigned long long* emit_lb = nullptr; // [emit_parts(n) + 1]
   uint32_t* dlb = nullptr;               // depth-sort look-back [4][dparts][256]
   uint32_t* plb = nullptr;               // pair-sort look-back [passes][pparts][256]
@@ -140,7 +141,9 @@ struct Work {
   DevBuf dmeans, dquats, dscales;          // deformed Gaussians
   DevBuf xy, co, rgb, depth, radius, rect; // projected
   DevBuf offsets, counters, hist;
-  DevBuf dkeys, dvals, dkeys_alt, dvals_alt;  // per-Gaussian depth sort
+  DevBuf dkeys, dvals, dkeys_alt, dvals_alt;  // per-Gaussian depth sort (dkeys_alt: or grouped by bucket)
+  DevBuf bpos, bstart;                     // place in the depth bucket; bucket starts
+  bool buckets = false;                    // the frame in flight takes its depth order by buckets
   DevBuf keys, values, keys_alt, values_alt;
   DevBuf sort_lb;
   DevBuf ranges, tile_order;
@@ -165,7 +168,7 @@ struct Work {
 void release_work(Work& w) {
   DevBuf* all[] = {&w.zero, &w.dmeans, &w.dquats, &w.dscales, &w.xy, &w.co, &w.rgb, &w.depth, &w.radius, &w.rect,
                    &w.offsets, &w.counters, &w.hist, &w.dkeys, &w.dvals, &w.dkeys_alt,
-                   &w.dvals_alt, &w.keys, &w.values, &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges,
+                   &w.dvals_alt, &w.bpos, &w.bstart, &w.keys, &w.values, &w.keys_alt, &w.values_alt, &w.sort_lb, &w.ranges,
                    &w.tile_order, &w.axis, &w.sxy, &w.sco, &w.srgb, &w.srect, &w.ts, &w.host_img, &w.grad_pair, &w.gd, &w.acts,
                    &w.wpartial, &w.fd, &w.dsh, &w.dop, &w.yparts, &w.spos, &w.srg, &w.band_pairs};
   for (DevBuf* b : all) release(*b);
@@ -195,6 +198,7 @@ size_t frame_zero_layout(int n, int n_tiles, long long cap, int pair_passes, uns
   const size_t o_cnt = take(4 * 96);
   const size_t o_np = take(16);
   const size_t o_tc = take(4 * (size_t)n_tiles);
+  const size_t o_bh = take(4 * (size_t)kBuckets);
   const size_t o_elb = take(8 * (size_t)(emit_parts(std::max(n, 1)) + 1));
   const size_t o_dlb = take(4 * 256 * 4 * (size_t)dparts);
   const size_t o_plb = take(4 * 256 * (size_t)pair_passes * pparts);
@@ -203,6 +207,7 @@ size_t frame_zero_layout(int n, int n_tiles, long long cap, int pair_passes, uns
     z->counters = reinterpret_cast<uint32_t*>(base + o_cnt);
     z->num_pairs = reinterpret_cast<uint32_t*>(base + o_np);
     z->tile_count = reinterpret_cast<uint32_t*>(base + o_tc);
+    z->bucket_hist = reinterpret_cast<uint32_t*>(base + o_bh);
     z->emit_lb = reinterpret_cast<unsigned long long*>(base + o_elb);
     z->dlb = reinterpret_cast<uint32_t*>(base + o_dlb);
     z->plb = reinterpret_cast<uint32_t*>(base + o_plb);
@@ -573,9 +578,11 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
     FS4D_CUDA(c, ensure(w.dvals, 4 * m));
     FS4D_CUDA(c, ensure(w.dkeys_alt, 8 * m));
     FS4D_CUDA(c, ensure(w.dvals_alt, 4 * m));
+    FS4D_CUDA(c, ensure(w.bpos, 4 * m));
     w.cap_n = n;
   }
   FS4D_CUDA(c, ensure(w.counters, 4 * kCounters));
+  FS4D_CUDA(c, ensure(w.bstart, 4 * (kBuckets + 4)));
   FS4D_CUDA(c, ensure(w.hist, 4 * 256 * kSortMaxPasses));
   if (n_tiles > w.cap_tiles) {
     FS4D_CUDA(c, ensure(w.ranges, 8 * (size_t)n_tiles));
@@ -630,8 +637,13 @@ SortWork sort_work(fs4d_ctx* c) {
 
 // The depth sort's and the pair sort's share of a frame's zeroed state (counters: words
 // 0..7 emission, 8..24 depth sort, 32..48 pair sort, 56 grid barrier, 64..95 length classes).
-SortWork depth_sort_work(const fs4d_ctx* c, const FrameZero& z) {
+SortWork depth_sort_work(const fs4d_ctx* c, Work& w) {
+  const FrameZero& z = w.z;
   SortWork sw;
+  if (w.buckets) {
+    sw.bucket_hist = z.bucket_hist; sw.bucket_pos = P<uint32_t>(w.bpos);
+    sw.bucketed = P<unsigned long long>(w.dkeys_alt); sw.bucket_start = P<uint32_t>(w.bstart);
+  }
   sw.hist = z.hist; sw.lookback = z.dlb; sw.part_counters = z.counters + 8; sw.max_parts = z.dparts;
   sw.prezeroed = true;
   sw.spin_limit = c->spin_limit;
@@ -776,6 +788,7 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
   // every buffer the frame needs at zero, in one allocation (cleared below)
   FrameZero& z = w.z;
   w.bmp = use_lists(c, w, N, tx, ty);
+  w.buckets = w.bmp && !y_parts && sort_by_buckets(N);  // (only the lists' gather reads buckets)
   frame_zero_layout(N, tx * ty, cap, w.bmp ? 0 : sort_passes(tile_bits), static_cast<unsigned char*>(w.zero.p), &z);
   if (z.bytes > w.zero.bytes) return fail(c, FS4D_ERR_INVALID_ARG, "frame work memory was not reserved");
   mark(e, 0);
@@ -816,7 +829,12 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
     pa.depth = P<float>(w.depth) + q.off; pa.radius = P<int>(w.radius) + q.off; pa.rect = P<int4>(w.rect) + q.off;
     pa.depth_keys = P<unsigned long long>(w.dkeys) + q.off; pa.depth_vals = P<uint32_t>(w.dvals) + q.off;
     pa.index_base = (uint32_t)q.off;
-    pa.depth_hist = z.hist;
+    if (w.buckets) {
+      pa.bucket_hist = z.bucket_hist;
+      pa.bucket_pos = P<uint32_t>(w.bpos) + q.off;
+    } else {
+      pa.depth_hist = z.hist;
+    }
     if (y_parts) pa.y_parts = y_parts + q.off;
     FS4D_CUDA(c, launch_project(pa, stream));
   }
@@ -824,7 +842,7 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
   // Gaussians in (float32 depth, index) order: the emission order
   bool dalt = false;
   FS4D_CUDA(c, launch_sort(P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), P<unsigned long long>(w.dkeys_alt),
-                           P<uint32_t>(w.dvals_alt), nullptr, N, 0, 32, true, depth_sort_work(c, z), e.status, stream, &dalt,
+                           P<uint32_t>(w.dvals_alt), nullptr, N, 0, 32, true, depth_sort_work(c, w), e.status, stream, &dalt,
                            dsel));
   mark(e, 3);
   return FS4D_OK;
@@ -873,6 +891,7 @@ fs4d_status frame_front(const Env& e, const FramePart* parts, int n_parts, fs4d_
   if (w.bmp) {  // lists of depth ranks into rank-ordered copies of the projected Gaussians
     ListArgs la{};
     la.n = N; la.order = ea.order; la.order_alt = ea.order_alt; la.order_sel = dsel;
+    if (w.buckets) la.buckets = BucketOrder{P<unsigned long long>(w.dkeys_alt), P<uint32_t>(w.bstart)};
     la.rect = P<int4>(w.rect); la.xy = P<float2>(w.xy); la.conic_opacity = P<float4>(w.co); la.rgb = P<float>(w.rgb);
     la.tiles_x = tx; la.tiles_y = ty; la.n_tiles = tx * ty;
     la.words = bitmap_words(N);
@@ -2069,16 +2088,19 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
   const bool bmp = use_lists(c, w, n, tiles_x, tiles_y);
   c->last_binning = bmp ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
   // everything that starts at zero, as a frame's (frame_depth_order)
+  w.buckets = bmp && sort_by_buckets(n);
   FrameZero& z = w.z;
   frame_zero_layout(n, n_tiles, capacity, bmp ? 0 : sort_passes(tile_bits), static_cast<unsigned char*>(w.zero.p), &z);
   if (z.bytes > w.zero.bytes) return fail(c, FS4D_ERR_INVALID_ARG, "bin_sort: work memory was not reserved");
   FS4D_CUDA(c, cudaMemsetAsync(w.zero.p, 0, z.bytes, c->stream));
   // Gaussians sorted by (float32 depth, index)
-  FS4D_CUDA(c, launch_depth_keys(d_depth, n, P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), z.hist, c->stream));
+  FS4D_CUDA(c, launch_depth_keys(d_depth, reinterpret_cast<const int4*>(d_rect), n, P<unsigned long long>(w.dkeys),
+                                 P<uint32_t>(w.dvals), z.hist, w.buckets ? z.bucket_hist : nullptr,
+                                 P<uint32_t>(w.bpos), c->stream));
   bool dalt = false;
   const uint32_t* dsel = nullptr;
   FS4D_CUDA(c, launch_sort(P<unsigned long long>(w.dkeys), P<uint32_t>(w.dvals), P<unsigned long long>(w.dkeys_alt),
-                           P<uint32_t>(w.dvals_alt), nullptr, n, 0, 32, true, depth_sort_work(c, z),
+                           P<uint32_t>(w.dvals_alt), nullptr, n, 0, 32, true, depth_sort_work(c, w),
                            P<uint32_t>(c->status), c->stream, &dalt, &dsel));
   const int4* rect = reinterpret_cast<const int4*>(d_rect);
   uint2* ranges = reinterpret_cast<uint2*>(d_ranges);
@@ -2086,6 +2108,8 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
   if (bmp) {  // lists of depth ranks in the work memory, then copied in tile order
     ListArgs la{};
     la.n = n; la.order = P<uint32_t>(w.dvals); la.order_alt = P<uint32_t>(w.dvals_alt); la.order_sel = dsel;
+    if (w.buckets) la.buckets = BucketOrder{P<unsigned long long>(w.dkeys_alt), P<uint32_t>(w.bstart)};
+    la.order_out = P<uint32_t>(w.offsets);
     la.rect = const_cast<int4*>(rect);  // (written only with offsets)
     la.depth = d_depth;
     la.tiles_x = tiles_x; la.tiles_y = tiles_y; la.n_tiles = n_tiles;

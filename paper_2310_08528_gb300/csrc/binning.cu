@@ -310,6 +310,23 @@ cudaError_t launch_tile_scan(const uint32_t* tile_count, int n_tiles, uint32_t* 
 
 namespace fs4d {
 namespace {
+__global__ void __launch_bounds__(256) depth_buckets_kernel(const float* __restrict__ depth,
+                                                            const int4* __restrict__ rect, int n,
+                                                            unsigned long long* __restrict__ keys,
+                                                            uint32_t* __restrict__ vals,
+                                                            uint32_t* __restrict__ bucket_hist,
+                                                            uint32_t* __restrict__ bucket_pos) {
+  pdl_wait();
+  pdl_trigger();
+  const int i = blockIdx.x * 256 + (int)threadIdx.x;
+  if (i >= n) return;
+  const uint32_t key = __float_as_uint(depth[i]);
+  const int4 r = rect[i];
+  keys[i] = key;
+  vals[i] = (uint32_t)i;
+  bucket_pos[i] = r.z > r.x && r.w > r.y ? atomicAdd(&bucket_hist[depth_bucket(key)], 1u) : kNoBucket;
+}
+
 __global__ void __launch_bounds__(256) depth_keys_kernel(const float* __restrict__ depth, int n,
                                                          unsigned long long* __restrict__ keys,
                                                          uint32_t* __restrict__ vals, uint32_t* __restrict__ hist) {
@@ -339,10 +356,12 @@ __global__ void __launch_bounds__(256) depth_keys_kernel(const float* __restrict
 }
 }  // namespace
 
-cudaError_t launch_depth_keys(const float* depth, int n, unsigned long long* keys, uint32_t* vals, uint32_t* hist,
-                              cudaStream_t s) {
+cudaError_t launch_depth_keys(const float* depth, const int4* rect, int n, unsigned long long* keys, uint32_t* vals,
+                              uint32_t* hist, uint32_t* bucket_hist, uint32_t* bucket_pos, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  return launch_pdl(depth_keys_kernel, (n + 255) / 256, 256, 0, s, depth, n, keys, vals, hist);
+  const unsigned grid = (unsigned)((n + 255) / 256);
+  return bucket_hist ? launch_pdl(depth_buckets_kernel, grid, 256, 0, s, depth, rect, n, keys, vals, bucket_hist, bucket_pos)
+                     : launch_pdl(depth_keys_kernel, grid, 256, 0, s, depth, n, keys, vals, hist);
 }
 
 }  // namespace fs4d

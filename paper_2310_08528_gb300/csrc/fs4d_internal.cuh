@@ -181,6 +181,15 @@ cudaError_t launch_color_heads(const ColorArgs& a, cudaStream_t s);
 // BF16 tcgen05 form (the BF16 path): k3 in {3, 12, 27, 48}; fd_tiles, sh, sh_out 16-byte aligned
 cudaError_t launch_color_heads_bf16(const ColorArgs& a, cudaStream_t s);
 
+// Depth buckets (sort.cu): 512 per power of two of the depth from 2^-7 to 2^9, in the order
+// of the depth keys; nearer and farther depths share the first and the last.
+constexpr int kBuckets = 8192;
+constexpr uint32_t kNoBucket = 0xffffffffu;
+constexpr int kBucketMost = 1024;  // a fuller bucket: the keys are radix-sorted instead
+__device__ __forceinline__ int depth_bucket(uint32_t key) {
+  return min(max((int)(key >> 14) - (0x3C000000 >> 14), 0), kBuckets - 1);
+}
+
 struct CamParams {
   int width, height;
   float fx, fy, cx, cy, znear;
@@ -210,6 +219,8 @@ struct ProjectArgs {
   uint32_t* depth_vals;            // optional [n]: Gaussian index (index_base + g)
   uint32_t index_base;             // index of this call's first Gaussian in the frame's set
   uint32_t* depth_hist;            // optional [4][256] (zeroed): byte histograms of the depth keys
+  uint32_t* bucket_hist;           // optional [kBuckets] (zeroed): visible Gaussians per depth bucket, and
+  uint32_t* bucket_pos;            // [n] each one's place in its bucket (kNoBucket: not visible)
   float2* y_parts;                 // optional [n]: (fy y, 1 / z) of the visible Gaussians, so that the mean's row
                                    // is y_parts.x * y_parts.y + cy for any cy; a Gaussian is then culled by its
                                    // columns only, and its rectangle's rows may be empty
@@ -251,6 +262,19 @@ struct SortWork {
   uint32_t spin_limit = kSpinLimit;  // polls of a look-back wait before it gives up
   uint32_t* grid_counter = nullptr;  // optional, zero (with prezeroed): lets a small sort with result_sel
                                      // run every pass in one launch, its CTAs meeting at a grid barrier
+  // optional, for a sort of few 32-bit keys (sort_by_buckets) without their histograms: the keys' buckets as ProjectArgs leaves them; see BucketOrder
+  const uint32_t* bucket_hist = nullptr;
+  const uint32_t* bucket_pos = nullptr;
+  unsigned long long* bucketed = nullptr;
+  uint32_t* bucket_start = nullptr;
+};
+bool sort_by_buckets(long long n);
+// What such a sort leaves: with start[kBuckets + 1] == 1 the (key << 32 | value) words of the
+// visible Gaussians grouped by bucket, bucket b in [start[b], start[b + 1]), not ordered within;
+// with 0 (some bucket is too full) the sorted values as ever.
+struct BucketOrder {
+  const unsigned long long* bucketed = nullptr;
+  const uint32_t* start = nullptr;   // [kBuckets + 2]
 };
 
 // ---------------------------------------------------------------- launchers
@@ -263,9 +287,10 @@ cudaError_t launch_project(const ProjectArgs& a, cudaStream_t s);
 
 int emit_parts(int n);          // scan partitions of the emit kernel
 // keys[i] = float bits of depth[i] (upper word 0), vals[i] = i: input of the depth sort;
-// hist [4][256] (zeroed): byte histograms of the keys
-cudaError_t launch_depth_keys(const float* depth, int n, unsigned long long* keys, uint32_t* vals, uint32_t* hist,
-                              cudaStream_t s);
+// hist [4][256] (zeroed): byte histograms of the keys; or with bucket_hist non-NULL the buckets
+// of the Gaussians with tiles (rect), as ProjectArgs
+cudaError_t launch_depth_keys(const float* depth, const int4* rect, int n, unsigned long long* keys, uint32_t* vals,
+                              uint32_t* hist, uint32_t* bucket_hist, uint32_t* bucket_pos, cudaStream_t s);
 cudaError_t launch_scan_emit(const EmitArgs& a, cudaStream_t s);
 // tile ranges (from the per-tile counts; all (0, 0) when num_pairs[1] == 0 < num_pairs[0]),
 // if hist != NULL the [passes][256] digit histograms of the pair sort on the tile bits, and
@@ -281,6 +306,8 @@ struct ListArgs {
   const uint32_t* order;        // depth order, as EmitArgs
   const uint32_t* order_alt;
   const uint32_t* order_sel;
+  BucketOrder buckets;          // or the depth order by buckets
+  uint32_t* order_out;          // optional [n]: the depth order
   int4* rect;                   // with offsets set to the cut rectangles, whose tiles the slots are
   const float2* xy;
   const float4* conic_opacity;

@@ -2,8 +2,9 @@
 // interval, so with one bit per depth rank the Gaussians of tile (tx, ty), in depth
 // order, are the set bits of columns[tx] & rows[ty]: exactly the order a stable sort of
 // (tile | depth) keys gives.  Three kernels:
-//   gather  one thread per depth rank: the rectangle and what the compositing reads,
-//           copied into rank order; pair count and slots;
+//   gather  one thread per Gaussian: its depth rank (from the sorted order, or within its
+//           depth bucket), the rectangle and what the compositing reads copied into rank
+//           order; pair count and slots;
 //   bits    the bit rows, by ballots over 32 ranks or one bit at a time;
 //   list    one CTA per tile, each warp an eighth of the ranks, 4096 ranks per step (a
 //           16-byte word of each bit row per lane): counted, placed and written.
@@ -47,17 +48,50 @@ __device__ __forceinline__ int4 cut_rect(int4 r, float2 p, float4 co) {
   return r.z > r.x && r.w > r.y ? r : make_int4(0, 0, 0, 0);
 }
 
-// Bound by the gathers' latency: everything is requested at once after the index.
+// Bound by the gathers' latency: everything is requested at once after the index.  The
+// words of a CTA are in shared memory while their ranks are counted (an object of 20,000
+// Gaussians has about 50 per bucket).
 __global__ void __launch_bounds__(kThreads) gather_kernel(const __grid_constant__ ListArgs a) {
   __shared__ uint32_t s_warp[kWarps], s_sum[kWarps], s_slot;
+  __shared__ unsigned long long s_kv[kThreads + 2 * kBucketMost];
   pdl_wait();
   pdl_trigger();
-  const uint32_t* order = (a.order_sel && *a.order_sel) ? a.order_alt : a.order;
-  const int pos = blockIdx.x * kThreads + (int)threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * kThreads + (int)threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int pos = i;  // depth rank
   uint32_t g = 0, cnt = 0;
+  bool live = i < a.n;
+  if (a.buckets.start && a.buckets.start[kBuckets + 1]) {
+    // grouped by depth bucket: the rank of a word is its bucket's start plus the smaller
+    // words (depth, then index) of the bucket; the CTA's words lie in whole buckets
+    const uint32_t seen = a.buckets.start[kBuckets], i0 = blockIdx.x * kThreads;
+    const unsigned long long* kv = a.buckets.bucketed;
+    live = (uint32_t)i < seen;
+    uint32_t lo = 0;
+    if (i0 < seen) {
+      lo = a.buckets.start[depth_bucket((uint32_t)(kv[i0] >> 32))];
+      const uint32_t hi = a.buckets.start[depth_bucket((uint32_t)(kv[min(i0 + kThreads, seen) - 1] >> 32)) + 1];
+      for (uint32_t j = lo + threadIdx.x; j < hi; j += kThreads) s_kv[j - lo] = kv[j];
+    }
+    __syncthreads();
+    if (live) {
+      const unsigned long long w = s_kv[(uint32_t)i - lo];
+      const int b = depth_bucket((uint32_t)(w >> 32));
+      const uint32_t s0 = a.buckets.start[b], s1 = a.buckets.start[b + 1];
+      uint32_t less = 0;
+#pragma unroll 8
+      for (uint32_t j = s0 - lo; j < s1 - lo; ++j) less += s_kv[j] < w ? 1u : 0u;
+      pos = (int)(s0 + less);
+      g = (uint32_t)w;
+    } else if (i < a.n) {
+      a.s_rect[i] = make_int4(0, 0, 0, 0);  // no Gaussian of this rank
+    }
+  } else if (live) {
+    const uint32_t* order = (a.order_sel && *a.order_sel) ? a.order_alt : a.order;
+    g = order[i];
+  }
   int4 cut = make_int4(0, 0, 0, 0);
-  if (pos < a.n) {
-    g = order[pos];
+  if (live) {
+    if (a.order_out) a.order_out[pos] = g;
     const int4 r = a.rect[g];
     cnt = (uint32_t)max(0, r.z - r.x) * (uint32_t)max(0, r.w - r.y);
     cut = cnt ? r : cut;
@@ -105,7 +139,7 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const __grid_constant_
   }
   if (!a.offsets) return;
   __syncthreads();
-  if (pos < a.n) {
+  if (live) {
     const uint32_t first = s_slot + before + incl - slots;
     a.offsets[g] = first;
     a.rect[g] = cut;
@@ -259,7 +293,7 @@ __global__ void __launch_bounds__(kThreads) list_keys_kernel(const __grid_consta
   const uint32_t tile = blockIdx.x;
   const uint2 from = a.ranges[tile], to = out[tile];
   if (to.y <= to.x) return;  // empty, or the pairs overflow the buffers
-  const uint32_t* order = (a.order_sel && *a.order_sel) ? a.order_alt : a.order;
+  const uint32_t* order = a.order_out;
   const uint32_t cnt = min(to.y - to.x, from.y - from.x), most = (uint32_t)a.n - 1u;
   constexpr int kU = 4;
   for (uint32_t i0 = threadIdx.x; i0 < cnt; i0 += kU * kThreads) {

@@ -191,6 +191,9 @@ __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   }
   }
 
+  if (a.bucket_hist && valid)
+    a.bucket_pos[g] = seen ? atomicAdd(&a.bucket_hist[depth_bucket(__float_as_uint(pz))], 1u) : kNoBucket;
+
   float r = 0.f, gg = 0.f, b = 0.f;
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   if (SHQ > 0) __syncthreads();  // the SH rows were copied by the whole CTA

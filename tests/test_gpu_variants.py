@@ -99,8 +99,9 @@ def test_lists_equal_sorted_pairs(n, tx, ty, side):
 def test_block_masks_miss_no_pixel(thin):
     """One Gaussian per tile, round to a thousand times longer than wide, its mean within a few
     of its sizes of the tile: every pixel whose alpha passes the threshold in 64 bits is
-    blended.  (alpha = 1.01 / 255 is a 1% margin on an exponent whose rounding is below 1e-7 of
-    the conic's terms, under 1e-2 here.)"""
+    blended, with that alpha, as far as float32 can tell: each term of the exponent is three
+    roundings (offset, product, sum) from its value twice over, so the exponent in powers of
+    two is within 10 2^-24 of the sum of its terms' magnitudes."""
     tiles = 48
     n = tiles * tiles
     rng = np.random.default_rng(int(thin))
@@ -128,6 +129,35 @@ def test_block_masks_miss_no_pixel(thin):
     dy = (xy[:, 1].astype(np.float64) - t // tiles * 16)[:, None, None] - px[None, :, None]
     A, B, C, O = [co[:, i].astype(np.float64)[:, None, None] for i in range(4)]
     alpha = np.minimum(0.99, O * np.exp(-0.5 * (A * dx * dx + 2 * B * dx * dy + C * dy * dy)))
-    need = alpha > 1.01 / 255
-    assert need.sum() > n
-    assert (np.abs(got - alpha)[need] <= 2e-2 * alpha[need]).all()
+    e = 10 * 2.0 ** -24 * 0.7213475 * (A * dx * dx + 2 * np.abs(B * dx * dy) + C * dy * dy) + 1e-6
+    need = alpha * 2.0 ** -e > 1 / 255
+    assert need.sum() > n / 2
+    assert (np.abs(got - alpha)[need] <= (alpha * (2.0 ** e - 1) + 1e-6)[need]).all()
+
+
+# depths by bucket (at most 1024 in one), a full bucket (radix sort after all), out of the buckets' range
+@pytest.mark.parametrize("n,lo,hi", [(1, 1.0, 1.0), (1000, 2.0, 2.0), (1024, 3.0, 3.0), (1025, 3.0, 3.0),
+                                     (100000, 2.0, 5.0), (100000, 4.0, 4.01), (60000, 1e-4, 3e3), (5000, -2.0, 2.0),
+                                     (20000, 1e-4, 3e3), (24576, 2.0, 5.0), (24577, 2.0, 5.0)])
+def test_depth_order_by_buckets(n, lo, hi):
+    """(depth bits, index) order of the Gaussians with tiles, whatever the depths: bin_sort with
+    lists against the sorted pairs."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    depth = lo + (hi - lo) * torch.rand(n, generator=g, device="cuda")
+    if n < 10000:
+        depth[::3] = float(depth[0])  # ties (more than a bucket holds, with 5000)
+    x = torch.randint(0, 9, (n, 1), generator=g, device="cuda")
+    size = torch.randint(0, 3, (n, 1), generator=g, device="cuda")
+    rect = torch.cat([x, x, torch.clamp(x + size, max=9), torch.clamp(x + size, max=9)], 1).int().contiguous()
+    cap = int(((rect[:, 2] - rect[:, 0]) * (rect[:, 3] - rect[:, 1])).sum())
+    ctx = fs4d.Context(0)
+    try:
+        ctx.set_binning(fs4d.BINNING_SORT)
+        want = [v.clone() if torch.is_tensor(v) else v for v in ctx.bin_sort(depth, rect, 9, 9, cap)]
+        ctx.set_binning(fs4d.BINNING_AUTO)
+        got = ctx.bin_sort(depth, rect, 9, 9, cap)
+        assert got[3] == want[3] == cap
+        for a, b in zip(got[:3], want[:3]):
+            assert torch.equal(a, b)
+    finally:
+        ctx.close()
