@@ -603,16 +603,22 @@ __device__ __forceinline__ float4 composite_coeffs(float2 p, float4 conic_opacit
 }
 __device__ __forceinline__ float composite_b2(float4 conic_opacity) { return -kLog2e * conic_opacity.y; }
 
-// alpha = min(0.99, o * G) of a term at offset (dx, dy) = mean - pixel centre,
-// or 0 when the term is skipped (alpha below 1/255).  The exponent
+// alpha = min(0.99, o * G) of a term at offset (dx, dy) = mean - pixel centre; the term
+// is skipped where alpha is below 1/255.  The exponent
 // dx (a2 dx + b2 dy) + c2 dy^2 is never positive: every Gaussian that reaches
 // compositing has a positive-definite conic (projection culls det <= 0, and the
 // 0.3 dilation keeps det >= 0.09), so no exponent-sign test is needed.
-__device__ __forceinline__ float composite_alpha(const float4& g0, float b2, float opacity, float dx, float dy,
-                                                 float& G) {
+__device__ __forceinline__ float composite_weight(const float4& g0, float b2, float opacity, float dx, float dy,
+                                                  float& G) {
   const float p = fmaf(fmaf(g0.z, dx, b2 * dy), dx, (g0.w * dy) * dy);
   G = ex2_approx(p);
-  const float alpha = fminf(0.99f, opacity * G);
+  return fminf(0.99f, opacity * G);
+}
+
+// The weight, or 0 where the term is skipped.
+__device__ __forceinline__ float composite_alpha(const float4& g0, float b2, float opacity, float dx, float dy,
+                                                 float& G) {
+  const float alpha = composite_weight(g0, b2, opacity, dx, dy, G);
   return alpha < 1.f / 255.f ? 0.f : alpha;
 }
 

@@ -9,7 +9,9 @@
 //    runs of equal digits are written contiguously;
 //  - or, for a sort whose 1024-key partitions are all resident at once (a frame's
 //    depth sort of up to ~150k keys), every pass in one launch: CTA b owns
-//    partition b in every pass and a bounded grid barrier separates the passes.
+//    partition b in every pass and a bounded grid barrier separates the passes;
+//  - or, for the depths of up to kBucketKeys Gaussians, one pass by depth buckets that
+//    the projection has counted (the list gather orders each bucket).
 // Only the key bits that can differ are sorted.  A frame sorts the N float32
 // depths (32 bits in 4 passes; a pass whose digit is the same for every key moves
 // nothing) and, on the key-emission route, the pairs on their tile bits only (the

@@ -1,7 +1,8 @@
-"""Variants of a stage that are chosen by size give the same bits.  Frames composited straight from the depth order: columns and rows of tiles as
-bits per depth rank.  A frame whose pairs exceed a band goes that way; its first
-band has the whole frame's principal point, so its pixels are the listed tiles'
-bit for bit, with full lists (the last contributors are list positions)."""
+"""Variants of a stage that are chosen by size give the same bits.  Frames composited
+straight from the depth order: columns and rows of tiles as bits per depth rank.  A frame
+whose pairs exceed a band goes that way; its first band has the whole frame's principal
+point, so its pixels are the listed tiles' bit for bit, with full lists (the last
+contributors are list positions)."""
 import numpy as np
 import pytest
 
@@ -161,3 +162,41 @@ def test_depth_order_by_buckets(n, lo, hi):
             assert torch.equal(a, b)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 8, 255, 256, 257, 259, 513, 1100])
+def test_composite_list_lengths(n):
+    """Lists that end anywhere in a step of the walk, a batch or after saturation (from about 300
+    terms): sums in float64.  Every term is far above 1/255, so only the cut at T < 1e-4 can fall
+    on the other side: it moves less than 0.08 * 1e-4.  Rounding of 600 terms' products: 1e-4."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    w, h = 27, 15  # a whole tile and a ragged one
+    xy = (torch.rand(n, 2, generator=g, device="cuda") * torch.tensor([27.0, 15.0], device="cuda")).contiguous()
+    conic = torch.tensor([1e-3, 2e-4, 2e-3], device="cuda").repeat(n, 1)
+    opac = 0.03 + 0.05 * torch.rand(n, 1, generator=g, device="cuda")
+    co = torch.cat([conic, opac], 1).contiguous()
+    rgb = torch.rand(n, 3, generator=g, device="cuda")
+    half = (n + 1) // 2
+    values = torch.cat([torch.arange(n), torch.arange(half)]).int().cuda()
+    ranges = torch.tensor([[0, n], [n, n + half]], dtype=torch.int32, device="cuda")
+    ctx = fs4d.Context(0)
+    try:
+        img, t_final, last = [v.cpu() for v in ctx.composite(w, h, ranges, values, xy, co, rgb)]
+    finally:
+        ctx.close()
+    p, c, col = xy.double().cpu(), co.double().cpu(), rgb.double().cpu()
+    yy, xx = torch.meshgrid(torch.arange(h) + 0.5, torch.arange(w) + 0.5, indexing="ij")
+    dx, dy = p[:, 0, None, None] - xx, p[:, 1, None, None] - yy
+    al = c[:, 3, None, None] * torch.exp(-0.5 * (1e-3 * dx * dx + 2 * 2e-4 * dx * dy + 2e-3 * dy * dy))
+    assert float(al.min()) > 2 / 255
+    al[half:, :, 16:] = 0  # the second tile's list is the first half
+    T = torch.cumprod(1 - al, 0)
+    before = torch.cat([torch.ones(1, h, w, dtype=torch.float64), T[:-1]])
+    live = T >= 1e-4
+    want = torch.einsum("nhw,nc->hwc", al * before * live, col)
+    assert float((img - want).abs().max()) < 1e-4 + 0.08 * 1e-4
+    count = torch.minimum(live.sum(0), torch.tensor([n] * 16 + [half] * 11))
+    assert int((last - count).abs().max()) <= 1
+    if n < 100:
+        assert torch.equal(last.long(), count)
+    assert float((t_final / T.gather(0, (last.long() - 1)[None])[0] - 1).abs().max()) < 1e-4
