@@ -53,37 +53,41 @@ __device__ __forceinline__ float warp_sum18(const float (&a)[kPairGrad], const f
 
 // The state of a pixel on its way back to front.
 struct PixelBack {
-  float T, b0, b1, b2;     // transmittance before the current term, colour blended behind it
+  float T;                 // transmittance behind the current term
+  float b0, b1, b2;        // minus the colour blended behind it
   float dC0, dC1, dC2;     // dL/dC
 };
 
-// The gradients of one blended term (alpha > 0) at offset (dx, dy), zero otherwise.
+// The gradients of one blended term (alpha > 0) at offset (dx, dy), zero otherwise, without
+// the opacity's factor, which is the same for every pixel and multiplies the sums: with
+// u = G dL/dalpha (0 where alpha is capped), u K d, u (dx^2, dx dy, dy^2), u, and dL/dcolour.
+// dL/dalpha = sum_k dC_k (col_k T - b_k) / (1 - alpha) rounds col_k T - b_k once, where
+// the two cancel.  The mean's u K d stays a per-pixel product: A sum(u dx) + B sum(u dy)
+// would cancel in thin, oblique ellipses (ten times the error at 1000:1).  Selects, no
+// branch: nine values under a divergent branch took 549 us where this takes 535.
 __device__ __forceinline__ void term_grads(PixelBack& p, float alpha, float G, const float4& co, const float4& col,
                                            float dx, float dy, float (&gr)[kPairGrad]) {
-#pragma unroll
-  for (int k = 0; k < kPairGrad; ++k) gr[k] = 0.f;
-  if (!(alpha > 0.f)) return;
+  const bool on = alpha > 0.f;
   const float inv = 1.f / (1.f - alpha);
-  const float Ti = p.T * inv;
-  const float dalpha = p.dC0 * (col.x * Ti - p.b0 * inv) + p.dC1 * (col.y * Ti - p.b1 * inv) +
-                       p.dC2 * (col.z * Ti - p.b2 * inv);
-  const float w = alpha * Ti;
-  gr[6] = p.dC0 * w;
-  gr[7] = p.dC1 * w;
-  gr[8] = p.dC2 * w;
-  p.b0 += col.x * w;
-  p.b1 += col.y * w;
-  p.b2 += col.z * w;
-  p.T = Ti;
-  if (co.w * G <= kAlphaMax) {
-    const float dpow = dalpha * co.w * G;
-    gr[0] = -dpow * (co.x * dx + co.y * dy);
-    gr[1] = -dpow * (co.z * dy + co.y * dx);
-    gr[2] = -0.5f * dpow * dx * dx;
-    gr[3] = -dpow * dx * dy;
-    gr[4] = -0.5f * dpow * dy * dy;
-    gr[5] = dalpha * G;
+  const float x0 = fmaf(col.x, p.T, p.b0), x1 = fmaf(col.y, p.T, p.b1), x2 = fmaf(col.z, p.T, p.b2);
+  const float dalpha = (p.dC0 * x0 + p.dC1 * x1 + p.dC2 * x2) * inv;
+  const float Ti = p.T * inv, w = alpha * Ti;
+  gr[6] = on ? p.dC0 * w : 0.f;
+  gr[7] = on ? p.dC1 * w : 0.f;
+  gr[8] = on ? p.dC2 * w : 0.f;
+  if (on) {
+    p.T = Ti;
+    p.b0 = fmaf(col.x, -w, p.b0);
+    p.b1 = fmaf(col.y, -w, p.b1);
+    p.b2 = fmaf(col.z, -w, p.b2);
   }
+  const float u = on && co.w * G <= kAlphaMax ? dalpha * G : 0.f, ux = u * dx, uy = u * dy;
+  gr[0] = u * (co.x * dx + co.y * dy);
+  gr[1] = u * (co.z * dy + co.y * dx);
+  gr[2] = ux * dx;
+  gr[3] = ux * dy;
+  gr[4] = uy * dy;
+  gr[5] = u;
 }
 
 // One CTA per tile in the forward's launch order (longest lists first), one pixel per
@@ -93,21 +97,22 @@ __device__ __forceinline__ void term_grads(PixelBack& p, float alpha, float G, c
 // one reduction for both.  A warp leaves its sums of a term in its own place in shared
 // memory (no atomics, nothing to clear: the output adds up the warps of the term's mask, in
 // order) and each (tile, Gaussian) slot is written once.  Bound by instruction issue, about
-// a hundred per term and warp: 240 -> 121 us at 800x800 / 100k, 992 -> 651 at 1352x1014 /
-// 300k against 16x2 blocks that test every term of a batch, reduce one term at a time and
-// add to shared memory with float atomics, in tile order.  At 80 registers and less (three,
-// four CTAs per SM): 123 and 660, 129 and 641.
+// ninety per term and warp: 240 -> 110 us at 800x800 / 100k, 992 -> 535 at 1352x1014 / 300k
+// against 16x2 blocks that test every term of a batch, reduce one term at a time and add to
+// shared memory with float atomics, in tile order.  (115 and 618 with byte indices, the
+// terms' products taken per pixel and branches; at the registers of three CTAs per SM 105
+// and 560: the few tiles of the small frame end later with four.)
 constexpr int kBack = 128;
 constexpr int kBackWarps = kBatch / 32;
-constexpr size_t kBackSmem = 4 * (size_t)kBackWarps * kBack * kPairGrad;
+constexpr size_t kBackSmem = 4 * (size_t)kBackWarps * (kBack + 1) * kPairGrad;
 
-__global__ void __launch_bounds__(kBatch, 2) composite_bwd_kernel(const __grid_constant__ CompositeBwdArgs a) {
-  extern __shared__ float s_part[];        // [kBackWarps][kBack][kPairGrad]
-  __shared__ float4 s_g0[kBack];           // x, y, a2, c2
-  __shared__ float4 s_co[kBack];           // conic, opacity
-  __shared__ float4 s_col[kBack];          // colour, b2
+__global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_constant__ CompositeBwdArgs a) {
+  extern __shared__ float s_part[];        // [kBackWarps][kBack + 1][kPairGrad]
+  __shared__ float4 s_g0[kBack + 1];       // x, y, a2, c2 (the last place: a term that adds nothing)
+  __shared__ float4 s_co[kBack + 1];       // conic, opacity
+  __shared__ float4 s_col[kBack + 1];      // colour, b2
   __shared__ uint32_t s_slot[kBack], s_mask[kBack];
-  __shared__ uint8_t s_list[kBackWarps][kBack];
+  __shared__ __align__(8) uint32_t s_list[kBackWarps][kBack];  // byte offsets of the warp's terms
   __shared__ int s_max_last;
   const int tile = a.order ? (int)a.order[blockIdx.x] : (int)blockIdx.x;
   const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
@@ -126,7 +131,10 @@ __global__ void __launch_bounds__(kBatch, 2) composite_bwd_kernel(const __grid_c
     p.dC1 = a.dl_dimage[3 * pix + 1];
     p.dC2 = a.dl_dimage[3 * pix + 2];
   }
-  if (threadIdx.x == 0) s_max_last = 0;
+  if (threadIdx.x == 0) {
+    s_max_last = 0;
+    s_g0[kBack] = s_co[kBack] = s_col[kBack] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   __syncthreads();
   const int wlast = __reduce_max_sync(0xffffffffu, last);
   if (lane == 0) atomicMax(&s_max_last, wlast);
@@ -163,48 +171,55 @@ __global__ void __launch_bounds__(kBatch, 2) composite_bwd_kernel(const __grid_c
       const int j = c0 + (int)lane;
       const bool hit = j < jend && ((s_mask[j] >> warp) & 1u);
       const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-      if (hit) s_list[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = (uint8_t)j;
+      if (hit) s_list[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = 16u * (uint32_t)j;
       cnt += __popc(bal);
     }
+    if ((cnt & 1) && lane == 0) s_list[warp][cnt] = 16u * (uint32_t)kBack;
     __syncwarp();
-    float* part = s_part + warp * kBack * kPairGrad;
-    for (int i = cnt - 1; i >= 0; i -= 2) {
-      const int ja = s_list[warp][i], jb = i > 0 ? s_list[warp][i - 1] : ja;
-      const float4 a0 = s_g0[ja], b0 = s_g0[jb], aco = s_co[ja], bco = s_co[jb], acol = s_col[ja], bcol = s_col[jb];
-      const float adx = a0.x - fx, ady = a0.y - fy, bdx = b0.x - fx, bdy = b0.y - fy;
+    char* part = reinterpret_cast<char*>(s_part + warp * (kBack + 1) * kPairGrad);
+    const int end = 16 * min(max(last - bstart, 0), kBack);  // byte offset past the pixel's last term
+    for (int i = (cnt - 1) & ~1; i >= 0; i -= 2) {
+      const uint2 l = *reinterpret_cast<const uint2*>(&s_list[warp][i]);  // l.y, the later one, first
+      const float4 a0 = staged4(s_g0, l.y), b0 = staged4(s_g0, l.x), aco = staged4(s_co, l.y), bco = staged4(s_co, l.x);
+      const float4 acol = staged4(s_col, l.y), bcol = staged4(s_col, l.x);
+      const float2 ad = __fadd2_rn(make_float2(a0.x, a0.y), make_float2(-fx, -fy));
+      const float2 bd = __fadd2_rn(make_float2(b0.x, b0.y), make_float2(-fx, -fy));
       float Ga, Gb;
-      float alpha_a = composite_alpha(a0, acol.w, aco.w, adx, ady, Ga);
-      float alpha_b = composite_alpha(b0, bcol.w, bco.w, bdx, bdy, Gb);
-      if (bstart + ja >= last) alpha_a = 0.f;
-      if (i == 0 || bstart + jb >= last) alpha_b = 0.f;
+      float alpha_a = composite_alpha(a0, acol.w, aco.w, ad.x, ad.y, Ga);
+      float alpha_b = composite_alpha(b0, bcol.w, bco.w, bd.x, bd.y, Gb);
+      if ((int)l.y >= end) alpha_a = 0.f;
+      if ((int)l.x >= end) alpha_b = 0.f;
+      // byte offset 16 j of term j is place (9/4) 16 j of its sums
+      float* pa = reinterpret_cast<float*>(part + (l.y >> 2) * kPairGrad);
+      float* pb = reinterpret_cast<float*>(part + (l.x >> 2) * kPairGrad);
       if (!__any_sync(0xffffffffu, alpha_a > 0.f || alpha_b > 0.f)) {
         if (lane < kPairGrad) {
-          part[ja * kPairGrad + lane] = 0.f;
-          part[jb * kPairGrad + lane] = 0.f;
+          pa[lane] = 0.f;
+          pb[lane] = 0.f;
         }
         continue;
       }
       float ga[kPairGrad], gb[kPairGrad], s8;
-      term_grads(p, alpha_a, Ga, aco, acol, adx, ady, ga);
-      term_grads(p, alpha_b, Gb, bco, bcol, bdx, bdy, gb);
+      term_grads(p, alpha_a, Ga, aco, acol, ad.x, ad.y, ga);
+      term_grads(p, alpha_b, Gb, bco, bcol, bd.x, bd.y, gb);
       const float s = warp_sum18(ga, gb, lane, s8);
-      float* dst = part + (lane < 16 ? ja : jb) * kPairGrad;
-      if (lane < 16 || i > 0) {
-        if ((lane & 1u) == 0u) dst[(lane >> 1) & 7u] = s;
-        if ((lane & 15u) == 0u) dst[8] = s8;
-      }
+      float* dst = lane < 16 ? pa : pb;
+      if ((lane & 1u) == 0u) dst[(lane >> 1) & 7u] = s;
+      if ((lane & 15u) == 0u) dst[8] = s8;
     }
     __syncthreads();
     if (term < jend) {  // half 0: values 0..3 of the term, half 1: values 4..8
       float v[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
       for (uint32_t m = s_mask[term]; m; m &= m - 1u) {
-        const float* src = s_part + ((__ffs((int)m) - 1) * kBack + term) * kPairGrad + 4 * half;
+        const float* src = s_part + ((__ffs((int)m) - 1) * (kBack + 1) + term) * kPairGrad + 4 * half;
 #pragma unroll
         for (int k = 0; k < 4; ++k) v[k] += src[k];
         if (half) v[4] += src[4];
       }
+      const float o = s_co[term].w, h = -0.5f * o;
       float4* dst = reinterpret_cast<float4*>(a.grad_pair + (size_t)s_slot[term] * kPairStride);
-      dst[half] = make_float4(v[0], v[1], v[2], v[3]);
+      dst[half] = half ? make_float4(h * v[0], v[1], v[2], v[3])
+                       : make_float4(-o * v[0], -o * v[1], h * v[2], -o * v[3]);
       if (half) dst[2] = make_float4(v[4], 0.f, 0.f, 0.f);
     }
   }

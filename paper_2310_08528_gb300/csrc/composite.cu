@@ -31,10 +31,6 @@ struct Staged {
   float4 blue[kSlots];  // .x
 };
 
-__device__ __forceinline__ float4 staged4(const float4* s, uint32_t byte) {
-  return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s) + byte);
-}
-
 // One staged batch of m Gaussians (list positions base .. base + m - 1) for the
 // calling thread's pixel: the warp compacts the batch to the Gaussians whose mask
 // holds its block (ballot, order kept) and walks them kStep at a time -- all weights

@@ -622,6 +622,11 @@ __device__ __forceinline__ float composite_alpha(const float4& g0, float b2, flo
   return alpha < 1.f / 255.f ? 0.f : alpha;
 }
 
+// The staged float4 at a byte offset.
+__device__ __forceinline__ float4 staged4(const float4* s, uint32_t byte) {
+  return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s) + byte);
+}
+
 // Natural-log exponent bound: a term reaches alpha >= 1/255 only where
 // -d^T K d / 2 >= ln(1/(255 o)); the bound minus 1e-3 (0.1% in alpha, far above
 // the rounding of either exponent form) is used for conservative culling.
