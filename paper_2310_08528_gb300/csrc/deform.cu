@@ -69,7 +69,7 @@ __device__ __forceinline__ void layer64(const float* __restrict__ Wt, const floa
 #pragma unroll
     for (int g = 0; g < GP; ++g) a2[g][o] = bo;
   }
-#pragma unroll 4
+#pragma unroll 8
   for (int i = 0; i < IN; ++i) {
     float xs[GP];
     if constexpr (GP == 4) {

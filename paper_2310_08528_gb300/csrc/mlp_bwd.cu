@@ -37,7 +37,7 @@ constexpr int delta_weights() {
 template <int LDW>
 __device__ __forceinline__ void back64(const float* __restrict__ W, const float* __restrict__ D, int g0, int i8,
                                        float2 (&acc)[4][4]) {
-#pragma unroll 4
+#pragma unroll 8
   for (int o = 0; o < kWidth; ++o) {
     const float4 x = *reinterpret_cast<const float4*>(D + o * kGS + g0);
     const float4 w0 = *reinterpret_cast<const float4*>(W + o * LDW + i8);
