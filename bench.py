@@ -7,8 +7,8 @@ sphere, SH degree 3, HexPlane spatial {64,128} x temporal 25 x 32 features, MLP
 width 64 -- rendered at 800x800 from 50 hemisphere cameras x 20 timestamps in
 [0,1] (view i = camera i % 50, timestamp (i // 50) % 20).  The scene stays
 resident in HBM; each timed frame uploads its camera and t, then replays one
-captured CUDA graph of deform -> project -> depth sort -> tile binning (tile
-bitmap: mark, tile scan, extract) -> composite.  L2 is flushed (a 256 MB device write) before every timed frame, and
+captured CUDA graph of deform -> project -> depth sort -> tile binning (gather,
+column and row bits, lists) -> composite.  L2 is flushed (a 256 MB device write) before every timed frame, and
 the flush is outside the timed interval.
 
 Prints ONE JSON line (rank 0).  --impl reference times the FP64 CPU oracle on
@@ -158,14 +158,16 @@ def load_peaks(sms: int = 152):
 
 
 def stage_work(stage: str, n: int, K: int, pixels: int, passes: int, prec: str, evals: int = 0,
-               bitmap: bool = True, visited: int = None, bands: int = 1):
+               bitmap: bool = True, visited: int = None, bands: int = 1, direct: bool = False):
     """Algorithmic bytes or FLOPs of one frame's launches of each stage (per-unit
     figures times the units processed).  Returns a list of (bound, work, unit);
     the first entry is the stage's primary bound; an empty list: the stage does
     no work of its own.  visited: tile pairs the compositing must read (each
     tile's list up to its last contributing Gaussian); bands: passes of the
-    per-Gaussian stages (a frame rendered in bands projects and depth-sorts once
-    per band)."""
+    per-Gaussian stages (a composed frame rendered in bands projects and depth-sorts
+    once per band); direct: a frame composited straight from the depth order."""
+    if direct:
+        bands = 1  # the bands share one projection and one depth order
     if stage == "deform":
         flops = 2 * (64 * 64 + 64 * 64 + 3 * 64 * 64 + 64 * 10) * n   # MLP contraction, 42,240 FLOP/Gaussian
         return [(("tensor" if prec == "bf16" else "alu"), flops, "FLOP"), ("hbm", 80 * n, "B")]
@@ -177,17 +179,23 @@ def stage_work(stage: str, n: int, K: int, pixels: int, passes: int, prec: str, 
         # 4 passes over 32-bit keys, each reading and writing an 8 B key and a 4 B index per Gaussian
         return [("hbm", bands * 4 * n * 24, "B")]
     if stage == "binning":
+        if direct:
+            # pairs per band: radius, rect, y parts per Gaussian
+            return [("hbm", n * (4 + 16 + 8), "B")]
         if bitmap:
-            # tile bitmap: order + rect in and the 36 B of projected data copied into rank order per
-            # Gaussian; per pair one 4 B bit-word update (read + write), the word read and cleared by the
-            # row walk and the rank written
-            return [("hbm", bands * n * (4 + 16 + 72) + K * (8 + 4 + 4 + 4), "B")]
+            # tile lists: order + rect + 36 B of projected data in, the same but the order out in rank
+            # order per Gaussian; a 4 B rank out per pair
+            return [("hbm", n * (4 + 52 + 52) + K * 4, "B")]
         # emission: order, rect, depth in + offset out per Gaussian; one 8 B (tile | index) word per pair
         # out (frames that keep no backward state sort these words without a value array)
         return [("hbm", bands * n * (4 + 16 + 4 + 4) + K * 8, "B")]
     if stage == "sort":
+        if direct:
+            # column and row bits: order, radius, rect, y parts, xy, conic + opacity, rgb in and 40 B out in
+            # rank order per Gaussian
+            return [("hbm", n * (4 + 4 + 16 + 8 + 8 + 16 + 12 + 40), "B")]
         if bitmap:
-            return []  # no pair sort: the bitmap rows list each tile's Gaussians in depth order
+            return []  # no pair sort: the column and row bits give each tile's Gaussians in depth order
         return [("hbm", passes * K * 16, "B")]                         # read + write 8 B per pair per pass
     if stage == "composite":
         # gather (idx + xy, conic/opacity, rgb) per visited pair and the rgb write per pixel; ~15 FLOP per
@@ -209,7 +217,7 @@ def _frac(bound, work, sec, peaks):
 
 SINGLE_KERNEL = {"deform": "deform_tc_kernel / deform_fp32_kernel", "project": "project_kernel",
                  "composite": "composite_kernel"}
-FUSED = {"sort": "tile bitmap binning: no pair sort (the binning stage lists each tile in depth order)"}
+FUSED = {"sort": "tile lists from column and row bits: no pair sort (the binning stage lists each tile in depth order)"}
 
 
 def visited_pairs(torch, nc, tile: int = 16) -> int:
@@ -222,10 +230,10 @@ def visited_pairs(torch, nc, tile: int = 16) -> int:
     return int(pad.view(ty, tile, tx, tile).amax(dim=(1, 3)).sum().item())
 
 
-def roofline(stage_ms, n, K, pixels, passes, prec, peaks, evals, bitmap=True, visited=None, bands=1):
+def roofline(stage_ms, n, K, pixels, passes, prec, peaks, evals, bitmap=True, visited=None, bands=1, direct=False):
     out = {}
     for st, ms in stage_ms.items():
-        work = stage_work(st, n, K, pixels, passes, prec, evals, bitmap, visited, bands)
+        work = stage_work(st, n, K, pixels, passes, prec, evals, bitmap, visited, bands, direct)
         if not work:
             out[st] = {"ms": ms, "fused": FUSED[st]}
             continue
@@ -559,7 +567,7 @@ def stress_bench(ctx, fs4d, torch, stream, peaks, frames=3):
                 K, bands = ctx.last_pairs(), ctx.last_bands()
                 vis, evals = visited_pairs(torch, nc), int(nc.sum().item())
             r["stages"] = roofline(st, n, K, w * h, _sort_passes(w, h, bands), "bf16", peaks, evals, bitmap=False,
-                                   visited=vis, bands=bands)
+                                   visited=vis, bands=bands, direct=bands > 1)
             r["tile_pairs"], r["tile_pairs_visited"], r["bands"] = K, vis, bands
             res[f"{w}x{h}"] = r
             del image, nc
@@ -832,8 +840,8 @@ def main():
         raise SystemExit("bf16 requested but the BF16 path is not available for this scene")
 
     # kernels of one graph-replayed frame, as the library counts them for the same call
-    # (deform, project, the depth sort, then bitmap: mark, tile scan, extract, or sort:
-    # emission, tile scan, pair-sort passes; then composite)
+    # (deform, project, the depth sort, then lists: gather, bits, lists, or sort: emission,
+    # tile scan, pair-sort passes; then composite)
     launches = {}
     with torch.cuda.stream(stream):
         dev = torch.device("cuda", torch.cuda.current_device())
@@ -907,7 +915,7 @@ def main():
         "warmup": args.warmup, "ms_per_step": results[head]["ms_per_step"], "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "bf16" if head == "bf16" else "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD, "n_gaussians": scene.n, "resolution": [WIDTH, HEIGHT],
-                   "binning": "tile bitmap" if bitmap else "radix sort",
+                   "binning": "tile lists from column and row bits" if bitmap else "radix sort",
                    "tile_pairs_mean": K, "tile_pairs_visited_mean": visited, "pixel_gaussian_tests_mean": evals, "pair_capacity": cap, "parallelism": f"replicas x{world}",
                    "l2": "flushed before every timed frame (256 MB device write, outside the timed interval)",
                    "timing": "CUDA events around camera upload + CUDA-graph replay of one frame (graph without "

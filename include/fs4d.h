@@ -308,10 +308,11 @@ FS4D_API fs4d_status fs4d_last_binning(const fs4d_ctx* ctx, int32_t* mode);
 /* Per-stage device timing of frames rendered by fs4d_render / fs4d_render_async
  * (also inside a captured CUDA graph): when enabled, CUDA events are recorded on
  * the context's stream around each stage.  fs4d_stage_times waits for the last
- * recorded frame and writes ms[6] = deform, project, depth sort, binning (key
- * emission or tile bitmap, with the tile scan that writes the ranges), pair sort,
- * composite (milliseconds, that frame only; for a frame rendered in bands of tile
- * rows, each stage summed over the bands). */
+ * recorded frame and writes ms[6] = deform, project, depth sort, binning (tile lists
+ * from column and row bits, or key emission with the tile scan that writes the ranges;
+ * for a frame composited straight from the depth order, the pair count of its bands),
+ * pair sort (there, the column and row bits), composite (milliseconds, that frame
+ * only; each stage summed over the bands of tile rows of a frame that has several). */
 FS4D_API fs4d_status fs4d_set_stage_timing(fs4d_ctx* ctx, int32_t enable);
 FS4D_API fs4d_status fs4d_stage_times(fs4d_ctx* ctx, float* h_ms);
 /* With stage timing enabled, the last fs4d_render_backward's stages: h_ms[4] =

@@ -1164,7 +1164,7 @@ fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_c
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
   c->stage_acc_valid = false;
   c->last_bands = 1;
-  // too many tiles x Gaussians for the tile bitmap, or more pairs than a band may hold last time
+  // too many tiles x Gaussians for tile lists, or more pairs than a band may hold last time
   const bool banded = c->band_hint > 1 && c->band_scene == s->id && c->band_w == cam->width && c->band_h == cam->height;
   if (banded || (c->binning != FS4D_BINNING_SORT && !use_lists(c, c->w, s->n, tx, ty)))
     return render_direct(c, s, prec, cam, t, true, d_image, d_t_final, d_n_contrib);

@@ -19,8 +19,8 @@
 //
 // Bound by the FP32 FMAs (21.1k per Gaussian) and, with one group of eight warps, by
 // their latency: a group's plane taps, barriers and output layers left the FMA pipe
-// idle.  Two groups fill it for each other: 417 -> 348 us for the 300k room (its FMAs alone
-// take 157), now at 73% of the shared-memory and L1 data pipe (a k-step of a warp costs
+// idle.  Two groups fill it for each other: 417 -> 348 us for the 300k room (343 with
+// the layers unrolled by eight; its FMAs alone take 157), now at 73% of the shared-memory and L1 data pipe (a k-step of a warp costs
 // four wavefronts for its activations and two for each weight load).
 // While every tile of 32 can run at once, a call takes those: more SMs share the chain of a
 // tile (2000 Gaussians 24.1 -> 15.0 us, 5000 32.4 -> 25.4, 9000 25.5; in two rounds, at 19,000,

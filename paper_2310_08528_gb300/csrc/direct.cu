@@ -9,7 +9,7 @@
 // depth rank: tiles_x + tiles_y bit rows (47 MB for that frame) in place of 8 bytes
 // per pair, no pair sort, and nothing to size by the number of pairs.  At 1920x1080 /
 // 2M the binning and pair sort of three bands took 27.6 ms (emission 6.3, sort
-// 21.3); pair counts and bit rows take the times given at their kernels.
+// 21.3); the pair counts take 17 us and the bit rows 181.
 #include "fs4d_internal.cuh"
 
 namespace fs4d {

@@ -475,7 +475,7 @@ class Context:
         self.call("fs4d_set_band_pairs", int(max_pairs))
 
     def set_binning(self, mode: int) -> None:
-        """BINNING_AUTO (tile bitmap when it fits) or BINNING_SORT (keys + radix sort)."""
+        """BINNING_AUTO (tile lists from column and row bits when they fit) or BINNING_SORT (keys + radix sort)."""
         self.call("fs4d_set_binning", int(mode))
 
     def last_binning(self) -> int:
