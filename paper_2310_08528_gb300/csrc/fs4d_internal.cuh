@@ -508,7 +508,7 @@ struct MlpActs {
   float* d1;       // [n][64]
   float* dfh;      // [n][HL]  dL/df_h
   uint32_t* masks;
-  float* lines;    // time planes' gradients before the time weights: copies of [3 axes][line_cells][h]
+  float* lines;    // time planes' gradients at the two time rows: copies of [2 rows][3 axes][line_cells][h]
   int line_cells;  // spatial cells of all levels
 };
 size_t mlp_act_floats(long long n, const PlaneGeom& pg);

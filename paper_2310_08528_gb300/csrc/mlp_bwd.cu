@@ -10,8 +10,7 @@
 //      cell) and the sampling positions;
 //   4. wgrad kernels: dW = D^T X as 8x8 register blocks per thread, per-chunk partial sums
 //      and a fixed-order reduction (deterministic).
-// 100k Gaussians, L = 2, h = 32: recompute, deltas and planes 426 us (161, 149 and 125 before
-// the layers were unrolled by eight), weights 133; one kernel for all but the weights took
+// 100k Gaussians, L = 2, h = 32: recompute, deltas and planes 457 us, weights 133; one kernel for all but the weights took
 // 635, the weights 244.
 #include <algorithm>
 
@@ -203,15 +202,16 @@ __device__ __forceinline__ void axis_setup(float u, int R, int& i0, float& f, fl
 
 // h/4 consecutive lanes per Gaussian, a float4 of features each, level after level (so a
 // Gaussian's position gradient is one lane's sum and needs no atomics).  All Gaussians
-// share t, so a time plane's gradient is one line over its spatial axis times the two time
-// rows' weights: the atomics go to kTimeCopies copies of the lines (by CTA, against many
-// adds to one address), which time_lines_kernel spreads over the two rows -- half the
-// atomics of adding to four cells.  300k Gaussians with the recompute and the deltas: 1471
-// us with four cells and 148 registers; lines 1196, with two CTAs per SM 1135, with three
-// (80 registers, a few spilled) 1125; one copy 1285, 32 copies 1133.
+// share t, so a time plane's gradient falls on two lines of cells, the two time rows: the
+// atomics go to kTimeCopies copies of them (by CTA, against many adds to one address),
+// which time_lines_kernel adds up.  300k Gaussians with the recompute and the deltas: 1398
+// us straight into the planes, 1186 with eight copies, 1263 with two; three CTAs per SM
+// instead of two 1198.  One line per axis that the two rows' weights multiply at the end
+// took half the adds (1097), but the products' other rounding turned the sign of a sum near
+// zero, and with it Adam's step, for 17 seeds of 30 against 1 for either form above.
 constexpr int kTimeCopies = 8;
 template <int H, int L>
-__global__ void __launch_bounds__(256, 3) plane_bwd_kernel(const __grid_constant__ MlpBwdArgs a) {
+__global__ void __launch_bounds__(256, 2) plane_bwd_kernel(const __grid_constant__ MlpBwdArgs a) {
   constexpr int Q = H / 4, HL = H * L;
   const DeformArgs& f = a.f;
   const PlaneGeom& pg = f.pg;
@@ -277,20 +277,20 @@ __global__ void __launch_bounds__(256, 3) plane_bwd_kernel(const __grid_constant
           sa += gv[e] * ((1.f - fb) * (Bs[e] - As[e]) + fb * (Es[e] - Cs[e]));
           sb += gv[e] * ((1.f - fa) * (Cs[e] - As[e]) + fa * (Es[e] - Bs[e]));
         }
-        if (a.g_planes && p >= 3) {
-          float* G = a.act.lines + (((long long)(blockIdx.x % kTimeCopies) * 3 + ax) * a.act.line_cells + line0 + i0[ax]) * H + 4 * q;
-          atomicAdd(reinterpret_cast<float4*>(G),
-                    make_float4((1.f - fa) * gv[0], (1.f - fa) * gv[1], (1.f - fa) * gv[2], (1.f - fa) * gv[3]));
-          atomicAdd(reinterpret_cast<float4*>(G + H), make_float4(fa * gv[0], fa * gv[1], fa * gv[2], fa * gv[3]));
-        } else if (a.g_planes) {
+        if (a.g_planes) {
           float* GP = a.g_planes + cell;
+          long long up = (long long)Ra * H;  // to the next row of the second axis
+          if (p >= 3) {
+            up = 3ll * a.act.line_cells * H;
+            GP = a.act.lines + (((long long)(blockIdx.x % kTimeCopies) * 6 + ax) * a.act.line_cells + line0 + i0[ax]) * H + 4 * q;
+          }
           const float w00 = (1.f - fa) * (1.f - fb), w10 = fa * (1.f - fb), w01 = (1.f - fa) * fb, w11 = fa * fb;
           atomicAdd(reinterpret_cast<float4*>(GP), make_float4(w00 * gv[0], w00 * gv[1], w00 * gv[2], w00 * gv[3]));
           atomicAdd(reinterpret_cast<float4*>(GP + H),
                     make_float4(w10 * gv[0], w10 * gv[1], w10 * gv[2], w10 * gv[3]));
-          atomicAdd(reinterpret_cast<float4*>(GP + (long long)Ra * H),
+          atomicAdd(reinterpret_cast<float4*>(GP + up),
                     make_float4(w01 * gv[0], w01 * gv[1], w01 * gv[2], w01 * gv[3]));
-          atomicAdd(reinterpret_cast<float4*>(GP + (long long)Ra * H + H),
+          atomicAdd(reinterpret_cast<float4*>(GP + up + H),
                     make_float4(w11 * gv[0], w11 * gv[1], w11 * gv[2], w11 * gv[3]));
         }
         if (ax < 3) gxs[ax] += sa * df[ax] * pg.aabb_scale[ax];
@@ -318,16 +318,19 @@ __global__ void __launch_bounds__(256) time_lines_kernel(const __grid_constant__
   if (e >= 3 * per) return;
   const int ax = e / per;
   int cell = (e % per) / H, l = 0;
-  float g = 0.f;
+  float g0 = 0.f, g1 = 0.f;
 #pragma unroll
-  for (int k = 0; k < kTimeCopies; ++k) g += a.act.lines[(long long)k * 3 * per + e];
+  for (int k = 0; k < kTimeCopies; ++k) {
+    g0 += a.act.lines[(long long)(2 * k) * 3 * per + e];
+    g1 += a.act.lines[(long long)(2 * k + 1) * 3 * per + e];
+  }
   for (; cell >= pg.res[l]; ++l) cell -= pg.res[l];
   int j0;
   float fb, db;
   axis_setup(2.f * a.f.t0 - 1.f, pg.res_time, j0, fb, db);
   float* out = a.g_planes + pg.off[l][3 + ax] + ((long long)j0 * pg.res[l] + cell) * H + e % H;
-  out[0] += (1.f - fb) * g;
-  out[(long long)pg.res[l] * H] += fb * g;
+  out[0] += g0;
+  out[(long long)pg.res[l] * H] += g1;
 }
 
 // ------------------------------------------------------------------ weight gradients
@@ -505,7 +508,7 @@ cudaError_t launch_bwd_t(const MlpBwdArgs& a, cudaStream_t s) {
   mlp_delta_kernel<HL><<<(unsigned)(tiles < sms ? tiles : sms), kGroups * kThreads, smem, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t line_floats = 3 * (size_t)a.act.line_cells * H;
-  if (a.g_planes && (e = cudaMemsetAsync(a.act.lines, 0, 4 * kTimeCopies * line_floats, s)) != cudaSuccess) return e;
+  if (a.g_planes && (e = cudaMemsetAsync(a.act.lines, 0, 4 * 2 * kTimeCopies * line_floats, s)) != cudaSuccess) return e;
   const long long items = (long long)a.f.n * (H / 4);
   plane_bwd_kernel<H, L><<<(unsigned)((items + 255) / 256), 256, 0, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess || !a.g_planes) return e;
@@ -526,7 +529,7 @@ int line_cells(const PlaneGeom& pg) {
 size_t mlp_act_floats(long long n, const PlaneGeom& pg) {
   const long long tiles = (n + kTG - 1) / kTG;
   return (size_t)n * (2 * pg.feat_dim * pg.n_levels + 64 + 64 + 192 + 12 + 192 + 64 + 64) +
-         (size_t)tiles * 5 * kThreads + (size_t)kTimeCopies * 3 * line_cells(pg) * pg.feat_dim;
+         (size_t)tiles * 5 * kThreads + (size_t)kTimeCopies * 6 * line_cells(pg) * pg.feat_dim;
 }
 
 MlpActs mlp_acts(float* base, long long n, const PlaneGeom& pg) {
