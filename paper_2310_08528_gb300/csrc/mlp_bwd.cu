@@ -10,8 +10,8 @@
 //      cell) and the sampling positions;
 //   4. wgrad kernels: dW = D^T X as 8x8 register blocks per thread, per-chunk partial sums
 //      and a fixed-order reduction (deterministic).
-// 100k Gaussians, L = 2, h = 32: recompute, deltas and planes 457 us, weights 133; one kernel for all but the weights took
-// 635, the weights 244.
+// 100k Gaussians, L = 2, h = 32: recompute, deltas and planes 457 us, weights 133; one
+// kernel for all but the weights took 635, the weights 244.
 #include <algorithm>
 
 #include "fs4d_internal.cuh"
