@@ -354,7 +354,7 @@ def training_bench(ctx, fs4d, torch, sid, scene, stream, steps=10, warmup=3):
         return {"workload": "one view of the 800x800 / 100k object, dL/dI ~ N(0,1), gradients of every parameter "
                             "group", "steps": steps, "forward_saved_ms": f, "backward_ms": b, "step_ms": f + b,
                 "views_per_s": 1e3 / (f + b), "backward_kernels_ms": per,
-                "note": "the forward keeps the backward's state (sort binning, emission offsets, copies)"}
+                "note": "the forward keeps the backward's state (full tile lists, written into the frame's own buffers)"}
     except Exception as exc:  # the headline line must still be printed
         return {"error": f"{type(exc).__name__}: {exc}"}
 
