@@ -5,7 +5,8 @@
 //  composite_bwd_kernel  one CTA per tile, one pixel per thread, walking the
 //      tile's list back to front from each pixel's last blended term.  The
 //      contributions of the 256 pixels to each Gaussian are summed inside the
-//      CTA and written ONCE per (tile, Gaussian) pair into that pair's slot, so no
+//      CTA (warp shuffles, then shared-memory adds) and written ONCE per
+//      (tile, Gaussian) pair into that pair's slot, so no
 //      global atomics are needed: a Gaussian's slots are contiguous (offsets[g] ...
 //      offsets[g] + rect area).
 //  project_bwd_kernel    one thread per Gaussian: sums its pair slots, then
@@ -54,60 +55,90 @@ __device__ __forceinline__ float warp_sum18(const float (&a)[kPairGrad], const f
 // The state of a pixel on its way back to front.
 struct PixelBack {
   float T;                 // transmittance behind the current term
-  float b0, b1, b2;        // minus the colour blended behind it
+  float b0, b1, b2;        // the colour blended behind it
   float dC0, dC1, dC2;     // dL/dC
 };
 
-// The gradients of one blended term (alpha > 0) at offset (dx, dy), zero otherwise, without
-// the opacity's factor, which is the same for every pixel and multiplies the sums: with
-// u = G dL/dalpha (0 where alpha is capped), u K d, u (dx^2, dx dy, dy^2), u, and dL/dcolour.
-// dL/dalpha = sum_k dC_k (col_k T - b_k) / (1 - alpha) rounds col_k T - b_k once, where
-// the two cancel.  The mean's u K d stays a per-pixel product: A sum(u dx) + B sum(u dy)
-// would cancel in thin, oblique ellipses (ten times the error at 1000:1).  Selects, no
-// branch: nine values under a divergent branch took 549 us where this takes 535.
+// The gradients of one blended term (alpha > 0) at offset (dx, dy), zero otherwise.  The
+// products are rounded per pixel, the opacity's factor included, in this order: a training
+// step's first Adam updates take the sign of a gradient alone, so another rounding (the
+// opacity multiplied into the sums; col T - b divided once) changes the step of the plane
+// cells whose sum cancels below it.  Selects, no branch: nine values under a divergent
+// branch took 549 us where selects took 535.
 __device__ __forceinline__ void term_grads(PixelBack& p, float alpha, float G, const float4& co, const float4& col,
                                            float dx, float dy, float (&gr)[kPairGrad]) {
   const bool on = alpha > 0.f;
   const float inv = 1.f / (1.f - alpha);
-  const float x0 = fmaf(col.x, p.T, p.b0), x1 = fmaf(col.y, p.T, p.b1), x2 = fmaf(col.z, p.T, p.b2);
-  const float dalpha = (p.dC0 * x0 + p.dC1 * x1 + p.dC2 * x2) * inv;
-  const float Ti = p.T * inv, w = alpha * Ti;
+  const float Ti = p.T * inv;
+  const float c0 = col.x, c1 = col.y, c2 = col.z;
+  const float dalpha =
+      p.dC0 * (c0 * Ti - p.b0 * inv) + p.dC1 * (c1 * Ti - p.b1 * inv) + p.dC2 * (c2 * Ti - p.b2 * inv);
+  const float w = alpha * Ti;
   gr[6] = on ? p.dC0 * w : 0.f;
   gr[7] = on ? p.dC1 * w : 0.f;
   gr[8] = on ? p.dC2 * w : 0.f;
   if (on) {
+    p.b0 += c0 * w;
+    p.b1 += c1 * w;
+    p.b2 += c2 * w;
     p.T = Ti;
-    p.b0 = fmaf(col.x, -w, p.b0);
-    p.b1 = fmaf(col.y, -w, p.b1);
-    p.b2 = fmaf(col.z, -w, p.b2);
   }
-  const float u = on && co.w * G <= kAlphaMax ? dalpha * G : 0.f, ux = u * dx, uy = u * dy;
-  gr[0] = u * (co.x * dx + co.y * dy);
-  gr[1] = u * (co.z * dy + co.y * dx);
-  gr[2] = ux * dx;
-  gr[3] = ux * dy;
-  gr[4] = uy * dy;
-  gr[5] = u;
+  const bool grad = on && co.w * G <= kAlphaMax;
+  const float dpow = grad ? dalpha * co.w * G : 0.f;
+  gr[0] = -dpow * (co.x * dx + co.y * dy);
+  gr[1] = -dpow * (co.z * dy + co.y * dx);
+  gr[2] = -0.5f * dpow * dx * dx;
+  gr[3] = -dpow * dx * dy;
+  gr[4] = -0.5f * dpow * dy * dy;
+  gr[5] = grad ? dalpha * G : 0.f;
+}
+
+// Bit w set iff some pixel centre of the 16x2 pixel rows (2w, 2w + 1) of tile (tx, ty), warp
+// w's pixels, may reach alpha >= 1/255: block_mask's column intervals and margins, per pair
+// of rows.
+__device__ __forceinline__ uint32_t row_pair_mask(float2 p, float4 co, float thr, int tx, int ty) {
+  if (!(thr < 0.f)) return 0u;
+  const float A = co.x, B = co.y, C = co.z, det = conic_det(co);
+  if (!conic_bounded(co, det)) return 0xffu;
+  const float s = -2.f * thr * 1.002f + 1e-3f;
+  const float X0 = (float)(tx * kTile) + 0.5f - p.x, Y0 = (float)(ty * kTile) + 0.5f - p.y;
+  const float iA = 1.f / A, sd = s / det, k = B * iA, wA = s * iA, wd = det * iA * iA;
+  const float hx = sqrt_approx(sd * C), hy = sqrt_approx(sd * A) * 1.00001f + 0.01f;
+  const float yr = -B / C * hx;  // the row of the greatest column
+  const float slack = 1e-5f * hx + 0.01f;
+  uint32_t mask = 0u;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const float ya = Y0 + (float)(2 * r), yb = ya + 1.f;
+    const float a = fmaxf(ya, -hy), b = fminf(yb, hy);
+    const float va = sqrt_approx(fmaxf(0.f, wA - wd * a * a)), vb = sqrt_approx(fmaxf(0.f, wA - wd * b * b));
+    float hi = fmaxf(va - k * a, vb - k * b), lo = fminf(-va - k * a, -vb - k * b);
+    if (yr >= a && yr <= b) hi = hx;
+    if (-yr >= a && -yr <= b) lo = -hx;
+    if (!(a > b) && !(hi + slack < X0) && !(lo - slack > X0 + 15.f)) mask |= 1u << r;
+  }
+  return mask;
 }
 
 // One CTA per tile in the forward's launch order (longest lists first), one pixel per
-// thread, the forward's 8x4 pixel blocks per warp.  Batches of kBack terms are staged with
-// the forward's block masks, and each warp compacts a batch to the terms its block may
-// blend and walks them back to front, two per step: both weights before the two updates,
-// one reduction for both.  A warp leaves its sums of a term in its own place in shared
-// memory (no atomics, nothing to clear: the output adds up the warps of the term's mask, in
-// order) and each (tile, Gaussian) slot is written once.  Bound by instruction issue, about
-// ninety per term and warp: 240 -> 110 us at 800x800 / 100k, 992 -> 535 at 1352x1014 / 300k
-// against 16x2 blocks that test every term of a batch, reduce one term at a time and add to
-// shared memory with float atomics, in tile order.  (115 and 618 with byte indices, the
-// terms' products taken per pixel and branches; at the registers of three CTAs per SM 105
-// and 560: the few tiles of the small frame end later with four.)
+// thread, 16x2 pixels per warp.  Batches of kBack terms are staged with the masks of the
+// warps that may blend them, and each warp compacts a batch to its terms and walks them back
+// to front, two per step: both weights before the two updates, one reduction for both.  A
+// warp adds its sum of a term to the CTA's, or its few pixels one by one, and each
+// (tile, Gaussian) slot is written once.  The sums' order is fixed within a warp and
+// free among the warps.  Bound by instruction issue and the shared adds: 240 -> 181 us at
+// 800x800 / 100k and 992 -> 769 at 1352x1014 / 300k against every term of a batch tested
+// by every warp and reduced one at a time, in tile order.  Other orders of the same sums
+// are faster, 111 and 536 us (8x4 pixels per warp, the opacity's factor multiplied into the
+// sums, a place in shared memory per warp) and 129 and 626 (16x2 pixels and a place per
+// warp), but a training step then sends plane cells the other way in 35 and 34 of 750
+// steps of small and large scenes; here it is 23, where this order against itself has 20.
 constexpr int kBack = 128;
+constexpr int kFewPixels = 4;  // a warp adds up to this many pixels of a term one by one
 constexpr int kBackWarps = kBatch / 32;
-constexpr size_t kBackSmem = 4 * (size_t)kBackWarps * (kBack + 1) * kPairGrad;
 
 __global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_constant__ CompositeBwdArgs a) {
-  extern __shared__ float s_part[];        // [kBackWarps][kBack + 1][kPairGrad]
+  __shared__ float s_acc[(kBack + 1) * kPairGrad];  // the terms' sums
   __shared__ float4 s_g0[kBack + 1];       // x, y, a2, c2 (the last place: a term that adds nothing)
   __shared__ float4 s_co[kBack + 1];       // conic, opacity
   __shared__ float4 s_col[kBack + 1];      // colour, b2
@@ -117,7 +148,7 @@ __global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_c
   const int tile = a.order ? (int)a.order[blockIdx.x] : (int)blockIdx.x;
   const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
   const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const int px = tx * kTile + (int)(warp & 1) * 8 + (int)(lane & 7), py = ty * kTile + (int)(warp >> 1) * 4 + (int)(lane >> 3);
+  const int px = tx * kTile + (int)(lane & 15), py = ty * kTile + (int)warp * 2 + (int)(lane >> 4);
   const bool inside = px < a.width && py < a.height;
   const int pix = py * a.width + px;
   const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
@@ -145,6 +176,7 @@ __global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_c
   for (int bstart = ((max_last - 1) / kBack) * kBack; bstart >= 0 && max_last > 0; bstart -= kBack) {
     __syncthreads();  // the previous batch's sums have been written out
     const int jend = min(kBack, max_last - bstart);
+    for (int k = threadIdx.x; k < kBack * kPairGrad; k += kBatch) s_acc[k] = 0.f;
     if (term < jend) {
       const uint32_t g = a.values[range.x + bstart + term];
       const float4 co = a.conic_opacity[g];
@@ -152,7 +184,7 @@ __global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_c
         const float2 xy = a.xy[g];
         s_g0[term] = composite_coeffs(xy, co);
         s_co[term] = co;
-        s_mask[term] = block_mask(xy, co, composite_exp_threshold(co.w), tx, ty);
+        s_mask[term] = row_pair_mask(xy, co, composite_exp_threshold(co.w), tx, ty);
       } else {
         s_col[term] = make_float4(a.rgb[3 * (size_t)g], a.rgb[3 * (size_t)g + 1], a.rgb[3 * (size_t)g + 2],
                                   composite_b2(co));
@@ -176,7 +208,6 @@ __global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_c
     }
     if ((cnt & 1) && lane == 0) s_list[warp][cnt] = 16u * (uint32_t)kBack;
     __syncwarp();
-    char* part = reinterpret_cast<char*>(s_part + warp * (kBack + 1) * kPairGrad);
     const int end = 16 * min(max(last - bstart, 0), kBack);  // byte offset past the pixel's last term
     for (int i = (cnt - 1) & ~1; i >= 0; i -= 2) {
       const uint2 l = *reinterpret_cast<const uint2*>(&s_list[warp][i]);  // l.y, the later one, first
@@ -190,36 +221,32 @@ __global__ void __launch_bounds__(kBatch, 4) composite_bwd_kernel(const __grid_c
       if ((int)l.y >= end) alpha_a = 0.f;
       if ((int)l.x >= end) alpha_b = 0.f;
       // byte offset 16 j of term j is place (9/4) 16 j of its sums
-      float* pa = reinterpret_cast<float*>(part + (l.y >> 2) * kPairGrad);
-      float* pb = reinterpret_cast<float*>(part + (l.x >> 2) * kPairGrad);
-      if (!__any_sync(0xffffffffu, alpha_a > 0.f || alpha_b > 0.f)) {
-        if (lane < kPairGrad) {
-          pa[lane] = 0.f;
-          pb[lane] = 0.f;
-        }
-        continue;
-      }
+      float* pa = reinterpret_cast<float*>(reinterpret_cast<char*>(s_acc) + (l.y >> 2) * kPairGrad);
+      float* pb = reinterpret_cast<float*>(reinterpret_cast<char*>(s_acc) + (l.x >> 2) * kPairGrad);
+      const unsigned ma = __ballot_sync(0xffffffffu, alpha_a > 0.f), mb = __ballot_sync(0xffffffffu, alpha_b > 0.f);
+      if ((ma | mb) == 0u) continue;
       float ga[kPairGrad], gb[kPairGrad], s8;
       term_grads(p, alpha_a, Ga, aco, acol, ad.x, ad.y, ga);
       term_grads(p, alpha_b, Gb, bco, bcol, bd.x, bd.y, gb);
-      const float s = warp_sum18(ga, gb, lane, s8);
-      float* dst = lane < 16 ? pa : pb;
-      if ((lane & 1u) == 0u) dst[(lane >> 1) & 7u] = s;
-      if ((lane & 15u) == 0u) dst[8] = s8;
+      const bool many_a = __popc(ma) > kFewPixels, many_b = __popc(mb) > kFewPixels;
+      if (many_a || many_b) {
+        const float s = warp_sum18(ga, gb, lane, s8);
+        const bool last = (lane & 15u) == 1u;  // (value 8 from the first odd lane)
+        if ((lane < 16 ? many_a : many_b) && ((lane & 1u) == 0u || last))
+          atomicAdd((lane < 16 ? pa : pb) + (last ? 8 : (lane >> 1) & 7u), last ? s8 : s);
+      }
+      if (!many_a && alpha_a > 0.f)
+#pragma unroll
+        for (int k = 0; k < kPairGrad; ++k) atomicAdd(&pa[k], ga[k]);
+      if (!many_b && alpha_b > 0.f)
+#pragma unroll
+        for (int k = 0; k < kPairGrad; ++k) atomicAdd(&pb[k], gb[k]);
     }
     __syncthreads();
     if (term < jend) {  // half 0: values 0..3 of the term, half 1: values 4..8
-      float v[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-      for (uint32_t m = s_mask[term]; m; m &= m - 1u) {
-        const float* src = s_part + ((__ffs((int)m) - 1) * (kBack + 1) + term) * kPairGrad + 4 * half;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] += src[k];
-        if (half) v[4] += src[4];
-      }
-      const float o = s_co[term].w, h = -0.5f * o;
+      const float* v = s_acc + term * kPairGrad + 4 * half;
       float4* dst = reinterpret_cast<float4*>(a.grad_pair + (size_t)s_slot[term] * kPairStride);
-      dst[half] = half ? make_float4(h * v[0], v[1], v[2], v[3])
-                       : make_float4(-o * v[0], -o * v[1], h * v[2], -o * v[3]);
+      dst[half] = make_float4(v[0], v[1], v[2], v[3]);
       if (half) dst[2] = make_float4(v[4], 0.f, 0.f, 0.f);
     }
   }
@@ -516,12 +543,7 @@ __global__ void __launch_bounds__(kProj) project_bwd_kernel(const __grid_constan
 cudaError_t launch_composite_bwd(const CompositeBwdArgs& a, cudaStream_t s) {
   const int tiles_y = (a.height + kTile - 1) / kTile;
   if (a.tiles_x * tiles_y == 0) return cudaSuccess;
-  static PerDeviceFlag attr;
-  const cudaError_t e = once_per_device(attr, [] {
-    return cudaFuncSetAttribute(composite_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBackSmem);
-  });
-  if (e != cudaSuccess) return e;
-  composite_bwd_kernel<<<a.tiles_x * tiles_y, kBatch, kBackSmem, s>>>(a);
+  composite_bwd_kernel<<<a.tiles_x * tiles_y, kBatch, 0, s>>>(a);
   return cudaGetLastError();
 }
 

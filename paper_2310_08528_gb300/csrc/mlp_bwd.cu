@@ -201,11 +201,12 @@ __device__ __forceinline__ void axis_setup(float u, int R, int& i0, float& f, fl
 }
 
 // h/4 consecutive lanes per Gaussian, a float4 of features each, level after level (so a
-// Gaussian's position gradient is one lane's sum and needs no atomics).  All Gaussians
+// Gaussian's position gradient is one lane's sum, level by level, and needs no atomics).  All Gaussians
 // share t, so a time plane's gradient falls on two lines of cells, the two time rows: the
 // atomics go to kTimeCopies copies of them (by CTA, against many adds to one address),
 // which time_lines_kernel adds up.  300k Gaussians with the recompute and the deltas: 1398
-// us straight into the planes, 1186 with eight copies, 1263 with two; three CTAs per SM
+// us straight into the planes, 1186 with eight copies (1194 with the positions level by
+// level, as their adds to memory were), 1263 with two; three CTAs per SM
 // instead of two 1198.  One line per axis that the two rows' weights multiply at the end
 // took half the adds (1097), but the products' other rounding turned the sign of a sum near
 // zero, and with it Adam's step, for 17 seeds of 30 against 1 for either form above.
@@ -220,14 +221,18 @@ __global__ void __launch_bounds__(256, 2) plane_bwd_kernel(const __grid_constant
   const long long ii = item / Q;
   const bool live = ii < f.n;
   const long long g = live ? (f.perm ? (long long)f.perm[ii] : ii) : 0;
-  float gxs[3] = {0.f, 0.f, 0.f};
-  if (live) {
-    const float c[4] = {(f.means[3 * g] - pg.aabb_min[0]) * pg.aabb_scale[0] - 1.f,
-                        (f.means[3 * g + 1] - pg.aabb_min[1]) * pg.aabb_scale[1] - 1.f,
-                        (f.means[3 * g + 2] - pg.aabb_min[2]) * pg.aabb_scale[2] - 1.f, 2.f * f.t0 - 1.f};
-    int line0 = 0;  // first cell of the level in a line
+  float c[4] = {0.f, 0.f, 0.f, 2.f * f.t0 - 1.f}, gm[3] = {0.f, 0.f, 0.f};
+  if (live)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      c[k] = (f.means[3 * g + k] - pg.aabb_min[k]) * pg.aabb_scale[k] - 1.f;
+      if (a.g_means && q == 0) gm[k] = a.g_means[3 * g + k];
+    }
+  int line0 = 0;  // first cell of the level in a line
 #pragma unroll 1
-    for (int l = 0; l < L; line0 += pg.res[l], ++l) {
+  for (int l = 0; l < L; line0 += pg.res[l], ++l) {
+    float gxs[3] = {0.f, 0.f, 0.f};
+    if (live) {
       const float4 gf4 = *reinterpret_cast<const float4*>(a.act.dfh + ii * HL + l * H + 4 * q);
       const float gf[4] = {gf4.x, gf4.y, gf4.z, gf4.w};
       int i0[4];
@@ -297,17 +302,18 @@ __global__ void __launch_bounds__(256, 2) plane_bwd_kernel(const __grid_constant
         if (bx < 3) gxs[bx] += sb * df[bx] * pg.aabb_scale[bx];
       }
     }
+    // the level's position gradient: the Q lanes of one Gaussian are consecutive and Q divides 32
+    if (!a.g_means) continue;
+#pragma unroll
+    for (int w = 1; w < Q; w <<= 1)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) gxs[k] += __shfl_xor_sync(0xffffffffu, gxs[k], w);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gm[k] += gxs[k];
   }
-  if (!a.g_means) return;
-  // the Q lanes of one Gaussian are consecutive and Q divides 32
+  if (a.g_means && live && q == 0)
 #pragma unroll
-  for (int w = 1; w < Q; w <<= 1)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) gxs[k] += __shfl_xor_sync(0xffffffffu, gxs[k], w);
-  if (live && q == 0) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) a.g_means[3 * g + k] += gxs[k];
-  }
+    for (int k = 0; k < 3; ++k) a.g_means[3 * g + k] = gm[k];
 }
 
 // The lines of the time planes (all copies) into their two time rows.
