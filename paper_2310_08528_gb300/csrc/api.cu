@@ -544,6 +544,8 @@ fs4d_status ensure_color(fs4d_ctx* c, Work& w, cudaStream_t stream, int n) {
   return FS4D_OK;
 }
 
+// Bytes of the tiles by length class, and of the bit rows.
+size_t class_bytes(long long n_tiles) { return 4 * 32 * (size_t)n_tiles; }
 size_t axis_bytes(int n, long long rows) { return 4 * (size_t)rows * (size_t)bitmap_words(std::max(n, 1)); }
 
 fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx, int ty, long long pairs) {
@@ -553,7 +555,7 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   const bool bits = image || (c->binning != FS4D_BINNING_SORT && bitmap_bytes(n, (long long)tx * ty) <= kBitmapMaxBytes);
   const long long rows = std::max(bits ? (long long)tx + ty : 0ll, w.cap_rows);
   const size_t axis = axis_bytes(std::max(n, w.cap_n), rows);
-  const size_t order = 4 * (size_t)n_tiles * (image ? 32 : 1);  // 32 length classes
+  const size_t order = image ? class_bytes(n_tiles) : 4 * (size_t)n_tiles;
   const bool grow = n > w.cap_n || n_tiles > w.cap_tiles || pairs > w.cap_pairs || axis > w.axis.bytes ||
                     order > w.tile_order.bytes;
   if (!grow) return FS4D_OK;
@@ -611,9 +613,14 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
 }
 
 // Whether a frame of n Gaussians over tx x ty tiles has tile lists from column and row bits.
-bool use_lists(const fs4d_ctx* c, const Work& w, int n, int tx, int ty) {
-  return c->binning != FS4D_BINNING_SORT && n > 0 && bitmap_bytes(n, (long long)tx * ty) <= kBitmapMaxBytes &&
-         axis_bytes(n, (long long)tx + ty) <= w.axis.bytes;
+// classes: with the tiles by length class (every frame; bin_sort lists have none).  A frame
+// that allocates nothing may be larger than what its buffers were sized for: then it has
+// lists by emission and sort, which need no more than cap_tiles says.
+bool use_lists(const fs4d_ctx* c, const Work& w, int n, int tx, int ty, bool classes = true) {
+  const long long n_tiles = (long long)tx * ty;
+  return c->binning != FS4D_BINNING_SORT && n > 0 && bitmap_bytes(n, n_tiles) <= kBitmapMaxBytes &&
+         axis_bytes(n, (long long)tx + ty) <= w.axis.bytes &&
+         (!classes || class_bytes(n_tiles) <= w.tile_order.bytes);
 }
 
 fs4d_status ensure_work(fs4d_ctx* c, int n, int tx, int ty, long long pairs) {
@@ -2085,7 +2092,7 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
   if (st != FS4D_OK) return st;
   Work& w = c->w;
   const int tile_bits = ceil_log2(n_tiles);
-  const bool bmp = use_lists(c, w, n, tiles_x, tiles_y);
+  const bool bmp = use_lists(c, w, n, tiles_x, tiles_y, false);
   c->last_binning = bmp ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
   // everything that starts at zero, as a frame's (frame_depth_order)
   w.buckets = bmp && sort_by_buckets(n);

@@ -1,0 +1,54 @@
+"""Work memory that calls of several kinds and sizes share: what one call sized is enough for
+the next, whatever came before it."""
+import numpy as np
+import pytest
+
+from paper_2310_08528_gb300 import scenegen as sg
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2310_08528_gb300 import fs4d  # noqa: E402
+
+
+@pytest.fixture()
+def ctx():
+    c = fs4d.Context(0)
+    yield c
+    c.close()
+
+
+def long_row(ctx, n, tiles):
+    """A bin_sort of n Gaussians over one row of tiles."""
+    depth = torch.linspace(1, 2, n, device="cuda")
+    x = (torch.arange(n, device="cuda") * (tiles // n)).int()
+    rect = torch.stack([x, 0 * x, x + 1, 0 * x + 1], 1).contiguous()
+    _, vals, _, k = ctx.bin_sort(depth, rect, tiles, 1, n)
+    assert k == n and torch.equal(vals, torch.arange(n, device="cuda", dtype=torch.int32))
+
+
+@pytest.mark.parametrize("tiles", [6000, 100_000])
+def test_async_frame_after_a_long_row_of_tiles(ctx, tiles):
+    """bin_sort sizes the tiles' buffers for a grid that is no image (without length classes); a
+    larger frame than the reserved one then has its lists by another route, with the same image."""
+    s = sg.make_object(3, n=3000, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=1200, height=1200, seed=3)[1]
+    sid = ctx.load_scene(s)
+    other = fs4d.Context(0)
+    try:
+        want = other.render(other.load_scene(s), cam, 0.3)
+        pairs = other.last_pairs()
+    finally:
+        other.close()
+    long_row(ctx, 1000, tiles)
+    ctx.reserve(sid, 64, 64, 2 * pairs)
+    d_cam = torch.from_numpy(np.frombuffer(bytes(fs4d.camera_struct(cam)), np.float32).copy()).cuda()
+    image = torch.empty(1200, 1200, 3, device="cuda")
+    ctx.render_async(sid, cam, d_cam, torch.tensor([0.3], device="cuda"), image)
+    assert ctx.last_binning() == fs4d.BINNING_SORT
+    torch.cuda.synchronize()
+    assert torch.equal(image, want)
+    ctx.check_device_status()
