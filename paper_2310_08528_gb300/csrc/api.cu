@@ -77,7 +77,10 @@ cudaError_t ensure(DevBuf& b, size_t bytes) {
   }
   if (bytes == 0) return cudaSuccess;
   cudaError_t e = cudaMalloc(&b.p, bytes + kCanaryBytes);
-  if (e == cudaSuccess) b.bytes = bytes;
+  if (e == cudaSuccess)
+    b.bytes = bytes;
+  else
+    (void)cudaGetLastError();  // (the caller reports it: the next launch check is not to find it again)
 #ifdef FS4D_CHECK_BOUNDS
   if (e == cudaSuccess) {
     e = cudaMemset(static_cast<unsigned char*>(b.p) + bytes, kCanary, kCanaryBytes);
@@ -162,7 +165,6 @@ struct Work {
   long long cap_pairs = 0;
   long long sort_parts_cap = 0;
   int cap_n = 0, cap_tiles = 0;
-  long long cap_rows = 0;                  // bit rows (tile columns + tile rows)
 };
 
 void release_work(Work& w) {
@@ -537,6 +539,7 @@ fs4d_status get_scene(fs4d_ctx* c, fs4d_scene_id id, Scene** out) {
 fs4d_status ensure_color(fs4d_ctx* c, Work& w, cudaStream_t stream, int n) {
   if (w.cap_color >= n) return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(stream));
+  w.cap_color = 0;
   FS4D_CUDA(c, ensure(w.fd, 4 * 64 * (size_t)n + 16384));  // + the last BF16 tile image's ragged end
   FS4D_CUDA(c, ensure(w.dsh, 4 * 48 * (size_t)n));
   FS4D_CUDA(c, ensure(w.dop, 4 * (size_t)n));
@@ -553,15 +556,19 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   // bit rows for an image's tiles, or for lists of any number of tiles (bin_sort)
   const bool image = tx <= kMaxTileRows && ty <= kMaxTileRows;
   const bool bits = image || (c->binning != FS4D_BINNING_SORT && bitmap_bytes(n, (long long)tx * ty) <= kBitmapMaxBytes);
-  const long long rows = std::max(bits ? (long long)tx + ty : 0ll, w.cap_rows);
-  const size_t axis = axis_bytes(std::max(n, w.cap_n), rows);
+  // (this call's rows and Gaussians: the largest of each, from calls of different kinds, could
+  // come to many gigabytes that no call needs)
+  const size_t axis = bits ? axis_bytes(n, (long long)tx + ty) : 0;
   const size_t order = image ? class_bytes(n_tiles) : 4 * (size_t)n_tiles;
   const bool grow = n > w.cap_n || n_tiles > w.cap_tiles || pairs > w.cap_pairs || axis > w.axis.bytes ||
-                    order > w.tile_order.bytes;
+                    order > w.tile_order.bytes || w.sort_parts_cap == 0 || !w.zero.p;
   if (!grow) return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(stream));
+  // a capacity is 0 while its buffers are reallocated: after a failure the next call allocates
+  // them again, for its own size
   if (n > w.cap_n) {
     const size_t m = (size_t)n;
+    w.cap_n = 0;
     FS4D_CUDA(c, ensure(w.dmeans, 12 * m));
     FS4D_CUDA(c, ensure(w.dquats, 16 * m));
     FS4D_CUDA(c, ensure(w.dscales, 12 * m));
@@ -586,12 +593,16 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   FS4D_CUDA(c, ensure(w.counters, 4 * kCounters));
   FS4D_CUDA(c, ensure(w.bstart, 4 * (kBuckets + 4)));
   FS4D_CUDA(c, ensure(w.hist, 4 * 256 * kSortMaxPasses));
-  if (n_tiles > w.cap_tiles) {
-    FS4D_CUDA(c, ensure(w.ranges, 8 * (size_t)n_tiles));
-    w.cap_tiles = n_tiles;
+  if (n_tiles > w.cap_tiles || order > w.tile_order.bytes) {
+    const int tiles = std::max(n_tiles, w.cap_tiles);
+    w.cap_tiles = 0;
+    FS4D_CUDA(c, ensure(w.ranges, 8 * (size_t)tiles));
+    FS4D_CUDA(c, ensure(w.tile_order, std::max(order, 4 * (size_t)tiles)));
+    w.cap_tiles = tiles;
   }
   if (pairs > w.cap_pairs) {
     const long long cap = std::max<long long>(pairs, 4096);
+    w.cap_pairs = 0;
     FS4D_CUDA(c, ensure(w.keys, 8 * (size_t)cap));
     FS4D_CUDA(c, ensure(w.values, 4 * (size_t)cap));
     FS4D_CUDA(c, ensure(w.keys_alt, 8 * (size_t)cap));
@@ -600,15 +611,14 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   }
   const long long parts = std::max(sort_parts(std::max<long long>(w.cap_pairs, 4096)), sort_parts(w.cap_n));
   if (parts > w.sort_parts_cap) {
+    w.sort_parts_cap = 0;
     FS4D_CUDA(c, ensure(w.sort_lb, 4 * 256 * (size_t)kSortMaxPasses * parts));
     w.sort_parts_cap = parts;
   }
   const size_t zb = frame_zero_layout(w.cap_n, w.cap_tiles, w.cap_pairs,
                                       sort_passes(ceil_log2(std::max(w.cap_tiles, 1))), nullptr, nullptr);
   FS4D_CUDA(c, ensure(w.zero, zb));
-  w.cap_rows = rows;
   FS4D_CUDA(c, ensure(w.axis, axis));
-  FS4D_CUDA(c, ensure(w.tile_order, order));
   return FS4D_OK;
 }
 
@@ -1029,7 +1039,7 @@ BandTab band_tab(const fs4d_camera* cam, const std::vector<std::pair<int, int>>&
 fs4d_status ensure_direct(fs4d_ctx* c, int n) {
   Work& w = c->w;
   const size_t m = (size_t)n;
-  if (w.yparts.bytes >= 8 * m && w.spos.bytes >= 16 * m && w.srg.bytes >= 8 * m && w.band_pairs.bytes > 0)
+  if (w.yparts.bytes >= 8 * m && w.spos.bytes >= 16 * m && w.srg.bytes >= 8 * m && w.band_pairs.bytes > 0 && c->h_band_pairs)
     return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
   FS4D_CUDA(c, ensure(w.yparts, 8 * m));
@@ -2368,14 +2378,15 @@ fs4d_status fit_slot(fs4d_server* sv, Slot* sl, int n, int w, int h, long long p
   fs4d_ctx* c = sv->c;
   const void* before[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.axis.p};
   fs4d_status st = ensure_work(c, sl->w, sl->stream, n, tiles_of(w), tiles_of(h), pairs);
-  if (st != FS4D_OK) return st;
-  if ((size_t)w * h * 12 > sl->image.bytes) FS4D_CUDA(c, ensure(sl->image, (size_t)w * h * 12));
+  if (st == FS4D_OK && ensure(sl->image, (size_t)w * h * 12) != cudaSuccess)
+    st = fail(c, FS4D_ERR_OOM, "server: slot image allocation failed");
   const void* after[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.axis.p};
   if (std::memcmp(before, after, sizeof(before)) != 0) {  // graphs captured on old buffers are stale
     cudaStreamSynchronize(sl->stream);
     for (auto& kv : sl->graphs) cudaGraphExecDestroy(kv.second);
     sl->graphs.clear();
   }
+  if (st != FS4D_OK) return st;  // (some of the buffers may have moved all the same)
   sl->cap_w = std::max(sl->cap_w, w);
   sl->cap_h = std::max(sl->cap_h, h);
   const size_t b = slot_bytes_for(sl->w.cap_n, sl->cap_w, sl->cap_h, sl->w.cap_pairs);

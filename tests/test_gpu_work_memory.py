@@ -52,3 +52,49 @@ def test_async_frame_after_a_long_row_of_tiles(ctx, tiles):
     torch.cuda.synchronize()
     assert torch.equal(image, want)
     ctx.check_device_status()
+
+
+def test_sizes_of_different_calls_do_not_multiply(ctx):
+    """Bit rows are sized for one call's tiles and Gaussians: many tiles with few Gaussians (128 MB
+    of bits) and many Gaussians with few tiles (1.3 MB) take no product of the two (25 GB)."""
+    s = sg.make_object(5, n=200_000, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=300, height=200, seed=3)[2]
+    sid = ctx.load_scene(s)
+    want = ctx.render(sid, cam, 0.6)
+    for _ in range(2):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        long_row(ctx, 1000, 1_000_000)
+        assert torch.equal(ctx.render(sid, cam, 0.6), want)
+        torch.cuda.synchronize()
+        assert free - torch.cuda.mem_get_info()[0] < 2 << 30
+    ctx.unload_scene(sid)
+    fresh = fs4d.Context(0)  # the other order
+    try:
+        long_row(fresh, 1000, 1_000_000)
+        free = torch.cuda.mem_get_info()[0]
+        assert torch.equal(fresh.render(fresh.load_scene(s), cam, 0.6), want)
+        assert free - torch.cuda.mem_get_info()[0] < 2 << 30
+    finally:
+        fresh.close()
+
+
+@pytest.mark.parametrize("before", [False, True])
+def test_a_failed_allocation_leaves_a_working_context(ctx, before):
+    """A capacity beyond the device's memory is refused, and the buffers that made room for it are
+    allocated again by the next call (before: the context has rendered already)."""
+    s = sg.make_object(6, n=5000, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=300, height=200, seed=3)[2]
+    sid = ctx.load_scene(s)
+    if before:
+        want = ctx.render(sid, cam, 0.6)
+    with pytest.raises(fs4d.Fs4dError):
+        ctx.reserve(sid, 300, 200, 40_000_000_000)
+    got = ctx.render(sid, cam, 0.6)
+    image, frame = ctx.render_saved(sid, cam, 0.6)
+    ctx.render_backward(frame, torch.ones_like(image), {"means": torch.zeros(s.n, 3, device="cuda")})
+    ctx.frame_free(frame)
+    assert torch.equal(got, image)
+    if before:
+        assert torch.equal(got, want)
+    ctx.check_device_status()
