@@ -834,6 +834,7 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
     if (s->color_heads) {  // App. B: this frame's deformed colour and opacity
       pa.opacity_logits = P<float>(w.dop) + q.off;
       pa.sh = P<float>(w.dsh) + 48 * q.off;
+      pa.sh_late = 1;
     }
     pa.cam = cam_params(shape);
     // world_to_cam applied to X + shift: the translation column absorbs W shift
@@ -2081,6 +2082,7 @@ fs4d_status fs4d_project(fs4d_ctx* c, int32_t n, const float* d_means, const flo
   ProjectArgs pa{};
   pa.n = n; pa.means = d_means; pa.quats = d_quats; pa.log_scales = d_log_scales;
   pa.opacity_logits = d_opacity_logits; pa.sh = d_sh; pa.sh_degree = sh_degree;
+  pa.sh_late = 1;  // (the caller's kernels may have written them just now)
   pa.cam = cam_params(*cam); pa.cam_dev = nullptr;
   pa.tiles_x = tiles_of(cam->width); pa.tiles_y = tiles_of(cam->height);
   pa.xy = reinterpret_cast<float2*>(out->xy); pa.conic_opacity = reinterpret_cast<float4*>(out->conic_opacity);

@@ -3,7 +3,8 @@
 // with coalesced loads (quaternions as one 128-bit load) and every output is a
 // coalesced store, written once.  Every input load is issued at the start: the SH rows
 // (the bulk of the bytes) go to shared memory by cp.async and are waited for only
-// when the colour is evaluated, so their latency overlaps the geometry.  Float32
+// when the colour is evaluated, so their latency overlaps the geometry (and, where they are
+// the scene's own, the end of the kernel before).  Float32
 // throughout.  Bound by memory (236 bytes in, 68 out at degree 3):
 // 2M Gaussians 121 us (150 with SH rows copied by the thread that reads them, 192 bytes
 // apart, and every output stored as zero first), 100k 12.
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   extern __shared__ float4 s_sh[];  // [256][SHQ + 1]
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = g < a.n;
+  if (a.sh_late) pdl_wait();
   if (SHQ > 0) {
     const long long g0 = (long long)blockIdx.x * 256;
     const int words = (int)min(256ll, a.n - g0) * SHQ;
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) c.m[4 * r + k] = d->world_to_cam[4 * r + k];
   }
-  pdl_wait();  // (the SH rows and the camera are inputs of the frame; the Gaussians come from the deformation)
+  pdl_wait();  // (the camera and, without sh_late, the SH rows are inputs of the frame; the Gaussians come from the deformation)
   pdl_trigger();
   float X0 = 0.f, X1 = 0.f, X2 = 0.f, logit = 0.f, ls0 = 0.f, ls1 = 0.f, ls2 = 0.f;
   float4 q4 = make_float4(1.f, 0.f, 0.f, 0.f);
