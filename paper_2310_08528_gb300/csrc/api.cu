@@ -115,6 +115,8 @@ struct Scene {
   size_t color_off = 0;
   std::atomic<int> refs{0};   // serving requests in flight on this scene
   bool dying = false;         // being unloaded: no new serving launches
+  std::atomic<bool> derived{false};  // the last kernel on the context's stream may be the one that writes
+                                     // the MLP's copies (a training step): the next deformation waits first
   // capacity-mode reservation
   long long reserved_pairs = 0;
   int reserved_w = 0, reserved_h = 0;
@@ -726,6 +728,12 @@ fs4d_status run_deform(fs4d_ctx* c, Scene* s, fs4d_precision prec, const DeformA
                        uint32_t* status) {
   DeformArgs b = a;
   b.status = status;
+  if (stream == c->stream && s->derived) {
+    b.mlp_late = 1;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;  // (a captured launch runs later)
+    FS4D_CUDA(c, cudaStreamIsCapturing(stream, &cs));
+    if (cs == cudaStreamCaptureStatusNone) s->derived = false;
+  }
   if (prec == FS4D_BF16) {
     if (!s->bf16_ok) return fail(c, FS4D_ERR_UNIMPLEMENTED, "BF16 deformation does not support this scene shape");
     FS4D_CUDA(c, launch_deform_bf16(b, stream));
@@ -2917,6 +2925,7 @@ fs4d_status fs4d_train_step(fs4d_trainer* tr, fs4d_precision prec, const fs4d_ca
                              P<float>(s->mlp), (int)s->mlp_floats, P<int4>(s->derive_tab), P<float>(s->mlp_t),
                              s->bf16_ok ? P<uint8_t>(s->tc_ops) : nullptr, s->bf16_ok ? P<float>(s->tc_bias) : nullptr,
                              c->stream));
+  s->derived = true;
   tr->step = step;
   return FS4D_OK;
 }

@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kThreads, 1) deform_tc_kernel(DeformArgs a) {
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // the weights by cp.async: every 16-byte copy in flight at once
+  if (a.mlp_late) pdl_wait();
   for (int i = tid; i < tg.bytes / 16; i += kThreads) cp_async(sB + 16 * i, a.tc_ops + 16 * i, 1);
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   for (int i = tid; i < kBiasFloats; i += kThreads) sBias[i] = a.tc_bias[i];

@@ -155,6 +155,7 @@ struct DeformArgs {
   float* act_a1;
   float* act_hid;
   uint32_t* act_masks;
+  int mlp_late;                 // the MLP's copies are written by the kernel before this one
   uint4* zero;                  // optional: zero_n16 16-byte words the kernel sets to 0 (a frame's counters
   long long zero_n16;           // and look-back tables, cleared here instead of by a separate memset)
   uint4* fd_tiles;              // BF16 kernel, optional: f_d of each tile of 128 work-order rows as its BF16
