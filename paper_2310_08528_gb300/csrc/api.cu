@@ -239,10 +239,16 @@ struct fs4d_frame {
   bool ranks = false;                          // the lists hold depth ranks
   DevBuf values, ranges;                       // sorted Gaussian indices, per-tile ranges
   DevBuf t_final, n_contrib;                   // per pixel
-  cudaStream_t stream = nullptr;               // the stream of every launch that used the buffers,
-  bool one_stream = true;                      // unless there were several
+  unsigned long long epoch = 0;                // the context's while every launch used the buffers,
+  bool one_epoch = true;                       // unless there were several
   int device = 0;
 };
+
+// A number no context has had yet: a stream's handle may be given out again.
+static unsigned long long next_epoch() {
+  static std::atomic<unsigned long long> last{0};
+  return ++last;
+}
 
 struct fs4d_server;
 
@@ -258,11 +264,13 @@ struct fs4d_ctx {
   DevBuf status;
   uint32_t* h_pinned = nullptr;  // [4] readback slots
   long long last_pairs = 0;
-  // Freed frames whose buffers the next saved frame takes over (at most kSpareFrames; all of
-  // their work is on `stream`, so the next frame's launches come after it).  A device
+  // Freed frames whose buffers the next saved frame takes over (at most kSpareFrames).  A device
   // allocation and its release cost a saved frame more than its kernels: 1.1 ms of the 2.65 ms
-  // of one 800x800 / 100k view and its backward went there.
+  // of one 800x800 / 100k view and its backward went there.  Only a frame of this epoch is taken
+  // over: all of its work is on `stream`, so the next frame's launches come after it.
+  std::mutex spare_mu;
   std::vector<fs4d_frame*> spare;
+  unsigned long long epoch = next_epoch();  // another number for each stream that the context is given
   int binning = FS4D_BINNING_AUTO;
   int last_binning = FS4D_BINNING_SORT;
   bool timing = false;
@@ -1229,12 +1237,41 @@ void release_frame(fs4d_frame& f) {
   for (DevBuf* b : all) release(*b);
 }
 
-void release_spare(fs4d_ctx* c) {  // (cudaFree waits for the work that uses the buffers)
-  for (fs4d_frame* f : c->spare) {
+// Gives the kept frames back (cudaFree waits for the work that uses the buffers).
+void release_spare(fs4d_ctx* c) {
+  std::vector<fs4d_frame*> all;
+  {
+    std::lock_guard<std::mutex> lock(c->spare_mu);
+    all.swap(c->spare);
+  }
+  for (fs4d_frame* f : all) {
     release_frame(*f);
     delete f;
   }
-  c->spare.clear();
+}
+
+// A kept frame that the context's stream may go on with, or NULL; those of other epochs are
+// given back (not in fs4d_set_stream: that is called within a capture, where nothing may be
+// freed, and a saved frame reads its pair count back, so none is rendered there).
+fs4d_frame* take_spare(fs4d_ctx* c) {
+  std::vector<fs4d_frame*> old;
+  fs4d_frame* f = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(c->spare_mu);
+    while (!f && !c->spare.empty()) {
+      fs4d_frame* q = c->spare.back();
+      c->spare.pop_back();
+      if (q->epoch == c->epoch)
+        f = q;
+      else
+        old.push_back(q);
+    }
+  }
+  for (fs4d_frame* q : old) {
+    release_frame(*q);
+    delete q;
+  }
+  return f;
 }
 
 // The buffers of a saved frame, grown where they are too small.
@@ -1269,8 +1306,8 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
   if (s->color_heads && (st = ensure_color(c, c->w, c->stream, s->n)) != FS4D_OK) return st;
   c->stage_acc_valid = false;
   c->last_bands = 1;
-  if (f->stream != c->stream && f->dmeans.p) f->one_stream = false;
-  f->stream = c->stream;
+  if (f->epoch != c->epoch && f->dmeans.p) f->one_epoch = false;
+  f->epoch = c->epoch;
   f->device = c->device;
   for (int pass = 0;; ++pass) {
     if ((st = ensure_frame(c, f, (size_t)s->n, (size_t)n_tiles, npix, (size_t)c->w.cap_pairs)) != FS4D_OK) return st;
@@ -1373,10 +1410,7 @@ const char* fs4d_last_error(const fs4d_ctx* c) { return c ? c->err.c_str() : "nu
 
 fs4d_status fs4d_set_stream(fs4d_ctx* c, void* cuda_stream) {
   if (!c) return FS4D_ERR_INVALID_ARG;
-  if (c->stream != reinterpret_cast<cudaStream_t>(cuda_stream) && !c->spare.empty()) {
-    DeviceGuard g(c->device);
-    release_spare(c);  // their work is on the old stream
-  }
+  if (c->stream != reinterpret_cast<cudaStream_t>(cuda_stream)) c->epoch = next_epoch();
   c->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   return FS4D_OK;
 }
@@ -1604,13 +1638,8 @@ fs4d_status render_impl(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision prec, cons
   DeviceGuard g(c->device);
   if (!saved) return render_sync(c, s, prec, cam, t, d_image, d_t_final, d_n_contrib);
   *saved = nullptr;
-  fs4d_frame* f = nullptr;
-  if (!c->spare.empty()) {
-    f = c->spare.back();
-    c->spare.pop_back();
-  } else {
-    f = new (std::nothrow) fs4d_frame();
-  }
+  fs4d_frame* f = take_spare(c);
+  if (!f) f = new (std::nothrow) fs4d_frame();
   if (!f) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
   st = render_into_frame(c, s, prec, cam, t, d_image, f, !d_n_contrib);
   if (st == FS4D_OK && d_t_final)
@@ -1874,7 +1903,7 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
     return fail(c, FS4D_ERR_UNIMPLEMENTED, "render_backward: no backward through the colour and opacity heads");
   if (s->n != f->n) return fail(c, FS4D_ERR_INVALID_ARG, "render_backward: the scene changed size since the frame");
   DeviceGuard g(c->device);
-  if (f->stream != c->stream) f->one_stream = false;
+  if (f->epoch != c->epoch) f->one_epoch = false;
   Work& w = c->w;
   const long long n = s->n, K = f->slots;
   const int hin = s->mg.hin;
@@ -1975,9 +2004,12 @@ fs4d_status fs4d_render_backward_stats(fs4d_ctx* c, fs4d_frame* f, const float* 
 fs4d_status fs4d_frame_free(fs4d_ctx* c, fs4d_frame* f) {
   if (!f) return FS4D_OK;
   // kept for the context's next saved frame if all of its work is on the context's stream
-  if (c && f->one_stream && f->stream == c->stream && f->device == c->device && c->spare.size() < kSpareFrames) {
-    c->spare.push_back(f);
-    return FS4D_OK;
+  if (c && f->one_epoch && f->epoch == c->epoch) {
+    std::lock_guard<std::mutex> lock(c->spare_mu);
+    if (c->spare.size() < kSpareFrames) {
+      c->spare.push_back(f);
+      return FS4D_OK;
+    }
   }
   {
     DeviceGuard g(c ? c->device : f->device);

@@ -98,3 +98,63 @@ def test_a_failed_allocation_leaves_a_working_context(ctx, before):
     if before:
         assert torch.equal(got, want)
     ctx.check_device_status()
+
+
+def test_set_stream_within_a_capture(ctx):
+    """A context that keeps freed frames may be given another stream inside a capture."""
+    s = sg.make_object(6, n=3000, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=160, height=120, seed=3)[2]
+    sid = ctx.load_scene(s)
+    want, frame = ctx.render_saved(sid, cam, 0.6)
+    ctx.reserve(sid, 160, 120, 2 * ctx.last_pairs())
+    d_cam = torch.from_numpy(np.frombuffer(bytes(fs4d.camera_struct(cam)), np.float32).copy()).cuda()
+    d_t, image = torch.tensor([0.6], device="cuda"), torch.zeros(120, 160, 3, device="cuda")
+    ctx.frame_free(frame)
+    torch.cuda.synchronize()
+    before, graph = ctx.stream, torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.set_stream(torch.cuda.current_stream())
+        ctx.render_async(sid, cam, d_cam, d_t, image)
+    ctx.set_stream(before)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(image, want)
+    # frames kept from before the other stream are not taken over, and the next ones are right
+    for _ in range(3):
+        again, frame = ctx.render_saved(sid, cam, 0.6)
+        assert torch.equal(again, want)
+        ctx.frame_free(frame)
+
+
+def test_saved_frames_on_two_streams(ctx):
+    """Frames rendered on one stream, used and freed on another."""
+    s = sg.make_object(8, n=20_000, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=320, height=240, seed=3)[2]
+    sid = ctx.load_scene(s)
+    dl = torch.ones(240, 320, 3, device="cuda")
+
+    def grads(frame):
+        g = {"sh": torch.zeros(s.sh.shape, device="cuda"), "opacity_logits": torch.zeros(s.n, device="cuda")}
+        torch.cuda.synchronize()
+        ctx.render_backward(frame, dl, g)
+        return g
+
+    image, frame = ctx.render_saved(sid, cam, 0.2)
+    want = grads(frame)
+    torch.cuda.synchronize()
+    ctx.frame_free(frame)
+    first, side = ctx.stream, torch.cuda.Stream()
+    for k in range(6):
+        got, frame = ctx.render_saved(sid, cam, 0.2)
+        torch.cuda.synchronize()
+        ctx.set_stream(side if ctx.stream is first else first)
+        g = grads(frame)
+        if k % 2:
+            ctx.frame_free(frame)
+        torch.cuda.synchronize()
+        if not k % 2:
+            ctx.frame_free(frame)
+        assert torch.equal(got, image)
+        for n, v in g.items():  # (the order among warps is free)
+            assert float((v - want[n]).abs().max()) <= 1e-5 * float(want[n].abs().max())
+    ctx.set_stream(first)
