@@ -279,6 +279,11 @@ FS4D_API fs4d_status fs4d_render_async(fs4d_ctx* ctx, fs4d_scene_id id, fs4d_pre
  * non-NULL pointers of *d_grads. */
 FS4D_API fs4d_status fs4d_render_backward(fs4d_ctx* ctx, fs4d_frame* saved, const float* d_dl_dimage,
                                  const fs4d_grads* d_grads);
+/* Frees a saved frame.  The context keeps the device buffers of up to two freed frames for
+ * its next saved frames (of any scene and size; about 130 bytes per Gaussian, 8 per pixel and
+ * 4 per listed tile pair each).  They are given back when an allocation of the context finds no
+ * room, when a scene is unloaded, with the first saved frame after the context was given another
+ * stream, and with the context. */
 FS4D_API fs4d_status fs4d_frame_free(fs4d_ctx* ctx, fs4d_frame* frame);
 /* Number of tile pairs K of a saved frame, and of the last render on the context:
  * the pairs of the Gaussians' tile rectangles (frames with lists from column and row bits that

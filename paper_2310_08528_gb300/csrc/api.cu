@@ -519,9 +519,37 @@ std::vector<int4> build_derive_tab(int hin, int W, const MlpGeomT& mg, const Mlp
   return tab;
 }
 
+void release_frame(fs4d_frame& f) {
+  DevBuf* all[] = {&f.dmeans, &f.dquats, &f.dscales, &f.xy, &f.co, &f.rgb, &f.radius, &f.rect, &f.offsets,
+                   &f.order, &f.sco, &f.slot, &f.values, &f.ranges, &f.t_final, &f.n_contrib};
+  for (DevBuf* b : all) release(*b);
+}
+
+// Gives the kept frames back (cudaFree waits for the work that uses the buffers); whether
+// there were any.
+bool release_spare(fs4d_ctx* c) {
+  std::vector<fs4d_frame*> all;
+  {
+    std::lock_guard<std::mutex> lock(c->spare_mu);
+    all.swap(c->spare);
+  }
+  for (fs4d_frame* f : all) {
+    release_frame(*f);
+    delete f;
+  }
+  return !all.empty();
+}
+
+// A buffer of the context's: with the kept frames given back if the device has no room else.
+cudaError_t ensure(fs4d_ctx* c, DevBuf& b, size_t bytes) {
+  cudaError_t e = ensure(b, bytes);
+  if (e == cudaErrorMemoryAllocation && release_spare(c)) e = ensure(b, bytes);
+  return e;
+}
+
 template <typename T>
 fs4d_status upload(fs4d_ctx* c, DevBuf& b, const T* h, size_t count, size_t* acc) {
-  FS4D_CUDA(c, ensure(b, sizeof(T) * std::max<size_t>(count, 1)));
+  FS4D_CUDA(c, ensure(c, b, sizeof(T) * std::max<size_t>(count, 1)));
   if (count) FS4D_CUDA(c, cudaMemcpy(b.p, h, sizeof(T) * count, cudaMemcpyHostToDevice));
   *acc += b.bytes;
   return FS4D_OK;
@@ -550,9 +578,9 @@ fs4d_status ensure_color(fs4d_ctx* c, Work& w, cudaStream_t stream, int n) {
   if (w.cap_color >= n) return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(stream));
   w.cap_color = 0;
-  FS4D_CUDA(c, ensure(w.fd, 4 * 64 * (size_t)n + 16384));  // + the last BF16 tile image's ragged end
-  FS4D_CUDA(c, ensure(w.dsh, 4 * 48 * (size_t)n));
-  FS4D_CUDA(c, ensure(w.dop, 4 * (size_t)n));
+  FS4D_CUDA(c, ensure(c, w.fd, 4 * 64 * (size_t)n + 16384));  // + the last BF16 tile image's ragged end
+  FS4D_CUDA(c, ensure(c, w.dsh, 4 * 48 * (size_t)n));
+  FS4D_CUDA(c, ensure(c, w.dop, 4 * (size_t)n));
   w.cap_color = n;
   return FS4D_OK;
 }
@@ -579,56 +607,56 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   if (n > w.cap_n) {
     const size_t m = (size_t)n;
     w.cap_n = 0;
-    FS4D_CUDA(c, ensure(w.dmeans, 12 * m));
-    FS4D_CUDA(c, ensure(w.dquats, 16 * m));
-    FS4D_CUDA(c, ensure(w.dscales, 12 * m));
-    FS4D_CUDA(c, ensure(w.xy, 8 * m));
-    FS4D_CUDA(c, ensure(w.co, 16 * m));
-    FS4D_CUDA(c, ensure(w.rgb, 12 * m));
-    FS4D_CUDA(c, ensure(w.depth, 4 * m));
-    FS4D_CUDA(c, ensure(w.radius, 4 * m));
-    FS4D_CUDA(c, ensure(w.rect, 16 * m));
-    FS4D_CUDA(c, ensure(w.sxy, 8 * m));
-    FS4D_CUDA(c, ensure(w.sco, 16 * m));
-    FS4D_CUDA(c, ensure(w.srgb, 12 * m));
-    FS4D_CUDA(c, ensure(w.srect, 16 * m));
-    FS4D_CUDA(c, ensure(w.offsets, 4 * m));
-    FS4D_CUDA(c, ensure(w.dkeys, 8 * m));
-    FS4D_CUDA(c, ensure(w.dvals, 4 * m));
-    FS4D_CUDA(c, ensure(w.dkeys_alt, 8 * m));
-    FS4D_CUDA(c, ensure(w.dvals_alt, 4 * m));
-    FS4D_CUDA(c, ensure(w.bpos, 4 * m));
+    FS4D_CUDA(c, ensure(c, w.dmeans, 12 * m));
+    FS4D_CUDA(c, ensure(c, w.dquats, 16 * m));
+    FS4D_CUDA(c, ensure(c, w.dscales, 12 * m));
+    FS4D_CUDA(c, ensure(c, w.xy, 8 * m));
+    FS4D_CUDA(c, ensure(c, w.co, 16 * m));
+    FS4D_CUDA(c, ensure(c, w.rgb, 12 * m));
+    FS4D_CUDA(c, ensure(c, w.depth, 4 * m));
+    FS4D_CUDA(c, ensure(c, w.radius, 4 * m));
+    FS4D_CUDA(c, ensure(c, w.rect, 16 * m));
+    FS4D_CUDA(c, ensure(c, w.sxy, 8 * m));
+    FS4D_CUDA(c, ensure(c, w.sco, 16 * m));
+    FS4D_CUDA(c, ensure(c, w.srgb, 12 * m));
+    FS4D_CUDA(c, ensure(c, w.srect, 16 * m));
+    FS4D_CUDA(c, ensure(c, w.offsets, 4 * m));
+    FS4D_CUDA(c, ensure(c, w.dkeys, 8 * m));
+    FS4D_CUDA(c, ensure(c, w.dvals, 4 * m));
+    FS4D_CUDA(c, ensure(c, w.dkeys_alt, 8 * m));
+    FS4D_CUDA(c, ensure(c, w.dvals_alt, 4 * m));
+    FS4D_CUDA(c, ensure(c, w.bpos, 4 * m));
     w.cap_n = n;
   }
-  FS4D_CUDA(c, ensure(w.counters, 4 * kCounters));
-  FS4D_CUDA(c, ensure(w.bstart, 4 * (kBuckets + 4)));
-  FS4D_CUDA(c, ensure(w.hist, 4 * 256 * kSortMaxPasses));
+  FS4D_CUDA(c, ensure(c, w.counters, 4 * kCounters));
+  FS4D_CUDA(c, ensure(c, w.bstart, 4 * (kBuckets + 4)));
+  FS4D_CUDA(c, ensure(c, w.hist, 4 * 256 * kSortMaxPasses));
   if (n_tiles > w.cap_tiles || order > w.tile_order.bytes) {
     const int tiles = std::max(n_tiles, w.cap_tiles);
     w.cap_tiles = 0;
-    FS4D_CUDA(c, ensure(w.ranges, 8 * (size_t)tiles));
-    FS4D_CUDA(c, ensure(w.tile_order, std::max(order, 4 * (size_t)tiles)));
+    FS4D_CUDA(c, ensure(c, w.ranges, 8 * (size_t)tiles));
+    FS4D_CUDA(c, ensure(c, w.tile_order, std::max(order, 4 * (size_t)tiles)));
     w.cap_tiles = tiles;
   }
   if (pairs > w.cap_pairs) {
     const long long cap = std::max<long long>(pairs, 4096);
     w.cap_pairs = 0;
-    FS4D_CUDA(c, ensure(w.keys, 8 * (size_t)cap));
-    FS4D_CUDA(c, ensure(w.values, 4 * (size_t)cap));
-    FS4D_CUDA(c, ensure(w.keys_alt, 8 * (size_t)cap));
-    FS4D_CUDA(c, ensure(w.values_alt, 4 * (size_t)cap));
+    FS4D_CUDA(c, ensure(c, w.keys, 8 * (size_t)cap));
+    FS4D_CUDA(c, ensure(c, w.values, 4 * (size_t)cap));
+    FS4D_CUDA(c, ensure(c, w.keys_alt, 8 * (size_t)cap));
+    FS4D_CUDA(c, ensure(c, w.values_alt, 4 * (size_t)cap));
     w.cap_pairs = cap;
   }
   const long long parts = std::max(sort_parts(std::max<long long>(w.cap_pairs, 4096)), sort_parts(w.cap_n));
   if (parts > w.sort_parts_cap) {
     w.sort_parts_cap = 0;
-    FS4D_CUDA(c, ensure(w.sort_lb, 4 * 256 * (size_t)kSortMaxPasses * parts));
+    FS4D_CUDA(c, ensure(c, w.sort_lb, 4 * 256 * (size_t)kSortMaxPasses * parts));
     w.sort_parts_cap = parts;
   }
   const size_t zb = frame_zero_layout(w.cap_n, w.cap_tiles, w.cap_pairs,
                                       sort_passes(ceil_log2(std::max(w.cap_tiles, 1))), nullptr, nullptr);
-  FS4D_CUDA(c, ensure(w.zero, zb));
-  FS4D_CUDA(c, ensure(w.axis, axis));
+  FS4D_CUDA(c, ensure(c, w.zero, zb));
+  FS4D_CUDA(c, ensure(c, w.axis, axis));
   return FS4D_OK;
 }
 
@@ -1059,10 +1087,10 @@ fs4d_status ensure_direct(fs4d_ctx* c, int n) {
   if (w.yparts.bytes >= 8 * m && w.spos.bytes >= 16 * m && w.srg.bytes >= 8 * m && w.band_pairs.bytes > 0 && c->h_band_pairs)
     return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
-  FS4D_CUDA(c, ensure(w.yparts, 8 * m));
-  FS4D_CUDA(c, ensure(w.spos, 16 * m));
-  FS4D_CUDA(c, ensure(w.srg, 8 * m));
-  FS4D_CUDA(c, ensure(w.band_pairs, 8 * kMaxTileRows));
+  FS4D_CUDA(c, ensure(c, w.yparts, 8 * m));
+  FS4D_CUDA(c, ensure(c, w.spos, 16 * m));
+  FS4D_CUDA(c, ensure(c, w.srg, 8 * m));
+  FS4D_CUDA(c, ensure(c, w.band_pairs, 8 * kMaxTileRows));
   if (!c->h_band_pairs) FS4D_CUDA(c, cudaMallocHost(&c->h_band_pairs, 8 * kMaxTileRows));
   return FS4D_OK;
 }
@@ -1231,25 +1259,6 @@ fs4d_status render_sync(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_c
 
 constexpr size_t kSpareFrames = 2;
 
-void release_frame(fs4d_frame& f) {
-  DevBuf* all[] = {&f.dmeans, &f.dquats, &f.dscales, &f.xy, &f.co, &f.rgb, &f.radius, &f.rect, &f.offsets,
-                   &f.order, &f.sco, &f.slot, &f.values, &f.ranges, &f.t_final, &f.n_contrib};
-  for (DevBuf* b : all) release(*b);
-}
-
-// Gives the kept frames back (cudaFree waits for the work that uses the buffers).
-void release_spare(fs4d_ctx* c) {
-  std::vector<fs4d_frame*> all;
-  {
-    std::lock_guard<std::mutex> lock(c->spare_mu);
-    all.swap(c->spare);
-  }
-  for (fs4d_frame* f : all) {
-    release_frame(*f);
-    delete f;
-  }
-}
-
 // A kept frame that the context's stream may go on with, or NULL; those of other epochs are
 // given back (not in fs4d_set_stream: that is called within a capture, where nothing may be
 // freed, and a saved frame reads its pair count back, so none is rendered there).
@@ -1288,7 +1297,7 @@ fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, siz
   if (!grow) return FS4D_OK;
   if (!first) FS4D_CUDA(c, cudaStreamSynchronize(c->stream));  // the old buffers may still be read
   for (const auto& q : need)
-    if (ensure(*q.first, q.second) != cudaSuccess) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
+    if (ensure(c, *q.first, q.second) != cudaSuccess) return fail(c, FS4D_ERR_OOM, "render: frame allocation failed");
   return FS4D_OK;
 }
 
@@ -1620,7 +1629,7 @@ fs4d_status fs4d_deform(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision prec, cons
   DeviceGuard g(c->device);
   if (c->w.ts.bytes < 4 * (size_t)n_t) {
     FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
-    FS4D_CUDA(c, ensure(c->w.ts, 4 * (size_t)n_t));
+    FS4D_CUDA(c, ensure(c, c->w.ts, 4 * (size_t)n_t));
   }
   FS4D_CUDA(c, cudaMemcpyAsync(c->w.ts.p, h_ts, 4 * (size_t)n_t, cudaMemcpyHostToDevice, c->stream));
   DeformArgs a = deform_args(s, P<float>(c->w.ts), 0.f, n_t, d_means, d_quats, d_log_scales);
@@ -1722,7 +1731,7 @@ fs4d_status fs4d_render_host(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision prec,
   const size_t bytes = (size_t)cam->width * cam->height * 12;
   if (img.bytes < bytes) {
     FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
-    FS4D_CUDA(c, ensure(img, bytes));
+    FS4D_CUDA(c, ensure(c, img, bytes));
   }
   // The whole frame is queued at the current pair capacity and the pair count comes
   // back with the image, so one host synchronisation per frame suffices; a frame
@@ -1763,7 +1772,7 @@ fs4d_status fs4d_render_host_batch(fs4d_ctx* c, fs4d_scene_id id, fs4d_precision
   if (img.bytes < 2 * bytes || c->h_pairs_cap < n || !c->copy_stream) {
     FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
     if (c->copy_stream) FS4D_CUDA(c, cudaStreamSynchronize(c->copy_stream));
-    FS4D_CUDA(c, ensure(img, 2 * bytes));
+    FS4D_CUDA(c, ensure(c, img, 2 * bytes));
     if (c->h_pairs_cap < n) {
       if (c->h_pairs) cudaFreeHost(c->h_pairs);
       c->h_pairs = nullptr;
@@ -1918,10 +1927,10 @@ static fs4d_status backward_impl(fs4d_ctx* c, fs4d_frame* f, const float* d_dl_d
   if (w.grad_pair.bytes < 4 * kPairStride * (size_t)std::max(K, 1ll) || w.gd.bytes < 40 * (size_t)n ||
       w.acts.bytes < 4 * act_floats || w.wpartial.bytes < 4 * wp) {
     FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
-    FS4D_CUDA(c, ensure(w.grad_pair, 4 * kPairStride * (size_t)std::max(K, 1ll)));
-    FS4D_CUDA(c, ensure(w.gd, 40 * (size_t)n));
-    FS4D_CUDA(c, ensure(w.acts, 4 * act_floats));
-    FS4D_CUDA(c, ensure(w.wpartial, 4 * wp));
+    FS4D_CUDA(c, ensure(c, w.grad_pair, 4 * kPairStride * (size_t)std::max(K, 1ll)));
+    FS4D_CUDA(c, ensure(c, w.gd, 40 * (size_t)n));
+    FS4D_CUDA(c, ensure(c, w.acts, 4 * act_floats));
+    FS4D_CUDA(c, ensure(c, w.wpartial, 4 * wp));
   }
   const int tx = tiles_of(f->cam.width);
   auto bmark = [&](int i) {
@@ -2420,7 +2429,7 @@ fs4d_status fit_slot(fs4d_server* sv, Slot* sl, int n, int w, int h, long long p
   fs4d_ctx* c = sv->c;
   const void* before[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.axis.p};
   fs4d_status st = ensure_work(c, sl->w, sl->stream, n, tiles_of(w), tiles_of(h), pairs);
-  if (st == FS4D_OK && ensure(sl->image, (size_t)w * h * 12) != cudaSuccess)
+  if (st == FS4D_OK && ensure(c, sl->image, (size_t)w * h * 12) != cudaSuccess)
     st = fail(c, FS4D_ERR_OOM, "server: slot image allocation failed");
   const void* after[6] = {sl->w.dmeans.p, sl->w.keys.p, sl->w.ranges.p, sl->w.zero.p, sl->image.p, sl->w.axis.p};
   if (std::memcmp(before, after, sizeof(before)) != 0) {  // graphs captured on old buffers are stale
@@ -2877,9 +2886,9 @@ fs4d_status fs4d_train_create(fs4d_ctx* c, fs4d_scene_id id, const fs4d_train_co
     total += (cnt[k] + 3) / 4 * 4;  // each group 16-byte aligned
   }
   const size_t parts = (size_t)train_partials();
-  if (ensure(tr->grad, 4 * total) != cudaSuccess || ensure(tr->m, 4 * total) != cudaSuccess ||
-      ensure(tr->v, 4 * total) != cudaSuccess || ensure(tr->partial, 4 * parts) != cudaSuccess ||
-      ensure(tr->losses, 16) != cudaSuccess || ensure(tr->stats, 8 * n) != cudaSuccess) {
+  if (ensure(c, tr->grad, 4 * total) != cudaSuccess || ensure(c, tr->m, 4 * total) != cudaSuccess ||
+      ensure(c, tr->v, 4 * total) != cudaSuccess || ensure(c, tr->partial, 4 * parts) != cudaSuccess ||
+      ensure(c, tr->losses, 16) != cudaSuccess || ensure(c, tr->stats, 8 * n) != cudaSuccess) {
     fs4d_train_destroy(tr);
     return fail(c, FS4D_ERR_OOM, "train_create: device allocation failed");
   }
@@ -2909,8 +2918,8 @@ fs4d_status fs4d_train_step(fs4d_trainer* tr, fs4d_precision prec, const fs4d_ca
   const size_t pix3 = 3 * (size_t)cam->width * cam->height;
   if (tr->image.bytes < 4 * pix3 || tr->dl.bytes < 4 * pix3) {
     FS4D_CUDA(c, cudaStreamSynchronize(c->stream));
-    FS4D_CUDA(c, ensure(tr->image, 4 * pix3));
-    FS4D_CUDA(c, ensure(tr->dl, 4 * pix3));
+    FS4D_CUDA(c, ensure(c, tr->image, 4 * pix3));
+    FS4D_CUDA(c, ensure(c, tr->dl, 4 * pix3));
   }
   float* losses = d_losses ? d_losses : P<float>(tr->losses);
   // 1. the frame, keeping the backward's state
@@ -3046,7 +3055,7 @@ fs4d_status fs4d_densify(fs4d_ctx* c, fs4d_scene_id id, const fs4d_densify_confi
   auto cleanup = [](std::initializer_list<DevBuf*> bufs) {
     for (DevBuf* b : bufs) release(*b);
   };
-  FS4D_CUDA(c, ensure(plan, 4 * (3 * (size_t)nb + 4)));
+  FS4D_CUDA(c, ensure(c, plan, 4 * (3 * (size_t)nb + 4)));
   DensifyArgs a{};
   a.n = n;
   a.log_scales = P<float>(s->log_scales);
@@ -3078,10 +3087,10 @@ fs4d_status fs4d_densify(fs4d_ctx* c, fs4d_scene_id id, const fs4d_densify_confi
   // the new arrays, the output map and the work order's sort buffers
   DevBuf map, nm, nls, nq, no, nsh, keys, perm;
   std::initializer_list<DevBuf*> fresh = {&map, &nm, &nls, &nq, &no, &nsh, &keys, &perm};
-  if (ensure(map, 8 * (size_t)m) != cudaSuccess || ensure(nm, 12 * (size_t)m) != cudaSuccess ||
-      ensure(nls, 12 * (size_t)m) != cudaSuccess || ensure(nq, 16 * (size_t)m) != cudaSuccess ||
-      ensure(no, 4 * (size_t)m) != cudaSuccess || ensure(nsh, 4 * (size_t)K3 * m) != cudaSuccess ||
-      ensure(keys, 8 * (size_t)m) != cudaSuccess || ensure(perm, 4 * (size_t)m) != cudaSuccess) {
+  if (ensure(c, map, 8 * (size_t)m) != cudaSuccess || ensure(c, nm, 12 * (size_t)m) != cudaSuccess ||
+      ensure(c, nls, 12 * (size_t)m) != cudaSuccess || ensure(c, nq, 16 * (size_t)m) != cudaSuccess ||
+      ensure(c, no, 4 * (size_t)m) != cudaSuccess || ensure(c, nsh, 4 * (size_t)K3 * m) != cudaSuccess ||
+      ensure(c, keys, 8 * (size_t)m) != cudaSuccess || ensure(c, perm, 4 * (size_t)m) != cudaSuccess) {
     cleanup({&plan});
     cleanup(fresh);
     return fail(c, FS4D_ERR_OOM, "densify: device allocation failed");
@@ -3137,8 +3146,8 @@ fs4d_status fs4d_densify(fs4d_ctx* c, fs4d_scene_id id, const fs4d_densify_confi
       tcnt[k] = cnt[k];
       total += (cnt[k] + 3) / 4 * 4;
     }
-    if (ensure(tg, 4 * total) != cudaSuccess || ensure(tm, 4 * total) != cudaSuccess ||
-        ensure(tv, 4 * total) != cudaSuccess || ensure(ts, 8 * (size_t)m) != cudaSuccess) {
+    if (ensure(c, tg, 4 * total) != cudaSuccess || ensure(c, tm, 4 * total) != cudaSuccess ||
+        ensure(c, tv, 4 * total) != cudaSuccess || ensure(c, ts, 8 * (size_t)m) != cudaSuccess) {
       cudaStreamSynchronize(c->stream);
       cleanup({&plan, &tg, &tm, &tv, &ts});
       cleanup(fresh);
