@@ -1283,11 +1283,11 @@ fs4d_frame* take_spare(fs4d_ctx* c) {
   return f;
 }
 
-// The buffers of a saved frame, grown where they are too small.
-fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, size_t npix, size_t pairs) {
+// The buffers of a saved frame but its list, grown where they are too small.
+fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, size_t npix) {
   const std::pair<DevBuf*, size_t> need[] = {
       {&f->dmeans, 12 * n}, {&f->dquats, 16 * n}, {&f->dscales, 12 * n}, {&f->xy, 8 * n},       {&f->co, 16 * n},
-      {&f->rgb, 12 * n},    {&f->radius, 4 * n},  {&f->rect, 16 * n},    {&f->offsets, 4 * n},  {&f->values, 4 * pairs},
+      {&f->rgb, 12 * n},    {&f->radius, 4 * n},  {&f->rect, 16 * n},    {&f->offsets, 4 * n},
       {&f->sco, 16 * n},    {&f->slot, 16 * n},   {&f->ranges, 8 * tiles}, {&f->order, 4 * tiles}, {&f->t_final, 4 * npix}, {&f->n_contrib, 4 * npix}};
   bool grow = false, first = true;
   for (const auto& q : need) {
@@ -1304,7 +1304,10 @@ fs4d_status ensure_frame(fs4d_ctx* c, fs4d_frame* f, size_t n, size_t tiles, siz
 // Render with the state the backward needs, into f (its buffers are reused and
 // grown when needed, so a frame object can serve one training step after another).
 // The frame's kernels write that state where it stays: they run on a view of the
-// work memory in which the frame's buffers stand in for the context's.
+// work memory in which the frame's buffers stand in for the context's.  A frame
+// without a list yet has it made in the work memory and copied once its length is
+// known, so that it holds what its list needs (and a quarter, for the next view) and
+// not what the context was reserved for.
 fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const fs4d_camera* cam, float t,
                               float* d_image, fs4d_frame* f, bool cull) {
   const size_t npix = (size_t)cam->width * cam->height;
@@ -1318,19 +1321,22 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
   if (f->epoch != c->epoch && f->dmeans.p) f->one_epoch = false;
   f->epoch = c->epoch;
   f->device = c->device;
+  if ((st = ensure_frame(c, f, (size_t)s->n, (size_t)n_tiles, npix)) != FS4D_OK) return st;
   for (int pass = 0;; ++pass) {
-    if ((st = ensure_frame(c, f, (size_t)s->n, (size_t)n_tiles, npix, (size_t)c->w.cap_pairs)) != FS4D_OK) return st;
     Work v = c->w;
     v.dmeans = f->dmeans; v.dquats = f->dquats; v.dscales = f->dscales;
     v.co = f->co; v.radius = f->radius; v.rect = f->rect;
     v.offsets = f->offsets; v.ranges = f->ranges; v.order_out = f->order;
     f->ranks = use_lists(c, c->w, s->n, tx, ty);
+    const long long own = (long long)(f->values.bytes / 4);
+    if (own > 0) {  // (a sorted list needs the keys' room beside it)
+      v.cap_pairs = f->ranks ? own : std::min(own, c->w.cap_pairs);
+      (!f->ranks && odd ? v.values_alt : v.values) = f->values;
+    }
     if (f->ranks) {
       v.sxy = f->xy; v.srgb = f->rgb; v.sco = f->sco; v.sslot = f->slot;
-      v.values = f->values;
     } else {
       v.xy = f->xy; v.rgb = f->rgb;
-      (odd ? v.values_alt : v.values) = f->values;
     }
     c->last_binning = f->ranks ? FS4D_BINNING_BITMAP : FS4D_BINNING_SORT;
     const Env e{c, &v, c->stream, P<uint32_t>(c->status), true};
@@ -1344,12 +1350,24 @@ fs4d_status render_into_frame(fs4d_ctx* c, Scene* s, fs4d_precision prec, const 
       return fail(c, FS4D_ERR_CAPACITY, "a frame saved for the backward must fit one band of tile pairs");
     f->pairs = c->last_pairs = K;
     f->slots = f->ranks ? (long long)c->h_pinned[2] : K;
-    if (K <= c->w.cap_pairs) {
-      if (values != f->values.p) return fail(c, FS4D_ERR_CUDA, "render: the frame's list is not where it belongs");
+    const long long listed = f->ranks ? (long long)c->h_pinned[1] : K;  // (both count on past the capacity)
+    const size_t room = 4 * (size_t)std::max(listed + listed / 4, 1ll);
+    if (listed <= v.cap_pairs) {
+      if (own > 0 && values != f->values.p)
+        return fail(c, FS4D_ERR_CUDA, "render: the frame's list is not where it belongs");
+      if (own > 0) break;
+      FS4D_CUDA(c, ensure(c, f->values, room));
+      FS4D_CUDA(c, cudaMemcpyAsync(f->values.p, values, 4 * (size_t)listed, cudaMemcpyDeviceToDevice, c->stream));
       break;
     }
     if (pass > 0) return fail(c, FS4D_ERR_CAPACITY, "render: the frame's pairs changed between two passes");
-    if ((st = ensure_work(c, s->n, tx, ty, std::min(K + K / 4, c->band_pairs))) != FS4D_OK) return st;
+    if (own > 0 && f->values.bytes < room) {
+      FS4D_CUDA(c, cudaStreamSynchronize(c->stream));  // the old list may still be read
+      FS4D_CUDA(c, ensure(c, f->values, room));
+    }
+    if ((own == 0 || !f->ranks) &&
+        (st = ensure_work(c, s->n, tx, ty, std::max(std::min(K + K / 4, c->band_pairs), c->w.cap_pairs))) != FS4D_OK)
+      return st;
   }
   f->scene = s->id;
   f->cam = *cam;

@@ -188,3 +188,53 @@ def test_kept_frames_make_room(ctx):
     finally:
         hogs.clear()
         torch.cuda.empty_cache()
+
+
+def view_gradients(ctx, sid, s, cam, t):
+    image, frame = ctx.render_saved(sid, cam, t)
+    g = {k: torch.zeros(np.shape(getattr(s, k)), device="cuda") for k in fs4d.PARAMS}
+    ctx.render_backward(frame, torch.ones_like(image), g)
+    ctx.frame_free(frame)
+    return image, g
+
+
+@pytest.mark.parametrize("modes", [(fs4d.BINNING_AUTO,), (fs4d.BINNING_SORT,), (fs4d.BINNING_AUTO, fs4d.BINNING_SORT)])
+def test_saved_frames_of_changing_size(ctx, modes):
+    """Frames that take over the buffers of frames of other sizes, scenes and binnings, growing
+    past their lists' capacity and shrinking again, are those of a context that has rendered
+    nothing yet."""
+    scenes = [sg.make_object(12, n=900, mlp_std=0.1), sg.make_object(13, n=15_000, log_scale_mean=-3.0, mlp_std=0.1)]
+    ids = [ctx.load_scene(s) for s in scenes]
+    turns = [(0, 64, 48), (1, 300, 200), (0, 500, 300), (1, 120, 500), (1, 640, 480), (0, 33, 17), (1, 300, 200)]
+    for k, (which, w, h) in enumerate(turns):
+        mode = modes[k % len(modes)]
+        cam = sg.hemisphere_cameras(5, width=w, height=h, seed=4)[k % 5]
+        fresh = fs4d.Context(0)
+        try:
+            fresh.set_binning(mode)
+            want, wg = view_gradients(fresh, fresh.load_scene(scenes[which]), scenes[which], cam, 0.3)
+        finally:
+            fresh.close()
+        ctx.set_binning(mode)
+        got, gg = view_gradients(ctx, ids[which], scenes[which], cam, 0.3)
+        assert torch.equal(got, want)
+        for n, v in wg.items():  # (the order among warps, and of a plane cell's terms, is free)
+            scale = float(v.abs().max())
+            assert float((gg[n] - v).abs().max()) <= 1e-4 * scale, (k, n)
+    ctx.check_device_status()
+
+
+def test_saved_frames_hold_what_their_lists_need(ctx):
+    """After a generous reservation a saved frame holds its own list, not the reserved one."""
+    s = sg.make_object(14, n=10_000, mlp_std=0.1)
+    cam = sg.hemisphere_cameras(5, width=200, height=150, seed=4)[1]
+    sid = ctx.load_scene(s)
+    ctx.reserve(sid, 200, 150, 100_000_000)
+    view_gradients(ctx, sid, s, cam, 0.3)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    frames = [ctx.render_saved(sid, cam, 0.1 * k)[1] for k in range(4)]
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 4 * (32 << 20)  # (their lists at the reservation: 400 MB each)
+    for f in frames:
+        ctx.frame_free(f)
