@@ -571,14 +571,16 @@ fs4d_status get_scene(fs4d_ctx* c, fs4d_scene_id id, Scene** out) {
   return FS4D_OK;
 }
 
-// Grow the per-Gaussian / per-tile / per-pair work buffers.
+constexpr size_t kColorTail = 16384;
+size_t color_bytes(int n) { return 4 * (64 + 48 + 1) * (size_t)n + kColorTail; }
+
 // Work memory of the colour and opacity heads for frames of up to n Gaussians
 // (allocated on the first frame of a scene with them; never during a capture).
 fs4d_status ensure_color(fs4d_ctx* c, Work& w, cudaStream_t stream, int n) {
   if (w.cap_color >= n) return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(stream));
   w.cap_color = 0;
-  FS4D_CUDA(c, ensure(c, w.fd, 4 * 64 * (size_t)n + 16384));  // + the last BF16 tile image's ragged end
+  FS4D_CUDA(c, ensure(c, w.fd, 4 * 64 * (size_t)n + kColorTail));  // + the last BF16 tile image's ragged end
   FS4D_CUDA(c, ensure(c, w.dsh, 4 * 48 * (size_t)n));
   FS4D_CUDA(c, ensure(c, w.dop, 4 * (size_t)n));
   w.cap_color = n;
@@ -589,6 +591,38 @@ fs4d_status ensure_color(fs4d_ctx* c, Work& w, cudaStream_t stream, int n) {
 size_t class_bytes(long long n_tiles) { return 4 * 32 * (size_t)n_tiles; }
 size_t axis_bytes(int n, long long rows) { return 4 * (size_t)rows * (size_t)bitmap_words(std::max(n, 1)); }
 
+// Work buffers by what they hold one element of.
+struct WorkItem {
+  DevBuf Work::*buf;
+  size_t bytes;
+};
+constexpr WorkItem kPerGaussian[] = {
+    {&Work::dmeans, 12}, {&Work::dquats, 16},    {&Work::dscales, 12}, {&Work::xy, 8},        {&Work::co, 16},
+    {&Work::rgb, 12},    {&Work::depth, 4},      {&Work::radius, 4},   {&Work::rect, 16},     {&Work::sxy, 8},
+    {&Work::sco, 16},    {&Work::srgb, 12},      {&Work::srect, 16},   {&Work::offsets, 4},   {&Work::dkeys, 8},
+    {&Work::dvals, 4},   {&Work::dkeys_alt, 8},  {&Work::dvals_alt, 4}, {&Work::bpos, 4}};
+constexpr WorkItem kPerPair[] = {
+    {&Work::keys, 8}, {&Work::values, 4}, {&Work::keys_alt, 8}, {&Work::values_alt, 4}};
+constexpr long long kMinPairs = 4096;
+
+long long look_back_parts(int n, long long pairs) {
+  return std::max(sort_parts(std::max(pairs, kMinPairs)), sort_parts(n));
+}
+
+// What ensure_work allocates for an image of tx x ty tiles.
+size_t work_bytes(int n, int tx, int ty, long long pairs) {
+  const int n_tiles = tx * ty;
+  n = std::max(n, 1);
+  pairs = std::max(pairs, kMinPairs);
+  size_t b = 4 * kCounters + 4 * (kBuckets + 4) + 4 * 256 * kSortMaxPasses + 8 * (size_t)n_tiles + class_bytes(n_tiles) +
+             axis_bytes(n, (long long)tx + ty) + 4 * 256 * (size_t)kSortMaxPasses * look_back_parts(n, pairs) +
+             frame_zero_layout(n, n_tiles, pairs, sort_passes(ceil_log2(std::max(n_tiles, 1))), nullptr, nullptr);
+  for (const WorkItem& q : kPerGaussian) b += q.bytes * (size_t)n;
+  for (const WorkItem& q : kPerPair) b += q.bytes * (size_t)pairs;
+  return b;
+}
+
+// Grow the per-Gaussian / per-tile / per-pair work buffers.
 fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx, int ty, long long pairs) {
   const int n_tiles = tx * ty;
   // bit rows for an image's tiles, or for lists of any number of tiles (bin_sort)
@@ -605,27 +639,8 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   // a capacity is 0 while its buffers are reallocated: after a failure the next call allocates
   // them again, for its own size
   if (n > w.cap_n) {
-    const size_t m = (size_t)n;
     w.cap_n = 0;
-    FS4D_CUDA(c, ensure(c, w.dmeans, 12 * m));
-    FS4D_CUDA(c, ensure(c, w.dquats, 16 * m));
-    FS4D_CUDA(c, ensure(c, w.dscales, 12 * m));
-    FS4D_CUDA(c, ensure(c, w.xy, 8 * m));
-    FS4D_CUDA(c, ensure(c, w.co, 16 * m));
-    FS4D_CUDA(c, ensure(c, w.rgb, 12 * m));
-    FS4D_CUDA(c, ensure(c, w.depth, 4 * m));
-    FS4D_CUDA(c, ensure(c, w.radius, 4 * m));
-    FS4D_CUDA(c, ensure(c, w.rect, 16 * m));
-    FS4D_CUDA(c, ensure(c, w.sxy, 8 * m));
-    FS4D_CUDA(c, ensure(c, w.sco, 16 * m));
-    FS4D_CUDA(c, ensure(c, w.srgb, 12 * m));
-    FS4D_CUDA(c, ensure(c, w.srect, 16 * m));
-    FS4D_CUDA(c, ensure(c, w.offsets, 4 * m));
-    FS4D_CUDA(c, ensure(c, w.dkeys, 8 * m));
-    FS4D_CUDA(c, ensure(c, w.dvals, 4 * m));
-    FS4D_CUDA(c, ensure(c, w.dkeys_alt, 8 * m));
-    FS4D_CUDA(c, ensure(c, w.dvals_alt, 4 * m));
-    FS4D_CUDA(c, ensure(c, w.bpos, 4 * m));
+    for (const WorkItem& q : kPerGaussian) FS4D_CUDA(c, ensure(c, w.*q.buf, q.bytes * (size_t)n));
     w.cap_n = n;
   }
   FS4D_CUDA(c, ensure(c, w.counters, 4 * kCounters));
@@ -639,15 +654,12 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
     w.cap_tiles = tiles;
   }
   if (pairs > w.cap_pairs) {
-    const long long cap = std::max<long long>(pairs, 4096);
+    const long long cap = std::max(pairs, kMinPairs);
     w.cap_pairs = 0;
-    FS4D_CUDA(c, ensure(c, w.keys, 8 * (size_t)cap));
-    FS4D_CUDA(c, ensure(c, w.values, 4 * (size_t)cap));
-    FS4D_CUDA(c, ensure(c, w.keys_alt, 8 * (size_t)cap));
-    FS4D_CUDA(c, ensure(c, w.values_alt, 4 * (size_t)cap));
+    for (const WorkItem& q : kPerPair) FS4D_CUDA(c, ensure(c, w.*q.buf, q.bytes * (size_t)cap));
     w.cap_pairs = cap;
   }
-  const long long parts = std::max(sort_parts(std::max<long long>(w.cap_pairs, 4096)), sort_parts(w.cap_n));
+  const long long parts = look_back_parts(w.cap_n, w.cap_pairs);
   if (parts > w.sort_parts_cap) {
     w.sort_parts_cap = 0;
     FS4D_CUDA(c, ensure(c, w.sort_lb, 4 * 256 * (size_t)kSortMaxPasses * parts));
@@ -1081,6 +1093,8 @@ BandTab band_tab(const fs4d_camera* cam, const std::vector<std::pair<int, int>>&
 }
 
 // Device memory of the frames composited straight from the depth order.
+size_t direct_bytes(int n) { return (8 + 16 + 8) * (size_t)n + 8 * kMaxTileRows; }
+
 fs4d_status ensure_direct(fs4d_ctx* c, int n) {
   Work& w = c->w;
   const size_t m = (size_t)n;
@@ -1625,13 +1639,11 @@ fs4d_status fs4d_scene_bytes(fs4d_ctx* c, fs4d_scene_id id, int32_t width, int32
   if (st != FS4D_OK) return st;
   if (resident) *resident = s->resident;
   if (per_frame) {
-    const size_t n = (size_t)s->n;
-    const size_t pairs = (size_t)(std::max(0.f, ppg) * (float)n) + 4096;
-    const size_t tiles = (size_t)tiles_of(width) * tiles_of(height);
-    const size_t bmp = bitmap_bytes((int)n, (long long)tiles);
-    *per_frame = (bmp <= kBitmapMaxBytes ? bmp + 36 * n : 0) + n * (12 + 16 + 12 + 8 + 16 + 12 + 4 + 4 + 16 + 4 + 24) + pairs * 24 +
-                 sort_parts((long long)pairs) * 256 * 4 * kSortMaxPasses + tiles * 8 +
-                 (size_t)width * height * 12;
+    const long long pairs = (long long)(std::max(0.f, ppg) * (float)s->n) + 4096;
+    const int tx = tiles_of(width), ty = tiles_of(height);
+    *per_frame = work_bytes(s->n, tx, ty, pairs) + (size_t)width * height * 12;
+    if (bitmap_bytes(s->n, (long long)tx * ty) > kBitmapMaxBytes) *per_frame += direct_bytes(s->n);
+    if (s->color_heads) *per_frame += color_bytes(s->n);
   }
   return FS4D_OK;
 }
@@ -2331,11 +2343,7 @@ struct Staging {
 };
 
 size_t slot_bytes_for(int n, int w, int h, long long pairs) {
-  const size_t tiles = (size_t)tiles_of(w) * tiles_of(h);
-  const size_t bmp = bitmap_bytes(n, (long long)tiles);
-  return (bmp <= kBitmapMaxBytes ? bmp + 36 * (size_t)n : 0) + (size_t)n * (12 + 16 + 12 + 8 + 16 + 12 + 4 + 4 + 16 + 4 + 24) + 8 * (size_t)(emit_parts(n) + 1) +
-         (size_t)pairs * 24 + 4 * 256 * (size_t)kSortMaxPasses * sort_parts(pairs) + tiles * 8 +
-         (size_t)w * h * 12 + 4096;
+  return work_bytes(n, tiles_of(w), tiles_of(h), pairs) + (size_t)w * h * 12 + 4096;
 }
 
 }  // namespace

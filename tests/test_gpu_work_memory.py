@@ -238,3 +238,17 @@ def test_saved_frames_hold_what_their_lists_need(ctx):
     assert free - torch.cuda.mem_get_info()[0] < 4 * (32 << 20)  # (their lists at the reservation: 400 MB each)
     for f in frames:
         ctx.frame_free(f)
+
+
+@pytest.mark.parametrize("n,w,h,ppg", [(1_000_000, 800, 600, 10.0), (600_000, 1920, 1080, 4.0)])
+def test_scene_bytes_are_what_a_frame_allocates(ctx, n, w, h, ppg):
+    """The per-frame figure that admission goes by, against the device memory that a reservation
+    of that size takes (allocations come in 2 MB, fewer than 40 of them)."""
+    sid = ctx.load_scene(sg.make_object(15, n=n, log_scale_mean=-7.0))
+    _, per_frame = ctx.scene_bytes(sid, w, h, ppg)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    ctx.reserve(sid, w, h, int(ppg * n) + 4096)
+    used = free - torch.cuda.mem_get_info()[0]
+    want = per_frame - w * h * 12  # (the image is the caller's)
+    assert want <= used <= want + 40 * (2 << 20)
