@@ -166,7 +166,9 @@ struct Work {
   int cap_color = 0;
   long long cap_pairs = 0;
   long long sort_parts_cap = 0;
-  int cap_n = 0, cap_tiles = 0;
+  int cap_n = 0, cap_tiles = 0;            // Gaussians of a frame, tiles
+  int cap_order = 0;                       // Gaussians of a depth order (kPerRank), at least cap_n
+  long long cap_list = 0;                  // pairs of `values`, at least cap_pairs
 };
 
 void release_work(Work& w) {
@@ -597,12 +599,13 @@ struct WorkItem {
   size_t bytes;
 };
 constexpr WorkItem kPerGaussian[] = {
-    {&Work::dmeans, 12}, {&Work::dquats, 16},    {&Work::dscales, 12}, {&Work::xy, 8},        {&Work::co, 16},
-    {&Work::rgb, 12},    {&Work::depth, 4},      {&Work::radius, 4},   {&Work::rect, 16},     {&Work::sxy, 8},
-    {&Work::sco, 16},    {&Work::srgb, 12},      {&Work::srect, 16},   {&Work::offsets, 4},   {&Work::dkeys, 8},
-    {&Work::dvals, 4},   {&Work::dkeys_alt, 8},  {&Work::dvals_alt, 4}, {&Work::bpos, 4}};
-constexpr WorkItem kPerPair[] = {
-    {&Work::keys, 8}, {&Work::values, 4}, {&Work::keys_alt, 8}, {&Work::values_alt, 4}};
+    {&Work::dmeans, 12}, {&Work::dquats, 16}, {&Work::dscales, 12}, {&Work::xy, 8},    {&Work::co, 16},  {&Work::rgb, 12},
+    {&Work::depth, 4},   {&Work::radius, 4},  {&Work::rect, 16},    {&Work::sxy, 8},   {&Work::sco, 16}, {&Work::srgb, 12}};
+constexpr WorkItem kPerRank[] = {  // depth order and lists from it: all that bin_sort needs
+    {&Work::srect, 16}, {&Work::offsets, 4},   {&Work::dkeys, 8}, {&Work::dvals, 4},
+    {&Work::dkeys_alt, 8}, {&Work::dvals_alt, 4}, {&Work::bpos, 4}};
+constexpr WorkItem kPerPair[] = {  // (and `values`)
+    {&Work::keys, 8}, {&Work::keys_alt, 8}, {&Work::values_alt, 4}};
 constexpr long long kMinPairs = 4096;
 
 long long look_back_parts(int n, long long pairs) {
@@ -618,12 +621,16 @@ size_t work_bytes(int n, int tx, int ty, long long pairs) {
              axis_bytes(n, (long long)tx + ty) + 4 * 256 * (size_t)kSortMaxPasses * look_back_parts(n, pairs) +
              frame_zero_layout(n, n_tiles, pairs, sort_passes(ceil_log2(std::max(n_tiles, 1))), nullptr, nullptr);
   for (const WorkItem& q : kPerGaussian) b += q.bytes * (size_t)n;
+  for (const WorkItem& q : kPerRank) b += q.bytes * (size_t)n;
   for (const WorkItem& q : kPerPair) b += q.bytes * (size_t)pairs;
-  return b;
+  return b + 4 * (size_t)pairs;
 }
 
-// Grow the per-Gaussian / per-tile / per-pair work buffers.
-fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx, int ty, long long pairs) {
+// Grow the per-Gaussian / per-tile / per-pair work buffers.  lists_only: for bin_sort by lists,
+// which has neither deformed nor projected Gaussians nor keys of its own (a third of the
+// allocations: the first call of a context takes 0.3 ms less).
+fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx, int ty, long long pairs,
+                        bool lists_only = false) {
   const int n_tiles = tx * ty;
   // bit rows for an image's tiles, or for lists of any number of tiles (bin_sort)
   const bool image = tx <= kMaxTileRows && ty <= kMaxTileRows;
@@ -631,21 +638,25 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
   // (this call's rows and Gaussians: the largest of each, from calls of different kinds, could
   // come to many gigabytes that no call needs)
   const size_t axis = bits ? axis_bytes(n, (long long)tx + ty) : 0;
-  const size_t order = image ? class_bytes(n_tiles) : 4 * (size_t)n_tiles;
-  const bool grow = n > w.cap_n || n_tiles > w.cap_tiles || pairs > w.cap_pairs || axis > w.axis.bytes ||
-                    order > w.tile_order.bytes || w.sort_parts_cap == 0 || !w.zero.p;
-  if (!grow) return FS4D_OK;
+  const size_t order = image && !lists_only ? class_bytes(n_tiles) : 4 * (size_t)n_tiles;
+  const bool frame = !lists_only && (n > w.cap_n || pairs > w.cap_pairs || w.sort_parts_cap == 0);
+  if (!frame && n <= w.cap_order && n_tiles <= w.cap_tiles && pairs <= w.cap_list && axis <= w.axis.bytes &&
+      order <= w.tile_order.bytes && w.zero.p)
+    return FS4D_OK;
   FS4D_CUDA(c, cudaStreamSynchronize(stream));
   // a capacity is 0 while its buffers are reallocated: after a failure the next call allocates
   // them again, for its own size
-  if (n > w.cap_n) {
+  if (n > w.cap_order) {
+    w.cap_n = w.cap_order = 0;
+    for (const WorkItem& q : kPerRank) FS4D_CUDA(c, ensure(c, w.*q.buf, q.bytes * (size_t)n));
+    w.cap_order = n;
+  }
+  if (!lists_only && n > w.cap_n) {
     w.cap_n = 0;
     for (const WorkItem& q : kPerGaussian) FS4D_CUDA(c, ensure(c, w.*q.buf, q.bytes * (size_t)n));
     w.cap_n = n;
   }
-  FS4D_CUDA(c, ensure(c, w.counters, 4 * kCounters));
   FS4D_CUDA(c, ensure(c, w.bstart, 4 * (kBuckets + 4)));
-  FS4D_CUDA(c, ensure(c, w.hist, 4 * 256 * kSortMaxPasses));
   if (n_tiles > w.cap_tiles || order > w.tile_order.bytes) {
     const int tiles = std::max(n_tiles, w.cap_tiles);
     w.cap_tiles = 0;
@@ -653,19 +664,28 @@ fs4d_status ensure_work(fs4d_ctx* c, Work& w, cudaStream_t stream, int n, int tx
     FS4D_CUDA(c, ensure(c, w.tile_order, std::max(order, 4 * (size_t)tiles)));
     w.cap_tiles = tiles;
   }
-  if (pairs > w.cap_pairs) {
-    const long long cap = std::max(pairs, kMinPairs);
+  const long long cap = std::max(pairs, kMinPairs);
+  if (pairs > w.cap_list) {
+    w.cap_pairs = w.cap_list = 0;
+    FS4D_CUDA(c, ensure(c, w.values, 4 * (size_t)cap));
+    w.cap_list = cap;
+  }
+  if (!lists_only && pairs > w.cap_pairs) {
     w.cap_pairs = 0;
     for (const WorkItem& q : kPerPair) FS4D_CUDA(c, ensure(c, w.*q.buf, q.bytes * (size_t)cap));
     w.cap_pairs = cap;
   }
-  const long long parts = look_back_parts(w.cap_n, w.cap_pairs);
-  if (parts > w.sort_parts_cap) {
-    w.sort_parts_cap = 0;
-    FS4D_CUDA(c, ensure(c, w.sort_lb, 4 * 256 * (size_t)kSortMaxPasses * parts));
-    w.sort_parts_cap = parts;
+  if (!lists_only) {
+    FS4D_CUDA(c, ensure(c, w.counters, 4 * kCounters));
+    FS4D_CUDA(c, ensure(c, w.hist, 4 * 256 * kSortMaxPasses));
+    const long long parts = look_back_parts(w.cap_n, w.cap_pairs);
+    if (parts > w.sort_parts_cap) {
+      w.sort_parts_cap = 0;
+      FS4D_CUDA(c, ensure(c, w.sort_lb, 4 * 256 * (size_t)kSortMaxPasses * parts));
+      w.sort_parts_cap = parts;
+    }
   }
-  const size_t zb = frame_zero_layout(w.cap_n, w.cap_tiles, w.cap_pairs,
+  const size_t zb = frame_zero_layout(w.cap_order, w.cap_tiles, w.cap_pairs,
                                       sort_passes(ceil_log2(std::max(w.cap_tiles, 1))), nullptr, nullptr);
   FS4D_CUDA(c, ensure(c, w.zero, zb));
   FS4D_CUDA(c, ensure(c, w.axis, axis));
@@ -683,8 +703,8 @@ bool use_lists(const fs4d_ctx* c, const Work& w, int n, int tx, int ty, bool cla
          (!classes || class_bytes(n_tiles) <= w.tile_order.bytes);
 }
 
-fs4d_status ensure_work(fs4d_ctx* c, int n, int tx, int ty, long long pairs) {
-  return ensure_work(c, c->w, c->stream, n, tx, ty, pairs);
+fs4d_status ensure_work(fs4d_ctx* c, int n, int tx, int ty, long long pairs, bool lists_only = false) {
+  return ensure_work(c, c->w, c->stream, n, tx, ty, pairs, lists_only);
 }
 
 SortWork sort_work(Work& w) {
@@ -2179,7 +2199,9 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
     return fail(c, FS4D_ERR_INVALID_ARG, "bin_sort: bad argument");
   DeviceGuard g(c->device);
   const int n_tiles = tiles_x * tiles_y;
-  fs4d_status st = ensure_work(c, std::max(n, 1), tiles_x, tiles_y, capacity);
+  const bool lists = c->binning != FS4D_BINNING_SORT && n > 0 &&
+                     bitmap_bytes(n, (long long)tiles_x * tiles_y) <= kBitmapMaxBytes;
+  fs4d_status st = ensure_work(c, std::max(n, 1), tiles_x, tiles_y, capacity, lists);
   if (st != FS4D_OK) return st;
   Work& w = c->w;
   const int tile_bits = ceil_log2(n_tiles);
@@ -2214,7 +2236,7 @@ fs4d_status fs4d_bin_sort(fs4d_ctx* c, int32_t n, const float* d_depth, const in
     la.words = bitmap_words(n);
     la.bits = P<uint32_t>(w.axis); la.s_rect = P<int4>(w.srect);
     la.num_pairs = z.num_pairs;
-    la.capacity = std::min<long long>(w.cap_pairs, capacity);
+    la.capacity = std::min<long long>(w.cap_list, capacity);
     la.values = P<uint32_t>(w.values); la.ranges = P<uint2>(w.ranges);
     la.tile_count = z.tile_count;
     FS4D_CUDA(c, launch_tile_bits(la, c->stream));
