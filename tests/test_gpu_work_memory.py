@@ -256,19 +256,20 @@ def test_scene_bytes_are_what_a_frame_allocates(ctx, n, w, h, ppg):
 
 def test_bin_sort_allocates_no_frame(ctx):
     """A context's first bin_sort takes the depth order, the lists and the bit rows (48 bytes per
-    Gaussian and pair, 13 MB of bits), none of a frame's 140 bytes per Gaussian and 20 per pair."""
+    Gaussian and pair, 10 MB of bits), none of a frame's 140 bytes per Gaussian and 20 per pair."""
     n = 1_000_000
     depth = torch.rand(n, device="cuda") + 1
-    x = (torch.arange(n, device="cuda") % 50).int()
-    y = (torch.arange(n, device="cuda") // 50 % 50).int()
+    x = (torch.arange(n, device="cuda") % 40).int()
+    y = (torch.arange(n, device="cuda") // 40 % 40).int()
     rect = torch.stack([x, y, x + 1, y + 1], 1).contiguous()
-    ctx.bin_sort(depth[:1], rect[:1].contiguous(), 50, 50, 1)  # (the modules are loaded)
-    warm = ctx.bin_sort(depth, rect, 50, 50, n)
+    ctx.bin_sort(depth[:1], rect[:1].contiguous(), 40, 40, 1)  # (the modules are loaded)
+    warm = ctx.bin_sort(depth, rect, 40, 40, n)
     torch.cuda.synchronize()
     other = fs4d.Context(0)
     try:
         free = torch.cuda.mem_get_info()[0]
-        got = other.bin_sort(depth, rect, 50, 50, n)
+        got = other.bin_sort(depth, rect, 40, 40, n)
+        assert other.last_binning() == fs4d.BINNING_BITMAP
         torch.cuda.synchronize()
         assert free - torch.cuda.mem_get_info()[0] < 120 << 20  # (12 bytes per pair of them torch's)
         assert all(torch.equal(a, b) for a, b in zip(got[:3], warm[:3]))
