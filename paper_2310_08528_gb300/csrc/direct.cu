@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads) axis_bits_kernel(const __grid_consta
     x0[k] = x1[k] = 0;
     fr[k] = fpy[k] = iz[k] = 0.f;
     if (pos < a.n) {
-      const uint32_t g = order[pos];
+      const uint32_t g = min(order[pos], (uint32_t)a.n - 1u);  // (a sort whose wait gave up leaves anything there)
       const int rad = a.radius[g];
       if (rad > 0) {  // (an invisible Gaussian has no bits, so its copies are never read)
         const int4 r = a.rect[g];

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const __grid_constant_
     }
   } else if (live) {
     const uint32_t* order = (a.order_sel && *a.order_sel) ? a.order_alt : a.order;
-    g = order[i];
+    g = min(order[i], (uint32_t)a.n - 1u);  // (a sort whose wait gave up leaves anything there)
   }
   int4 cut = make_int4(0, 0, 0, 0);
   if (live) {
