@@ -158,26 +158,23 @@ def load_peaks(sms: int = 152):
 
 
 def stage_work(stage: str, n: int, K: int, pixels: int, passes: int, prec: str, evals: int = 0,
-               bitmap: bool = True, visited: int = None, bands: int = 1, direct: bool = False):
+               bitmap: bool = True, visited: int = None, direct: bool = False):
     """Algorithmic bytes or FLOPs of one frame's launches of each stage (per-unit
     figures times the units processed).  Returns a list of (bound, work, unit);
     the first entry is the stage's primary bound; an empty list: the stage does
     no work of its own.  visited: tile pairs the compositing must read (each
-    tile's list up to its last contributing Gaussian); bands: passes of the
-    per-Gaussian stages (a composed frame rendered in bands projects and depth-sorts
-    once per band); direct: a frame composited straight from the depth order."""
-    if direct:
-        bands = 1  # the bands share one projection and one depth order
+    tile's list up to its last contributing Gaussian); direct: a frame composited
+    straight from the depth order (its bands share one projection and one depth order)."""
     if stage == "deform":
         flops = 2 * (64 * 64 + 64 * 64 + 3 * 64 * 64 + 64 * 10) * n   # MLP contraction, 42,240 FLOP/Gaussian
         return [(("tensor" if prec == "bf16" else "alu"), flops, "FLOP"), ("hbm", 80 * n, "B")]
     if stage == "project":
         # read: mean, quaternion, log-scale, opacity logit, 48 SH floats; written: xy, conic + opacity,
         # rgb, depth, radius, tile rectangle, depth-sort key and index
-        return [("hbm", bands * (n * (12 + 16 + 12 + 4 + 48 * 4) + n * (8 + 16 + 12 + 4 + 4 + 16 + 4 + 4)), "B")]
+        return [("hbm", n * (12 + 16 + 12 + 4 + 48 * 4) + n * (8 + 16 + 12 + 4 + 4 + 16 + 4 + 4), "B")]
     if stage == "depth_sort":
         # 4 passes over 32-bit keys, each reading and writing an 8 B key and a 4 B index per Gaussian
-        return [("hbm", bands * 4 * n * 24, "B")]
+        return [("hbm", 4 * n * 24, "B")]
     if stage == "binning":
         if direct:
             # pairs per band: radius, rect, y parts per Gaussian
@@ -188,7 +185,7 @@ def stage_work(stage: str, n: int, K: int, pixels: int, passes: int, prec: str, 
             return [("hbm", n * (4 + 52 + 52) + K * 4, "B")]
         # emission: order, rect, depth in + offset out per Gaussian; one 8 B (tile | index) word per pair
         # out (frames that keep no backward state sort these words without a value array)
-        return [("hbm", bands * n * (4 + 16 + 4 + 4) + K * 8, "B")]
+        return [("hbm", n * (4 + 16 + 4 + 4) + K * 8, "B")]
     if stage == "sort":
         if direct:
             # column and row bits: order, radius, rect, y parts, xy, conic + opacity, rgb in and 40 B out in
@@ -230,10 +227,10 @@ def visited_pairs(torch, nc, tile: int = 16) -> int:
     return int(pad.view(ty, tile, tx, tile).amax(dim=(1, 3)).sum().item())
 
 
-def roofline(stage_ms, n, K, pixels, passes, prec, peaks, evals, bitmap=True, visited=None, bands=1, direct=False):
+def roofline(stage_ms, n, K, pixels, passes, prec, peaks, evals, bitmap=True, visited=None, direct=False):
     out = {}
     for st, ms in stage_ms.items():
-        work = stage_work(st, n, K, pixels, passes, prec, evals, bitmap, visited, bands, direct)
+        work = stage_work(st, n, K, pixels, passes, prec, evals, bitmap, visited, direct)
         if not work:
             out[st] = {"ms": ms, "fused": FUSED[st]}
             continue
@@ -354,7 +351,7 @@ def training_bench(ctx, fs4d, torch, sid, scene, stream, steps=10, warmup=3):
         return {"workload": "one view of the 800x800 / 100k object, dL/dI ~ N(0,1), gradients of every parameter "
                             "group", "steps": steps, "forward_saved_ms": f, "backward_ms": b, "step_ms": f + b,
                 "views_per_s": 1e3 / (f + b), "backward_kernels_ms": per,
-                "note": "the forward keeps the backward's state (full tile lists, written into the frame's own buffers)"}
+                "note": "the forward keeps the backward's state (tile lists cut to each ellipse's box, written into the frame's own buffers)"}
     except Exception as exc:  # the headline line must still be printed
         return {"error": f"{type(exc).__name__}: {exc}"}
 
@@ -508,7 +505,7 @@ def stress_bench(ctx, fs4d, torch, stream, peaks, frames=3):
     precisions) and frames at 1080p and 4K.  Every input is far larger than L2
     (2M Gaussians; 1.3e9 and 5e9 tile pairs per frame), so no flush is needed.
     Frames with more pairs than one pair-sort pass counts render in bands of
-    tile rows (each band projects and depth-sorts the 2M Gaussians again)."""
+    tile rows, which share one projection and one depth order."""
     from paper_2310_08528_gb300 import scenegen as sg
     try:
         scene = sg.make_stress(0)
@@ -565,9 +562,10 @@ def stress_bench(ctx, fs4d, torch, stream, peaks, frames=3):
                 st = ctx.stage_times()
                 ctx.set_stage_timing(False)
                 K, bands = ctx.last_pairs(), ctx.last_bands()
+                direct = ctx.last_binning() == fs4d.BINNING_SORT  # (no lists: of AUTO's frames, these)
                 vis, evals = visited_pairs(torch, nc), int(nc.sum().item())
             r["stages"] = roofline(st, n, K, w * h, _sort_passes(w, h, bands), "bf16", peaks, evals, bitmap=False,
-                                   visited=vis, bands=bands, direct=bands > 1)
+                                   visited=vis, direct=direct)
             r["tile_pairs"], r["tile_pairs_visited"], r["bands"] = K, vis, bands
             res[f"{w}x{h}"] = r
             del image, nc

@@ -75,6 +75,9 @@ typedef enum fs4d_binning {
                               and (tile row, depth rank), ANDed and read in rank order; frames too large
                               for it report FS4D_BINNING_SORT */
 } fs4d_binning;
+/* Frames composited straight from the depth order (too large for lists, or with more pairs than
+ * one band may hold) have neither lists nor sorted pairs: they report FS4D_BINNING_SORT, as they
+ * do when that mode is forced. */
 
 typedef struct fs4d_ctx fs4d_ctx;     /* one device + one stream; not thread-safe */
 typedef struct fs4d_frame fs4d_frame; /* saved forward state of one render, for the backward */

@@ -815,7 +815,6 @@ fs4d_status run_deform(fs4d_ctx* c, Scene* s, fs4d_precision prec, const DeformA
   return run_deform(c, s, prec, a, c->stream, P<uint32_t>(c->status));
 }
 
-// Everything of a frame up to (and including) the key emission.
 // One scene's share of a frame's Gaussian set: its deformed Gaussians and
 // projections sit at [off, off + n) of the work arrays; shift translates the
 // scene in the world (composition, Sec. 5.4: G' = {G'_1, ..., G'_n}).
@@ -942,8 +941,8 @@ fs4d_status frame_depth_order(const Env& e, const FramePart* parts, int n_parts,
   return FS4D_OK;
 }
 
-// Everything of a frame up to (and including) the key emission, over the union of
-// the parts' Gaussians.
+// Everything of a frame up to (and including) its tile lists or the key emission, over
+// the union of the parts' Gaussians.
 // saved: keep what the backward needs (each Gaussian's pair slots).
 // cull: the tile lists may leave out Gaussians that no pixel of the tile blends
 // (same image; list positions, and so last-contributor indices, differ).

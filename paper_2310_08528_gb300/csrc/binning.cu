@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(const uint32_t*
                                                                  uint32_t* __restrict__ num_pairs,
                                                                  uint2* __restrict__ ranges, uint32_t* __restrict__ hist,
                                                                  int passes, uint32_t* __restrict__ order,
-                                                                 long long capacity, uint32_t* __restrict__ status) {
+                                                                 long long capacity) {
   __shared__ uint32_t s_warp[kScanThreads / 32];
   __shared__ uint32_t s_hist[kMaxPasses][256];
   __shared__ uint32_t s_len[33];          // tiles per length class floor(log2(count)) + 1 (0: empty)
@@ -231,10 +231,7 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(const uint32_t*
     total += s_warp[w];
   }
   const bool overflow = capacity < 0 ? sort_overflow : (long long)total > capacity;
-  if (capacity >= 0 && tid == 0) {
-    num_pairs[1] = overflow ? 0u : (uint32_t)total;
-    if (overflow && status) atomicOr(status, kStatusCapacity);
-  }
+  if (capacity >= 0 && tid == 0) num_pairs[1] = overflow ? 0u : (uint32_t)total;
   for (int t = t0; t < t1; ++t) {
     const uint32_t c = tile_count[t];
     if (ranges) ranges[t] = (overflow || c == 0) ? make_uint2(0u, 0u) : make_uint2(run, run + c);
@@ -299,11 +296,10 @@ cudaError_t launch_scan_emit(const EmitArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_tile_scan(const uint32_t* tile_count, int n_tiles, uint32_t* num_pairs, uint2* ranges,
-                             uint32_t* hist, int passes, uint32_t* order, cudaStream_t s, long long capacity,
-                             uint32_t* status) {
+                             uint32_t* hist, int passes, uint32_t* order, cudaStream_t s, long long capacity) {
   if (passes > kMaxPasses || n_tiles < 1) return cudaErrorInvalidValue;
   return launch_pdl(tile_scan_kernel, 1, kScanThreads, 0, s, tile_count, n_tiles, num_pairs, ranges, hist, passes, order,
-                    capacity, status);
+                    capacity);
 }
 
 }  // namespace fs4d

@@ -298,10 +298,9 @@ cudaError_t launch_scan_emit(const EmitArgs& a, cudaStream_t s);
 // if hist != NULL the [passes][256] digit histograms of the pair sort on the tile bits, and
 // if order != NULL a permutation of the tiles, longest lists first (compositing launch order)
 // capacity >= 0: the overflow test is the tiles' total > capacity instead (num_pairs[1] is then
-// written as the total, or 0 on overflow, and status, if non-NULL, gets kStatusCapacity)
+// written as the total, or 0 on overflow)
 cudaError_t launch_tile_scan(const uint32_t* tile_count, int n_tiles, uint32_t* num_pairs, uint2* ranges,
-                             uint32_t* hist, int passes, uint32_t* order, cudaStream_t s, long long capacity = -1,
-                             uint32_t* status = nullptr);
+                             uint32_t* hist, int passes, uint32_t* order, cudaStream_t s, long long capacity = -1);
 // Tile lists from column and row bits (lists.cu), the alternative to emission + pair sort.
 struct ListArgs {
   int n;

@@ -298,12 +298,6 @@ __device__ __forceinline__ void grid_sync(uint32_t* counter, uint32_t target, ui
   __syncthreads();
 }
 
-// Every pass of a sort small enough that all its 1024-key partitions are resident
-// at once (a frame's depth sort: 100k keys, 98 partitions) in one launch: CTA b owns
-// partition b in every pass and a grid barrier separates the passes, so the passes
-// need no further launch and no ticket.  A pass whose digit every key shares moves
-// nothing (the same decision in every CTA: it comes from the global histogram);
-// *a.sel_out records whether the result ended in the alternate buffers.
 // The keys' buckets: every CTA scans the histogram for itself and puts its keys at their
 // buckets' places (bucket start + place in the bucket), one pass where the radix sort
 // takes three and two grid barriers.  False if some bucket holds more than kBucketMost
@@ -358,6 +352,13 @@ __device__ __forceinline__ bool bucket_pass(const BucketArgs& b, const PassArgs&
   return true;
 }
 
+// Every pass of a sort small enough that all its 1024-key partitions are resident
+// at once (a frame's depth sort: 100k keys, 98 partitions) in one launch: CTA b owns
+// partition b in every pass and a grid barrier separates the passes, so the passes
+// need no further launch and no ticket.  A pass whose digit every key shares moves
+// nothing (the same decision in every CTA: it comes from the global histogram);
+// *a.sel_out records whether the result ended in the alternate buffers.
+// With bucket.hist the keys go to their buckets instead (bucket_pass), unless one is too full.
 __global__ void __launch_bounds__(kThreads) onesweep_fused_kernel(PassArgs a, int passes, int first_bit,
                                                                   int key_bits, uint32_t* grid_counter,
                                                                   BucketArgs bucket) {
