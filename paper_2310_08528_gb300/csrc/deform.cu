@@ -176,7 +176,6 @@ __global__ void __launch_bounds__(GROUPS * kThreads, 1) deform_fp32_kernel(const
   float4* sRowX = reinterpret_cast<float4*>(sw + mlp_floats(HL) + (size_t)GROUPS * (XR + kWidth) * kGS) + grp * TG;
   // the weights by cp.async (every 16-byte copy in flight at once), waited for
   // before the first tile's MLP below
-  if (a.mlp_late) pdl_wait();
   for (int i = threadIdx.x; i < a.mg.total / 4; i += GROUPS * kThreads) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem4 + i);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(reinterpret_cast<const float4*>(a.mlp_t) + i)
@@ -369,7 +368,7 @@ cudaError_t launch_tg(const DeformArgs& a, cudaStream_t s) {
   const long long total = (long long)a.n * a.n_t;
   const long long need = (total + TG - 1) / TG;
   const int grid = (int)(need < sms ? need : sms);
-  return launch_pdl(deform_fp32_kernel<H, L, TG, GROUPS, ACT>, grid, GROUPS * kThreads, smem, s, a);
+  return launch_kernel(!a.mlp_late, deform_fp32_kernel<H, L, TG, GROUPS, ACT>, dim3((unsigned)grid), GROUPS * kThreads, smem, s, a);
 }
 
 template <int H, int L>

@@ -107,7 +107,6 @@ __global__ void __launch_bounds__(kThreads, 1) deform_tc_kernel(DeformArgs a) {
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // the weights by cp.async: every 16-byte copy in flight at once
-  if (a.mlp_late) pdl_wait();
   for (int i = tid; i < tg.bytes / 16; i += kThreads) cp_async(sB + 16 * i, a.tc_ops + 16 * i, 1);
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   for (int i = tid; i < kBiasFloats; i += kThreads) sBias[i] = a.tc_bias[i];
@@ -351,7 +350,7 @@ cudaError_t launch_t(const DeformArgs& a, cudaStream_t s) {
   const int sms = device_sm_count();
   const long long tiles = ((long long)a.n * a.n_t + kRows - 1) / kRows;
   const int grid = (int)(tiles < sms ? tiles : sms);
-  return launch_pdl(deform_tc_kernel<H, L>, grid, kThreads, smem, s, a);
+  return launch_kernel(!a.mlp_late, deform_tc_kernel<H, L>, dim3((unsigned)grid), kThreads, smem, s, a);
 }
 
 }  // namespace

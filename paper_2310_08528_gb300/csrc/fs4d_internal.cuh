@@ -40,9 +40,10 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // kernels all are): the render entry points report a frame's count from it.
 extern thread_local unsigned long long g_kernel_launches;
 
+// early: with the attribute (a launch without it starts after everything before it on the stream)
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_2d(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
-                                 Args... args) {
+inline cudaError_t launch_kernel(bool early, void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
+                                 cudaStream_t s, Args... args) {
   ++g_kernel_launches;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -55,8 +56,14 @@ inline cudaError_t launch_pdl_2d(void (*kernel)(KArgs...), dim3 grid, unsigned b
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) return cudaGetLastError();
   cfg.attrs = attr;
-  cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
+  cfg.numAttrs = early && cs == cudaStreamCaptureStatusNone ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_2d(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                                 Args... args) {
+  return launch_kernel(true, kernel, grid, block, smem, s, args...);
 }
 
 template <typename... KArgs, typename... Args>
@@ -155,7 +162,7 @@ struct DeformArgs {
   float* act_a1;
   float* act_hid;
   uint32_t* act_masks;
-  int mlp_late;                 // the MLP's copies are written by the kernel before this one
+  int mlp_late;                 // the MLP's copies, read before the wait, are written by the kernel before this one
   uint4* zero;                  // optional: zero_n16 16-byte words the kernel sets to 0 (a frame's counters
   long long zero_n16;           // and look-back tables, cleared here instead of by a separate memset)
   uint4* fd_tiles;              // BF16 kernel, optional: f_d of each tile of 128 work-order rows as its BF16
@@ -218,7 +225,7 @@ struct ProjectArgs {
   int4* rect;
   unsigned long long* depth_keys;  // optional [n]: float bits of depth, for the depth sort
   uint32_t* depth_vals;            // optional [n]: Gaussian index (index_base + g)
-  int sh_late;                     // the SH rows are written by the kernels before this one
+  int sh_late;                     // the SH rows, read before the wait, are written by the kernels before this one
   uint32_t index_base;             // index of this call's first Gaussian in the frame's set
   uint32_t* depth_hist;            // optional [4][256] (zeroed): byte histograms of the depth keys
   uint32_t* bucket_hist;           // optional [kBuckets] (zeroed): visible Gaussians per depth bucket, and
