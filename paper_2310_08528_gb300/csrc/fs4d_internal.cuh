@@ -225,7 +225,7 @@ struct ProjectArgs {
   int4* rect;
   unsigned long long* depth_keys;  // optional [n]: float bits of depth, for the depth sort
   uint32_t* depth_vals;            // optional [n]: Gaussian index (index_base + g)
-  int sh_late;                     // the SH rows, read before the wait, are written by the kernels before this one
+  int sh_late;                     // the SH rows are written by the kernels before this one: the wait comes first
   uint32_t index_base;             // index of this call's first Gaussian in the frame's set
   uint32_t* depth_hist;            // optional [4][256] (zeroed): byte histograms of the depth keys
   uint32_t* bucket_hist;           // optional [kBuckets] (zeroed): visible Gaussians per depth bucket, and

@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(256) project_kernel(ProjectArgs a) {
   extern __shared__ float4 s_sh[];  // [256][SHQ + 1]
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = g < a.n;
+  if (a.sh_late) pdl_wait();
   if (SHQ > 0) {
     const long long g0 = (long long)blockIdx.x * 256;
     const int words = (int)min(256ll, a.n - g0) * SHQ;
@@ -261,7 +262,7 @@ cudaError_t launch_project_deg(const ProjectArgs& a, unsigned grid, cudaStream_t
     });
     if (e != cudaSuccess) return e;
   }
-  return launch_kernel(!a.sh_late, project_kernel<DEG>, dim3(grid), 256, smem, s, a);
+  return launch_pdl(project_kernel<DEG>, grid, 256, smem, s, a);
 }
 
 cudaError_t launch_project(const ProjectArgs& a, cudaStream_t s) {
